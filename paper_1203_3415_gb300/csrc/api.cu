@@ -10,13 +10,17 @@
 #include "common.cuh"
 #include "context.cuh"
 #include "formula.cuh"
+#include "partial.cuh"
 #include "randomise.cuh"
 
 using namespace acc;
 
 namespace {
 
-constexpr unsigned long long kQueueCap = 1ull << 22;
+#ifndef ACC_QUEUE_CAP
+#define ACC_QUEUE_CAP (1ull << 22)
+#endif
+constexpr unsigned long long kQueueCap = ACC_QUEUE_CAP;
 // ACC_ADJ_AUTO: count-mode probes read hashed tables for sets whose largest
 // graph has at least this many vertices (k = 5; k = 3, 4), where the dense
 // block's probes (n^2/4 bytes, out of L2) get slower than the hashed ones
@@ -57,6 +61,7 @@ struct SharedTable {
     int refs = 0;
     int16_t *lut = nullptr, *lut_sv = nullptr;
     uint32_t *class_code = nullptr;
+    uint32_t *inv = nullptr;  // k = 3, 4: partial_matrix
     int16_t *lut_host = nullptr;
     uint32_t *class_code_host = nullptr;
 };
@@ -72,7 +77,7 @@ int build_table(int k, cudaStream_t s, SharedTable &t) {
     uint32_t *canon = nullptr;
     int *rank = nullptr;
     int16_t *lut = nullptr, *lut_sv = nullptr;
-    uint32_t *cc = nullptr;
+    uint32_t *cc = nullptr, *inv = nullptr;
     int16_t *lut_host = new (std::nothrow) int16_t[ncodes];
     uint32_t *cc_host = new (std::nothrow) uint32_t[ncls];
     int rc = ACC_ERR_NOMEM;
@@ -99,11 +104,21 @@ int build_table(int k, cudaStream_t s, SharedTable &t) {
             goto fail;
         }
     }
+    if (k <= 4) {
+        std::vector<uint32_t> m;
+        partial_matrix(k, lut_host, cc_host, m);
+        if (!ok(cudaMalloc(&inv, m.size() * 4)) ||
+            !ok(cudaMemcpy(inv, m.data(), m.size() * 4, cudaMemcpyHostToDevice))) {
+            rc = inv ? ACC_ERR_CUDA : ACC_ERR_NOMEM;
+            goto fail;
+        }
+    }
     cudaFree(canon);
     cudaFree(rank);
     t.lut = lut;
     t.lut_sv = lut_sv;
     t.class_code = cc;
+    t.inv = inv;
     t.lut_host = lut_host;
     t.class_code_host = cc_host;
     return ACC_OK;
@@ -114,6 +129,7 @@ fail:
     cudaFree(lut);
     cudaFree(lut_sv);
     cudaFree(cc);
+    cudaFree(inv);
     delete[] lut_host;
     delete[] cc_host;
     return rc;
@@ -132,6 +148,7 @@ int ensure_lut(acc_ctx *c, int k, cudaStream_t s) {
     c->lut[k] = t.lut;
     c->lut_sv[k] = t.lut_sv;
     c->class_code_dev[k] = t.class_code;
+    c->inv[k] = t.inv;
     c->lut_host[k] = t.lut_host;
     c->class_code_host[k] = t.class_code_host;
     return ACC_OK;
@@ -147,12 +164,14 @@ void release_luts(acc_ctx *c) {
             cudaFree(t.lut);
             cudaFree(t.lut_sv);
             cudaFree(t.class_code);
+            cudaFree(t.inv);
             delete[] t.lut_host;
             delete[] t.class_code_host;
             t = SharedTable();
         }
         c->lut[k] = c->lut_sv[k] = nullptr;
         c->class_code_dev[k] = nullptr;
+        c->inv[k] = nullptr;
         c->lut_host[k] = nullptr;
         c->class_code_host[k] = nullptr;
     }
@@ -193,6 +212,25 @@ bool uses_hash(const acc_ctx *c, int k, int max_n) {
 #endif
 bool uses_rev(const acc_ctx *c, long long arcs) { return ACC_REV && count_family(c) && arcs >= ACC_REV_MIN_ARCS; }
 
+// The automatic mode takes the k = 3 formula path on graphs of up to
+// kAutoFormulaMaxN vertices (measured faster there than the count mode's
+// scan: 0.028 against 0.034 ms at 1000 vertices, 0.065 against 0.100 at 5000;
+// slower at 20000 with hubs of degree 470, 0.208 against 0.181).
+bool uses_formula(const acc_ctx *c, int k, int max_n) {
+    return c->mode == ACC_MODE_FORMULA || (c->mode == ACC_MODE_AUTO && k == 3 && max_n <= kAutoFormulaMaxN &&
+                                           !sparse_build(c, max_n) && !uses_hash(c, k, max_n));
+}
+
+// The count mode of k = 3, 4 counts by partial patterns (partial.cu) on sets
+// whose vertices are renumbered by degree, from ACC_PARTIAL_MIN_ARCS arcs on
+// (smaller sets are bound by their launches either way and scan their lists).
+#ifndef ACC_PARTIAL_MIN_ARCS
+#define ACC_PARTIAL_MIN_ARCS 8192
+#endif
+bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel) {
+    return count_family(c) && k <= 4 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS && !uses_formula(c, k, max_n);
+}
+
 // Size limit of one graph: the dense block's, or the sparse build's for the
 // count mode (local ids fill 26 bits of the extension-list entries).
 int size_check(const acc_ctx *c, long long n) {
@@ -208,9 +246,18 @@ long long sparse_list_entries(int maxdeg) { return (3LL * maxdeg + 64 + 31) & ~3
 
 // Workspace for a set of NV vertices in blocks of state_words words, with at
 // most `arcs` arcs and graphs of at most max_n vertices.
-int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long arcs, int max_n, int k) {
+int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long arcs, int max_n, int k, int B,
+                     bool relabel) {
     int rc;
     const bool sparse = sparse_build(c, max_n);
+    const bool partial = uses_partial(c, k, max_n, arcs, relabel);
+    if (partial) {
+        if ((rc = grow(&c->pp_nd, &c->pp_nd_cap, (size_t)NV + 1))) return rc;
+        if ((rc = grow(&c->pp_part, &c->pp_part_cap, (size_t)B * num_classes(k)))) return rc;
+        if ((rc = grow(&c->pp_done, &c->pp_done_cap, (size_t)B))) return rc;
+        if (k == 4 && (rc = grow(&c->pp_wedges, &c->pp_wedges_cap, (size_t)NV + 1))) return rc;
+        if (k == 4 && (rc = grow(&c->pp_tri, &c->pp_tri_cap, 3 * (size_t)(2 * arcs) + 1))) return rc;
+    }
     if (uses_hash(c, k, max_n) && (rc = grow(&c->nh, &c->nh_cap, (size_t)kNhWords * (size_t)(2 * arcs) + 4)))
         return rc;
     if (sparse) {
@@ -251,7 +298,7 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
     if ((rc = grow(&c->f5_pre, &c->f5_pre_cap, (size_t)NV + 1))) return rc;
     if ((rc = grow(&c->nbr, &c->nbr_cap, (size_t)(2 * arcs) + 1))) return rc;
     if ((rc = grow(&c->src, &c->src_cap, (size_t)(2 * arcs) + 1))) return rc;
-    if (uses_rev(c, arcs) && (rc = grow(&c->rev, &c->rev_cap, (size_t)(2 * arcs) + 1))) return rc;
+    if ((uses_rev(c, arcs) || (partial && k == 4)) && (rc = grow(&c->rev, &c->rev_cap, (size_t)(2 * arcs) + 1))) return rc;
     if (!sparse && (rc = grow(&c->occ, &c->occ_cap, (size_t)NV * (size_t)occ_words(max_n) + 1))) return rc;
     if (!c->info) {
         if (!ok(cudaMalloc(&c->info, sizeof(GraphInfo)))) return ACC_ERR_NOMEM;
@@ -267,8 +314,8 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
     const int warps = enum_grid_warps(k, c->num_sms);
     if (warps < 0) return warps;
     // the sparse build sizes the overflow lists by the largest degree, once
-    // it is known (run_set)
-    if (!sparse && (rc = grow(&c->scratch, &c->scratch_cap, (size_t)scratch_per_warp(max_n) * (size_t)warps)))
+    // it is known (run_set); partial patterns have no extension lists
+    if (!sparse && !partial && (rc = grow(&c->scratch, &c->scratch_cap, (size_t)scratch_per_warp(max_n) * (size_t)warps)))
         return rc;
     if (!c->maxdeg_host && !ok(cudaMallocHost(&c->maxdeg_host, sizeof(int)))) return ACC_ERR_NOMEM;
     return ACC_OK;
@@ -301,6 +348,19 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     bb.occ_w = occ_words(max_n);
     bb.info = c->info;
     bb.k = k;
+    bool partial = gs.NV > 0 && uses_partial(c, k, max_n, gs.M, relabel);
+    if (partial) {
+        bb.zero[0] = reinterpret_cast<int *>(c->pp_nd);
+        bb.nzero[0] = 2 * gs.NV;
+        bb.zero[1] = reinterpret_cast<int *>(c->pp_part);
+        bb.nzero[1] = 2ll * gs.B * num_classes(k);
+        bb.zero[2] = c->pp_done;
+        bb.nzero[2] = gs.B;
+        if (k == 4) {
+            bb.zero[3] = reinterpret_cast<int *>(c->pp_wedges);
+            bb.nzero[3] = gs.NV;
+        }
+    }
     int rc;
     if (sparse) {
         const SparseBufs sb = {c->sp_raw, c->sp_merged, c->sp_roff, c->sp_big};
@@ -318,27 +378,22 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         if (!ok(cudaMemcpyAsync(c->maxdeg_host, &c->info->maxdeg, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
             !ok(cudaStreamSynchronize(s)))
             return ACC_ERR_CUDA;
+        if (*c->maxdeg_host > kNdMax) partial = false;  // its packed degree counts hold kNdMax
         spw = 2 * sparse_list_entries(*c->maxdeg_host) + 2 * kPartBRows;
         const int warps = enum_grid_warps(k, c->num_sms);
         if (warps < 0) return warps;
-        if ((rc = grow(&c->scratch, &c->scratch_cap, (size_t)spw * (size_t)warps))) return rc;
+        if (!partial && (rc = grow(&c->scratch, &c->scratch_cap, (size_t)spw * (size_t)warps))) return rc;
     }
     // count mode on a large set: probes read hashed tables, built from the
     // sorted neighbour lists
     const bool hash = gs.NV > 0 && uses_hash(c, k, max_n);
-    // the automatic mode takes the k = 3 formula path on graphs of up to
-    // kAutoFormulaMaxN vertices (measured faster there: 0.028 against 0.034 ms
-    // at 1000 vertices, 0.065 against 0.100 at 5000; slower at 20000 with
-    // hubs of degree 470, 0.208 against 0.181)
     if (hash) {
         rc = launch_nh_build(c->nptr, c->deg, c->nbr, c->src, c->info, 2 * gs.M, c->nh, c->num_sms, s);
         if (rc < 0) return rc;
         launches += rc;
     }
-    const bool formula = c->mode == ACC_MODE_FORMULA ||
-                         (c->mode == ACC_MODE_AUTO && k == 3 && max_n <= kAutoFormulaMaxN && !sparse &&
-                          !uses_hash(c, k, max_n));
-    const bool rev = gs.NV > 0 && !formula && uses_rev(c, gs.M);
+    const bool formula = uses_formula(c, k, max_n);
+    const bool rev = gs.NV > 0 && !formula && !partial && uses_rev(c, gs.M);
     if (rev) {
         rc = launch_rev_build(gs, c->nptr, c->deg, c->nbr, c->src, c->info, 2 * gs.M, c->rev, c->num_sms, s);
         if (rc < 0) return rc;
@@ -368,7 +423,36 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     a.counts = reinterpret_cast<unsigned long long *>(counts);
     a.status = status;
     const bool any = gs.NV > 0;
-    if (any && formula) {
+    if (partial) {
+        PartialArgs p;
+        p.state = c->state;
+        p.state_w = c->state;
+        p.deg = c->deg;
+        p.lo = c->lo;
+        p.nptr = c->nptr;
+        p.nbr = c->nbr;
+        p.src = c->src;
+        p.nh = hash ? c->nh : nullptr;
+        p.lut = c->lut_sv[k];
+        p.inv = c->inv[k];
+        p.gs = gs;
+        p.info = c->info;
+        p.queue = c->queue;
+        p.queue_cap = c->queue_cap;
+        p.rev = c->rev;
+        p.nd = c->pp_nd;
+        p.wedges = c->pp_wedges;
+        p.tri = c->pp_tri;
+        p.part = c->pp_part;
+        p.done = c->pp_done;
+        p.counts = reinterpret_cast<unsigned long long *>(counts);
+        p.status = status;
+        p.occ = sparse ? nullptr : c->occ;
+        p.occ_w = occ_words(max_n);
+        rc = launch_partial(k, p, 2 * gs.M, c->num_sms, s, c->grid_num, c->grid_den);
+        if (rc < 0) return rc;
+        launches += rc;
+    } else if (any && formula) {
         if (k == 3)
             rc = launch_formula3(gs, c->state, c->nptr, c->deg, c->lo, c->nbr, c->lut[3],
                                  reinterpret_cast<unsigned long long *>(counts), status, c->num_sms, s);
@@ -386,16 +470,18 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         launches += rc;
     }
     if (c->timing && !ok(cudaEventRecord(c->ev[3], s))) return ACC_ERR_CUDA;
-    if (any && !formula) {
+    if (any && !formula && !partial) {
         rc = launch_enumerate(k, a, c->num_sms, 2, s, c->grid_num, c->grid_den);
         if (rc < 0) return rc;
         launches += rc;
     }
     if (c->timing && !ok(cudaEventRecord(c->ev[2], s))) return ACC_ERR_CUDA;
     if (!sparse) {
-        rc = launch_clear_graph(gs, c->state, c->occ, occ_words(max_n), c->num_sms, s);
-        if (rc < 0) return rc;
-        launches += rc;
+        if (!partial) {  // (its last kernel clears the block)
+            rc = launch_clear_graph(gs, c->state, c->occ, occ_words(max_n), c->num_sms, s);
+            if (rc < 0) return rc;
+            launches += rc;
+        }
         c->state_clean = true;
     }
     c->last_launches = launches;
@@ -424,7 +510,8 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     int rc = ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
-    if ((rc = ensure_workspace(c, n, sparse_build(c, n) ? 0 : (long long)n * pitch, m, n, k))) return rc;
+    if ((rc = ensure_workspace(c, n, sparse_build(c, n) ? 0 : (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN)))
+        return rc;
     GSet gs = {};
     gs.one.rowptr = reinterpret_cast<const long long *>(rowptr);
     gs.one.col = col;
@@ -459,9 +546,10 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
         key.grid_num = c->grid_num;
         key.grid_den = c->grid_den;
         key.adjacency = c->adjacency;
-        const void *ws[21] = {c->state, c->deg, c->lo, c->label, c->deg_in, c->nptr, c->tiles, c->nbr, c->occ,
+        const void *ws[25] = {c->state, c->deg, c->lo, c->label, c->deg_in, c->nptr, c->tiles, c->nbr, c->occ,
                               c->info, c->queue, c->scratch, c->lut[k], c->lut_sv[k], c->class_code_dev[k],
-                              c->f5_pre, c->status_dev, c->src, c->nh, c->rev, nullptr};
+                              c->f5_pre, c->status_dev, c->src, c->nh, c->rev, c->pp_nd, c->pp_tri, c->pp_part,
+                              c->pp_wedges, c->pp_done};
         memcpy(key.ws, ws, sizeof(ws));
         bool have = c->cg_exec && memcmp(&key, &c->cg_key, sizeof(key)) == 0;
         // capture only when a count repeats: a one-off count runs one by one
@@ -514,7 +602,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
 int batch_workspace(acc_ctx *c) {
     if (size_check(c, c->batch_max_n)) return ACC_ERR_TOO_LARGE;
     return ensure_workspace(c, c->batch_set.NV, sparse_build(c, c->batch_max_n) ? 0 : c->batch_words, c->batch_arcs,
-                            c->batch_max_n, c->batch_k);
+                            c->batch_max_n, c->batch_k, c->batch_set.B, true);
 }
 
 }  // namespace
@@ -530,11 +618,15 @@ long long ctx_footprint(const acc_ctx *c, long long n, long long m, int k) {
     // offsets instead of the dense block and its bitmap; its overflow lists
     // are bounded by the largest degree, itself at most 2m and n
     const long long list_n = sparse ? (2 * m < n ? 2 * m : n) : n;
+    const long long lists = (sparse ? 2 * sparse_list_entries((int)list_n) + 2 * kPartBRows : scratch_per_warp((int)n)) *
+                            (warps > 0 ? warps : 0) * 4;
+    // k = 3, 4 by partial patterns hold counters per entry instead of the
+    // scan's lists; a slot is sized for either, so that admission does not
+    // depend on the path
+    const long long counters = 12 * (n + 1) + (k == 4 ? (24 + 8) * (2 * m + 1) : 0);
     const long long bytes = (sparse ? 16 * (m + 1) + 8 * (n + 1) : n * pitch * 4 + 4 * n * occ_words((int)n)) +
                             5 * 4 * (n + 1) + 8 * (n + 1) + (uses_rev(c, m) ? 16 : 8) * (2 * m + 1) + hash_bytes +
-                            (long long)kQueueCap * 16 +
-                            (sparse ? 2 * sparse_list_entries((int)list_n) + 2 * kPartBRows : scratch_per_warp((int)n)) *
-                                (warps > 0 ? warps : 0) * 4;
+                            (long long)kQueueCap * 16 + (lists > counters ? lists : counters);
     return bytes + bytes / 4;
 }
 
@@ -544,7 +636,7 @@ int ctx_reserve(acc_ctx *c, long long n, long long m, int k) {
         const int rc = ensure_lut(c, kk, c->own);
         if (rc) return rc;
     }
-    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k);
+    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, n >= kRelabelMinN);
 }
 
 }  // namespace acc
@@ -605,6 +697,11 @@ void acc_ctx_destroy(acc_ctx *c) {
     cudaFree(c->src);
     cudaFree(c->rev);
     cudaFree(c->nh);
+    cudaFree(c->pp_nd);
+    cudaFree(c->pp_tri);
+    cudaFree(c->pp_part);
+    cudaFree(c->pp_wedges);
+    cudaFree(c->pp_done);
     cudaFree(c->sp_raw);
     cudaFree(c->sp_merged);
     cudaFree(c->sp_roff);
@@ -711,7 +808,7 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     if (!ok(cudaStreamSynchronize(s))) return ACC_ERR_CUDA;
     int rc = ensure_lut(c, k, s);
     if (rc) return rc;
-    if ((rc = ensure_workspace(c, NV, sparse_build(c, max_n) ? 0 : words, arcs, max_n, k))) return rc;
+    if ((rc = ensure_workspace(c, NV, sparse_build(c, max_n) ? 0 : words, arcs, max_n, k, B, true))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;
     if ((rc = grow(&c->gid, &c->gid_cap, (size_t)NV + 1))) return rc;
     if (B > 0 && !ok(cudaMemcpy(c->meta_dev, metas.data(), sizeof(GMeta) * (size_t)B, cudaMemcpyHostToDevice)))

@@ -137,6 +137,28 @@ inline int occ_words(int max_n) {
     return (int)((chunks + 31) / 32 > 0 ? (chunks + 31) / 32 : 1);
 }
 
+// Zero the 32-word chunks of the set's pair-state rows that the occupancy
+// bitmap marks (every word the ingest set lies in one): warp `warp` of
+// `nwarps` takes every nwarps-th row, lane j the j-th marked chunk of a
+// bitmap word.  The buffer is all zero afterwards.
+__device__ __forceinline__ void clear_chunks(const GSet &gs, uint32_t *state, const uint32_t *__restrict__ occ, int occ_w,
+                                             long long warp, long long nwarps, int lane) {
+    for (long long v = warp; v < gs.NV; v += nwarps) {
+        const GMeta mt = gs.meta(gs.graph_of((int)v));
+        const int quads = (((mt.n + 15) >> 4) + 3) >> 2;
+        uint4 *row4 = reinterpret_cast<uint4 *>(state + mt.soff + (long long)(v - mt.voff) * mt.pitch);
+        for (int mw = 0; mw < occ_w; mw++) {
+            const uint32_t mask = occ[v * occ_w + mw];
+            if (lane < __popc(mask)) {
+                const int q0 = (mw * 32 + (int)__fns(mask, 0, lane + 1)) * 8;
+#pragma unroll
+                for (int g = 0; g < 8; g++)
+                    if (q0 + g < quads) row4[q0 + g] = make_uint4(0, 0, 0, 0);
+            }
+        }
+    }
+}
+
 // Bit of the adjacency code for the arc from tuple slot i to slot j.
 __host__ __device__ constexpr int code_bit(int k, int i, int j) {
     return i * (k - 1) + (j - (j > i ? 1 : 0));
@@ -199,6 +221,13 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+// Orders this thread's writes before its later ones for the whole device.
+__device__ __forceinline__ void fence_device() {
+#ifdef __CUDA_ARCH__
+    __threadfence();
+#endif
+}
+
 // First-error-wins status update.
 __device__ inline void set_status(int *status, int err) {
     if (status) atomicCAS(status, 0, err);
@@ -229,6 +258,8 @@ struct BuildBufs {
     uint32_t *occ;           // NV * occ_words(max_n)
     int occ_w;               // occ_words(max_n)
     GraphInfo *info;
+    int *zero[4] = {};       // further arrays to clear with the counts (NULL: none) ...
+    long long nzero[4] = {}; // ... and their lengths
     int k = 0;               // 3..5: refuse (ACC_ERR_OVERFLOW) a set whose count bound
                              // exceeds kCountLimit; 0: no check
 };

@@ -22,6 +22,7 @@ struct acc_ctx {
     int16_t *lut[6] = {};
     int16_t *lut_sv[6] = {};
     uint32_t *class_code_dev[6] = {};
+    uint32_t *inv[6] = {};  // k = 3, 4: partial counts to induced ones (partial.cuh)
     int16_t *lut_host[6] = {};
     uint32_t *class_code_host[6] = {};
 
@@ -60,6 +61,13 @@ struct acc_ctx {
     unsigned long long queue_cap = 0;
     uint32_t *scratch = nullptr;
     size_t scratch_cap = 0;
+    // partial patterns (partial.cu)
+    unsigned long long *pp_nd = nullptr, *pp_tri = nullptr, *pp_part = nullptr;
+    size_t pp_nd_cap = 0, pp_tri_cap = 0, pp_part_cap = 0;
+    uint32_t *pp_wedges = nullptr;
+    size_t pp_wedges_cap = 0;
+    int *pp_done = nullptr;
+    size_t pp_done_cap = 0;
     int mode = 0;             // ACC_MODE_COUNT, _ENUMERATE, _FORMULA or _AUTO
     long long sched_light = 0;   // enumeration schedule (0: the kernels' default)
     long long sched_target = 0;
@@ -106,7 +114,7 @@ struct acc_ctx {
         const void *rowptr, *col, *counts, *status;
         long long m, light, target;
         int n, k, mode, grid_num, grid_den, adjacency;
-        const void *ws[21];
+        const void *ws[25];
     } cg_key = {}, cg_seen = {};  // the captured graph's key; the last key counted one by one
     int cg_launches = 0;
     long long cg_units = 0;

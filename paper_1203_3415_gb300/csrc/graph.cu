@@ -49,9 +49,10 @@ __device__ __forceinline__ int warp_excl_scan(int x, int lane, int *total) {
     return incl - x;
 }
 
+constexpr int kRanges = 8;
 struct IntRanges {
-    int *p[4];
-    long long n[4];
+    int *p[kRanges];
+    long long n[kRanges];
 };
 
 __global__ void k_zero(uint4 *p, size_t n16, unsigned char *tail, size_t ntail, int *status,
@@ -63,7 +64,7 @@ __global__ void k_zero(uint4 *p, size_t n16, unsigned char *tail, size_t ntail, 
     if (i < ntail) tail[i] = 0;
     for (size_t j = i; j < (size_t)ncounts; j += stride) counts[j] = 0;
 #pragma unroll
-    for (int r = 0; r < 4; r++)
+    for (int r = 0; r < kRanges; r++)
         for (size_t j = i; j < (size_t)ints.n[r]; j += stride) ints.p[r][j] = 0;
     if (i == 0 && status) *status = 0;
 }
@@ -172,28 +173,11 @@ __global__ void k_ingest(GSet gs, uint32_t *state, const int *__restrict__ label
     });
 }
 
-// Warp per global row: zero the 32-word chunks of the row that the occupancy
-// bitmap marks (every word the ingest set lies in one), lane j taking the
-// j-th marked chunk of a bitmap word.  The buffer is all zero afterwards.
+// The marked chunks of the set's pair-state rows back to zero (clear_chunks).
 __global__ void k_clear_chunks(GSet gs, uint32_t *state, const uint32_t *__restrict__ occ, int occ_w) {
     grid_dep_wait();
-    const int lane = threadIdx.x & 31;
-    const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
-    const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
-    for (long long v = warp; v < gs.NV; v += nwarps) {
-        const GMeta mt = gs.meta(gs.graph_of((int)v));
-        const int quads = (((mt.n + 15) >> 4) + 3) >> 2;
-        uint4 *row4 = reinterpret_cast<uint4 *>(state + mt.soff + (long long)(v - mt.voff) * mt.pitch);
-        for (int mw = 0; mw < occ_w; mw++) {
-            const uint32_t mask = occ[v * occ_w + mw];
-            if (lane < __popc(mask)) {
-                const int q0 = (mw * 32 + (int)__fns(mask, 0, lane + 1)) * 8;
-#pragma unroll
-                for (int g = 0; g < 8; g++)
-                    if (q0 + g < quads) row4[q0 + g] = make_uint4(0, 0, 0, 0);
-            }
-        }
-    }
+    clear_chunks(gs, state, occ, occ_w, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
+                 ((long long)gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
 // Per-graph histogram dhist[voff + key] of the renumbering keys (clamped to
@@ -926,11 +910,23 @@ int grid_for(long long work_items, int per_block, int num_sms) {
     return (int)b;
 }
 
+// Append the caller's arrays to a build's cleared ranges; the longest.
+long long more_ranges(const BuildBufs &bb, IntRanges &r) {
+    long long longest = 0;
+    for (int i = 0; i < 4; i++)
+        if (bb.zero[i]) {
+            r.p[4 + i] = bb.zero[i];
+            r.n[4 + i] = bb.nzero[i];
+            longest = max(longest, bb.nzero[i]);
+        }
+    return longest;
+}
+
 }  // namespace
 
 int launch_zero(void *p, size_t bytes, int num_sms, cudaStream_t s, int *status, unsigned long long *counts,
                 long long ncounts, int *ints, long long nints) {
-    IntRanges r = {{ints, nullptr, nullptr, nullptr}, {ints ? nints : 0, 0, 0, 0}};
+    IntRanges r = {{ints}, {ints ? nints : 0}};
     const size_t n16 = bytes / 16, ntail = bytes % 16;
     const int grid = grid_for((long long)(n16 > 0 ? n16 : 1), 256 * 4, num_sms);
     launch_pdl(k_zero, grid, 256, 0, s, reinterpret_cast<uint4 *>(p), n16,
@@ -967,8 +963,9 @@ int launch_build_graph(const GSet &gs, const BuildBufs &bb, int max_n, int *stat
         const long long nocc = NV * bb.occ_w;
         IntRanges r = {{bb.deg, bb.lo, bb.deg_in, reinterpret_cast<int *>(bb.occ)},
                        {NV, NV, relabel ? NV : 0, nocc}};
+        const long long extra = more_ranges(bb, r);
         const size_t n16 = bytes / 16, ntail = bytes % 16;
-        const long long items = (long long)max((size_t)1, max(n16, (size_t)max(max(NV, ncounts), nocc)));
+        const long long items = (long long)max((size_t)1, max(n16, (size_t)max(max(max(NV, ncounts), nocc), extra)));
         launch_pdl(k_zero, grid_for(items, 256 * 4, num_sms), 256, 0, s, reinterpret_cast<uint4 *>(bb.state), n16,
                                                                  reinterpret_cast<unsigned char *>(bb.state) + n16 * 16,
                                                                  ntail, status, counts, ncounts, r);
@@ -1047,7 +1044,7 @@ int launch_build_graph_sparse(const GSet &gs, const BuildBufs &bb, const SparseB
     int *cnt = bb.lo, *cur = bb.deg;  // raw entries per row, then the final neighbours below each vertex
     {
         IntRanges r = {{bb.deg, bb.lo, bb.deg_in, nullptr}, {NV, NV, relabel ? NV : 0, 0}};
-        const long long items = max(NV, ncounts) > 0 ? max(NV, ncounts) : 1;
+        const long long items = max(max(max(NV, ncounts), more_ranges(bb, r)), 1ll);
         launch_pdl(k_zero, grid_for(items, 256 * 4, num_sms), 256, 0, s, nullptr, 0, nullptr, 0, status, counts, ncounts, r);
         if (!launch_ok()) return ACC_ERR_CUDA;
         launches++;

@@ -1,0 +1,1126 @@
+// Counting by partial patterns (k = 3, 4): the count mode of sets of at least
+// kPartialMinArcs arcs whose vertices are renumbered by descending degree.
+//
+// A partial pattern fixes the pair states of some pairs of a k-set (its
+// edges, which connect the set) and leaves the other pairs open.  With P(c)
+// the number of k-sets in which class c occurs as a partial pattern (each
+// occurrence counted) and I(c) the induced count the library reports, a set
+// of class c' contains c once for every subset of its G* edges whose pattern
+// is c, so by inclusion and exclusion over the edges left out
+//   I(c) = sum over c' and edge subsets S of c' with class(S) = c of
+//          (-1)^(edges of c' - |S|) P(c').
+// The partial counts need no walk over the k-sets, as the paper's set-size
+// formulas do not (Table starb, Table ept): a path or a star is a product of
+// typed degrees, a triangle with a pendant arc one of a typed triangle count
+// and a degree, and what has to be visited is only
+//   wedges v - u - w with v the smallest id (k = 4, for the 4-cycles: the
+//   wedges of one v that end in the same w, by their two states),
+//   triangles, and for the 4-cliques the common neighbours of a triangle.
+// In degree order those are few: on 20000 vertices and 100000 arcs (Chung-Lu,
+// degrees up to 500) 1.35e6 wedges and 1.5e4 triangles, where the scan of
+// the extension lists (enum.cu) reads 8.6e7 entries.
+//
+// Every sum is exact modulo 2^64, and the reported counts are below 2^62.
+#include <type_traits>
+
+#include "common.cuh"
+#include "partial.cuh"
+
+namespace acc {
+
+namespace {
+
+constexpr int kPWarps = 4;           // warps per block
+constexpr int kPThreads = kPWarps * kWarp;
+// Wedge tables, 16 bytes a slot: one a warp for the roots with few wedges, one
+// a block for the others.
+constexpr int kSlots = 192;
+constexpr int kFill = 144;           // most keys a warp's table takes
+constexpr int kBlockSlots = 1024;
+constexpr int kBlockFill = kBlockSlots * 2 / 3;
+constexpr int kWideSlots = kBlockSlots / 2;  // 28-byte slots: key, three words of 21-bit counts
+constexpr int kWideFill = kWideSlots * 2 / 3;
+constexpr int kFieldMax = 1023;      // largest count of a 16-byte slot's fields
+constexpr int kRingP = 64;           // rows staged for the flat scan
+constexpr int kRingArrays = 5;       // (k = 4: 4, the root is packed into the entry)
+constexpr int kRoots = 16;           // roots that share a table pass
+constexpr int kHits = 96;            // triangles held before they are counted, two words each
+constexpr int kFThreads = 256;       // threads per block of the finish
+
+__device__ __forceinline__ uint32_t swap_state(uint32_t s) { return ((s & 1u) << 1) | (s >> 1); }
+
+// One graph's arrays by local vertex (neighbour-list positions are global).
+struct PView {
+    const uint32_t *state;
+    long long pitch;
+    const long long *nptr;
+    const int *deg, *lo;
+    const unsigned long long *nd;
+    const uint32_t *nh;
+    int n;
+};
+
+__device__ __forceinline__ PView pview(const PartialArgs &a, const GMeta &mt) {
+    return PView{a.state + mt.soff, mt.pitch,        a.nptr + mt.voff, a.deg + mt.voff,
+                 a.lo + mt.voff,    a.nd + mt.voff, a.nh,             mt.n};
+}
+
+// state(x, y): the dense block, or x's hashed table (enum.cu, nh.cu).
+template <bool HASH>
+__device__ __forceinline__ uint32_t pstate(const PView &g, uint32_t x, uint32_t y) {
+    if constexpr (HASH) {
+        const uint32_t lg = nh_lg(g.deg[x]), m = (1u << lg) - 1u;
+        const uint4 *tab = reinterpret_cast<const uint4 *>(g.nh + (long long)kNhWords * g.nptr[x]);
+        uint32_t k = nh_bucket(y, lg);
+        for (uint32_t tries = 0; tries <= m; tries++, k = (k + 1u) & m) {
+            const uint4 q = __ldg(tab + k);
+            if ((q.x >> 2) == y) return q.x & 3u;
+            if ((q.y >> 2) == y) return q.y & 3u;
+            if ((q.z >> 2) == y) return q.z & 3u;
+            if ((q.w >> 2) == y) return q.w & 3u;
+            if (!q.w) return 0u;
+        }
+        return 0u;
+    } else {
+        return (__ldg(g.state + (long long)x * g.pitch + (y >> 4)) >> ((y & 15u) << 1)) & 3u;
+    }
+}
+
+// First index of the sorted entries e[0..n) (u << 2 | state) with u >= id.
+__device__ __forceinline__ int lower_id(const uint32_t *__restrict__ e, int n, uint32_t id) {
+    const uint32_t key = id << 2;
+    int lo = 0, hi = n;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (__ldg(e + mid) < key) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+__device__ __forceinline__ int warp_excl(int x, int lane, int *total) {
+    int incl = x;
+#pragma unroll
+    for (int d = 1; d < kWarp; d <<= 1) {
+        const int y = __shfl_up_sync(kFull, incl, d);
+        if (lane >= d) incl += y;
+    }
+    *total = __shfl_sync(kFull, incl, kWarp - 1);
+    return incl - x;
+}
+
+// 64-bit histogram bin in shared memory as two words (the hardware adds 32
+// bits natively): the add that carries out of the low word raises the high.
+__device__ __forceinline__ void hist_add(uint32_t *h, int bin, unsigned long long d) {
+    const uint32_t lo = (uint32_t)d;
+    uint32_t hi = (uint32_t)(d >> 32);
+    if (lo) {
+        const uint32_t old = atomicAdd(&h[2 * bin], lo);
+        if (old > ~lo) hi++;
+    }
+    if (hi) atomicAdd(&h[2 * bin + 1], hi);
+}
+
+// ---------------------------------------------------------------------------
+// Preparation: typed degrees, and for k = 4 the reverse positions of the upper
+// entries (v -> u with u above v: the part of N*(u) above v, as k_rev gives
+// it for every entry), the wedges of each v, and cleared triangle counters.
+// Thread per neighbour entry; bound by the dependent loads of its search.
+// ---------------------------------------------------------------------------
+template <int K>
+__global__ void k_partial_prep(PartialArgs a) {
+    grid_dep_wait();
+    const long long nnz = a.info->nnz;
+    const int lane = threadIdx.x & 31;
+    for (long long p0 = blockIdx.x * (long long)blockDim.x + threadIdx.x - lane; p0 < nnz;
+         p0 += (long long)gridDim.x * blockDim.x) {
+        const long long pos = p0 + lane;
+        const bool ok = pos < nnz;
+        const uint32_t r = ok ? a.src[pos] : 0xFFFFFFFFu, v = r & 0x7FFFFFFFu;
+        const uint32_t e = ok ? a.nbr[pos] : 0u;
+        // a row's entries sit on consecutive lanes: one add per row and warp
+        // (an add per entry took 25 us at 1.9e5 entries: a hub row's adds meet
+        // in one word)
+        const unsigned same = __match_any_sync(kFull, (int)v);
+        const bool leader = ok && lane == __ffs(same) - 1;
+        const unsigned m1 = __ballot_sync(kFull, (e & 3u) == 1u), m2 = __ballot_sync(kFull, (e & 3u) == 2u),
+                       m3 = __ballot_sync(kFull, (e & 3u) == 3u);
+        if (leader)
+            atomicAdd(&a.nd[v], (unsigned long long)__popc(same & m1) |
+                                    ((unsigned long long)__popc(same & m2) << kNdBits) |
+                                    ((unsigned long long)__popc(same & m3) << (2 * kNdBits)));
+        if constexpr (K == 4) {
+            uint2 rv = make_uint2(0u, 0u);
+            if (ok && !(r >> 31)) {
+                const int voff = a.gs.meta(a.gs.graph_of((int)v)).voff;
+                const uint32_t u = (uint32_t)voff + (e >> 2);
+                const long long base = a.nptr[u];
+                // v is among the neighbours of u below u
+                const int i = lower_id(a.nbr + base, a.lo[u], v - (uint32_t)voff);
+                rv = make_uint2((uint32_t)(base + i + 1), (uint32_t)(a.deg[u] - i - 1));
+#pragma unroll
+                for (int j = 0; j < 3; j++) a.tri[3 * pos + j] = 0ull;
+            }
+            if (ok) a.rev[pos] = rv;
+            uint32_t incl = rv.y;
+#pragma unroll
+            for (int d = 1; d < kWarp; d <<= 1) {
+                const uint32_t y = __shfl_up_sync(kFull, incl, d);
+                if (lane >= d) incl += y;
+            }
+            const int last = lane + __popc(same >> lane) - 1;  // (the row's last lane, seen from its first)
+            const uint32_t sum = __shfl_sync(kFull, incl, last) - incl + rv.y;
+            if (leader && sum) atomicAdd(&a.wedges[v], sum);
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Wedges and triangles
+// ---------------------------------------------------------------------------
+
+// A warp's working storage and the graph it counts.
+template <int K, bool HASH>
+struct Walker {
+    const PartialArgs *a;
+    PView g;
+    uint32_t *hist;   // this warp's histogram of partial counts (two words a class)
+    uint4 *tab;       // k = 4: (key, three words of three 10-bit counts)
+    uint32_t slots;   // the table's slots
+    uint32_t *ring;   // flat start, entry offset, row position, row entry[, row vertex]
+    uint32_t *hq;     // k = 4: triangles held (positions of v -> u and u -> w)
+    int held;
+    int gcur;
+    unsigned long long scanned;
+    int lane;
+
+    __device__ __forceinline__ int cls(uint32_t code) const { return (int)__ldg(a->lut + code); }
+    __device__ __forceinline__ void add(uint32_t code, unsigned long long d) {
+        const int c = cls(code);
+        if (c < 0) set_status(a->status, ACC_ERR_INTERNAL);
+        else hist_add(hist, c, d);
+    }
+
+    // the histogram into graph gcur's partial counts (whole warp)
+    __device__ __forceinline__ void drain() {
+        constexpr int N = num_classes(K);
+        if (K == 4 && held) triangles(held);
+        held = 0;
+        __syncwarp();
+        if (gcur >= 0)
+            for (int c = lane; c < N; c += kWarp) {
+                const unsigned long long v =
+                    (unsigned long long)hist[2 * c] | ((unsigned long long)hist[2 * c + 1] << 32);
+                if (v) {
+                    hist[2 * c] = hist[2 * c + 1] = 0u;
+                    atomicAdd(&a->part[(size_t)gcur * N + c], v);
+                }
+            }
+        __syncwarp();
+    }
+
+    __device__ __forceinline__ void switch_graph(int gi) {
+        if (gi == gcur) return;
+        drain();
+        gcur = gi;
+        g = pview(*a, a->gs.meta(gi));
+    }
+
+    // k = 4: the last n <= 32 triangles held (v < u < w), a lane each.  Each
+    // edge's typed counter of common neighbours takes the third vertex (edge
+    // b < c, common neighbour x: word state(b, x), field state(c, x)), and the
+    // 4-cliques v < u < w < x are found among the neighbours of w above w: the
+    // triangles' lists as one flat sequence, kAhead entries a lane in flight
+    // (phase 2 of 20000 vertices, 1.5e4 triangles: 109 us; 190 us with a lane
+    // walking its own triangle's list, which waits for one entry at a time).
+    __device__ __forceinline__ void triangles(int n) {
+        constexpr int kAhead = 4;
+        __syncwarp();
+        uint32_t v = 0, u = 0, code = 0, off = 0;
+        int len = 0;
+        if (lane < n) {
+            const uint32_t pvu = hq[2 * (held - n + lane)], puw = hq[2 * (held - n + lane) + 1];
+            const uint32_t e1 = __ldg(a->nbr + pvu), e2 = __ldg(a->nbr + puw), w = e2 >> 2;
+            v = (__ldg(a->src + pvu) & 0x7FFFFFFFu) - (uint32_t)(g.deg - a->deg);
+            u = e1 >> 2;
+            const uint32_t svu = e1 & 3u, suw = e2 & 3u, svw = pstate<HASH>(g, v, w);
+            const long long vb = g.nptr[v];
+            const uint32_t pvw = (uint32_t)(vb + lower_id(a->nbr + vb, g.deg[v], w));
+            atomicAdd(&a->tri[3ll * pvu + svw - 1u], 1ull << (kNdBits * (suw - 1u)));
+            atomicAdd(&a->tri[3ll * pvw + svu - 1u], 1ull << (kNdBits * (swap_state(suw) - 1u)));
+            atomicAdd(&a->tri[3ll * puw + swap_state(svu) - 1u], 1ull << (kNdBits * (swap_state(svw) - 1u)));
+            code = (svu << 10) | ((svw | (suw << 2)) << 6);
+            const int l = g.lo[w];
+            off = (uint32_t)(g.nptr[w] + l);
+            len = g.deg[w] - l;
+        }
+        int tot;
+        const int pre = warp_excl(len, lane, &tot);
+        off -= (uint32_t)pre;
+        for (int t0 = 0; t0 < tot; t0 += kWarp * kAhead) {
+            uint32_t x[kAhead], hv[kAhead], hu[kAhead], hc[kAhead], sv[kAhead];
+#pragma unroll
+            for (int i = 0; i < kAhead; i++) {
+                const int t = t0 + i * kWarp + lane;
+                int r = 0;  // the last triangle whose list starts at or before t
+#pragma unroll
+                for (int d = 16; d; d >>= 1)
+                    if (__shfl_sync(kFull, pre, r + d) <= t) r += d;
+                hv[i] = __shfl_sync(kFull, v, r);
+                hu[i] = __shfl_sync(kFull, u, r);
+                hc[i] = __shfl_sync(kFull, code, r);
+                const uint32_t o = __shfl_sync(kFull, off, r);
+                x[i] = t < tot ? __ldg(a->nbr + (o + (uint32_t)t)) : 0u;
+            }
+#pragma unroll
+            for (int i = 0; i < kAhead; i++) sv[i] = x[i] ? pstate<HASH>(g, hv[i], x[i] >> 2) : 0u;
+#pragma unroll
+            for (int i = 0; i < kAhead; i++) {
+                if (!sv[i]) continue;
+                const uint32_t su = pstate<HASH>(g, hu[i], x[i] >> 2);
+                if (su) add(hc[i] | sv[i] | (su << 2) | ((x[i] & 3u) << 4), 1ull);
+            }
+        }
+        __syncwarp();
+    }
+
+    // One wedge end into the table: its key, the wedge's type (s1, s2).
+    template <bool WIDE>
+    __device__ __forceinline__ void put(uint32_t key, uint32_t s1, uint32_t s2) {
+        constexpr int S = WIDE ? 1 : 4;  // words from one key to the next
+        uint32_t *t = reinterpret_cast<uint32_t *>(tab);
+        const uint32_t h = key * 0x9E3779B1u;
+        uint32_t i = (uint32_t)(((unsigned long long)h * slots) >> 32);
+        // (slots is 2^x or 3 2^x: 6 y + 1 steps through all of it)
+        const uint32_t step = 6u * ((h >> 4) & 15u) + 1u;
+        for (uint32_t tries = 0; tries < slots; tries++, i = i + step < slots ? i + step : i + step - slots) {
+            const uint32_t old = atomicCAS(&t[S * i], 0u, key);
+            if (old == 0u || old == key) {
+                if constexpr (WIDE)
+                    atomicAdd(reinterpret_cast<unsigned long long *>(t + kWideSlots) + 3 * i + (s1 - 1u),
+                              1ull << (kNdBits * (s2 - 1u)));
+                else
+                    atomicAdd(&t[4 * i + s1], 1u << (10 * (s2 - 1u)));
+                return;
+            }
+        }
+        set_status(a->status, ACC_ERR_INTERNAL);  // (more keys than slots: the callers bound them)
+    }
+
+    // Pairs of wedges with the same ends are 4-cycles v-b-w-d, typed by the
+    // two wedges' states: field 3 (s1 - 1) + s2 - 1 of the three words w0, w1,
+    // w2 (fields of B bits) counts the wedges of a type.
+    template <int B, typename Word>
+    __device__ __forceinline__ void cycles(Word w0, Word w1, Word w2) {
+        constexpr Word mask = (Word(1) << B) - 1;
+        uint32_t types = 0;
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+            types |= (((w0 >> (B * j)) & mask) ? 1u << j : 0u) | (((w1 >> (B * j)) & mask) ? 8u << j : 0u) |
+                     (((w2 >> (B * j)) & mask) ? 64u << j : 0u);
+        auto field = [&](uint32_t t) -> Word {
+            const uint32_t i = t / 3u;
+            const Word w = i == 0u ? w0 : (i == 1u ? w1 : w2);
+            return (w >> (B * (t - 3u * i))) & mask;
+        };
+        for (uint32_t m = types; m; m &= m - 1u) {
+            const uint32_t t = (uint32_t)__ffs((int)m) - 1u;
+            const unsigned long long ct = field(t);
+            const uint32_t c1 = ((t / 3u + 1u) << 10) | ((t % 3u + 1u) << 8);  // slots v, b, w
+            for (uint32_t r = m; r; r &= r - 1u) {
+                const uint32_t q = (uint32_t)__ffs((int)r) - 1u;
+                const unsigned long long pairs = q == t ? ct * (ct - 1u) / 2 : ct * field(q);
+                if (pairs) add(c1 | (q / 3u + 1u) | (swap_state(q % 3u + 1u) << 4), pairs);
+            }
+        }
+    }
+
+    // Count the 4-cycles of slots i0, i0 + step, ... (i0 by lane) and empty
+    // them.  Most ends take one wedge: the others are gathered in the (idle)
+    // ring and counted 32 at a time.
+    template <bool WIDE>
+    __device__ __forceinline__ void sweep(int i0, int step) {
+        if constexpr (WIDE) {
+            uint32_t *t = reinterpret_cast<uint32_t *>(tab);
+            for (int i = i0; i < (int)slots; i += step) {
+                if (!t[i]) continue;
+                unsigned long long *w = reinterpret_cast<unsigned long long *>(t + kWideSlots) + 3 * i;
+                cycles<kNdBits>(w[0], w[1], w[2]);
+                t[i] = 0u;
+                w[0] = w[1] = w[2] = 0ull;
+            }
+        } else {
+            int kept = 0;  // slots gathered, 3 words each
+            for (int b = i0 - lane; b < (int)slots; b += step) {
+                const int i = b + lane;  // (the tables hold a multiple of 32 slots)
+                const uint4 q = tab[i];
+                if (q.x) tab[i] = make_uint4(0u, 0u, 0u, 0u);
+                const uint32_t s = q.y + q.z + q.w;
+                const bool many = q.x && (s & 1023u) + ((s >> 10) & 1023u) + (s >> 20) != 1u;
+                const unsigned mm = __ballot_sync(kFull, many);
+                if (many) {
+                    uint32_t *h = ring + 3 * (kept + __popc(mm & ((1u << lane) - 1u)));
+                    h[0] = q.y;
+                    h[1] = q.z;
+                    h[2] = q.w;
+                }
+                kept += __popc(mm);
+                __syncwarp();
+                if (kept >= kWarp) {
+                    kept -= kWarp;
+                    const uint32_t *h = ring + 3 * (kept + lane);
+                    cycles<10>(h[0], h[1], h[2]);
+                    __syncwarp();
+                }
+            }
+            if (lane < kept) cycles<10>(ring[3 * lane], ring[3 * lane + 1], ring[3 * lane + 2]);
+            __syncwarp();
+        }
+    }
+
+    // The part of row entry p's list that the scan takes: k = 3 the
+    // neighbours of u above u (triangles v < u < w); k = 4 those of u above
+    // v, within [lo, hi) when RANGED.
+    template <bool RANGED>
+    __device__ __forceinline__ int row_part(long long p, uint32_t lo, uint32_t hi, uint32_t *first) const {
+        if constexpr (K == 3) {
+            const uint32_t r = __ldg(a->src + p);
+            if (r >> 31) return 0;
+            const uint32_t u = __ldg(a->nbr + p) >> 2;
+            const int l = g.lo[u];
+            *first = (uint32_t)(g.nptr[u] + l);
+            return g.deg[u] - l;
+        } else {
+            const uint2 r = __ldg(a->rev + p);
+            *first = r.x;
+            int cnt = (int)r.y;
+            if constexpr (RANGED) {
+                if (cnt) {
+                    const int i = lower_id(a->nbr + r.x, cnt, lo);
+                    cnt = lower_id(a->nbr + r.x + i, cnt - i, hi);
+                    *first = r.x + (uint32_t)i;
+                }
+            }
+            return cnt;
+        }
+    }
+
+    // Scan rows p0, p0 + step, ... (nrows of them) as one flat sequence of
+    // 32-entry windows, a lane an entry, across row boundaries (the staging
+    // and row lookup of enum.cu's count_leaves), two windows at a time.
+    // k = 4: the rows' roots are v0, v0 + 1, ... (at most kRoots of them; one
+    // when the end vertices are restricted to [lo, hi)).
+    template <bool RANGED, bool WIDE>
+    __device__ __forceinline__ void scan(long long p0, long long step, int nrows, uint32_t v0, uint32_t lo, uint32_t hi) {
+        constexpr int RM = kRingP - 1;
+        constexpr int W = 2;
+        uint32_t *rS = ring, *rO = ring + kRingP, *rP = ring + 2 * kRingP, *rE = ring + 3 * kRingP,
+                 *rV = ring + 4 * kRingP;
+        uint32_t T = 0, F = 0;
+        int tail = 0, cur = -1, jb = 0;
+        const uint32_t voff = (uint32_t)(g.deg - a->deg);
+        for (;;) {
+            while (jb < nrows && T - F < 32u * W && tail - cur + kWarp <= kRingP) {
+                const long long p = p0 + (long long)(jb + lane) * step;
+                int cnt = 0;
+                uint32_t first = 0;
+                if (jb + lane < nrows) cnt = row_part<RANGED>(p, lo, hi, &first);
+                const unsigned nz = __ballot_sync(kFull, cnt > 0);
+                jb += kWarp;
+                if (!nz) continue;
+                int tot;
+                const int pre = warp_excl(cnt, lane, &tot);
+                if (cnt > 0) {
+                    const int slot = (tail + __popc(nz & ((1u << lane) - 1u))) & RM;
+                    const uint32_t sflat = T + (uint32_t)pre;
+                    rS[slot] = sflat;
+                    rO[slot] = first - sflat;
+                    rP[slot] = (uint32_t)p;
+                    const uint32_t v = (__ldg(a->src + p) & 0x7FFFFFFFu) - voff;
+                    if (K == 3) {
+                        rE[slot] = __ldg(a->nbr + p);
+                        rV[slot] = v;
+                    } else {
+                        rE[slot] = __ldg(a->nbr + p) | ((v - v0) << 28);  // (ids have 26 bits)
+                    }
+                }
+                tail += __popc(nz);
+                T += (uint32_t)tot;
+            }
+            const uint32_t pend = T - F;
+            if (!pend) break;
+            __syncwarp();
+            uint32_t v[W], e1[W], pvu[W], puw[W], e2[W], svw[W];
+            bool ok[W];
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                const uint32_t t0 = F + 32u * w;
+                uint32_t bit = 0;
+                const int r = cur + 1 + lane;
+                if (r < tail) {
+                    const uint32_t sd = rS[r & RM] - t0;
+                    if (sd < 32u) bit = 1u << sd;
+                }
+                const uint32_t starts = __reduce_or_sync(kFull, bit);
+                const int row = (cur + __popc(starts & (0xFFFFFFFFu >> (31 - lane)))) & RM;
+                cur += __popc(starts);
+                ok[w] = 32u * w + (uint32_t)lane < pend;
+                e1[w] = rE[row];
+                if (K == 3) {
+                    v[w] = rV[row];
+                } else {
+                    v[w] = e1[w] >> 28;
+                    e1[w] &= 0x0FFFFFFFu;
+                }
+                pvu[w] = rP[row];
+                puw[w] = rO[row] + t0 + (uint32_t)lane;
+                e2[w] = ok[w] ? __ldg(a->nbr + puw[w]) : 0u;
+            }
+#pragma unroll
+            for (int w = 0; w < W; w++)
+                svw[w] = ok[w] && (K == 3 || (e2[w] >> 2) > (e1[w] >> 2)) ? pstate<HASH>(g, K == 3 ? v[w] : v0 + v[w], e2[w] >> 2) : 0u;
+            if constexpr (K == 4) {
+#pragma unroll
+                for (int w = 0; w < W; w++)
+                    if (ok[w])
+                        put<WIDE>(RANGED ? (e2[w] >> 2) + 1u : ((v[w] + 1u) << 26) | (e2[w] >> 2), e1[w] & 3u,
+                                  e2[w] & 3u);
+            }
+#pragma unroll
+            for (int w = 0; w < W; w++) {
+                const uint32_t e = (e1[w] & 3u) << 4 | svw[w] | (e2[w] & 3u) << 2;
+                if constexpr (K == 3) {
+                    if (svw[w]) add(e, 1ull);
+                } else {
+                    const unsigned m = __ballot_sync(kFull, svw[w] != 0u);
+                    if (svw[w]) {
+                        uint32_t *h = hq + 2 * (held + __popc(m & ((1u << lane) - 1u)));
+                        h[0] = pvu[w];
+                        h[1] = puw[w];
+                    }
+                    held += __popc(m);
+                }
+            }
+            if constexpr (K == 4)
+                while (held >= kWarp) {
+                    triangles(kWarp);
+                    held -= kWarp;
+                }
+            F += pend < 32u * W ? pend : 32u * W;
+        }
+        scanned += T;
+    }
+};
+
+// k = 4.  Phase 1: up to 32 consecutive vertices a grab; roots with few wedges
+// share passes over the warp's table (up to kFill wedges a pass), a root
+// with more is queued in parts, ranges of end vertices that carry about
+// equal neighbour entries (a wedge ends in w about in proportion to w's
+// degree).  Phase 2: a block per part, whose warps fill one table of
+// kBlockSlots slots; the rows are dealt to the warps one by one, since a
+// root's first neighbours are hubs with the longest rows.
+//
+// Bound by the latency of list entry, state and table (L2, shared memory).
+// A part re-reads the root's rows (two binary searches a row), so parts are
+// as long as the table allows: on 20000 vertices and 1.35e6 wedges, parts of
+// 160 wedges on one warp's table executed 83e6 warp instructions, this 27e6.
+// Blocks of 16 warps and 4096 slots took 18.2 ms on a set of 4008 graphs (1.4e8
+// wedges of such roots, 900 a root) against 10.6 with 4 warps: their fixed work
+// per warp and part outweighs the fewer searches.
+constexpr int kPart = kBlockFill * 7 / 8, kWidePart = kWideFill * 7 / 8;
+
+template <int PHASE, bool HASH>
+__global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
+    grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem[];
+    __shared__ uint4 item;
+    __shared__ uint32_t bounds[2];
+    __shared__ unsigned long long sizes[kPWarps];
+    constexpr int N = num_classes(4);
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
+    if (PHASE == 2 && a.info->queue_tail == 0) return;
+    uint4 *tabs = reinterpret_cast<uint4 *>(smem);
+    Walker<4, HASH> wk;
+    wk.a = &a;
+    constexpr int kTab = PHASE == 1 ? kPWarps * kSlots : kBlockSlots;
+    wk.tab = PHASE == 1 ? tabs + wib * kSlots : tabs;
+    wk.slots = kSlots;
+    uint32_t *words = reinterpret_cast<uint32_t *>(smem + kTab * 16);
+    wk.ring = words + wib * kRingP * 4;
+    wk.hq = words + kPWarps * kRingP * 4 + wib * 2 * kHits;
+    // (phase 2: the block is at one graph at a time, one histogram)
+    wk.hist = words + kPWarps * (kRingP * 4 + 2 * kHits) + (PHASE == 1 ? wib * 2 * N : 0);
+    wk.held = 0;
+    wk.gcur = -1;
+    wk.scanned = 0;
+    wk.lane = lane;
+    for (int i = threadIdx.x; i < kTab; i += kPThreads) tabs[i] = make_uint4(0u, 0u, 0u, 0u);
+    for (int i = lane; i < 2 * N; i += kWarp) wk.hist[i] = 0u;
+    __syncthreads();
+    // parts of a root with W wedges and d rows
+    auto parts_of = [](uint32_t W, int d) -> uint32_t {
+        return d > kFieldMax ? (W <= (uint32_t)kWideFill ? 1u : (W + kWidePart - 1) / kWidePart)
+                             : (W <= (uint32_t)kBlockFill ? 1u : (W + kPart - 1) / kPart);
+    };
+    if constexpr (PHASE == 1) {
+        // vertices a grab: up to 32, fewer while that leaves warps without any
+        const long long warps = (long long)gridDim.x * kPWarps;
+        const int grab = (int)min(max((a.gs.NV + warps - 1) / warps, 1ll), (long long)kWarp);
+        for (;;) {
+            unsigned long long u0 = 0;
+            if (lane == 0) u0 = atomicAdd(&a.info->unit_ctr, (unsigned long long)grab);
+            u0 = __shfl_sync(kFull, u0, 0);
+            if ((long long)u0 >= a.gs.NV) break;
+            const long long vg = (long long)u0 + lane;
+            uint32_t W = 0;
+            int gi = 0;
+            if (lane < grab && vg < a.gs.NV) {
+                W = a.wedges[vg];
+                if (W) gi = a.gs.graph_of((int)vg);
+            }
+            const bool big = W > (uint32_t)kFill;
+            const unsigned heavy = __ballot_sync(kFull, big);
+            if (heavy) {
+                // (a queued root's count is cleared: what the queue could not
+                // take is found by its count at the end of phase 2)
+                const uint32_t parts = big ? parts_of(W, a.deg[vg] - a.lo[vg]) : 0u;
+                int tot;
+                const int pre = warp_excl((int)parts, lane, &tot);
+                unsigned long long base = 0;
+                if (lane == 0) base = atomicAdd(&a.info->queue_tail, (unsigned long long)tot);
+                base = __shfl_sync(kFull, base, 0) + (unsigned long long)pre;
+                if (base + parts <= a.queue_cap) {
+                    for (uint32_t c = 0; c < parts; c++)
+                        a.queue[base + c] = make_uint4((uint32_t)vg, parts == 1u ? W : c, parts, (uint32_t)gi);
+                    if (parts) a.wedges[vg] = 0u;
+                } else {
+                    for (uint32_t c = 0; c < parts; c++)
+                        if (base + c < a.queue_cap) a.queue[base + c] = make_uint4(0u, 0u, 0u, 0u);
+                }
+            }
+            unsigned todo = __ballot_sync(kFull, W > 0u) & ~heavy;
+            while (todo) {
+                // the roots from the first one on, of one graph, up to the next
+                // queued root and kFill wedges
+                const int s = __ffs(todo) - 1;
+                const int gs = __shfl_sync(kFull, gi, s);
+                const unsigned after = heavy & ~((1u << s) - 1u);
+                const int lim = after ? __ffs(after) - 1 : kWarp;
+                const bool in = ((todo >> lane) & 1u) && gi == gs && lane < lim && lane < s + kRoots;
+                int tot;
+                const int pre = warp_excl(in ? (int)W : 0, lane, &tot);
+                const bool ok = in && pre + (int)W <= kFill;
+                const unsigned take = __ballot_sync(kFull, ok);
+                const int e = __reduce_max_sync(kFull, ok ? lane : 0);
+                wk.switch_graph(gs);
+                const uint32_t voff = (uint32_t)a.gs.meta(gs).voff, v0 = (uint32_t)u0 + s - voff,
+                               v1 = (uint32_t)u0 + e - voff;
+                const long long p0 = wk.g.nptr[v0] + wk.g.lo[v0], p1 = wk.g.nptr[v1] + wk.g.deg[v1];
+                wk.template scan<false, false>(p0, 1, (int)(p1 - p0), v0, 0u, 0u);
+                __syncwarp();
+                wk.template sweep<false>(lane, kWarp);
+                __syncwarp();
+                todo &= ~take;
+            }
+        }
+    } else {
+        // part `part` of `parts` of global root vg of graph gi, W wedges when
+        // it is the only one (whole block)
+        auto run_part = [&](uint32_t vg, uint32_t W, uint32_t part, uint32_t parts, int gi) {
+            if (gi != wk.gcur) {
+                // every warp's triangles are counted before the histogram moves on
+                if (wk.held) wk.triangles(wk.held);
+                wk.held = 0;
+                __syncthreads();
+                if (wib == 0) wk.drain();
+                wk.gcur = gi;
+                wk.g = pview(a, a.gs.meta(gi));
+                __syncthreads();
+            }
+            const uint32_t v = vg - (uint32_t)(wk.g.deg - a.deg), n = (uint32_t)wk.g.n;
+            const long long pb = wk.g.nptr[v] + wk.g.lo[v];
+            const int rows = wk.g.deg[v] - wk.g.lo[v];
+            const bool wide = rows > kFieldMax;
+            const uint32_t fill = wide ? kWideFill : kBlockFill;
+            const long long p0 = pb + wib;
+            const int nr = rows > wib ? (rows - wib + kPWarps - 1) / kPWarps : 0;
+            // one pass over the root's rows, of at most `keys` distinct ends
+            auto pass = [&](auto ranged, uint32_t keys, uint32_t lo, uint32_t hi) {
+                constexpr bool R = decltype(ranged)::value;
+                // the least of 192, 256, 384, ... that is at most two thirds full
+                uint32_t sl = 192;
+                while (2u * sl < 3u * keys) sl = sl % 3u ? sl + sl / 2u : sl / 3u * 4u;
+                wk.slots = sl;
+                if (wide) wk.template scan<R, true>(p0, kPWarps, nr, v, lo, hi);
+                else wk.template scan<R, false>(p0, kPWarps, nr, v, lo, hi);
+                __syncthreads();
+                if (wide) wk.template sweep<true>(threadIdx.x, kPThreads);
+                else wk.template sweep<false>(threadIdx.x, kPThreads);
+                __syncthreads();
+            };
+            // (a range's wedges may all end in one vertex: its counts fit the
+            // fields, each at most the root's rows)
+            if (parts == 1u) {
+                pass(std::false_type{}, W < n ? W : n, 0u, 0u);
+                return;
+            }
+            // ends [bound(part), bound(part + 1)): bound(c) is the first vertex
+            // after v whose entries start at that share of the entries after v's
+            if (threadIdx.x < 2) {
+                const uint32_t c = part + threadIdx.x;
+                const long long q0 = wk.g.nptr[v + 1], q1 = wk.g.nptr[n];
+                const long long want = q0 + (q1 - q0) * (long long)c / (long long)parts;
+                uint32_t x = v + 1u, y = n;
+                if (c == 0) y = x;
+                if (c == parts) x = y;
+                while (x < y) {
+                    const uint32_t mid = (x + y) >> 1;
+                    if (wk.g.nptr[mid] < want) x = mid + 1u;
+                    else y = mid;
+                }
+                bounds[threadIdx.x] = x;
+            }
+            __syncthreads();
+            uint32_t lo = bounds[0], end = bounds[1];
+            const uint32_t hi = end;
+            while (lo < hi) {
+                // wedges that end in [lo, end); when they and their ends are
+                // more than the table takes, the range is halved
+                const uint32_t width = end - lo;
+                unsigned long long S = 0;
+                for (int r = threadIdx.x; r < rows; r += kPThreads) {
+                    uint32_t first;
+                    S += (unsigned long long)wk.template row_part<true>(pb + r, lo, end, &first);
+                }
+#pragma unroll
+                for (int d = 16; d; d >>= 1) S += __shfl_xor_sync(kFull, S, d);
+                if (lane == 0) sizes[wib] = S;
+                __syncthreads();
+                S = 0;
+                for (int w = 0; w < kPWarps; w++) S += sizes[w];
+                __syncthreads();
+                const unsigned long long keys = S < width ? S : width;
+                if (keys > fill) {
+                    end = lo + width / 2;
+                    continue;
+                }
+                if (S) pass(std::true_type{}, (uint32_t)keys, lo, end);
+                lo = end;
+                end = hi - lo > 2u * width ? lo + 2u * width : hi;
+            }
+        };
+        const unsigned long long pushed = a.info->queue_tail, tail = min(pushed, a.queue_cap);
+        for (;;) {
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                const unsigned long long idx = atomicAdd(&a.info->queue_head, 1ull);
+                item = idx < tail ? a.queue[idx] : make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
+            }
+            __syncthreads();
+            const uint4 it = item;
+            if (it.x == 0xFFFFFFFFu) break;
+            if (it.z) run_part(it.x, it.y, it.y, it.z, (int)it.w);
+        }
+        if (pushed > a.queue_cap) {
+            for (long long vg = blockIdx.x; vg < a.gs.NV; vg += gridDim.x)
+                for (uint32_t c = 0; c < 2u && a.wedges[vg] > (uint32_t)kFill; c++)
+                    run_part((uint32_t)vg, 0u, c, 2u, a.gs.graph_of((int)vg));
+        }
+    }
+    if (PHASE == 2) {
+        if (wk.held) wk.triangles(wk.held);
+        wk.held = 0;
+        __syncthreads();
+    }
+    if (PHASE == 1 || wib == 0) wk.drain();
+    if (lane == 0 && wk.scanned) atomicAdd(&a.info->scanned, wk.scanned);
+}
+
+// k = 3: the triangles, 32 rows (neighbour entries) a grab.  The rows of one
+// graph are dealt out with a stride, so that the hubs' rows, which come first
+// and are the longest, end up in different grabs; a set of several graphs
+// takes consecutive entries (few graph switches).
+template <bool HASH>
+__global__ void __launch_bounds__(kPThreads, 8) k_partial3(PartialArgs a) {
+    grid_dep_wait();
+    constexpr int N = num_classes(3);
+    __shared__ uint32_t rings[kPWarps][kRingP * kRingArrays];
+    __shared__ uint32_t hists[kPWarps][2 * N];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
+    Walker<3, HASH> wk;
+    wk.a = &a;
+    wk.tab = nullptr;
+    wk.slots = 0;
+    wk.hq = nullptr;
+    wk.held = 0;
+    wk.ring = rings[wib];
+    wk.hist = hists[wib];
+    wk.gcur = -1;
+    wk.scanned = 0;
+    wk.lane = lane;
+    if (lane < 2 * N) wk.hist[lane] = 0u;
+    __syncwarp();
+    const long long nnz = a.info->nnz, units = (nnz + kWarp - 1) / kWarp;
+    for (;;) {
+        unsigned long long q = 0;
+        if (lane == 0) q = atomicAdd(&a.info->unit_ctr, 1ull);
+        q = __shfl_sync(kFull, q, 0);
+        if ((long long)q >= units) break;
+        if (a.gs.B == 1) {
+            wk.switch_graph(0);
+            wk.template scan<false, false>((long long)q, units, (int)((nnz - (long long)q + units - 1) / units), 0u, 0u, 0u);
+            continue;
+        }
+        const long long end = min(((long long)q + 1) * kWarp, nnz);
+        for (long long p = (long long)q * kWarp; p < end;) {
+            wk.switch_graph(a.gs.graph_of((int)(a.src[p] & 0x7FFFFFFFu)));
+            const long long e = min(end, wk.g.nptr[wk.g.n]);
+            wk.template scan<false, false>(p, 1, (int)(e - p), 0u, 0u, 0u);
+            p = e;
+        }
+    }
+    wk.drain();
+    if (lane == 0 && wk.scanned) atomicAdd(&a.info->scanned, wk.scanned);
+}
+
+// ---------------------------------------------------------------------------
+// Finish: the partial counts that are products of degrees and triangle
+// counters, then the induced counts.
+// ---------------------------------------------------------------------------
+
+__device__ __forceinline__ unsigned long long nd_of(unsigned long long nd, uint32_t s) {
+    return (nd >> (kNdBits * (s - 1u))) & ((1ull << kNdBits) - 1ull);
+}
+
+// Adds a per-thread sum to one class of the block's histogram (whole warp).
+__device__ __forceinline__ void warp_add(uint32_t *hist, const int16_t *lut, int lane, uint32_t code,
+                                         unsigned long long x) {
+#pragma unroll
+    for (int d = 16; d; d >>= 1) x += __shfl_xor_sync(kFull, x, d);
+    if (lane == 0 && x) hist_add(hist, __ldg(lut + code), x);
+}
+
+// One undirected edge b - c of G*, seen from the end where its state is 1 or 3:
+// its state s, the neighbours of b other than c and of c other than b by state.
+struct EdgeEnds {
+    uint32_t s;
+    bool flip;
+    unsigned long long b[3], c[3];
+};
+
+__device__ __forceinline__ EdgeEnds edge_ends(uint32_t s, unsigned long long nb, unsigned long long nc) {
+    EdgeEnds x;
+    x.flip = s == 2u;
+    x.s = x.flip ? 1u : s;
+    const uint32_t r = swap_state(x.s);
+    const unsigned long long n0 = x.flip ? nc : nb, n1 = x.flip ? nb : nc;
+#pragma unroll
+    for (uint32_t i = 0; i < 3; i++) {
+        x.b[i] = nd_of(n0, i + 1u) - (x.s == i + 1u ? 1u : 0u);
+        x.c[i] = nd_of(n1, i + 1u) - (r == i + 1u ? 1u : 0u);
+    }
+    return x;
+}
+
+// The terms of an edge with common neighbours (tw: their counts by state to
+// each end): paths that close (a = d, taken out), diamonds on the edge, and
+// triangles on the edge with a pendant at one end (each of those seen from two
+// edges: these counts are twice the real ones).
+__device__ __forceinline__ void edge_triangles(uint32_t *hist, const int16_t *lut, const EdgeEnds &x,
+                                               unsigned long long t0, unsigned long long t1, unsigned long long t2) {
+    const uint32_t f1 = x.s << 10;
+    uint32_t types = 0;
+#pragma unroll
+    for (uint32_t j = 0; j < 3; j++)
+        types |= (nd_of(t0, j + 1u) ? 1u << j : 0u) | (nd_of(t1, j + 1u) ? 8u << j : 0u) |
+                 (nd_of(t2, j + 1u) ? 64u << j : 0u);
+    auto count = [&](uint32_t t) -> unsigned long long {
+        const uint32_t i = t / 3u;
+        return nd_of(i == 0u ? t0 : (i == 1u ? t1 : t2), t - 3u * i + 1u);
+    };
+    // states of a common neighbour to the ends the edge is seen from
+    auto state_b = [&](uint32_t t) -> uint32_t { return x.flip ? t % 3u : t / 3u; };
+    auto state_c = [&](uint32_t t) -> uint32_t { return x.flip ? t / 3u : t % 3u; };
+    for (uint32_t m = types; m; m &= m - 1u) {
+        const uint32_t t = (uint32_t)__ffs((int)m) - 1u, i = state_b(t), j = state_c(t);
+        const unsigned long long n = count(t);
+        hist_add(hist, __ldg(lut + (f1 | ((i + 1u) << 6) | ((j + 1u) << 2))), 0ull - n);
+        const uint32_t code = f1 | (((i + 1u) | ((j + 1u) << 2)) << 6);
+        for (uint32_t r = m; r; r &= r - 1u) {
+            const uint32_t q = (uint32_t)__ffs((int)r) - 1u;
+            const unsigned long long pairs = q == t ? n * (n - 1u) / 2 : n * count(q);
+            if (pairs) hist_add(hist, __ldg(lut + (code | (state_b(q) + 1u) | ((state_c(q) + 1u) << 2))), pairs);
+        }
+#pragma unroll
+        for (uint32_t e = 0; e < 3; e++) {
+            const unsigned long long xb = n * (x.b[e] - (e == i ? 1u : 0u)), xc = n * (x.c[e] - (e == j ? 1u : 0u));
+            if (xb) hist_add(hist, __ldg(lut + (code | (e + 1u))), xb);
+            if (xc) hist_add(hist, __ldg(lut + (code | ((e + 1u) << 2))), xc);
+        }
+    }
+}
+
+// Induced counts of one graph from its partial counts (whole block), by the
+// entries of partial_matrix.
+template <int K>
+__device__ void induced(const PartialArgs &a, int g, uint32_t *res, unsigned long long *P) {
+    constexpr int N = num_classes(K);
+    for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) res[i] = 0u;
+    // (read past the L1: other blocks wrote these sums)
+    for (int i = threadIdx.x; i < N; i += blockDim.x) P[i] = atomicAdd(&a.part[(size_t)g * N + i], 0ull);
+    __syncthreads();
+    const int entries = (int)__ldg(a.inv);
+#pragma unroll 4
+    for (int i = threadIdx.x; i < entries; i += blockDim.x) {
+        const uint32_t e = __ldg(a.inv + 1 + i);
+        const unsigned long long x = P[(e >> 16) & 255u];
+        if (x) hist_add(res, (int)(e >> 24), x * (unsigned long long)((long long)(e & 0xFFFFu) - 32768ll));
+    }
+    __syncthreads();
+    for (int c = threadIdx.x; c < N; c += blockDim.x) {
+        const unsigned long long x = (unsigned long long)res[2 * c] | ((unsigned long long)res[2 * c + 1] << 32);
+        a.counts[(size_t)g * N + c] = K == 4 ? x >> 1 : x;  // (k = 4: twice the counts, see partial_matrix)
+    }
+    __syncthreads();
+}
+
+// Block per (graph, slice of its vertices and edges); the block that ends a
+// graph's last slice turns the partial counts into induced ones.  On the
+// dense block it also zeroes the marked chunks (k_clear_chunks).
+template <int K>
+__global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) {
+    grid_dep_wait();
+    constexpr int N = num_classes(K);
+    __shared__ uint32_t hist[2 * N];
+    __shared__ unsigned long long sums[N];
+    __shared__ uint32_t lists[kFThreads / kWarp][2 * kWarp];
+    __shared__ int last;
+    const int lane = threadIdx.x & 31;
+    const bool refused = a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW;
+    for (long long item = blockIdx.x; !refused && item < (long long)a.gs.B * a.slices; item += gridDim.x) {
+        const int g = (int)(item / a.slices), sl = (int)(item % a.slices);
+        const GMeta mt = a.gs.meta(g);
+        for (int i = threadIdx.x; i < 2 * N; i += blockDim.x) hist[i] = 0u;
+        __syncthreads();
+        // stars (k = 3: the open triples) from the typed degrees
+        const int v0 = (int)((long long)mt.n * sl / a.slices), v1 = (int)((long long)mt.n * (sl + 1) / a.slices);
+        unsigned long long st[10] = {};
+        for (int v = v0 + (int)threadIdx.x; v < v1; v += blockDim.x) {
+            const unsigned long long nd = a.nd[mt.voff + v];
+            const unsigned long long n1 = nd_of(nd, 1u), n2 = nd_of(nd, 2u), n3 = nd_of(nd, 3u);
+            const unsigned long long p1 = n1 * (n1 - 1) / 2, p2 = n2 * (n2 - 1) / 2, p3 = n3 * (n3 - 1) / 2;
+            if (K == 3) {
+                st[0] += p1;
+                st[1] += p2;
+                st[2] += p3;
+                st[3] += n1 * n2;
+                st[4] += n1 * n3;
+                st[5] += n2 * n3;
+            } else {
+                // (n (n - 1) / 2 is 0 for n = 0 modulo 2^64 too: n - 1 wraps and 0 times it is 0)
+                st[0] += n1 > 2 ? n1 * (n1 - 1) / 2 * (n1 - 2) / 3 : 0ull;
+                st[1] += n2 > 2 ? n2 * (n2 - 1) / 2 * (n2 - 2) / 3 : 0ull;
+                st[2] += n3 > 2 ? n3 * (n3 - 1) / 2 * (n3 - 2) / 3 : 0ull;
+                st[3] += p1 * n2;
+                st[4] += p1 * n3;
+                st[5] += p2 * n1;
+                st[6] += p2 * n3;
+                st[7] += p3 * n1;
+                st[8] += p3 * n2;
+                st[9] += n1 * n2 * n3;
+            }
+        }
+        if (K == 3) {
+            const uint32_t f[6] = {0x11, 0x22, 0x33, 0x12, 0x13, 0x23};  // (slot 1, slot 2) states
+#pragma unroll
+            for (int i = 0; i < 6; i++) warp_add(hist, a.lut, lane, ((f[i] >> 4) << 4) | (f[i] & 15u), st[i]);
+        } else {
+            const uint32_t f[10] = {0x111, 0x222, 0x333, 0x112, 0x113, 0x221, 0x223, 0x331, 0x332, 0x123};
+#pragma unroll
+            for (int i = 0; i < 10; i++)
+                warp_add(hist, a.lut, lane, ((f[i] >> 8) << 10) | (((f[i] >> 4) & 15u) << 6) | (f[i] & 15u), st[i]);
+            // paths, diamonds and triangles with a pendant from the edges
+            unsigned long long p4[18] = {};
+            // (slices of entries, not of vertices: a hub's row is as long as many others)
+            const long long b0 = a.nptr[mt.voff], nb = a.nptr[mt.voff + mt.n] - b0;
+            const long long e0 = b0 + nb * sl / a.slices, e1 = b0 + nb * (sl + 1) / a.slices;
+            // edges with common neighbours are few in a sparse graph: a warp
+            // gathers them and counts 32 at a time
+            uint32_t *list = lists[threadIdx.x >> 5];
+            int kept = 0;
+            auto closed = [&](int n) {  // the last n <= 32 gathered
+                __syncwarp();
+                if (lane < n) {
+                    const long long pos = e0 + list[kept - n + lane];
+                    const uint32_t e = a.nbr[pos];
+                    const EdgeEnds x = edge_ends(e & 3u, a.nd[a.src[pos]], a.nd[mt.voff + (e >> 2)]);
+                    edge_triangles(hist, a.lut, x, a.tri[3 * pos], a.tri[3 * pos + 1], a.tri[3 * pos + 2]);
+                }
+                __syncwarp();
+            };
+            for (long long w0 = e0 + threadIdx.x - lane; w0 < e1; w0 += blockDim.x) {
+                const long long pos = w0 + lane;
+                const uint32_t r = pos < e1 ? a.src[pos] : 0x80000000u;
+                bool tri = false;
+                if (!(r >> 31)) {  // each edge once, from its smaller end
+                    const uint32_t e = a.nbr[pos];
+                    const EdgeEnds x = edge_ends(e & 3u, a.nd[r], a.nd[mt.voff + (e >> 2)]);
+                    tri = (a.tri[3 * pos] | a.tri[3 * pos + 1] | a.tri[3 * pos + 2]) != 0ull;
+#pragma unroll
+                    for (int i = 0; i < 3; i++)
+#pragma unroll
+                        for (int j = 0; j < 3; j++) {
+                            const unsigned long long y = x.b[i] * x.c[j];
+                            p4[3 * i + j] += x.s == 3u ? 0ull : y;
+                            p4[9 + 3 * i + j] += x.s == 3u ? y : 0ull;
+                        }
+                }
+                const unsigned mm = __ballot_sync(kFull, tri);
+                if (tri) list[kept + __popc(mm & ((1u << lane) - 1u))] = (uint32_t)(pos - e0);
+                kept += __popc(mm);
+                if (kept >= kWarp) {
+                    closed(kWarp);
+                    kept -= kWarp;
+                }
+            }
+            closed(kept);
+#pragma unroll
+            for (uint32_t i = 0; i < 18; i++)
+                warp_add(hist, a.lut, lane, ((i < 9 ? 1u : 3u) << 10) | (((i % 9) / 3 + 1u) << 6) | ((i % 3 + 1u) << 2),
+                         p4[i]);
+        }
+        __syncthreads();
+        for (int c = threadIdx.x; c < N; c += blockDim.x) {
+            const unsigned long long x = (unsigned long long)hist[2 * c] | ((unsigned long long)hist[2 * c + 1] << 32);
+            if (x) atomicAdd(&a.part[(size_t)g * N + c], x);
+        }
+        fence_device();
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(&a.done[g], 1) == a.slices - 1;
+        __syncthreads();
+        if (last) {
+            fence_device();
+            induced<K>(a, g, hist, sums);
+        }
+        __syncthreads();
+    }
+    if (a.occ)
+        clear_chunks(a.gs, a.state_w, a.occ, a.occ_w, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
+                     ((long long)gridDim.x * blockDim.x) >> 5, lane);
+}
+
+bool launched() {
+    if (cudaPeekAtLastError() == cudaSuccess) return true;
+    cudaGetLastError();
+    return false;
+}
+
+constexpr size_t kSmem1 = kPWarps * (kSlots * 16 + kRingP * 16 + 8 * kHits + 8 * num_classes(4)),
+                 kSmem2 = kBlockSlots * 16 + kPWarps * (kRingP * 16 + 8 * kHits) + 8 * num_classes(4);
+
+// The persistent grid times grid_num / grid_den, at least a block per SM.
+int scaled_grid(int per_sm, int num_sms, int grid_num, int grid_den) {
+    const long long g = (long long)num_sms * per_sm * grid_num / grid_den;
+    return (int)(g < num_sms ? num_sms : g);
+}
+
+template <bool HASH>
+int partial4(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+    static bool smem_opt_in = false;
+    if (!smem_opt_in) {
+        if (cudaFuncSetAttribute(k_partial4<1, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1) != cudaSuccess ||
+            cudaFuncSetAttribute(k_partial4<2, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem2) != cudaSuccess)
+            return ACC_ERR_CUDA;
+        smem_opt_in = true;
+    }
+    // (no kernel waits on another block, so the grid need not be resident as a whole)
+    const int grid = scaled_grid(8, num_sms, grid_num, grid_den);
+    launch_pdl(k_partial4<1, HASH>, grid, kPThreads, kSmem1, s, a);
+    if (!launched()) return ACC_ERR_CUDA;
+    launch_pdl(k_partial4<2, HASH>, grid, kPThreads, kSmem2, s, a);
+    return launched() ? 2 : ACC_ERR_CUDA;
+}
+
+}  // namespace
+
+// k = 4: a partial count of a triangle with a pendant is kept doubled (see
+// edge_triangles), so the matrix holds twice the coefficients of the other classes
+// and yields twice the counts.
+void partial_matrix(int k, const int16_t *lut, const uint32_t *class_code, std::vector<uint32_t> &out) {
+    const int N = num_classes(k);
+    std::vector<int> coef((size_t)N * N, 0);
+    for (int c = 0; c < N; c++) {
+        const uint32_t code = class_code[c];
+        uint32_t edge[10];
+        int edges = 0, deg[5] = {};
+        for (int i = 0; i < k; i++)
+            for (int j = i + 1; j < k; j++) {
+                const uint32_t bits = code & ((1u << code_bit(k, i, j)) | (1u << code_bit(k, j, i)));
+                if (!bits) continue;
+                edge[edges++] = bits;
+                deg[i]++;
+                deg[j]++;
+            }
+        bool deg3 = false;
+        for (int i = 0; i < k; i++) deg3 = deg3 || deg[i] == 3;
+        const int unit = k == 4 && !(edges == 4 && deg3) ? 2 : 1;
+        for (uint32_t sub = 0; sub < 1u << edges; sub++) {
+            uint32_t kept = 0;
+            int left = edges;
+            for (int e = 0; e < edges; e++)
+                if ((sub >> e) & 1u) {
+                    kept |= edge[e];
+                    left--;
+                }
+            const int to = lut[kept];
+            if (to >= 0) coef[(size_t)to * N + c] += left & 1 ? -unit : unit;
+        }
+    }
+    out.assign(1, 0u);
+    for (int to = 0; to < N; to++)
+        for (int c = 0; c < N; c++)
+            if (coef[(size_t)to * N + c])
+                out.push_back(((uint32_t)to << 24) | ((uint32_t)c << 16) | (uint32_t)(coef[(size_t)to * N + c] + 32768));
+    out[0] = (uint32_t)out.size() - 1u;
+}
+
+int launch_partial(int k, PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num,
+                   int grid_den) {
+    int launches = 0;
+    long long grid = (max_entries + 255) / 256;
+    if (grid > (long long)num_sms * 8) grid = (long long)num_sms * 8;
+    if (grid < 1) grid = 1;
+    if (k == 3) launch_pdl(k_partial_prep<3>, (int)grid, 256, 0, s, a);
+    else launch_pdl(k_partial_prep<4>, (int)grid, 256, 0, s, a);
+    if (!launched()) return ACC_ERR_CUDA;
+    launches++;
+    if (k == 3) {
+        const int g3 = scaled_grid(8, num_sms, grid_num, grid_den);
+        if (a.nh) launch_pdl(k_partial3<true>, g3, kPThreads, 0, s, a);
+        else launch_pdl(k_partial3<false>, g3, kPThreads, 0, s, a);
+        if (!launched()) return ACC_ERR_CUDA;
+        launches++;
+    } else {
+        const int rc = a.nh ? partial4<true>(a, num_sms, s, grid_num, grid_den)
+                            : partial4<false>(a, num_sms, s, grid_num, grid_den);
+        if (rc < 0) return rc;
+        launches += rc;
+    }
+    // slices of a graph: about four blocks per SM over the set, of at least
+    // 512 entries each
+    long long sl = (4ll * num_sms + a.gs.B - 1) / a.gs.B;
+    const long long per = max_entries / a.gs.B / 512 + 1;
+    if (sl > per) sl = per;
+    a.slices = (int)(sl < 1 ? 1 : sl);
+    long long fin = (long long)a.gs.B * a.slices;
+    const long long rows = (a.gs.NV * kWarp + kFThreads - 1) / kFThreads;  // a warp a row to clear
+    if (a.occ && fin < rows) fin = rows;
+    if (fin > (long long)num_sms * 8) fin = (long long)num_sms * 8;
+    if (k == 3) launch_pdl(k_partial_finish<3>, (int)fin, kFThreads, 0, s, a);
+    else launch_pdl(k_partial_finish<4>, (int)fin, kFThreads, 0, s, a);
+    return launched() ? launches + 1 : ACC_ERR_CUDA;
+}
+
+}  // namespace acc
