@@ -62,6 +62,7 @@ struct SharedTable {
     int16_t *lut = nullptr, *lut_sv = nullptr;
     uint32_t *class_code = nullptr;
     uint32_t *inv = nullptr;  // k = 3, 4: partial_matrix
+    unsigned char *tab5 = nullptr;  // k = 5: partial5_tables
     int16_t *lut_host = nullptr;
     uint32_t *class_code_host = nullptr;
 };
@@ -135,6 +136,39 @@ fail:
     return rc;
 }
 
+int ensure_lut(acc_ctx *c, int k, cudaStream_t s);
+
+// k = 5 by partial patterns reads the tables of every k, and each class's
+// divisor and the smaller classes' automorphisms (built with the k = 5 table).
+int ensure_tab5(acc_ctx *c, cudaStream_t s) {
+    for (int k = 3; k <= 5; k++) {
+        const int rc = ensure_lut(c, k, s);
+        if (rc) return rc;
+    }
+    if (c->tab5) return ACC_OK;
+    std::lock_guard<std::mutex> lock(g_tables_mu);
+    SharedTable &t = g_tables[c->device][5];
+    if (!t.tab5) {
+        std::vector<unsigned char> div5, aut4, aut3;
+        partial5_tables(c->class_code_host[5], c->class_code_host[4], c->class_code_host[3], div5, aut4, aut3);
+        div5.insert(div5.end(), aut4.begin(), aut4.end());
+        div5.insert(div5.end(), aut3.begin(), aut3.end());
+        unsigned char *d = nullptr;
+        if (!ok(cudaMalloc(&d, div5.size()))) {
+            cudaGetLastError();
+            return ACC_ERR_NOMEM;
+        }
+        if (!ok(cudaMemcpy(d, div5.data(), div5.size(), cudaMemcpyHostToDevice))) {
+            cudaGetLastError();
+            cudaFree(d);
+            return ACC_ERR_CUDA;
+        }
+        t.tab5 = d;
+    }
+    c->tab5 = t.tab5;  // (the context holds a reference to the k = 5 table)
+    return ACC_OK;
+}
+
 int ensure_lut(acc_ctx *c, int k, cudaStream_t s) {
     if (c->lut[k]) return ACC_OK;
     if (c->device < 0 || c->device >= kTableDevices) return ACC_ERR_ARG;
@@ -165,6 +199,7 @@ void release_luts(acc_ctx *c) {
             cudaFree(t.lut_sv);
             cudaFree(t.class_code);
             cudaFree(t.inv);
+            cudaFree(t.tab5);
             delete[] t.lut_host;
             delete[] t.class_code_host;
             t = SharedTable();
@@ -172,6 +207,7 @@ void release_luts(acc_ctx *c) {
         c->lut[k] = c->lut_sv[k] = nullptr;
         c->class_code_dev[k] = nullptr;
         c->inv[k] = nullptr;
+        if (k == 5) c->tab5 = nullptr;
         c->lut_host[k] = nullptr;
         c->class_code_host[k] = nullptr;
     }
@@ -231,6 +267,14 @@ bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relab
     return count_family(c) && k <= 4 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS && !uses_formula(c, k, max_n);
 }
 
+// The same for k = 5 (partial5.cu), of one graph; its launches are followed by
+// the scan's, which run only when the device finds that it must (more
+// triangles than the list holds, a root with over 1023 neighbours above it, a
+// count bound near the 64-bit limit).
+bool uses_partial5(const acc_ctx *c, int k, long long arcs, bool relabel, int B) {
+    return count_family(c) && k == 5 && B == 1 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS;
+}
+
 // Size limit of one graph: the dense block's, or the sparse build's for the
 // count mode (local ids fill 26 bits of the extension-list entries).
 int size_check(const acc_ctx *c, long long n) {
@@ -251,12 +295,17 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
     int rc;
     const bool sparse = sparse_build(c, max_n);
     const bool partial = uses_partial(c, k, max_n, arcs, relabel);
-    if (partial) {
+    const bool partial5 = uses_partial5(c, k, arcs, relabel, B);
+    if (partial5) {
+        if ((rc = grow(&c->p5_vert, &c->p5_vert_cap, 3 * ((size_t)NV + 1)))) return rc;
+        if ((rc = grow(&c->p5_sums, &c->p5_sums_cap, (size_t)num_classes(5) + 16 + kCtrs))) return rc;
+    }
+    if (partial || partial5) {
         if ((rc = grow(&c->pp_nd, &c->pp_nd_cap, (size_t)NV + 1))) return rc;
-        if ((rc = grow(&c->pp_part, &c->pp_part_cap, (size_t)B * num_classes(k)))) return rc;
+        if ((rc = grow(&c->pp_part, &c->pp_part_cap, (size_t)B * num_classes(k == 5 ? 4 : k)))) return rc;
         if ((rc = grow(&c->pp_done, &c->pp_done_cap, (size_t)B))) return rc;
-        if (k == 4 && (rc = grow(&c->pp_wedges, &c->pp_wedges_cap, (size_t)NV + 1))) return rc;
-        if (k == 4 && (rc = grow(&c->pp_tri, &c->pp_tri_cap, 3 * (size_t)(2 * arcs) + 1))) return rc;
+        if (k >= 4 && (rc = grow(&c->pp_wedges, &c->pp_wedges_cap, (size_t)NV + 1))) return rc;
+        if (k >= 4 && (rc = grow(&c->pp_tri, &c->pp_tri_cap, 3 * (size_t)(2 * arcs) + 1))) return rc;
     }
     if (uses_hash(c, k, max_n) && (rc = grow(&c->nh, &c->nh_cap, (size_t)kNhWords * (size_t)(2 * arcs) + 4)))
         return rc;
@@ -298,7 +347,7 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
     if ((rc = grow(&c->f5_pre, &c->f5_pre_cap, (size_t)NV + 1))) return rc;
     if ((rc = grow(&c->nbr, &c->nbr_cap, (size_t)(2 * arcs) + 1))) return rc;
     if ((rc = grow(&c->src, &c->src_cap, (size_t)(2 * arcs) + 1))) return rc;
-    if ((uses_rev(c, arcs) || (partial && k == 4)) && (rc = grow(&c->rev, &c->rev_cap, (size_t)(2 * arcs) + 1))) return rc;
+    if ((uses_rev(c, arcs) || (partial && k == 4) || partial5) && (rc = grow(&c->rev, &c->rev_cap, (size_t)(2 * arcs) + 1))) return rc;
     if (!sparse && (rc = grow(&c->occ, &c->occ_cap, (size_t)NV * (size_t)occ_words(max_n) + 1))) return rc;
     if (!c->info) {
         if (!ok(cudaMalloc(&c->info, sizeof(GraphInfo)))) return ACC_ERR_NOMEM;
@@ -349,14 +398,22 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     bb.info = c->info;
     bb.k = k;
     bool partial = gs.NV > 0 && uses_partial(c, k, max_n, gs.M, relabel);
-    if (partial) {
+    bool partial5 = gs.NV > 0 && uses_partial5(c, k, gs.M, relabel, gs.B);
+    if (partial5) {
+        if (!c->tab5) return ACC_ERR_INTERNAL;  // (the callers ensure it)
+        bb.zero[4] = c->p5_vert;
+        bb.nzero[4] = 3 * gs.NV;
+        bb.zero[5] = reinterpret_cast<int *>(c->p5_sums);
+        bb.nzero[5] = 2ll * (num_classes(5) + 16 + kCtrs);
+    }
+    if (partial || partial5) {
         bb.zero[0] = reinterpret_cast<int *>(c->pp_nd);
         bb.nzero[0] = 2 * gs.NV;
         bb.zero[1] = reinterpret_cast<int *>(c->pp_part);
-        bb.nzero[1] = 2ll * gs.B * num_classes(k);
+        bb.nzero[1] = 2ll * gs.B * num_classes(k == 5 ? 4 : k);
         bb.zero[2] = c->pp_done;
         bb.nzero[2] = gs.B;
-        if (k == 4) {
+        if (k >= 4) {
             bb.zero[3] = reinterpret_cast<int *>(c->pp_wedges);
             bb.nzero[3] = gs.NV;
         }
@@ -378,7 +435,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         if (!ok(cudaMemcpyAsync(c->maxdeg_host, &c->info->maxdeg, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
             !ok(cudaStreamSynchronize(s)))
             return ACC_ERR_CUDA;
-        if (*c->maxdeg_host > kNdMax) partial = false;  // its packed degree counts hold kNdMax
+        if (*c->maxdeg_host > kNdMax) partial = partial5 = false;  // its packed degree counts hold kNdMax
         spw = 2 * sparse_list_entries(*c->maxdeg_host) + 2 * kPartBRows;
         const int warps = enum_grid_warps(k, c->num_sms);
         if (warps < 0) return warps;
@@ -393,7 +450,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         launches += rc;
     }
     const bool formula = uses_formula(c, k, max_n);
-    const bool rev = gs.NV > 0 && !formula && !partial && uses_rev(c, gs.M);
+    const bool rev = gs.NV > 0 && !formula && !partial && !partial5 && uses_rev(c, gs.M);
     if (rev) {
         rc = launch_rev_build(gs, c->nptr, c->deg, c->nbr, c->src, c->info, 2 * gs.M, c->rev, c->num_sms, s);
         if (rc < 0) return rc;
@@ -408,7 +465,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     a.nbr = c->nbr;
     a.src = c->src;
     a.nh = hash ? reinterpret_cast<const uint4 *>(c->nh) : nullptr;
-    a.rev = rev ? c->rev : nullptr;
+    a.rev = rev || partial5 ? c->rev : nullptr;
     a.lut = c->lut_sv[k];
     a.gs = gs;
     a.max_n = max_n;
@@ -423,8 +480,8 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     a.counts = reinterpret_cast<unsigned long long *>(counts);
     a.status = status;
     const bool any = gs.NV > 0;
-    if (partial) {
-        PartialArgs p;
+    PartialArgs p = {};
+    if (partial || partial5) {
         p.state = c->state;
         p.state_w = c->state;
         p.deg = c->deg;
@@ -433,8 +490,8 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         p.nbr = c->nbr;
         p.src = c->src;
         p.nh = hash ? c->nh : nullptr;
-        p.lut = c->lut_sv[k];
-        p.inv = c->inv[k];
+        p.lut = c->lut_sv[k == 5 ? 4 : k];
+        p.inv = c->inv[k == 5 ? 4 : k];
         p.gs = gs;
         p.info = c->info;
         p.queue = c->queue;
@@ -449,9 +506,37 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         p.status = status;
         p.occ = sparse ? nullptr : c->occ;
         p.occ_w = occ_words(max_n);
-        rc = launch_partial(k, p, 2 * gs.M, c->num_sms, s, c->grid_num, c->grid_den);
+        if (partial5) {
+            Partial5 &q = p.p5;
+            q.sums = c->p5_sums;
+            q.small = c->p5_sums + num_classes(5);
+            q.ctr = q.small + 16;
+            // the triangles are listed where the scan, if it runs after all,
+            // keeps its overflow lists
+            q.tris = reinterpret_cast<uint4 *>(c->scratch);
+            q.tri_cap = c->scratch_cap / 4;
+            q.in_tri = c->p5_vert;
+            q.pair_wedges = reinterpret_cast<uint32_t *>(c->p5_vert + gs.NV);
+            q.cycle_wedges = reinterpret_cast<uint32_t *>(c->p5_vert + 2 * gs.NV);
+            q.lut5 = c->lut_sv[5];
+            q.lut5_canon = c->lut[5];
+            q.lut4_canon = c->lut[4];
+            q.lut3 = c->lut_sv[3];
+            q.lut3_canon = c->lut[3];
+            q.code5 = c->class_code_dev[5];
+            q.div5 = c->tab5;
+            q.aut4 = c->tab5 + num_classes(5);
+            q.aut3 = q.aut4 + num_classes(4);
+            a.run = q.ctr + kCtrScan;
+            rc = launch_partial5(p, 2 * gs.M, c->num_sms, s, c->grid_num, c->grid_den);
+        } else {
+            rc = launch_partial(k, p, 2 * gs.M, c->num_sms, s, c->grid_num, c->grid_den);
+        }
         if (rc < 0) return rc;
         launches += rc;
+    }
+    if (partial) {
+        // counted
     } else if (any && formula) {
         if (k == 3)
             rc = launch_formula3(gs, c->state, c->nptr, c->deg, c->lo, c->nbr, c->lut[3],
@@ -472,6 +557,11 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     if (c->timing && !ok(cudaEventRecord(c->ev[3], s))) return ACC_ERR_CUDA;
     if (any && !formula && !partial) {
         rc = launch_enumerate(k, a, c->num_sms, 2, s, c->grid_num, c->grid_den);
+        if (rc < 0) return rc;
+        launches += rc;
+    }
+    if (partial5) {
+        rc = launch_partial5_counts(p, c->num_sms, s);
         if (rc < 0) return rc;
         launches += rc;
     }
@@ -507,7 +597,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     if (n < 0 || m < 0 || m >= (1ll << 31)) return ACC_ERR_INPUT;
     if (size_check(c, n)) return ACC_ERR_TOO_LARGE;
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
-    int rc = ensure_lut(c, k, s);
+    int rc = uses_partial5(c, k, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
     if ((rc = ensure_workspace(c, n, sparse_build(c, n) ? 0 : (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN)))
@@ -546,10 +636,10 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
         key.grid_num = c->grid_num;
         key.grid_den = c->grid_den;
         key.adjacency = c->adjacency;
-        const void *ws[25] = {c->state, c->deg, c->lo, c->label, c->deg_in, c->nptr, c->tiles, c->nbr, c->occ,
+        const void *ws[28] = {c->state, c->deg, c->lo, c->label, c->deg_in, c->nptr, c->tiles, c->nbr, c->occ,
                               c->info, c->queue, c->scratch, c->lut[k], c->lut_sv[k], c->class_code_dev[k],
                               c->f5_pre, c->status_dev, c->src, c->nh, c->rev, c->pp_nd, c->pp_tri, c->pp_part,
-                              c->pp_wedges, c->pp_done};
+                              c->pp_wedges, c->pp_done, c->p5_vert, c->p5_sums, c->tab5};
         memcpy(key.ws, ws, sizeof(ws));
         bool have = c->cg_exec && memcmp(&key, &c->cg_key, sizeof(key)) == 0;
         // capture only when a count repeats: a one-off count runs one by one
@@ -632,10 +722,8 @@ long long ctx_footprint(const acc_ctx *c, long long n, long long m, int k) {
 
 int ctx_reserve(acc_ctx *c, long long n, long long m, int k) {
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
-    for (int kk = 3; kk <= 5; kk++) {
-        const int rc = ensure_lut(c, kk, c->own);
-        if (rc) return rc;
-    }
+    const int rc = ensure_tab5(c, c->own);
+    if (rc) return rc;
     return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, n >= kRelabelMinN);
 }
 
@@ -702,6 +790,8 @@ void acc_ctx_destroy(acc_ctx *c) {
     cudaFree(c->pp_part);
     cudaFree(c->pp_wedges);
     cudaFree(c->pp_done);
+    cudaFree(c->p5_vert);
+    cudaFree(c->p5_sums);
     cudaFree(c->sp_raw);
     cudaFree(c->sp_merged);
     cudaFree(c->sp_roff);
@@ -735,7 +825,7 @@ int acc_motif_prepare(acc_ctx *c, int k, void *stream) {
     if (!valid_k(k)) return ACC_ERR_K;
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = ensure_lut(c, k, s);
+    int rc = k == 5 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     return ok(cudaStreamSynchronize(s)) ? ACC_OK : ACC_ERR_CUDA;
 }
@@ -806,7 +896,8 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     // word) may still read the descriptors and graph ids rewritten below;
     // the pageable copy would not wait for it
     if (!ok(cudaStreamSynchronize(s))) return ACC_ERR_CUDA;
-    int rc = ensure_lut(c, k, s);
+    // (k = 5: also for a run after the mode changed to the count mode)
+    int rc = k == 5 && B == 1 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     if ((rc = ensure_workspace(c, NV, sparse_build(c, max_n) ? 0 : words, arcs, max_n, k, B, true))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;

@@ -55,6 +55,7 @@ struct GraphInfo {
     unsigned big_rows;              // sparse build: rows listed for the block sort
     unsigned big_head;              // sparse build: listed rows taken
     float bound[3];                 // degree sums of the count bound (count_bound_terms)
+    int large;                      // the count bound exceeds kCountLimit / 32
 };
 
 // Largest count the library reports: a set whose upper bound on N_k (below)
@@ -258,8 +259,8 @@ struct BuildBufs {
     uint32_t *occ;           // NV * occ_words(max_n)
     int occ_w;               // occ_words(max_n)
     GraphInfo *info;
-    int *zero[4] = {};       // further arrays to clear with the counts (NULL: none) ...
-    long long nzero[4] = {}; // ... and their lengths
+    int *zero[6] = {};       // further arrays to clear with the counts (NULL: none) ...
+    long long nzero[6] = {}; // ... and their lengths
     int k = 0;               // 3..5: refuse (ACC_ERR_OVERFLOW) a set whose count bound
                              // exceeds kCountLimit; 0: no check
 };
@@ -333,6 +334,7 @@ struct EnumArgs {
     long long target;           // schedule: work of one queued chunk of a heavy unit
     unsigned long long *counts; // int64[B * num_classes]
     int *status;
+    const unsigned long long *run = nullptr;  // not NULL: nothing to do while it points to 0
 };
 // batch.cu: Z-scores of each group's real graph against its randomisations.
 int launch_zscores(const long long *counts, int groups, int group_size, int K, double *z, cudaStream_t s);

@@ -22,6 +22,7 @@ struct acc_ctx {
     int16_t *lut[6] = {};
     int16_t *lut_sv[6] = {};
     uint32_t *class_code_dev[6] = {};
+    unsigned char *tab5 = nullptr;  // k = 5: divisors, automorphisms (partial5_tables)
     uint32_t *inv[6] = {};  // k = 3, 4: partial counts to induced ones (partial.cuh)
     int16_t *lut_host[6] = {};
     uint32_t *class_code_host[6] = {};
@@ -68,6 +69,10 @@ struct acc_ctx {
     size_t pp_wedges_cap = 0;
     int *pp_done = nullptr;
     size_t pp_done_cap = 0;
+    int *p5_vert = nullptr;  // k = 5: three words a vertex
+    size_t p5_vert_cap = 0;
+    unsigned long long *p5_sums = nullptr;  // k = 5: sums, small patterns, counters
+    size_t p5_sums_cap = 0;
     int mode = 0;             // ACC_MODE_COUNT, _ENUMERATE, _FORMULA or _AUTO
     long long sched_light = 0;   // enumeration schedule (0: the kernels' default)
     long long sched_target = 0;
@@ -114,7 +119,7 @@ struct acc_ctx {
         const void *rowptr, *col, *counts, *status;
         long long m, light, target;
         int n, k, mode, grid_num, grid_den, adjacency;
-        const void *ws[25];
+        const void *ws[28];
     } cg_key = {}, cg_seen = {};  // the captured graph's key; the last key counted one by one
     int cg_launches = 0;
     long long cg_units = 0;

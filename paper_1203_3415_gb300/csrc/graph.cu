@@ -49,7 +49,7 @@ __device__ __forceinline__ int warp_excl_scan(int x, int lane, int *total) {
     return incl - x;
 }
 
-constexpr int kRanges = 8;
+constexpr int kRanges = 10;
 struct IntRanges {
     int *p[kRanges];
     long long n[kRanges];
@@ -335,7 +335,9 @@ __global__ void __launch_bounds__(1024) k_scan_degrees(const int *__restrict__ d
             float tb[3] = {0.0f, 0.0f, 0.0f};
             for (int w = 0; w < (int)(blockDim.x >> 5); w++)
                 for (int j = 0; j < 3; j++) tb[j] += warp_bound[w][j];
-            if (count_bound(k, max_n, warp_max[0], tb) > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
+            const double bound = count_bound(k, max_n, warp_max[0], tb);
+            if (bound > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
+            info->large = bound > kCountLimit / 32;
         }
         info->maxdeg = warp_max[0];
         info->big_rows = 0;
@@ -441,7 +443,11 @@ __global__ void __launch_bounds__(1024) k_scan_top(long long *tile_sum, int ntil
         run += v;
     }
     if (t == 0) {
-        if (k && count_bound(k, max_n, info->maxdeg, info->bound) > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
+        if (k) {
+            const double bound = count_bound(k, max_n, info->maxdeg, info->bound);
+            if (bound > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
+            info->large = bound > kCountLimit / 32;
+        }
         info->big_rows = 0;
         info->big_head = 0;
         info->queue_tail = 0;
@@ -913,7 +919,7 @@ int grid_for(long long work_items, int per_block, int num_sms) {
 // Append the caller's arrays to a build's cleared ranges; the longest.
 long long more_ranges(const BuildBufs &bb, IntRanges &r) {
     long long longest = 0;
-    for (int i = 0; i < 4; i++)
+    for (int i = 0; i < 6; i++)
         if (bb.zero[i]) {
             r.p[4 + i] = bb.zero[i];
             r.n[4 + i] = bb.nzero[i];

@@ -30,8 +30,9 @@ namespace acc {
 
 namespace {
 
-constexpr int kPWarps = 4;           // warps per block
+constexpr int kPWarps = 4;           // warps per block (k = 5: twice as many share the block's sums)
 constexpr int kPThreads = kPWarps * kWarp;
+__host__ __device__ constexpr int warps_of(int K) { return K == 5 ? 2 * kPWarps : kPWarps; }
 // Wedge tables, 16 bytes a slot: one a warp for the roots with few wedges, one
 // a block for the others.
 constexpr int kSlots = 192;
@@ -47,80 +48,6 @@ constexpr int kRoots = 16;           // roots that share a table pass
 constexpr int kHits = 96;            // triangles held before they are counted, two words each
 constexpr int kFThreads = 256;       // threads per block of the finish
 
-__device__ __forceinline__ uint32_t swap_state(uint32_t s) { return ((s & 1u) << 1) | (s >> 1); }
-
-// One graph's arrays by local vertex (neighbour-list positions are global).
-struct PView {
-    const uint32_t *state;
-    long long pitch;
-    const long long *nptr;
-    const int *deg, *lo;
-    const unsigned long long *nd;
-    const uint32_t *nh;
-    int n;
-};
-
-__device__ __forceinline__ PView pview(const PartialArgs &a, const GMeta &mt) {
-    return PView{a.state + mt.soff, mt.pitch,        a.nptr + mt.voff, a.deg + mt.voff,
-                 a.lo + mt.voff,    a.nd + mt.voff, a.nh,             mt.n};
-}
-
-// state(x, y): the dense block, or x's hashed table (enum.cu, nh.cu).
-template <bool HASH>
-__device__ __forceinline__ uint32_t pstate(const PView &g, uint32_t x, uint32_t y) {
-    if constexpr (HASH) {
-        const uint32_t lg = nh_lg(g.deg[x]), m = (1u << lg) - 1u;
-        const uint4 *tab = reinterpret_cast<const uint4 *>(g.nh + (long long)kNhWords * g.nptr[x]);
-        uint32_t k = nh_bucket(y, lg);
-        for (uint32_t tries = 0; tries <= m; tries++, k = (k + 1u) & m) {
-            const uint4 q = __ldg(tab + k);
-            if ((q.x >> 2) == y) return q.x & 3u;
-            if ((q.y >> 2) == y) return q.y & 3u;
-            if ((q.z >> 2) == y) return q.z & 3u;
-            if ((q.w >> 2) == y) return q.w & 3u;
-            if (!q.w) return 0u;
-        }
-        return 0u;
-    } else {
-        return (__ldg(g.state + (long long)x * g.pitch + (y >> 4)) >> ((y & 15u) << 1)) & 3u;
-    }
-}
-
-// First index of the sorted entries e[0..n) (u << 2 | state) with u >= id.
-__device__ __forceinline__ int lower_id(const uint32_t *__restrict__ e, int n, uint32_t id) {
-    const uint32_t key = id << 2;
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(e + mid) < key) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
-__device__ __forceinline__ int warp_excl(int x, int lane, int *total) {
-    int incl = x;
-#pragma unroll
-    for (int d = 1; d < kWarp; d <<= 1) {
-        const int y = __shfl_up_sync(kFull, incl, d);
-        if (lane >= d) incl += y;
-    }
-    *total = __shfl_sync(kFull, incl, kWarp - 1);
-    return incl - x;
-}
-
-// 64-bit histogram bin in shared memory as two words (the hardware adds 32
-// bits natively): the add that carries out of the low word raises the high.
-__device__ __forceinline__ void hist_add(uint32_t *h, int bin, unsigned long long d) {
-    const uint32_t lo = (uint32_t)d;
-    uint32_t hi = (uint32_t)(d >> 32);
-    if (lo) {
-        const uint32_t old = atomicAdd(&h[2 * bin], lo);
-        if (old > ~lo) hi++;
-    }
-    if (hi) atomicAdd(&h[2 * bin + 1], hi);
-}
-
 // ---------------------------------------------------------------------------
 // Preparation: typed degrees, and for k = 4 the reverse positions of the upper
 // entries (v -> u with u above v: the part of N*(u) above v, as k_rev gives
@@ -132,6 +59,9 @@ __global__ void k_partial_prep(PartialArgs a) {
     grid_dep_wait();
     const long long nnz = a.info->nnz;
     const int lane = threadIdx.x & 31;
+    // k = 5: sums near the 64-bit limit (a pattern's sum counts an occurrence
+    // up to 24 times before it is divided) are left to the scan
+    if (K == 5 && blockIdx.x == 0 && threadIdx.x == 0 && a.info->large) a.p5.ctr[kCtrScan] = 1ull;
     for (long long p0 = blockIdx.x * (long long)blockDim.x + threadIdx.x - lane; p0 < nnz;
          p0 += (long long)gridDim.x * blockDim.x) {
         const long long pos = p0 + lane;
@@ -149,28 +79,37 @@ __global__ void k_partial_prep(PartialArgs a) {
             atomicAdd(&a.nd[v], (unsigned long long)__popc(same & m1) |
                                     ((unsigned long long)__popc(same & m2) << kNdBits) |
                                     ((unsigned long long)__popc(same & m3) << (2 * kNdBits)));
-        if constexpr (K == 4) {
+        if constexpr (K >= 4) {
             uint2 rv = make_uint2(0u, 0u);
-            if (ok && !(r >> 31)) {
+            if (ok && (K == 5 || !(r >> 31))) {
                 const int voff = a.gs.meta(a.gs.graph_of((int)v)).voff;
                 const uint32_t u = (uint32_t)voff + (e >> 2);
                 const long long base = a.nptr[u];
-                // v is among the neighbours of u below u
-                const int i = lower_id(a.nbr + base, a.lo[u], v - (uint32_t)voff);
+                // (k = 4: v is among the neighbours of u below u)
+                const int i = lower_id(a.nbr + base, K == 5 ? a.deg[u] : a.lo[u], v - (uint32_t)voff);
                 rv = make_uint2((uint32_t)(base + i + 1), (uint32_t)(a.deg[u] - i - 1));
+                if (!(r >> 31))
 #pragma unroll
-                for (int j = 0; j < 3; j++) a.tri[3 * pos + j] = 0ull;
+                    for (int j = 0; j < 3; j++) a.tri[3 * pos + j] = 0ull;
             }
             if (ok) a.rev[pos] = rv;
-            uint32_t incl = rv.y;
+            auto row_sum = [&](uint32_t x) -> uint32_t {  // of the row's lanes, seen from its first
+                uint32_t incl = x;
 #pragma unroll
-            for (int d = 1; d < kWarp; d <<= 1) {
-                const uint32_t y = __shfl_up_sync(kFull, incl, d);
-                if (lane >= d) incl += y;
-            }
-            const int last = lane + __popc(same >> lane) - 1;  // (the row's last lane, seen from its first)
-            const uint32_t sum = __shfl_sync(kFull, incl, last) - incl + rv.y;
+                for (int d = 1; d < kWarp; d <<= 1) {
+                    const uint32_t y = __shfl_up_sync(kFull, incl, d);
+                    if (lane >= d) incl += y;
+                }
+                const int last = lane + __popc(same >> lane) - 1;
+                return __shfl_sync(kFull, incl, last) - incl + x;
+            };
+            const uint32_t sum = row_sum(r >> 31 ? 0u : rv.y);
             if (leader && sum) atomicAdd(&a.wedges[v], sum);
+            if constexpr (K == 5) {
+                if (leader && sum) atomicAdd(&a.p5.cycle_wedges[v], sum);
+                const uint32_t all = row_sum(rv.y);
+                if (leader && all) atomicAdd(&a.p5.pair_wedges[v], all);
+            }
         }
     }
 }
@@ -185,7 +124,8 @@ struct Walker {
     const PartialArgs *a;
     PView g;
     uint32_t *hist;   // this warp's histogram of partial counts (two words a class)
-    uint4 *tab;       // k = 4: (key, three words of three 10-bit counts)
+    Bins5 bins;       // k = 5: the block's sums
+    uint4 *tab;       // k = 4, 5: (key, three words of three 10-bit counts)
     uint32_t slots;   // the table's slots
     uint32_t *ring;   // flat start, entry offset, row position, row entry[, row vertex]
     uint32_t *hq;     // k = 4: triangles held (positions of v -> u and u -> w)
@@ -196,6 +136,10 @@ struct Walker {
 
     __device__ __forceinline__ int cls(uint32_t code) const { return (int)__ldg(a->lut + code); }
     __device__ __forceinline__ void add(uint32_t code, unsigned long long d) {
+        if constexpr (K == 5) {
+            bins.add(code, d);
+            return;
+        }
         const int c = cls(code);
         if (c < 0) set_status(a->status, ACC_ERR_INTERNAL);
         else hist_add(hist, c, d);
@@ -203,6 +147,7 @@ struct Walker {
 
     // the histogram into graph gcur's partial counts (whole warp)
     __device__ __forceinline__ void drain() {
+        if constexpr (K == 5) return;  // (one graph; the block flushes its sums)
         constexpr int N = num_classes(K);
         if (K == 4 && held) triangles(held);
         held = 0;
@@ -250,6 +195,12 @@ struct Walker {
             atomicAdd(&a->tri[3ll * pvw + svu - 1u], 1ull << (kNdBits * (swap_state(suw) - 1u)));
             atomicAdd(&a->tri[3ll * puw + swap_state(svu) - 1u], 1ull << (kNdBits * (swap_state(svw) - 1u)));
             code = (svu << 10) | ((svw | (suw << 2)) << 6);
+            if (a->p5.tris) {  // counting k = 5: the triangle is listed
+                const unsigned long long i = atomicAdd(&a->p5.ctr[kCtrTris], 1ull);
+                if (i < a->p5.tri_cap) a->p5.tris[i] = make_uint4(pvu, puw, pvw, 0u);
+                else a->p5.ctr[kCtrScan] = 1ull;
+                a->p5.in_tri[v] = a->p5.in_tri[u] = a->p5.in_tri[w] = 1;
+            }
             const int l = g.lo[w];
             off = (uint32_t)(g.nptr[w] + l);
             len = g.deg[w] - l;
@@ -307,6 +258,22 @@ struct Walker {
         set_status(a->status, ACC_ERR_INTERNAL);  // (more keys than slots: the callers bound them)
     }
 
+    // The slot that holds key, or -1.
+    template <bool WIDE>
+    __device__ __forceinline__ int find(uint32_t key) const {
+        constexpr int S = WIDE ? 1 : 4;
+        const uint32_t *t = reinterpret_cast<const uint32_t *>(tab);
+        const uint32_t h = key * 0x9E3779B1u;
+        uint32_t i = (uint32_t)(((unsigned long long)h * slots) >> 32);
+        const uint32_t step = 6u * ((h >> 4) & 15u) + 1u;
+        for (uint32_t tries = 0; tries < slots; tries++, i = i + step < slots ? i + step : i + step - slots) {
+            const uint32_t k = t[S * i];
+            if (k == key) return (int)i;
+            if (!k) return -1;
+        }
+        return -1;
+    }
+
     // Pairs of wedges with the same ends are 4-cycles v-b-w-d, typed by the
     // two wedges' states: field 3 (s1 - 1) + s2 - 1 of the three words w0, w1,
     // w2 (fields of B bits) counts the wedges of a type.
@@ -335,22 +302,131 @@ struct Walker {
         }
     }
 
-    // Count the 4-cycles of slots i0, i0 + step, ... (i0 by lane) and empty
+    // k = 5: the wedges of one pair {v, w} (words as above).  Three of them are
+    // a K_{2,3}; two are a 4-cycle, and with a pendant at v or w a banner (its
+    // other ends may coincide with the pendant; twice, as the cycle's two
+    // middles may be swapped).
+    template <int B, typename Word>
+    __device__ __forceinline__ void pair_terms(Word w0, Word w1, Word w2, uint32_t v, uint32_t w) {
+        constexpr Word mask = (Word(1) << B) - 1;
+        uint32_t types = 0;
+#pragma unroll
+        for (int j = 0; j < 3; j++)
+            types |= (((w0 >> (B * j)) & mask) ? 1u << j : 0u) | (((w1 >> (B * j)) & mask) ? 8u << j : 0u) |
+                     (((w2 >> (B * j)) & mask) ? 64u << j : 0u);
+        auto field = [&](uint32_t t) -> unsigned long long {
+            const uint32_t i = t / 3u;
+            const Word x = i == 0u ? w0 : (i == 1u ? w1 : w2);
+            return (x >> (B * (t - 3u * i))) & mask;
+        };
+        auto middle = [](int m, uint32_t t) -> uint32_t {  // K_{2,3} with ends 0, 1
+            return e5(0, m, t / 3u + 1u) | e5(1, m, swap_state(t % 3u + 1u));
+        };
+        const unsigned long long nv = g.nd[v], nw = g.nd[w];
+        for (uint32_t m = types; m; m &= m - 1u) {
+            const uint32_t t = (uint32_t)__ffs((int)m) - 1u;
+            const unsigned long long ct = field(t);
+            for (uint32_t r = m; r; r &= r - 1u) {
+                const uint32_t q = (uint32_t)__ffs((int)r) - 1u;
+                const unsigned long long cq = field(q), pairs = q == t ? ct * (ct - 1u) / 2 : ct * cq;
+                if (!pairs) continue;
+                const uint32_t cyc = e5(0, 1, t / 3u + 1u) | e5(1, 2, t % 3u + 1u) | e5(0, 3, q / 3u + 1u) |
+                                     e5(2, 3, swap_state(q % 3u + 1u));
+#pragma unroll
+                for (uint32_t s = 1; s <= 3; s++) {
+                    const unsigned long long xv = nd_of(nv, s), xw = nd_of(nw, s);
+                    if (xv) add(cyc | e5(0, 4, s), 2u * pairs * xv);
+                    if (xw) add(cyc | e5(2, 4, s), 2u * pairs * xw);
+                }
+                for (uint32_t z = r; z; z &= z - 1u) {
+                    const uint32_t y = (uint32_t)__ffs((int)z) - 1u;
+                    const unsigned long long cy = field(y);
+                    unsigned long long n;
+                    if (y == q) n = q == t ? (ct > 2 ? ct * (ct - 1u) / 2 * (ct - 2u) / 3 : 0ull) : ct * (cq * (cq - 1u) / 2);
+                    else n = pairs * cy;
+                    if (n) add(middle(2, t) | middle(3, q) | middle(4, y), n);
+                }
+            }
+        }
+    }
+
+    // k = 5: houses.  A wedge v - b - w, another wedge v - d - w of the table,
+    // and a common neighbour of v and b, or of b and w (which may coincide
+    // with w or d, or v or d).  Rows as in scan, of the middles in a triangle.
+    template <bool RANGED, bool WIDE>
+    __device__ __forceinline__ void houses(long long p0, long long step, int nrows, uint32_t v0, uint32_t lo, uint32_t hi) {
+        for (int jb = 0; jb < nrows; jb += kWarp) {
+            const long long pl = p0 + (long long)(jb + lane) * step;
+            int cl = 0;
+            uint32_t fl = 0, el = 0;
+            if (jb + lane < nrows) {
+                el = __ldg(a->nbr + pl);
+                if (a->p5.in_tri[el >> 2]) cl = row_part<RANGED>(pl, lo, hi, &fl);
+            }
+            for (unsigned rows = __ballot_sync(kFull, cl > 0); rows; rows &= rows - 1u) {
+                const int r = __ffs(rows) - 1;
+                const long long p = p0 + (long long)(jb + r) * step;
+                const int cnt = __shfl_sync(kFull, cl, r);
+                const uint32_t first = __shfl_sync(kFull, fl, r), e1 = __shfl_sync(kFull, el, r);
+                const uint32_t src = __ldg(a->src + p), v = (src & 0x7FFFFFFFu), b = e1 >> 2, s1 = e1 & 3u;
+                const EdgeTri tv = edge_tri(*a, p, !(src >> 31));
+                const uint32_t mv = types_of(tv);
+                for (int q = lane; q < cnt; q += kWarp) {
+                    const uint32_t pos = first + (uint32_t)q, e2 = __ldg(a->nbr + pos), w = e2 >> 2, s2 = e2 & 3u;
+                    const int i = find<WIDE>(((v - v0 + 1u) << 26) | w);
+                    if (i < 0) continue;
+                    const EdgeTri tw = edge_tri(*a, pos, b < w);
+                    const uint32_t mw = types_of(tw);
+                    if (!(mv | mw)) continue;
+                    const uint32_t *t = reinterpret_cast<const uint32_t *>(tab);
+                    auto count = [&](uint32_t y) -> unsigned long long {  // wedges of type y but this one
+                        const uint32_t own = y == 3u * (s1 - 1u) + s2 - 1u ? 1u : 0u;
+                        if constexpr (WIDE)
+                            return nd_of(reinterpret_cast<const unsigned long long *>(t + kWideSlots)[3 * i + y / 3u], y % 3u + 1u) - own;
+                        else
+                            return ((t[4 * i + 1 + y / 3u] >> (10 * (y % 3u))) & 1023u) - own;
+                    };
+                    for (uint32_t y = 0; y < 9; y++) {
+                        const unsigned long long c = count(y);
+                        if (!c) continue;
+                        const uint32_t cyc = e5(0, 1, s1) | e5(1, 2, s2) | e5(0, 3, y / 3u + 1u) |
+                                             e5(2, 3, swap_state(y % 3u + 1u));
+                        for (uint32_t m = mv; m; m &= m - 1u) {
+                            const uint32_t z = next_bit(m);
+                            add(cyc | e5(0, 4, z / 3u + 1u) | e5(1, 4, z % 3u + 1u), c * tv.get(z / 3u, z % 3u));
+                        }
+                        for (uint32_t m = mw; m; m &= m - 1u) {
+                            const uint32_t z = next_bit(m);
+                            add(cyc | e5(1, 4, z / 3u + 1u) | e5(2, 4, z % 3u + 1u), c * tw.get(z / 3u, z % 3u));
+                        }
+                    }
+                }
+            }
+        }
+    }
+
+    // Count the terms of slots i0, i0 + step, ... (i0 by lane) and empty
     // them.  Most ends take one wedge: the others are gathered in the (idle)
     // ring and counted 32 at a time.
     template <bool WIDE>
-    __device__ __forceinline__ void sweep(int i0, int step) {
+    __device__ __forceinline__ void sweep(int i0, int step, uint32_t v0) {
         if constexpr (WIDE) {
             uint32_t *t = reinterpret_cast<uint32_t *>(tab);
             for (int i = i0; i < (int)slots; i += step) {
                 if (!t[i]) continue;
                 unsigned long long *w = reinterpret_cast<unsigned long long *>(t + kWideSlots) + 3 * i;
-                cycles<kNdBits>(w[0], w[1], w[2]);
+                if constexpr (K == 5) pair_terms<kNdBits>(w[0], w[1], w[2], v0 + (t[i] >> 26) - 1u, t[i] & 0x3FFFFFFu);
+                else cycles<kNdBits>(w[0], w[1], w[2]);
                 t[i] = 0u;
                 w[0] = w[1] = w[2] = 0ull;
             }
         } else {
-            int kept = 0;  // slots gathered, 3 words each
+            constexpr int H = K == 5 ? 4 : 3;
+            int kept = 0;  // slots gathered, H words each
+            auto count = [&](const uint32_t *h) {
+                if constexpr (K == 5) pair_terms<10>(h[0], h[1], h[2], v0 + (h[3] >> 26) - 1u, h[3] & 0x3FFFFFFu);
+                else cycles<10>(h[0], h[1], h[2]);
+            };
             for (int b = i0 - lane; b < (int)slots; b += step) {
                 const int i = b + lane;  // (the tables hold a multiple of 32 slots)
                 const uint4 q = tab[i];
@@ -359,21 +435,21 @@ struct Walker {
                 const bool many = q.x && (s & 1023u) + ((s >> 10) & 1023u) + (s >> 20) != 1u;
                 const unsigned mm = __ballot_sync(kFull, many);
                 if (many) {
-                    uint32_t *h = ring + 3 * (kept + __popc(mm & ((1u << lane) - 1u)));
+                    uint32_t *h = ring + H * (kept + __popc(mm & ((1u << lane) - 1u)));
                     h[0] = q.y;
                     h[1] = q.z;
                     h[2] = q.w;
+                    if (K == 5) h[H - 1] = q.x;
                 }
                 kept += __popc(mm);
                 __syncwarp();
                 if (kept >= kWarp) {
                     kept -= kWarp;
-                    const uint32_t *h = ring + 3 * (kept + lane);
-                    cycles<10>(h[0], h[1], h[2]);
+                    count(ring + H * (kept + lane));
                     __syncwarp();
                 }
             }
-            if (lane < kept) cycles<10>(ring[3 * lane], ring[3 * lane + 1], ring[3 * lane + 2]);
+            if (lane < kept) count(ring + H * lane);
             __syncwarp();
         }
     }
@@ -391,6 +467,8 @@ struct Walker {
             *first = (uint32_t)(g.nptr[u] + l);
             return g.deg[u] - l;
         } else {
+            // (entries below the row's vertex lie between the rows of a shared pass)
+            if (K == 4 && (__ldg(a->src + p) >> 31)) return 0;
             const uint2 r = __ldg(a->rev + p);
             *first = r.x;
             int cnt = (int)r.y;
@@ -478,14 +556,15 @@ struct Walker {
             }
 #pragma unroll
             for (int w = 0; w < W; w++)
-                svw[w] = ok[w] && (K == 3 || (e2[w] >> 2) > (e1[w] >> 2)) ? pstate<HASH>(g, K == 3 ? v[w] : v0 + v[w], e2[w] >> 2) : 0u;
-            if constexpr (K == 4) {
+                svw[w] = K < 5 && ok[w] && (K == 3 || (e2[w] >> 2) > (e1[w] >> 2)) ? pstate<HASH>(g, K == 3 ? v[w] : v0 + v[w], e2[w] >> 2) : 0u;
+            if constexpr (K >= 4) {
 #pragma unroll
                 for (int w = 0; w < W; w++)
                     if (ok[w])
-                        put<WIDE>(RANGED ? (e2[w] >> 2) + 1u : ((v[w] + 1u) << 26) | (e2[w] >> 2), e1[w] & 3u,
+                        put<WIDE>(((v[w] + 1u) << 26) | (e2[w] >> 2), e1[w] & 3u,
                                   e2[w] & 3u);
             }
+            if constexpr (K < 5)
 #pragma unroll
             for (int w = 0; w < W; w++) {
                 const uint32_t e = (e1[w] & 3u) << 4 | svw[w] | (e2[w] & 3u) << 2;
@@ -529,19 +608,30 @@ struct Walker {
 // per warp and part outweighs the fewer searches.
 constexpr int kPart = kBlockFill * 7 / 8, kWidePart = kWideFill * 7 / 8;
 
-template <int PHASE, bool HASH>
-__global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
+//
+// k = 5 runs the same passes over the wedges with any middle and the root as
+// the smaller end (K_{2,3}, banners and houses), for one graph.
+template <int K, int PHASE, bool HASH>
+__global__ void __launch_bounds__(warps_of(K) * kWarp, K == 5 ? 3 : 8) k_wedges(PartialArgs a) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint4 item;
     __shared__ uint32_t bounds[2];
+    constexpr int kPWarps = warps_of(K), kPThreads = kPWarps * kWarp;
     __shared__ unsigned long long sizes[kPWarps];
     constexpr int N = num_classes(4);
+    unsigned long long *ctr = a.p5.ctr;
+    // (counting k = 5, the scan's counters stay as the build left them)
+    unsigned long long *unit = K == 5 ? ctr + kCtrPairUnit : (ctr ? ctr + kCtrUnit4 : &a.info->unit_ctr),
+                       *qtail = K == 5 ? ctr + kCtrPairTail : (ctr ? ctr + kCtrTail4 : &a.info->queue_tail),
+                       *qhead = K == 5 ? ctr + kCtrPairHead : (ctr ? ctr + kCtrHead4 : &a.info->queue_head);
+    uint32_t *root_wedges = K == 5 ? a.p5.pair_wedges : a.wedges;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
-    if (PHASE == 2 && a.info->queue_tail == 0) return;
+    if (K == 5 && *(volatile unsigned long long *)(ctr + kCtrScan)) return;
+    if (PHASE == 2 && *qtail == 0) return;
     uint4 *tabs = reinterpret_cast<uint4 *>(smem);
-    Walker<4, HASH> wk;
+    Walker<K, HASH> wk;
     wk.a = &a;
     constexpr int kTab = PHASE == 1 ? kPWarps * kSlots : kBlockSlots;
     wk.tab = PHASE == 1 ? tabs + wib * kSlots : tabs;
@@ -550,33 +640,39 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
     wk.ring = words + wib * kRingP * 4;
     wk.hq = words + kPWarps * kRingP * 4 + wib * 2 * kHits;
     // (phase 2: the block is at one graph at a time, one histogram)
-    wk.hist = words + kPWarps * (kRingP * 4 + 2 * kHits) + (PHASE == 1 ? wib * 2 * N : 0);
+    wk.hist = words + kPWarps * (kRingP * 4 + (K == 4 ? 2 * kHits : 0)) + (PHASE == 1 && K == 4 ? wib * 2 * N : 0);
+    wk.bins = Bins5{wk.hist, a.p5.sums, a.p5.lut5, a.status};  // (k = 5: one histogram a block)
     wk.held = 0;
     wk.gcur = -1;
     wk.scanned = 0;
     wk.lane = lane;
     for (int i = threadIdx.x; i < kTab; i += kPThreads) tabs[i] = make_uint4(0u, 0u, 0u, 0u);
-    for (int i = lane; i < 2 * N; i += kWarp) wk.hist[i] = 0u;
+    if constexpr (K == 5) wk.bins.clear();
+    else
+        for (int i = lane; i < 2 * N; i += kWarp) wk.hist[i] = 0u;
     __syncthreads();
+    // first row of root v (k = 4: of the vertices above it)
+    auto first_row = [&](uint32_t v) -> long long { return wk.g.nptr[v] + (K == 5 ? 0 : wk.g.lo[v]); };
     // parts of a root with W wedges and d rows
     auto parts_of = [](uint32_t W, int d) -> uint32_t {
         return d > kFieldMax ? (W <= (uint32_t)kWideFill ? 1u : (W + kWidePart - 1) / kWidePart)
                              : (W <= (uint32_t)kBlockFill ? 1u : (W + kPart - 1) / kPart);
     };
     if constexpr (PHASE == 1) {
-        // vertices a grab: up to 32, fewer while that leaves warps without any
-        const long long warps = (long long)gridDim.x * kPWarps;
+        // vertices a grab: up to 32, and at least four grabs a warp (neighbouring
+        // roots are similar work, and a warp takes them pass after pass)
+        const long long warps = 4ll * gridDim.x * kPWarps;
         const int grab = (int)min(max((a.gs.NV + warps - 1) / warps, 1ll), (long long)kWarp);
         for (;;) {
             unsigned long long u0 = 0;
-            if (lane == 0) u0 = atomicAdd(&a.info->unit_ctr, (unsigned long long)grab);
+            if (lane == 0) u0 = atomicAdd(unit, (unsigned long long)grab);
             u0 = __shfl_sync(kFull, u0, 0);
             if ((long long)u0 >= a.gs.NV) break;
             const long long vg = (long long)u0 + lane;
             uint32_t W = 0;
             int gi = 0;
             if (lane < grab && vg < a.gs.NV) {
-                W = a.wedges[vg];
+                W = root_wedges[vg];
                 if (W) gi = a.gs.graph_of((int)vg);
             }
             const bool big = W > (uint32_t)kFill;
@@ -584,16 +680,16 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
             if (heavy) {
                 // (a queued root's count is cleared: what the queue could not
                 // take is found by its count at the end of phase 2)
-                const uint32_t parts = big ? parts_of(W, a.deg[vg] - a.lo[vg]) : 0u;
+                const uint32_t parts = big ? parts_of(W, a.deg[vg] - (K == 5 ? 0 : a.lo[vg])) : 0u;
                 int tot;
                 const int pre = warp_excl((int)parts, lane, &tot);
                 unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(&a.info->queue_tail, (unsigned long long)tot);
+                if (lane == 0) base = atomicAdd(qtail, (unsigned long long)tot);
                 base = __shfl_sync(kFull, base, 0) + (unsigned long long)pre;
                 if (base + parts <= a.queue_cap) {
                     for (uint32_t c = 0; c < parts; c++)
                         a.queue[base + c] = make_uint4((uint32_t)vg, parts == 1u ? W : c, parts, (uint32_t)gi);
-                    if (parts) a.wedges[vg] = 0u;
+                    if (parts) root_wedges[vg] = 0u;
                 } else {
                     for (uint32_t c = 0; c < parts; c++)
                         if (base + c < a.queue_cap) a.queue[base + c] = make_uint4(0u, 0u, 0u, 0u);
@@ -616,10 +712,15 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
                 wk.switch_graph(gs);
                 const uint32_t voff = (uint32_t)a.gs.meta(gs).voff, v0 = (uint32_t)u0 + s - voff,
                                v1 = (uint32_t)u0 + e - voff;
-                const long long p0 = wk.g.nptr[v0] + wk.g.lo[v0], p1 = wk.g.nptr[v1] + wk.g.deg[v1];
+                const long long p0 = first_row(v0), p1 = wk.g.nptr[v1] + wk.g.deg[v1];
                 wk.template scan<false, false>(p0, 1, (int)(p1 - p0), v0, 0u, 0u);
                 __syncwarp();
-                wk.template sweep<false>(lane, kWarp);
+                if constexpr (K == 5)
+                    if (ctr[kCtrTris]) {
+                        wk.template houses<false, false>(p0, 1, (int)(p1 - p0), v0, 0u, 0u);
+                        __syncwarp();
+                    }
+                wk.template sweep<false>(lane, kWarp, v0);
                 __syncwarp();
                 todo &= ~take;
             }
@@ -630,7 +731,8 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
         auto run_part = [&](uint32_t vg, uint32_t W, uint32_t part, uint32_t parts, int gi) {
             if (gi != wk.gcur) {
                 // every warp's triangles are counted before the histogram moves on
-                if (wk.held) wk.triangles(wk.held);
+                if constexpr (K == 4)
+                    if (wk.held) wk.triangles(wk.held);
                 wk.held = 0;
                 __syncthreads();
                 if (wib == 0) wk.drain();
@@ -639,8 +741,8 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
                 __syncthreads();
             }
             const uint32_t v = vg - (uint32_t)(wk.g.deg - a.deg), n = (uint32_t)wk.g.n;
-            const long long pb = wk.g.nptr[v] + wk.g.lo[v];
-            const int rows = wk.g.deg[v] - wk.g.lo[v];
+            const long long pb = first_row(v);
+            const int rows = (int)(wk.g.nptr[v] + wk.g.deg[v] - pb);
             const bool wide = rows > kFieldMax;
             const uint32_t fill = wide ? kWideFill : kBlockFill;
             const long long p0 = pb + wib;
@@ -655,8 +757,14 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
                 if (wide) wk.template scan<R, true>(p0, kPWarps, nr, v, lo, hi);
                 else wk.template scan<R, false>(p0, kPWarps, nr, v, lo, hi);
                 __syncthreads();
-                if (wide) wk.template sweep<true>(threadIdx.x, kPThreads);
-                else wk.template sweep<false>(threadIdx.x, kPThreads);
+                if constexpr (K == 5)
+                    if (ctr[kCtrTris]) {
+                        if (wide) wk.template houses<R, true>(p0, kPWarps, nr, v, lo, hi);
+                        else wk.template houses<R, false>(p0, kPWarps, nr, v, lo, hi);
+                        __syncthreads();
+                    }
+                if (wide) wk.template sweep<true>(threadIdx.x, kPThreads, v);
+                else wk.template sweep<false>(threadIdx.x, kPThreads, v);
                 __syncthreads();
             };
             // (a range's wedges may all end in one vertex: its counts fit the
@@ -710,11 +818,11 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
                 end = hi - lo > 2u * width ? lo + 2u * width : hi;
             }
         };
-        const unsigned long long pushed = a.info->queue_tail, tail = min(pushed, a.queue_cap);
+        const unsigned long long pushed = *qtail, tail = min(pushed, a.queue_cap);
         for (;;) {
             __syncthreads();
             if (threadIdx.x == 0) {
-                const unsigned long long idx = atomicAdd(&a.info->queue_head, 1ull);
+                const unsigned long long idx = atomicAdd(qhead, 1ull);
                 item = idx < tail ? a.queue[idx] : make_uint4(0xFFFFFFFFu, 0u, 0u, 0u);
             }
             __syncthreads();
@@ -724,16 +832,18 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial4(PartialArgs a) {
         }
         if (pushed > a.queue_cap) {
             for (long long vg = blockIdx.x; vg < a.gs.NV; vg += gridDim.x)
-                for (uint32_t c = 0; c < 2u && a.wedges[vg] > (uint32_t)kFill; c++)
+                for (uint32_t c = 0; c < 2u && root_wedges[vg] > (uint32_t)kFill; c++)
                     run_part((uint32_t)vg, 0u, c, 2u, a.gs.graph_of((int)vg));
         }
     }
     if (PHASE == 2) {
-        if (wk.held) wk.triangles(wk.held);
+        if constexpr (K == 4)
+            if (wk.held) wk.triangles(wk.held);
         wk.held = 0;
         __syncthreads();
     }
-    if (PHASE == 1 || wib == 0) wk.drain();
+    if constexpr (K == 5) wk.bins.flush();
+    else if (PHASE == 1 || wib == 0) wk.drain();
     if (lane == 0 && wk.scanned) atomicAdd(&a.info->scanned, wk.scanned);
 }
 
@@ -789,10 +899,6 @@ __global__ void __launch_bounds__(kPThreads, 8) k_partial3(PartialArgs a) {
 // Finish: the partial counts that are products of degrees and triangle
 // counters, then the induced counts.
 // ---------------------------------------------------------------------------
-
-__device__ __forceinline__ unsigned long long nd_of(unsigned long long nd, uint32_t s) {
-    return (nd >> (kNdBits * (s - 1u))) & ((1ull << kNdBits) - 1ull);
-}
 
 // Adds a per-thread sum to one class of the block's histogram (whole warp).
 __device__ __forceinline__ void warp_add(uint32_t *hist, const int16_t *lut, int lane, uint32_t code,
@@ -889,7 +995,7 @@ __device__ void induced(const PartialArgs &a, int g, uint32_t *res, unsigned lon
 // Block per (graph, slice of its vertices and edges); the block that ends a
 // graph's last slice turns the partial counts into induced ones.  On the
 // dense block it also zeroes the marked chunks (k_clear_chunks).
-template <int K>
+template <int K, bool INDUCED>
 __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) {
     grid_dep_wait();
     constexpr int N = num_classes(K);
@@ -996,6 +1102,10 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
             const unsigned long long x = (unsigned long long)hist[2 * c] | ((unsigned long long)hist[2 * c + 1] << 32);
             if (x) atomicAdd(&a.part[(size_t)g * N + c], x);
         }
+        if (!INDUCED) {  // (k = 5 reads the partial counts)
+            __syncthreads();
+            continue;
+        }
         fence_device();
         __syncthreads();
         if (threadIdx.x == 0) last = atomicAdd(&a.done[g], 1) == a.slices - 1;
@@ -1006,7 +1116,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
         }
         __syncthreads();
     }
-    if (a.occ)
+    if (INDUCED && a.occ)
         clear_chunks(a.gs, a.state_w, a.occ, a.occ_w, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
                      ((long long)gridDim.x * blockDim.x) >> 5, lane);
 }
@@ -1017,8 +1127,11 @@ bool launched() {
     return false;
 }
 
-constexpr size_t kSmem1 = kPWarps * (kSlots * 16 + kRingP * 16 + 8 * kHits + 8 * num_classes(4)),
-                 kSmem2 = kBlockSlots * 16 + kPWarps * (kRingP * 16 + 8 * kHits) + 8 * num_classes(4);
+// Dynamic shared memory of k_wedges.
+constexpr size_t wedge_smem(int K, int phase) {
+    return (phase == 1 ? warps_of(K) * kSlots : kBlockSlots) * 16 + warps_of(K) * (kRingP * 16 + (K == 4 ? 8 * kHits : 0)) +
+           (K == 5 ? 4 * num_classes(5) : (phase == 1 ? kPWarps : 1) * 8 * num_classes(4));
+}
 
 // The persistent grid times grid_num / grid_den, at least a block per SM.
 int scaled_grid(int per_sm, int num_sms, int grid_num, int grid_den) {
@@ -1026,21 +1139,43 @@ int scaled_grid(int per_sm, int num_sms, int grid_num, int grid_den) {
     return (int)(g < num_sms ? num_sms : g);
 }
 
-template <bool HASH>
-int partial4(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+template <int K, bool HASH>
+int wedges(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
     static bool smem_opt_in = false;
     if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_partial4<1, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem1) != cudaSuccess ||
-            cudaFuncSetAttribute(k_partial4<2, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem2) != cudaSuccess)
+        if (cudaFuncSetAttribute(k_wedges<K, 1, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)wedge_smem(K, 1)) != cudaSuccess ||
+            cudaFuncSetAttribute(k_wedges<K, 2, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)wedge_smem(K, 2)) != cudaSuccess)
             return ACC_ERR_CUDA;
         smem_opt_in = true;
     }
     // (no kernel waits on another block, so the grid need not be resident as a whole)
-    const int grid = scaled_grid(8, num_sms, grid_num, grid_den);
-    launch_pdl(k_partial4<1, HASH>, grid, kPThreads, kSmem1, s, a);
+    const int grid = scaled_grid(K == 5 ? 3 : 8, num_sms, grid_num, grid_den);
+    launch_pdl(k_wedges<K, 1, HASH>, grid, warps_of(K) * kWarp, wedge_smem(K, 1), s, a);
     if (!launched()) return ACC_ERR_CUDA;
-    launch_pdl(k_partial4<2, HASH>, grid, kPThreads, kSmem2, s, a);
+    launch_pdl(k_wedges<K, 2, HASH>, grid, warps_of(K) * kWarp, wedge_smem(K, 2), s, a);
     return launched() ? 2 : ACC_ERR_CUDA;
+}
+
+int grid_prep(long long max_entries, int num_sms) {
+    long long grid = (max_entries + 255) / 256;
+    if (grid > (long long)num_sms * 8) grid = (long long)num_sms * 8;
+    return (int)(grid < 1 ? 1 : grid);
+}
+
+// Blocks of the finish, its slices of a graph: about four blocks per SM over
+// the set, of at least 512 entries each.
+int finish_grid(PartialArgs &a, long long max_entries, int num_sms) {
+    long long sl = (4ll * num_sms + a.gs.B - 1) / a.gs.B;
+    const long long per = max_entries / a.gs.B / 512 + 1;
+    if (sl > per) sl = per;
+    a.slices = (int)(sl < 1 ? 1 : sl);
+    long long fin = (long long)a.gs.B * a.slices;
+    const long long rows = (a.gs.NV * kWarp + kFThreads - 1) / kFThreads;  // a warp a row to clear
+    if (a.occ && fin < rows) fin = rows;
+    if (fin > (long long)num_sms * 8) fin = (long long)num_sms * 8;
+    return (int)fin;
 }
 
 }  // namespace
@@ -1089,11 +1224,8 @@ void partial_matrix(int k, const int16_t *lut, const uint32_t *class_code, std::
 int launch_partial(int k, PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num,
                    int grid_den) {
     int launches = 0;
-    long long grid = (max_entries + 255) / 256;
-    if (grid > (long long)num_sms * 8) grid = (long long)num_sms * 8;
-    if (grid < 1) grid = 1;
-    if (k == 3) launch_pdl(k_partial_prep<3>, (int)grid, 256, 0, s, a);
-    else launch_pdl(k_partial_prep<4>, (int)grid, 256, 0, s, a);
+    if (k == 3) launch_pdl(k_partial_prep<3>, grid_prep(max_entries, num_sms), 256, 0, s, a);
+    else launch_pdl(k_partial_prep<4>, grid_prep(max_entries, num_sms), 256, 0, s, a);
     if (!launched()) return ACC_ERR_CUDA;
     launches++;
     if (k == 3) {
@@ -1103,24 +1235,32 @@ int launch_partial(int k, PartialArgs &a, long long max_entries, int num_sms, cu
         if (!launched()) return ACC_ERR_CUDA;
         launches++;
     } else {
-        const int rc = a.nh ? partial4<true>(a, num_sms, s, grid_num, grid_den)
-                            : partial4<false>(a, num_sms, s, grid_num, grid_den);
+        const int rc = a.nh ? wedges<4, true>(a, num_sms, s, grid_num, grid_den)
+                            : wedges<4, false>(a, num_sms, s, grid_num, grid_den);
         if (rc < 0) return rc;
         launches += rc;
     }
-    // slices of a graph: about four blocks per SM over the set, of at least
-    // 512 entries each
-    long long sl = (4ll * num_sms + a.gs.B - 1) / a.gs.B;
-    const long long per = max_entries / a.gs.B / 512 + 1;
-    if (sl > per) sl = per;
-    a.slices = (int)(sl < 1 ? 1 : sl);
-    long long fin = (long long)a.gs.B * a.slices;
-    const long long rows = (a.gs.NV * kWarp + kFThreads - 1) / kFThreads;  // a warp a row to clear
-    if (a.occ && fin < rows) fin = rows;
-    if (fin > (long long)num_sms * 8) fin = (long long)num_sms * 8;
-    if (k == 3) launch_pdl(k_partial_finish<3>, (int)fin, kFThreads, 0, s, a);
-    else launch_pdl(k_partial_finish<4>, (int)fin, kFThreads, 0, s, a);
+    const int fin = finish_grid(a, max_entries, num_sms);
+    if (k == 3) launch_pdl(k_partial_finish<3, true>, fin, kFThreads, 0, s, a);
+    else launch_pdl(k_partial_finish<4, true>, fin, kFThreads, 0, s, a);
     return launched() ? launches + 1 : ACC_ERR_CUDA;
+}
+
+int launch_partial5_wedges(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num,
+                           int grid_den) {
+    launch_pdl(k_partial_prep<5>, grid_prep(max_entries, num_sms), 256, 0, s, a);
+    if (!launched()) return ACC_ERR_CUDA;
+    const int rc = a.nh ? wedges<4, true>(a, num_sms, s, grid_num, grid_den)
+                        : wedges<4, false>(a, num_sms, s, grid_num, grid_den);
+    if (rc < 0) return rc;
+    const int fin = finish_grid(a, max_entries, num_sms);
+    launch_pdl(k_partial_finish<4, false>, fin, kFThreads, 0, s, a);
+    return launched() ? rc + 2 : ACC_ERR_CUDA;
+}
+
+int launch_partial5_pairs(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+    return a.nh ? wedges<5, true>(a, num_sms, s, grid_num, grid_den)
+                : wedges<5, false>(a, num_sms, s, grid_num, grid_den);
 }
 
 }  // namespace acc

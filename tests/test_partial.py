@@ -1,5 +1,5 @@
-"""The k = 3, 4 counts by partial patterns (csrc/partial.cu), exact integers
-throughout, on graphs at the edges of its tables: roots with as many wedges
+"""The counts by partial patterns (csrc/partial.cu, csrc/partial5.cu), exact
+integers throughout, on graphs at the edges of its tables: roots with as many wedges
 as a warp's or a block's table takes and one more, roots cut into ranges of
 end vertices, roots with more rows than a table's 10-bit fields count, ends
 shared by all rows of a root, and queues too short for every part.
@@ -53,6 +53,11 @@ def fan(rows, ends, pool, seed, filler=0):
 def small_sets(k):
     rng = np.random.default_rng(70 + k)
     gs = []
+    if k == 5:  # (the host runs about 10^5 device threads a graph: few and small ones)
+        s, d = random_digraph(rng, 14, p=0.4, recip=0.5)
+        gs.append((14, np.asarray(s, np.int64), np.asarray(d, np.int64)))
+        g = synth.chung_lu(150, 500, 2.1, 60, 20, 4)
+        return gs + [(g.n, g.src, g.dst), fan(13, 12, 20, 1)]
     for _ in range(7):
         n = int(rng.integers(2, 32))
         s, d = random_digraph(rng, n, p=float(rng.uniform(0.02, 0.6)), recip=float(rng.random()))
@@ -68,7 +73,8 @@ def small_sets(k):
     return gs
 
 
-@pytest.fixture(scope="module", params=["", "-DACC_QUEUE_CAP=3ull"], ids=["queue", "short_queue"])
+@pytest.fixture(scope="module", params=["-DACC_CYCLE_SLOTS=256", "-DACC_QUEUE_CAP=3ull"],
+                ids=["short_tables", "short_queue"])
 def host_lib(request, tmp_path_factory):
     if shutil.which("g++") is None:
         pytest.skip("g++ not available")
@@ -82,7 +88,7 @@ def host_lib(request, tmp_path_factory):
     asan = subprocess.run(["g++", "-print-file-name=libasan.so"], capture_output=True, text=True).stdout.strip()
     san = ["-fsanitize=address", "-DEMU_EXACT_ALLOC", "-DEMU_LANE_STACK=65536"] if os.path.isabs(asan) else []
     procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0",
-                               *filter(None, [request.param]), "-I", EMU, "-I", os.path.join(EMU, "fake"), "-I", CSRC, "-c", u,
+                               request.param, "-I", EMU, "-I", os.path.join(EMU, "fake"), "-I", CSRC, "-c", u,
                                "-o", str(out / f"u{i}.o")], stderr=subprocess.PIPE, text=True) for i, u in enumerate(units)]
     for p in procs:
         err = p.communicate()[1]
@@ -93,7 +99,7 @@ def host_lib(request, tmp_path_factory):
     return so, dict(os.environ, PYTHONPATH=ROOT, **({"LD_PRELOAD": asan, "ASAN_OPTIONS": "detect_leaks=0"} if san else {}))
 
 
-@pytest.mark.parametrize("k", [3, 4])
+@pytest.mark.parametrize("k", [3, 4, 5])
 def test_partial_patterns_on_the_host(host_lib, k):
     so, env = host_lib
     r = subprocess.run([sys.executable, os.path.abspath(__file__), so, str(k)], cwd=ROOT, env=env, capture_output=True,
@@ -107,18 +113,20 @@ def host_main(so, k):
     lib = acc.declare(ctypes.CDLL(so))
     gs = small_sets(k)
     want = [oracle.count(n, s, d, k) for n, s, d in gs]
-    for adj in (acc.ACC_ADJ_AUTO, acc.ACC_ADJ_HASH, acc.ACC_ADJ_SPARSE):
+    for adj in (acc.ACC_ADJ_AUTO, acc.ACC_ADJ_HASH, acc.ACC_ADJ_SPARSE)[k == 5:]:
         c = Ctx(lib)
         ok(lib.acc_ctx_set_adjacency(c.h, adj), "set_adjacency")
-        descs, keep = _descs(gs)
-        ok(lib.acc_motif_batch_prepare(c.h, descs, len(gs), k, None), "batch_prepare")
-        for rep in range(2):
-            out, st = np.zeros((len(gs), NCLS[k]), np.int64), np.full(1, -1, np.int32)
-            ok(lib.acc_motif_batch_run(c.h, None, P(out), P(st)), "batch_run")
-            sync(lib)
-            assert st[0] == 0
-            for i, w in enumerate(want):
-                assert np.array_equal(out[i], w), (adj, rep, i)
+        # (a set of several graphs for k = 3, 4, one graph at a time for k = 5)
+        for sets in ([list(range(len(gs)))] if k < 5 else [[i] for i in range(len(gs))]):
+            descs, keep = _descs([gs[i] for i in sets])
+            ok(lib.acc_motif_batch_prepare(c.h, descs, len(sets), k, None), "batch_prepare")
+            for rep in range(2 if k < 5 else 1):
+                out, st = np.zeros((len(sets), NCLS[k]), np.int64), np.full(1, -1, np.int32)
+                ok(lib.acc_motif_batch_run(c.h, None, P(out), P(st)), "batch_run")
+                sync(lib)
+                assert st[0] == 0
+                for o, i in zip(out, sets):
+                    assert np.array_equal(o, want[i]), (adj, rep, i)
         c.close()
 
 
@@ -133,7 +141,8 @@ def test_partial_patterns_equal_the_walk(rows, ends, pool):
     n, s, d = fan(rows, ends, pool, rows + ends, filler=3000)
     c = acc.Counter(0)
     try:
-        for k in (3, 4):
+        # (k = 5: not where the walk would visit 10^12 subsets; 1024 rows go to the scan)
+        for k in (3, 4, 5) if rows * ends < 10000 and pool > 60 else (3, 4):
             c.set_mode(acc.ACC_MODE_ENUMERATE)
             c.set_adjacency(acc.ACC_ADJ_AUTO)
             want = gpu_count(c, n, s, d, k).tolist()
