@@ -259,12 +259,21 @@ bool uses_formula(const acc_ctx *c, int k, int max_n) {
 
 // The count mode of k = 3, 4 counts by partial patterns (partial.cu) on sets
 // whose vertices are renumbered by degree, from ACC_PARTIAL_MIN_ARCS arcs on
-// (smaller sets are bound by their launches either way and scan their lists).
+// for k = 3 and sets of several graphs, from ACC_PARTIAL_MIN_ARCS1 for one graph
+// of k = 4, 5: the passes of a small graph take longer than its list scan
+// (scan / partial, us: k = 4, 8300 arcs on 4000 vertices 60 / 69 uniform, 73 / 82
+// with hubs; 12000 on 3000 65 / 67 and 117 / 104; 20000 on 5000 78 / 80 and 199 /
+// 119; k = 5, 9000 uniform arcs on 6000 vertices 105 / 145, 12000 on 3000 300 /
+// 186).
 #ifndef ACC_PARTIAL_MIN_ARCS
 #define ACC_PARTIAL_MIN_ARCS 8192
 #endif
-bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel) {
-    return count_family(c) && k <= 4 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS && !uses_formula(c, k, max_n);
+#ifndef ACC_PARTIAL_MIN_ARCS1
+#define ACC_PARTIAL_MIN_ARCS1 (ACC_PARTIAL_MIN_ARCS * 3 / 2)
+#endif
+bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
+    return count_family(c) && k <= 4 && relabel && !uses_formula(c, k, max_n) &&
+           arcs >= (k == 4 && B == 1 ? ACC_PARTIAL_MIN_ARCS1 : ACC_PARTIAL_MIN_ARCS);
 }
 
 // The same for k = 5 (partial5.cu), of one graph; its launches are followed by
@@ -272,7 +281,7 @@ bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relab
 // triangles than the list holds, a root with over 1023 neighbours above it, a
 // count bound near the 64-bit limit).
 bool uses_partial5(const acc_ctx *c, int k, long long arcs, bool relabel, int B) {
-    return count_family(c) && k == 5 && B == 1 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS;
+    return count_family(c) && k == 5 && B == 1 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS1;
 }
 
 // Size limit of one graph: the dense block's, or the sparse build's for the
@@ -294,7 +303,7 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
                      bool relabel) {
     int rc;
     const bool sparse = sparse_build(c, max_n);
-    const bool partial = uses_partial(c, k, max_n, arcs, relabel);
+    const bool partial = uses_partial(c, k, max_n, arcs, relabel, B);
     const bool partial5 = uses_partial5(c, k, arcs, relabel, B);
     if (partial5) {
         if ((rc = grow(&c->p5_vert, &c->p5_vert_cap, 3 * ((size_t)NV + 1)))) return rc;
@@ -397,7 +406,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     bb.occ_w = occ_words(max_n);
     bb.info = c->info;
     bb.k = k;
-    bool partial = gs.NV > 0 && uses_partial(c, k, max_n, gs.M, relabel);
+    bool partial = gs.NV > 0 && uses_partial(c, k, max_n, gs.M, relabel, gs.B);
     bool partial5 = gs.NV > 0 && uses_partial5(c, k, gs.M, relabel, gs.B);
     if (partial5) {
         if (!c->tab5) return ACC_ERR_INTERNAL;  // (the callers ensure it)
@@ -527,7 +536,6 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
             q.div5 = c->tab5;
             q.aut4 = c->tab5 + num_classes(5);
             q.aut3 = q.aut4 + num_classes(4);
-            a.run = q.ctr + kCtrScan;
             rc = launch_partial5(p, 2 * gs.M, c->num_sms, s, c->grid_num, c->grid_den);
         } else {
             rc = launch_partial(k, p, 2 * gs.M, c->num_sms, s, c->grid_num, c->grid_den);

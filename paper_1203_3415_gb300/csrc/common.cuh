@@ -334,7 +334,6 @@ struct EnumArgs {
     long long target;           // schedule: work of one queued chunk of a heavy unit
     unsigned long long *counts; // int64[B * num_classes]
     int *status;
-    const unsigned long long *run = nullptr;  // not NULL: nothing to do while it points to 0
 };
 // batch.cu: Z-scores of each group's real graph against its randomisations.
 int launch_zscores(const long long *counts, int groups, int group_size, int K, double *z, cudaStream_t s);

@@ -1528,7 +1528,6 @@ __global__ void __launch_bounds__(kThreads, K == 5 ? ACC_MINB5 : (COUNT ? (SET ?
     uint32_t *rings = reinterpret_cast<uint32_t *>(smem + L::lut + L::pending + L::hist + L::ebuf + L::groups);
     const int tid = threadIdx.x, lane = tid & 31, wib = tid >> 5;
     constexpr bool several = SET;
-    if (a.run && *(const volatile unsigned long long *)a.run == 0ull) return;  // counted by partial patterns
     // phase 2 with nothing queued: no table to stage, nothing to flush
     if constexpr (PHASE == 2)
         if (a.info->queue_tail == 0) return;

@@ -180,31 +180,57 @@ __global__ void k_clear_chunks(GSet gs, uint32_t *state, const uint32_t *__restr
                  ((long long)gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
 }
 
-// Per-graph histogram dhist[voff + key] of the renumbering keys (clamped to
-// n - 1: the out- plus in-degree can exceed it).
-__global__ void k_dhist(GSet gs, const int *__restrict__ key, int *dhist) {
+// Renumbering of large graphs (above kRelabelSmemMax vertices) by descending
+// key, in classes of equal key: kKeyClasses of them per graph, the last one
+// holding every key from kKeyClasses - 1 on (out- plus in-degrees of 4095 and
+// more are few, and any order of theirs serves).
+constexpr int kKeyClasses = 4096;
+__device__ __forceinline__ int key_classes(int n) { return min(n, kKeyClasses); }
+
+// dhist[voff + class] (class = key, clamped).  One graph: each block counts its
+// tile of vertices in shared memory first (at 10^6 vertices an add per vertex
+// took 195 us, most vertices sharing a few classes).
+constexpr int kKeyTile = 2048;
+__global__ void __launch_bounds__(1024) k_dhist(GSet gs, const int *__restrict__ key, int *dhist) {
     grid_dep_wait();
+    __shared__ int h[kKeyClasses];
+    if (gs.B == 1) {
+        const int C = key_classes(gs.one.n);
+        for (int i = threadIdx.x; i < C; i += blockDim.x) h[i] = 0;
+        __syncthreads();
+        const long long v0 = (long long)blockIdx.x * kKeyTile;
+        for (long long v = v0 + threadIdx.x; v < min(v0 + kKeyTile, gs.NV); v += blockDim.x)
+            atomicAdd(&h[min(key[v], C - 1)], 1);
+        __syncthreads();
+        for (int i = threadIdx.x; i < C; i += blockDim.x)
+            if (h[i]) atomicAdd(&dhist[i], h[i]);
+        return;
+    }
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < gs.NV;
          v += (long long)gridDim.x * blockDim.x) {
         const GMeta mt = gs.meta(gs.graph_of((int)v));
-        atomicAdd(&dhist[mt.voff + min(key[v], mt.n - 1)], 1);
+        atomicAdd(&dhist[mt.voff + min(key[v], key_classes(mt.n) - 1)], 1);
     }
 }
 
-// Block per graph: start[voff + d] = vertices of the graph with degree above d.
+// Block per graph: start[voff + c] = vertices of the graph with class above c.
 __global__ void __launch_bounds__(1024) k_desc_starts(GSet gs, const int *__restrict__ dhist, int *start) {
     grid_dep_wait();
     __shared__ int warp_sum[32];
     const GMeta mt = gs.meta(blockIdx.x);
-    const int n = mt.n;
+    const int C = key_classes(mt.n);
     const int *h = dhist + mt.voff;
     int *st = start + mt.voff;
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
-    const int chunk = (n + blockDim.x - 1) / blockDim.x;
-    // position i of the scan is degree n - 1 - i
-    const int b = min(n, t * chunk), e = min(n, b + chunk);
-    int s = 0;
-    for (int i = b; i < e; i++) s += h[n - 1 - i];
+    constexpr int kPer = kKeyClasses / 1024;
+    // position i of the scan is class C - 1 - i
+    int x[kPer], s = 0;
+#pragma unroll
+    for (int j = 0; j < kPer; j++) {
+        const int i = t * kPer + j;
+        x[j] = i < C ? h[C - 1 - i] : 0;
+        s += x[j];
+    }
     int incl = s;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
@@ -214,32 +240,53 @@ __global__ void __launch_bounds__(1024) k_desc_starts(GSet gs, const int *__rest
     if (lane == 31) warp_sum[wid] = incl;
     __syncthreads();
     if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-        const int ws = lane < nw ? warp_sum[lane] : 0;
+        const int ws = warp_sum[lane];
         int wi = ws;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const int y = __shfl_up_sync(kFull, wi, d);
             if (lane >= d) wi += y;
         }
-        if (lane < nw) warp_sum[lane] = wi - ws;
+        warp_sum[lane] = wi - ws;
     }
     __syncthreads();
     int run = warp_sum[wid] + (incl - s);
-    for (int i = b; i < e; i++) {
-        st[n - 1 - i] = run;
-        run += h[n - 1 - i];
+#pragma unroll
+    for (int j = 0; j < kPer; j++) {
+        const int i = t * kPer + j;
+        if (i < C) st[C - 1 - i] = run;
+        run += x[j];
     }
 }
 
-// label[v] = voff + the next free position of v's key class in its graph
-// (ties in any order); also zeroes dhist (dead once the starts exist).
-__global__ void k_desc_scatter(GSet gs, const int *__restrict__ key, int *start, int *label, int *dhist) {
+// label[v] = voff + the next free position of v's class in its graph (ties in
+// any order).  One graph: a block takes the places of its tile class by class,
+// then deals them out in shared memory.  Also zeroes dhist (dead once the
+// starts exist).
+__global__ void __launch_bounds__(1024) k_desc_scatter(GSet gs, const int *__restrict__ key, int *start, int *label,
+                                                       int *dhist) {
     grid_dep_wait();
+    __shared__ int h[kKeyClasses];
+    if (gs.B == 1) {
+        const int C = key_classes(gs.one.n);
+        for (int i = threadIdx.x; i < C; i += blockDim.x) h[i] = 0;
+        __syncthreads();
+        const long long v0 = (long long)blockIdx.x * kKeyTile, v1 = min(v0 + kKeyTile, gs.NV);
+        for (long long v = v0 + threadIdx.x; v < v1; v += blockDim.x) atomicAdd(&h[min(key[v], C - 1)], 1);
+        __syncthreads();
+        for (int i = threadIdx.x; i < C; i += blockDim.x)
+            if (h[i]) h[i] = atomicAdd(&start[i], h[i]);
+        __syncthreads();
+        for (long long v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+            label[v] = atomicAdd(&h[min(key[v], C - 1)], 1);
+            dhist[v] = 0;
+        }
+        return;
+    }
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < gs.NV;
          v += (long long)gridDim.x * blockDim.x) {
         const GMeta mt = gs.meta(gs.graph_of((int)v));
-        label[v] = mt.voff + atomicAdd(&start[mt.voff + min(key[v], mt.n - 1)], 1);
+        label[v] = mt.voff + atomicAdd(&start[mt.voff + min(key[v], key_classes(mt.n) - 1)], 1);
         dhist[v] = 0;
     }
 }
@@ -991,11 +1038,12 @@ int launch_build_graph(const GSet &gs, const BuildBufs &bb, int max_n, int *stat
         } else {
             int *dhist = bb.deg;  // zeroed above, zeroed again by k_desc_scatter
             int *start = reinterpret_cast<int *>(bb.nptr);
-            launch_pdl(k_dhist, grid_for(NV, 256, num_sms), 256, 0, s, gs, bb.deg_in, dhist);
+            const int key_grid = gs.B == 1 ? (int)((NV + kKeyTile - 1) / kKeyTile) : grid_for(NV, 1024, num_sms);
+            launch_pdl(k_dhist, key_grid, 1024, 0, s, gs, bb.deg_in, dhist);
             if (!launch_ok()) return ACC_ERR_CUDA;
             launch_pdl(k_desc_starts, gs.B, 1024, 0, s, gs, dhist, start);
             if (!launch_ok()) return ACC_ERR_CUDA;
-            launch_pdl(k_desc_scatter, grid_for(NV, 256, num_sms), 256, 0, s, gs, bb.deg_in, start, bb.label, dhist);
+            launch_pdl(k_desc_scatter, key_grid, 1024, 0, s, gs, bb.deg_in, start, bb.label, dhist);
             if (!launch_ok()) return ACC_ERR_CUDA;
             launches += 3;
         }
@@ -1066,11 +1114,12 @@ int launch_build_graph_sparse(const GSet &gs, const BuildBufs &bb, const SparseB
         } else {
             int *dhist = bb.deg;  // zeroed above, zeroed again by k_desc_scatter
             int *start = reinterpret_cast<int *>(bb.nptr);
-            launch_pdl(k_dhist, grid_for(NV, 256, num_sms), 256, 0, s, gs, bb.deg_in, dhist);
+            const int key_grid = gs.B == 1 ? (int)((NV + kKeyTile - 1) / kKeyTile) : grid_for(NV, 1024, num_sms);
+            launch_pdl(k_dhist, key_grid, 1024, 0, s, gs, bb.deg_in, dhist);
             if (!launch_ok()) return ACC_ERR_CUDA;
             launch_pdl(k_desc_starts, gs.B, 1024, 0, s, gs, dhist, start);
             if (!launch_ok()) return ACC_ERR_CUDA;
-            launch_pdl(k_desc_scatter, grid_for(NV, 256, num_sms), 256, 0, s, gs, bb.deg_in, start, bb.label, dhist);
+            launch_pdl(k_desc_scatter, key_grid, 1024, 0, s, gs, bb.deg_in, start, bb.label, dhist);
             if (!launch_ok()) return ACC_ERR_CUDA;
             launches += 3;
         }

@@ -30,17 +30,15 @@ namespace acc {
 
 namespace {
 
-constexpr int kPWarps = 4;           // warps per block (k = 5: twice as many share the block's sums)
+constexpr int kPWarps = 8;           // warps per block
 constexpr int kPThreads = kPWarps * kWarp;
-__host__ __device__ constexpr int warps_of(int K) { return K == 5 ? 2 * kPWarps : kPWarps; }
 // Wedge tables, 16 bytes a slot: one a warp for the roots with few wedges, one
-// a block for the others.
+// a block for the others (k = 5: smaller, beside the block's sums).
 constexpr int kSlots = 192;
 constexpr int kFill = 144;           // most keys a warp's table takes
-constexpr int kBlockSlots = 1024;
-constexpr int kBlockFill = kBlockSlots * 2 / 3;
-constexpr int kWideSlots = kBlockSlots / 2;  // 28-byte slots: key, three words of 21-bit counts
-constexpr int kWideFill = kWideSlots * 2 / 3;
+__host__ __device__ constexpr int block_slots(int K) { return K == 5 ? 1024 : 2048; }
+__host__ __device__ constexpr int wide_slots(int K) { return block_slots(K) / 2; }  // 28-byte slots: key, three words of 21-bit counts
+constexpr int kRowParts = 1024;      // k = 4: rows whose part of a range of ends is kept
 constexpr int kFieldMax = 1023;      // largest count of a 16-byte slot's fields
 constexpr int kRingP = 64;           // rows staged for the flat scan
 constexpr int kRingArrays = 5;       // (k = 4: 4, the root is packed into the entry)
@@ -121,12 +119,15 @@ __global__ void k_partial_prep(PartialArgs a) {
 // A warp's working storage and the graph it counts.
 template <int K, bool HASH>
 struct Walker {
+    static constexpr int kWideSlots = wide_slots(K);
     const PartialArgs *a;
     PView g;
     uint32_t *hist;   // this warp's histogram of partial counts (two words a class)
     Bins5 bins;       // k = 5: the block's sums
     uint4 *tab;       // k = 4, 5: (key, three words of three 10-bit counts)
     uint32_t slots;   // the table's slots
+    const uint2 *parts = nullptr;  // the rows' parts of the range, from row parts0 on, or NULL
+    long long parts0 = 0;
     uint32_t *ring;   // flat start, entry offset, row position, row entry[, row vertex]
     uint32_t *hq;     // k = 4: triangles held (positions of v -> u and u -> w)
     int held;
@@ -467,18 +468,19 @@ struct Walker {
             *first = (uint32_t)(g.nptr[u] + l);
             return g.deg[u] - l;
         } else {
+            if constexpr (RANGED && K == 4)
+                if (parts) {
+                    const uint2 x = parts[p - parts0];
+                    *first = x.x;
+                    return (int)x.y;
+                }
             // (entries below the row's vertex lie between the rows of a shared pass)
             if (K == 4 && (__ldg(a->src + p) >> 31)) return 0;
             const uint2 r = __ldg(a->rev + p);
             *first = r.x;
             int cnt = (int)r.y;
-            if constexpr (RANGED) {
-                if (cnt) {
-                    const int i = lower_id(a->nbr + r.x, cnt, lo);
-                    cnt = lower_id(a->nbr + r.x + i, cnt - i, hi);
-                    *first = r.x + (uint32_t)i;
-                }
-            }
+            if constexpr (RANGED)
+                if (cnt) cnt = id_range(a->nbr, cnt, lo, hi, first);
             return cnt;
         }
     }
@@ -600,24 +602,24 @@ struct Walker {
 // root's first neighbours are hubs with the longest rows.
 //
 // Bound by the latency of list entry, state and table (L2, shared memory).
-// A part re-reads the root's rows (two binary searches a row), so parts are
-// as long as the table allows: on 20000 vertices and 1.35e6 wedges, parts of
-// 160 wedges on one warp's table executed 83e6 warp instructions, this 27e6.
-// Blocks of 16 warps and 4096 slots took 18.2 ms on a set of 4008 graphs (1.4e8
-// wedges of such roots, 900 a root) against 10.6 with 4 warps: their fixed work
-// per warp and part outweighs the fewer searches.
-constexpr int kPart = kBlockFill * 7 / 8, kWidePart = kWideFill * 7 / 8;
-
+// A part re-reads the root's rows (two binary searches a row, side by side, and
+// kept for the scan), so parts are as long as the table allows: on 20000 vertices
+// and 1.35e6 wedges, parts of 160 wedges on one warp's table executed 83e6 warp
+// instructions, this about 27e6.  Measured with blocks of 16 warps and 4096 slots
+// / 4 and 1024 / 8 and 2048: 4008 graphs (1.4e8 wedges of such roots, 900 a root)
+// 18.2 / 10.6 / 10.6 ms in phase 2, and the whole count of 10^6 vertices - /
+// 3.64 / 3.09 ms.
 //
 // k = 5 runs the same passes over the wedges with any middle and the root as
 // the smaller end (K_{2,3}, banners and houses), for one graph.
 template <int K, int PHASE, bool HASH>
-__global__ void __launch_bounds__(warps_of(K) * kWarp, K == 5 ? 3 : 8) k_wedges(PartialArgs a) {
+__global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArgs a) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint4 item;
     __shared__ uint32_t bounds[2];
-    constexpr int kPWarps = warps_of(K), kPThreads = kPWarps * kWarp;
+    constexpr int kBlockSlots = block_slots(K), kBlockFill = kBlockSlots * 2 / 3, kWideFill = wide_slots(K) * 2 / 3,
+                  kPart = kBlockFill * 7 / 8, kWidePart = kWideFill * 7 / 8;
     __shared__ unsigned long long sizes[kPWarps];
     constexpr int N = num_classes(4);
     unsigned long long *ctr = a.p5.ctr;
@@ -639,9 +641,12 @@ __global__ void __launch_bounds__(warps_of(K) * kWarp, K == 5 ? 3 : 8) k_wedges(
     uint32_t *words = reinterpret_cast<uint32_t *>(smem + kTab * 16);
     wk.ring = words + wib * kRingP * 4;
     wk.hq = words + kPWarps * kRingP * 4 + wib * 2 * kHits;
-    // (phase 2: the block is at one graph at a time, one histogram)
-    wk.hist = words + kPWarps * (kRingP * 4 + (K == 4 ? 2 * kHits : 0)) + (PHASE == 1 && K == 4 ? wib * 2 * N : 0);
+    // (one histogram a block when its warps are at one graph at a time: with
+    // one a warp, 4864 warps add to the same few sums at the end)
+    const bool one_hist = PHASE == 2 || K == 5 || a.gs.B == 1;
+    wk.hist = words + kPWarps * (kRingP * 4 + (K == 4 ? 2 * kHits : 0)) + (one_hist ? 0 : wib * 2 * N);
     wk.bins = Bins5{wk.hist, a.p5.sums, a.p5.lut5, a.status};  // (k = 5: one histogram a block)
+    uint2 *row_parts = reinterpret_cast<uint2 *>(wk.hist + (PHASE == 2 && K == 4 ? 2 * N : 0));
     wk.held = 0;
     wk.gcur = -1;
     wk.scanned = 0;
@@ -797,9 +802,16 @@ __global__ void __launch_bounds__(warps_of(K) * kWarp, K == 5 ? 3 : 8) k_wedges(
                 // more than the table takes, the range is halved
                 const uint32_t width = end - lo;
                 unsigned long long S = 0;
+                wk.parts = nullptr;
                 for (int r = threadIdx.x; r < rows; r += kPThreads) {
-                    uint32_t first;
-                    S += (unsigned long long)wk.template row_part<true>(pb + r, lo, end, &first);
+                    uint32_t first = 0;
+                    const int cnt = wk.template row_part<true>(pb + r, lo, end, &first);
+                    if (K == 4 && rows <= kRowParts) row_parts[r] = make_uint2(first, (uint32_t)cnt);
+                    S += (unsigned long long)cnt;
+                }
+                if (K == 4 && rows <= kRowParts) {
+                    wk.parts = row_parts;
+                    wk.parts0 = pb;
                 }
 #pragma unroll
                 for (int d = 16; d; d >>= 1) S += __shfl_xor_sync(kFull, S, d);
@@ -836,14 +848,18 @@ __global__ void __launch_bounds__(warps_of(K) * kWarp, K == 5 ? 3 : 8) k_wedges(
                     run_part((uint32_t)vg, 0u, c, 2u, a.gs.graph_of((int)vg));
         }
     }
-    if (PHASE == 2) {
+    if (one_hist) {
         if constexpr (K == 4)
             if (wk.held) wk.triangles(wk.held);
         wk.held = 0;
         __syncthreads();
     }
-    if constexpr (K == 5) wk.bins.flush();
-    else if (PHASE == 1 || wib == 0) wk.drain();
+    if constexpr (K == 5) {
+        wk.bins.flush();
+    } else {
+        if (one_hist) wk.gcur = PHASE == 1 ? 0 : wk.gcur;
+        if (!one_hist || wib == 0) wk.drain();
+    }
     if (lane == 0 && wk.scanned) atomicAdd(&a.info->scanned, wk.scanned);
 }
 
@@ -852,7 +868,7 @@ __global__ void __launch_bounds__(warps_of(K) * kWarp, K == 5 ? 3 : 8) k_wedges(
 // and are the longest, end up in different grabs; a set of several graphs
 // takes consecutive entries (few graph switches).
 template <bool HASH>
-__global__ void __launch_bounds__(kPThreads, 8) k_partial3(PartialArgs a) {
+__global__ void __launch_bounds__(kPThreads, 4) k_partial3(PartialArgs a) {
     grid_dep_wait();
     constexpr int N = num_classes(3);
     __shared__ uint32_t rings[kPWarps][kRingP * kRingArrays];
@@ -905,7 +921,7 @@ __device__ __forceinline__ void warp_add(uint32_t *hist, const int16_t *lut, int
                                          unsigned long long x) {
 #pragma unroll
     for (int d = 16; d; d >>= 1) x += __shfl_xor_sync(kFull, x, d);
-    if (lane == 0 && x) hist_add(hist, __ldg(lut + code), x);
+    if (lane == 0 && x) hist_add(hist, lut[code], x);
 }
 
 // One undirected edge b - c of G*, seen from the end where its state is 1 or 3:
@@ -930,41 +946,30 @@ __device__ __forceinline__ EdgeEnds edge_ends(uint32_t s, unsigned long long nb,
     return x;
 }
 
-// The terms of an edge with common neighbours (tw: their counts by state to
-// each end): paths that close (a = d, taken out), diamonds on the edge, and
+// The terms of an edge with common neighbours (t: their counts by state to the
+// ends the edge is seen from) that involve their kth nonzero type: paths that
+// close (taken out), diamonds on the edge with a type not before it, and
 // triangles on the edge with a pendant at one end (each of those seen from two
 // edges: these counts are twice the real ones).
-__device__ __forceinline__ void edge_triangles(uint32_t *hist, const int16_t *lut, const EdgeEnds &x,
-                                               unsigned long long t0, unsigned long long t1, unsigned long long t2) {
+__device__ __forceinline__ void edge_triangles(uint32_t *hist, const int16_t *lut, const EdgeEnds &x, const EdgeTri &t,
+                                               int kth) {
     const uint32_t f1 = x.s << 10;
-    uint32_t types = 0;
+    uint32_t m = types_of(t);
+    for (int i = 0; i < kth; i++) m &= m - 1u;
+    const uint32_t z = next_bit(m), i = z / 3u, j = z % 3u;
+    const unsigned long long n = t.get(i, j);
+    hist_add(hist, lut[f1 | ((i + 1u) << 6) | ((j + 1u) << 2)], 0ull - n);
+    const uint32_t code = f1 | (((i + 1u) | ((j + 1u) << 2)) << 6);
+    for (uint32_t r = m; r; r &= r - 1u) {
+        const uint32_t q = next_bit(r);
+        const unsigned long long pairs = q == z ? n * (n - 1u) / 2 : n * t.get(q / 3u, q % 3u);
+        if (pairs) hist_add(hist, lut[code | (q / 3u + 1u) | ((q % 3u + 1u) << 2)], pairs);
+    }
 #pragma unroll
-    for (uint32_t j = 0; j < 3; j++)
-        types |= (nd_of(t0, j + 1u) ? 1u << j : 0u) | (nd_of(t1, j + 1u) ? 8u << j : 0u) |
-                 (nd_of(t2, j + 1u) ? 64u << j : 0u);
-    auto count = [&](uint32_t t) -> unsigned long long {
-        const uint32_t i = t / 3u;
-        return nd_of(i == 0u ? t0 : (i == 1u ? t1 : t2), t - 3u * i + 1u);
-    };
-    // states of a common neighbour to the ends the edge is seen from
-    auto state_b = [&](uint32_t t) -> uint32_t { return x.flip ? t % 3u : t / 3u; };
-    auto state_c = [&](uint32_t t) -> uint32_t { return x.flip ? t / 3u : t % 3u; };
-    for (uint32_t m = types; m; m &= m - 1u) {
-        const uint32_t t = (uint32_t)__ffs((int)m) - 1u, i = state_b(t), j = state_c(t);
-        const unsigned long long n = count(t);
-        hist_add(hist, __ldg(lut + (f1 | ((i + 1u) << 6) | ((j + 1u) << 2))), 0ull - n);
-        const uint32_t code = f1 | (((i + 1u) | ((j + 1u) << 2)) << 6);
-        for (uint32_t r = m; r; r &= r - 1u) {
-            const uint32_t q = (uint32_t)__ffs((int)r) - 1u;
-            const unsigned long long pairs = q == t ? n * (n - 1u) / 2 : n * count(q);
-            if (pairs) hist_add(hist, __ldg(lut + (code | (state_b(q) + 1u) | ((state_c(q) + 1u) << 2))), pairs);
-        }
-#pragma unroll
-        for (uint32_t e = 0; e < 3; e++) {
-            const unsigned long long xb = n * (x.b[e] - (e == i ? 1u : 0u)), xc = n * (x.c[e] - (e == j ? 1u : 0u));
-            if (xb) hist_add(hist, __ldg(lut + (code | (e + 1u))), xb);
-            if (xc) hist_add(hist, __ldg(lut + (code | ((e + 1u) << 2))), xc);
-        }
+    for (uint32_t e = 0; e < 3; e++) {
+        const unsigned long long xb = n * (x.b[e] - (e == i ? 1u : 0u)), xc = n * (x.c[e] - (e == j ? 1u : 0u));
+        if (xb) hist_add(hist, lut[code | (e + 1u)], xb);
+        if (xc) hist_add(hist, lut[code | ((e + 1u) << 2)], xc);
     }
 }
 
@@ -1002,8 +1007,12 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
     __shared__ uint32_t hist[2 * N];
     __shared__ unsigned long long sums[N];
     __shared__ uint32_t lists[kFThreads / kWarp][2 * kWarp];
+    __shared__ __align__(16) int16_t lut_s[1 << code_bits(K)];
     __shared__ int last;
     const int lane = threadIdx.x & 31;
+    if ((long long)blockIdx.x < (long long)a.gs.B * a.slices)
+        for (int i = threadIdx.x; i < (1 << code_bits(K)) / 8; i += blockDim.x)
+            reinterpret_cast<uint4 *>(lut_s)[i] = __ldg(reinterpret_cast<const uint4 *>(a.lut) + i);
     const bool refused = a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW;
     for (long long item = blockIdx.x; !refused && item < (long long)a.gs.B * a.slices; item += gridDim.x) {
         const int g = (int)(item / a.slices), sl = (int)(item % a.slices);
@@ -1041,28 +1050,47 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
         if (K == 3) {
             const uint32_t f[6] = {0x11, 0x22, 0x33, 0x12, 0x13, 0x23};  // (slot 1, slot 2) states
 #pragma unroll
-            for (int i = 0; i < 6; i++) warp_add(hist, a.lut, lane, ((f[i] >> 4) << 4) | (f[i] & 15u), st[i]);
+            for (int i = 0; i < 6; i++) warp_add(hist, lut_s, lane, ((f[i] >> 4) << 4) | (f[i] & 15u), st[i]);
         } else {
             const uint32_t f[10] = {0x111, 0x222, 0x333, 0x112, 0x113, 0x221, 0x223, 0x331, 0x332, 0x123};
 #pragma unroll
             for (int i = 0; i < 10; i++)
-                warp_add(hist, a.lut, lane, ((f[i] >> 8) << 10) | (((f[i] >> 4) & 15u) << 6) | (f[i] & 15u), st[i]);
+                warp_add(hist, lut_s, lane, ((f[i] >> 8) << 10) | (((f[i] >> 4) & 15u) << 6) | (f[i] & 15u), st[i]);
             // paths, diamonds and triangles with a pendant from the edges
             unsigned long long p4[18] = {};
             // (slices of entries, not of vertices: a hub's row is as long as many others)
             const long long b0 = a.nptr[mt.voff], nb = a.nptr[mt.voff + mt.n] - b0;
             const long long e0 = b0 + nb * sl / a.slices, e1 = b0 + nb * (sl + 1) / a.slices;
             // edges with common neighbours are few in a sparse graph: a warp
-            // gathers them and counts 32 at a time
+            // gathers them, and takes 32 at a time by their (edge, type) pairs
+            // (a lane an edge waited for up to a hundred adds one by one)
             uint32_t *list = lists[threadIdx.x >> 5];
             int kept = 0;
+            auto edge_at = [&](uint32_t at, EdgeEnds *x) -> EdgeTri {
+                const long long pos = e0 + at;
+                const uint32_t e = a.nbr[pos];
+                *x = edge_ends(e & 3u, a.nd[a.src[pos]], a.nd[mt.voff + (e >> 2)]);
+                EdgeTri t = edge_tri(a, pos, true);
+                t.flip = x->flip;
+                return t;
+            };
             auto closed = [&](int n) {  // the last n <= 32 gathered
                 __syncwarp();
-                if (lane < n) {
-                    const long long pos = e0 + list[kept - n + lane];
-                    const uint32_t e = a.nbr[pos];
-                    const EdgeEnds x = edge_ends(e & 3u, a.nd[a.src[pos]], a.nd[mt.voff + (e >> 2)]);
-                    edge_triangles(hist, a.lut, x, a.tri[3 * pos], a.tri[3 * pos + 1], a.tri[3 * pos + 2]);
+                EdgeEnds x;
+                const int own = lane < n ? __popc(types_of(edge_at(list[kept - n + lane], &x))) : 0;
+                int tot;
+                const int pre = warp_excl(own, lane, &tot);
+                for (int q0 = 0; q0 < tot; q0 += kWarp) {
+                    const int q = q0 + lane;
+                    int r = 0;
+#pragma unroll
+                    for (int d = 16; d; d >>= 1)
+                        if (__shfl_sync(kFull, pre, r + d) <= q) r += d;
+                    const int k = q - __shfl_sync(kFull, pre, r);
+                    if (q < tot) {
+                        const EdgeTri t = edge_at(list[kept - n + r], &x);
+                        edge_triangles(hist, lut_s, x, t, k);
+                    }
                 }
                 __syncwarp();
             };
@@ -1094,7 +1122,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
             closed(kept);
 #pragma unroll
             for (uint32_t i = 0; i < 18; i++)
-                warp_add(hist, a.lut, lane, ((i < 9 ? 1u : 3u) << 10) | (((i % 9) / 3 + 1u) << 6) | ((i % 3 + 1u) << 2),
+                warp_add(hist, lut_s, lane, ((i < 9 ? 1u : 3u) << 10) | (((i % 9) / 3 + 1u) << 6) | ((i % 3 + 1u) << 2),
                          p4[i]);
         }
         __syncthreads();
@@ -1129,8 +1157,9 @@ bool launched() {
 
 // Dynamic shared memory of k_wedges.
 constexpr size_t wedge_smem(int K, int phase) {
-    return (phase == 1 ? warps_of(K) * kSlots : kBlockSlots) * 16 + warps_of(K) * (kRingP * 16 + (K == 4 ? 8 * kHits : 0)) +
-           (K == 5 ? 4 * num_classes(5) : (phase == 1 ? kPWarps : 1) * 8 * num_classes(4));
+    return (phase == 1 ? kPWarps * kSlots : block_slots(K)) * 16 + kPWarps * (kRingP * 16 + (K == 4 ? 8 * kHits : 0)) +
+           (K == 5 ? 4 * num_classes(5) : (phase == 1 ? kPWarps : 1) * 8 * num_classes(4)) +
+           (phase == 2 && K == 4 ? 8 * kRowParts : 0);
 }
 
 // The persistent grid times grid_num / grid_den, at least a block per SM.
@@ -1151,10 +1180,10 @@ int wedges(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int 
         smem_opt_in = true;
     }
     // (no kernel waits on another block, so the grid need not be resident as a whole)
-    const int grid = scaled_grid(K == 5 ? 3 : 8, num_sms, grid_num, grid_den);
-    launch_pdl(k_wedges<K, 1, HASH>, grid, warps_of(K) * kWarp, wedge_smem(K, 1), s, a);
+    const int grid = scaled_grid(K == 5 ? 3 : 4, num_sms, grid_num, grid_den);
+    launch_pdl(k_wedges<K, 1, HASH>, grid, kPThreads, wedge_smem(K, 1), s, a);
     if (!launched()) return ACC_ERR_CUDA;
-    launch_pdl(k_wedges<K, 2, HASH>, grid, warps_of(K) * kWarp, wedge_smem(K, 2), s, a);
+    launch_pdl(k_wedges<K, 2, HASH>, grid, kPThreads, wedge_smem(K, 2), s, a);
     return launched() ? 2 : ACC_ERR_CUDA;
 }
 
@@ -1229,7 +1258,7 @@ int launch_partial(int k, PartialArgs &a, long long max_entries, int num_sms, cu
     if (!launched()) return ACC_ERR_CUDA;
     launches++;
     if (k == 3) {
-        const int g3 = scaled_grid(8, num_sms, grid_num, grid_den);
+        const int g3 = scaled_grid(4, num_sms, grid_num, grid_den);
         if (a.nh) launch_pdl(k_partial3<true>, g3, kPThreads, 0, s, a);
         else launch_pdl(k_partial3<false>, g3, kPThreads, 0, s, a);
         if (!launched()) return ACC_ERR_CUDA;

@@ -113,6 +113,30 @@ __device__ __forceinline__ int lower_id(const uint32_t *__restrict__ e, int n, u
     return lo;
 }
 
+// The part of the sorted entries e[*first .. *first + n) with ids in [lo, hi):
+// its length, *first moved to its start (both ends searched side by side: the
+// loads of one wait beside the other's).
+__device__ __forceinline__ int id_range(const uint32_t *__restrict__ e, int n, uint32_t lo, uint32_t hi,
+                                        uint32_t *first) {
+    const uint32_t *__restrict__ x = e + *first;
+    const uint32_t k0 = lo << 2, k1 = hi << 2;
+    int a0 = 0, b0 = n, a1 = 0, b1 = n;
+    while (a0 < b0 || a1 < b1) {
+        const int m0 = (a0 + b0) >> 1, m1 = (a1 + b1) >> 1;
+        const uint32_t y0 = a0 < b0 ? __ldg(x + m0) : 0u, y1 = a1 < b1 ? __ldg(x + m1) : 0u;
+        if (a0 < b0) {
+            if (y0 < k0) a0 = m0 + 1;
+            else b0 = m0;
+        }
+        if (a1 < b1) {
+            if (y1 < k1) a1 = m1 + 1;
+            else b1 = m1;
+        }
+    }
+    *first += (uint32_t)a0;
+    return a1 - a0;
+}
+
 __device__ __forceinline__ int warp_excl(int x, int lane, int *total) {
     int incl = x;
 #pragma unroll

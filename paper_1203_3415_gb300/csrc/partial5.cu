@@ -578,10 +578,7 @@ struct CycleWarp {
     __device__ __forceinline__ int part(long long p, uint32_t lo, uint32_t hi, bool all, uint32_t *first) const {
         const uint2 r = __ldg(a->rev + p);
         *first = r.x;
-        if (all || !r.y) return (int)r.y;
-        const int i = lower_id(a->nbr + r.x, (int)r.y, lo);
-        *first = r.x + (uint32_t)i;
-        return lower_id(a->nbr + r.x + i, (int)r.y - i, hi);
+        return all || !r.y ? (int)r.y : id_range(a->nbr, (int)r.y, lo, hi, first);
     }
     __device__ __forceinline__ void fill(long long p0, long long step, int nrows, uint32_t v0, uint32_t lo, uint32_t hi,
                                          bool all) {
@@ -867,6 +864,8 @@ __device__ __forceinline__ uint32_t partition_of(int i) {
 __global__ void k_quotients(PartialArgs a) {
     grid_dep_wait();
     if (scan_instead(a)) return;
+    // the scan's kernels, launched next, find no unit left
+    if (blockIdx.x == 0 && threadIdx.x == 0) a.info->unit_ctr = 1ull << 62;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kSigma * kParts; i += gridDim.x * blockDim.x) {
         int part = i % kParts, sig = i / kParts, sh = 0;
         constexpr int sizes[kShapes] = {81, 81, 243, 243, 243, 243, 729, 729, 729, 729, 2187};
@@ -1071,14 +1070,14 @@ int launch_partial5(PartialArgs &a, long long max_entries, int num_sms, cudaStre
     launch_pdl(k_cycles5<1>, share(3, num_sms, grid_num, grid_den), kCThreads, cycle_smem(1), s, a);
     if (!launched()) return ACC_ERR_CUDA;
     launch_pdl(k_cycles5<2>, share(2, num_sms, grid_num, grid_den), kCThreads, cycle_smem(2), s, a);
-    return launched() ? launches + 5 : ACC_ERR_CUDA;
+    if (!launched()) return ACC_ERR_CUDA;
+    launch_pdl(k_quotients, num_sms * 4, 256, 0, s, a);
+    return launched() ? launches + 6 : ACC_ERR_CUDA;
 }
 
 int launch_partial5_counts(const PartialArgs &a, int num_sms, cudaStream_t s) {
-    launch_pdl(k_quotients, num_sms * 4, 256, 0, s, a);
-    if (!launched()) return ACC_ERR_CUDA;
     launch_pdl(k_counts5, num_sms * 4, 256, kN5 * 4, s, a);
-    return launched() ? 2 : ACC_ERR_CUDA;
+    return launched() ? 1 : ACC_ERR_CUDA;
 }
 
 }  // namespace acc

@@ -138,7 +138,7 @@ def test_partial_patterns_equal_the_walk(rows, ends, pool):
     build.build()
     import paper_1203_3415_gb300 as acc
     from tests.gpu_helpers import gpu_count
-    n, s, d = fan(rows, ends, pool, rows + ends, filler=3000)
+    n, s, d = fan(rows, ends, pool, rows + ends, filler=6000)
     c = acc.Counter(0)
     try:
         # (k = 5: not where the walk would visit 10^12 subsets; 1024 rows go to the scan)
