@@ -260,11 +260,10 @@ bool uses_formula(const acc_ctx *c, int k, int max_n) {
 // The count mode of k = 3, 4 counts by partial patterns (partial.cu) on sets
 // whose vertices are renumbered by degree, from ACC_PARTIAL_MIN_ARCS arcs on
 // for k = 3 and sets of several graphs, from ACC_PARTIAL_MIN_ARCS1 for one graph
-// of k = 4, 5: the passes of a small graph take longer than its list scan
+// of k = 4: the passes of a small graph take longer than its list scan
 // (scan / partial, us: k = 4, 8300 arcs on 4000 vertices 60 / 69 uniform, 73 / 82
 // with hubs; 12000 on 3000 65 / 67 and 117 / 104; 20000 on 5000 78 / 80 and 199 /
-// 119; k = 5, 9000 uniform arcs on 6000 vertices 105 / 145, 12000 on 3000 300 /
-// 186).
+// 119).
 #ifndef ACC_PARTIAL_MIN_ARCS
 #define ACC_PARTIAL_MIN_ARCS 8192
 #endif
@@ -280,8 +279,12 @@ bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relab
 // the scan's, which run only when the device finds that it must (more
 // triangles than the list holds, a root with over 1023 neighbours above it, a
 // count bound near the 64-bit limit).
-bool uses_partial5(const acc_ctx *c, int k, long long arcs, bool relabel, int B) {
-    return count_family(c) && k == 5 && B == 1 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS1;
+// From ACC_PARTIAL_MIN_ARCS arcs on, of at least two a vertex below
+// ACC_PARTIAL_MIN_ARCS1 (scan / partial, us: 8300 uniform arcs on 4000 vertices 182 /
+// 150, 9000 on 6000 105 / 145; with hubs 820 / 312 and 702 / 246).
+bool uses_partial5(const acc_ctx *c, int k, int n, long long arcs, bool relabel, int B) {
+    return count_family(c) && k == 5 && B == 1 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS &&
+           (arcs >= 2ll * n || arcs >= ACC_PARTIAL_MIN_ARCS1);
 }
 
 // Size limit of one graph: the dense block's, or the sparse build's for the
@@ -304,7 +307,7 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
     int rc;
     const bool sparse = sparse_build(c, max_n);
     const bool partial = uses_partial(c, k, max_n, arcs, relabel, B);
-    const bool partial5 = uses_partial5(c, k, arcs, relabel, B);
+    const bool partial5 = uses_partial5(c, k, max_n, arcs, relabel, B);
     if (partial5) {
         if ((rc = grow(&c->p5_vert, &c->p5_vert_cap, 3 * ((size_t)NV + 1)))) return rc;
         if ((rc = grow(&c->p5_sums, &c->p5_sums_cap, (size_t)num_classes(5) + 16 + kCtrs))) return rc;
@@ -407,7 +410,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     bb.info = c->info;
     bb.k = k;
     bool partial = gs.NV > 0 && uses_partial(c, k, max_n, gs.M, relabel, gs.B);
-    bool partial5 = gs.NV > 0 && uses_partial5(c, k, gs.M, relabel, gs.B);
+    bool partial5 = gs.NV > 0 && uses_partial5(c, k, max_n, gs.M, relabel, gs.B);
     if (partial5) {
         if (!c->tab5) return ACC_ERR_INTERNAL;  // (the callers ensure it)
         bb.zero[4] = c->p5_vert;
@@ -605,7 +608,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     if (n < 0 || m < 0 || m >= (1ll << 31)) return ACC_ERR_INPUT;
     if (size_check(c, n)) return ACC_ERR_TOO_LARGE;
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
-    int rc = uses_partial5(c, k, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
+    int rc = uses_partial5(c, k, n, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
     if ((rc = ensure_workspace(c, n, sparse_build(c, n) ? 0 : (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN)))

@@ -204,6 +204,24 @@ __device__ __forceinline__ void grid_dep_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 #endif
 }
+// Lets the stream's next launch_pdl kernel begin beside this one (from where
+// every block has called it or ended).
+__device__ __forceinline__ void grid_dep_launch() {
+#ifdef __CUDA_ARCH__
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+#endif
+}
+// Kernels that run side by side: the first one waits for its predecessor, then
+// lets the next begin; that one (JoinsPrevious) does not wait at its start,
+// since what it reads was complete before the first one let it begin, and waits
+// before it ends, so that whatever follows finds both complete.
+struct JoinsPrevious {
+    __device__ __forceinline__ JoinsPrevious() { grid_dep_launch(); }
+    __device__ __forceinline__ ~JoinsPrevious() { grid_dep_wait(); }
+};
+struct WaitsForPrevious {
+    __device__ __forceinline__ WaitsForPrevious() { grid_dep_wait(); }
+};
 #ifdef __CUDACC__
 template <typename... KArgs, typename... Args>
 inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,

@@ -53,6 +53,7 @@ constexpr int kRanges = 10;
 struct IntRanges {
     int *p[kRanges];
     long long n[kRanges];
+    int count = 4;  // ranges in use, at least 4
 };
 
 __global__ void k_zero(uint4 *p, size_t n16, unsigned char *tail, size_t ntail, int *status,
@@ -64,7 +65,9 @@ __global__ void k_zero(uint4 *p, size_t n16, unsigned char *tail, size_t ntail, 
     if (i < ntail) tail[i] = 0;
     for (size_t j = i; j < (size_t)ncounts; j += stride) counts[j] = 0;
 #pragma unroll
-    for (int r = 0; r < kRanges; r++)
+    for (int r = 0; r < 4; r++)
+        for (size_t j = i; j < (size_t)ints.n[r]; j += stride) ints.p[r][j] = 0;
+    for (int r = 4; r < ints.count; r++)
         for (size_t j = i; j < (size_t)ints.n[r]; j += stride) ints.p[r][j] = 0;
     if (i == 0 && status) *status = 0;
 }
@@ -726,10 +729,18 @@ __device__ __forceinline__ void flip_sort(uint32_t *x, int n, int t, int nt, Syn
     }
 }
 
-// Warp per row of at most kSortSmall raw entries (longer rows are listed in
-// big[] for k_sp_sort_big): sort in the warp's shared buffer, then OR every
-// entry into merged[roff[v] + (its neighbour's rank in the row)] (merged is
-// zero beforehand); deg[v], lo[v] = neighbours of v, those below v.
+// Rows of at most kSortSmall raw entries (longer rows are listed in big[] for
+// k_sp_sort_big): sorted, then every entry OR'ed into merged[roff[v] + (its
+// neighbour's rank in the row)] (merged is zero beforehand); deg[v], lo[v] =
+// neighbours of v, those below v.
+//
+// Rows of more than 32 entries: a warp each, sorted in its shared buffer (the
+// rows of one warp lie a grid apart: the hubs, whose rows are long, come
+// first).  Shorter rows: consecutive ones share a warp, an entry a lane, up to
+// 32 entries and 16 rows, sorted across the lanes by (row, entry).  With a warp
+// per row all through, 10^6 vertices of 6 entries took 705 us, most lanes idle;
+// now SORTUS.
+constexpr int kPackRows = 16;  // rows that share a warp: 4 bits beside an entry's 28
 __global__ void __launch_bounds__(kSortWarps * kWarp) k_sp_sort_small(GSet gs, const long long *__restrict__ roff,
                                                                    const uint32_t *__restrict__ raw,
                                                                    uint32_t *merged, int *deg, int *lo, int *big,
@@ -738,33 +749,92 @@ __global__ void __launch_bounds__(kSortWarps * kWarp) k_sp_sort_small(GSet gs, c
     __shared__ uint32_t buf[kSortWarps][kSortSmall];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     uint32_t *x = buf[wib];
-    const long long nw = (long long)gridDim.x * kSortWarps;
-    for (long long v = blockIdx.x * (long long)kSortWarps + wib; v < gs.NV; v += nw) {
-        const long long r0 = roff[v];
-        const int R = (int)(roff[v + 1] - r0);
-        if (R > kSortSmall) {
-            if (lane == 0) big[atomicAdd(&info->big_rows, 1u)] = (int)v;
-            continue;
+    const long long nw = (long long)gridDim.x * kSortWarps, gw = blockIdx.x * (long long)kSortWarps + wib;
+    for (long long i0 = 0; i0 * nw < gs.NV; i0 += kWarp) {
+        const long long vl = (i0 + lane) * nw + gw;
+        const long long Rl = vl < gs.NV ? roff[vl + 1] - roff[vl] : 0;
+        if (Rl > kSortSmall) big[atomicAdd(&info->big_rows, 1u)] = (int)vl;
+        for (unsigned m = __ballot_sync(kFull, Rl > kWarp && Rl <= kSortSmall); m; m &= m - 1u) {
+            const long long v = (i0 + __ffs(m) - 1) * nw + gw;
+            const long long r0 = roff[v];
+            const int R = (int)(roff[v + 1] - r0);
+            for (int i = lane; i < R; i += kWarp) x[i] = raw[r0 + i];
+            __syncwarp();
+            flip_sort(x, R, lane, kWarp, [] { __syncwarp(); });
+            const uint32_t vloc = (uint32_t)((int)v - gs.meta(gs.graph_of((int)v)).voff);
+            int runs = 0, below = 0;
+            for (int c0 = 0; c0 < R; c0 += kWarp) {
+                const int i = c0 + lane;
+                const uint32_t e = i < R ? x[i] : 0u;
+                const bool start = i < R && (i == 0 || (x[i - 1] >> 2) != (e >> 2));
+                const unsigned ball = __ballot_sync(kFull, start);
+                if (i < R) atomicOr(&merged[r0 + runs + __popc(ball & (0xFFFFFFFFu >> (31 - lane))) - 1], e);
+                below += __popc(__ballot_sync(kFull, start && (e >> 2) < vloc));
+                runs += __popc(ball);
+            }
+            if (lane == 0) {
+                deg[v] = runs;
+                lo[v] = below;
+            }
+            __syncwarp();
         }
-        for (int i = lane; i < R; i += kWarp) x[i] = raw[r0 + i];
-        __syncwarp();
-        flip_sort(x, R, lane, kWarp, [] { __syncwarp(); });
-        const uint32_t vloc = (uint32_t)((int)v - gs.meta(gs.graph_of((int)v)).voff);
-        int runs = 0, below = 0;
-        for (int c0 = 0; c0 < R; c0 += kWarp) {
-            const int i = c0 + lane;
-            const uint32_t e = i < R ? x[i] : 0u;
-            const bool start = i < R && (i == 0 || (x[i - 1] >> 2) != (e >> 2));
+    }
+    for (long long v0 = gw * kWarp; v0 < gs.NV; v0 += nw * kWarp) {
+        const long long v = v0 + lane;
+        const long long r0 = v < gs.NV ? roff[v] : 0;
+        const long long Rl = v < gs.NV ? roff[v + 1] - r0 : 0;
+        uint32_t vloc = 0;
+        if (v < gs.NV) vloc = (uint32_t)((int)v - gs.meta(gs.graph_of((int)v)).voff);
+        const unsigned shorts = __ballot_sync(kFull, v < gs.NV && Rl <= kWarp);
+        for (unsigned todo = shorts; todo;) {
+            // rows s .. s + n - 1, all short
+            const int s = __ffs(todo) - 1;
+            const unsigned gap = ~todo & ~((1u << s) - 1u);
+            const int lim = min(gap ? __ffs(gap) - 1 : kWarp, s + kPackRows);
+            int tot;
+            const int pre = warp_excl_scan(lane >= s && lane < lim ? (int)Rl : 0, lane, &tot);
+            const bool in = lane >= s && lane < lim && pre + (int)Rl <= kWarp;
+            const unsigned take = __ballot_sync(kFull, in);  // (consecutive lanes: pre grows)
+            todo &= ~take;
+            // this lane's entry: the last taken row that starts at or before it
+            int row = s, end = 0;
+#pragma unroll
+            for (int d = 8; d; d >>= 1) {
+                const int c = row + d;
+                const int p = __shfl_sync(kFull, pre, c & 31);
+                if (c < kWarp && ((take >> c) & 1u) && p <= lane) row = c;
+            }
+            end = __shfl_sync(kFull, pre + (int)Rl, row);
+            const long long rb = __shfl_sync(kFull, r0, row);
+            const int first = __shfl_sync(kFull, pre, row);
+            const bool ok = lane >= first && lane < end;
+            uint32_t key = ok ? ((uint32_t)(row - s) << 28) | raw[rb + (lane - first)] : 0xFFFFFFFFu;
+#pragma unroll
+            for (int k = 2; k <= kWarp; k <<= 1)
+#pragma unroll
+                for (int j = k >> 1; j; j >>= 1) {
+                    const uint32_t o = __shfl_xor_sync(kFull, key, j);
+                    const bool up = (lane & k) == 0, lower = (lane & j) == 0;
+                    const uint32_t mn = key < o ? key : o, mx = key < o ? o : key;
+                    key = lower == up ? mn : mx;
+                }
+            // (rows keep their places: the sort is by row first)
+            const uint32_t e = key & 0x0FFFFFFFu, prev = __shfl_up_sync(kFull, key, 1);
+            const bool start = ok && (lane == 0 || (prev >> 2) != (key >> 2));
             const unsigned ball = __ballot_sync(kFull, start);
-            if (i < R) atomicOr(&merged[r0 + runs + __popc(ball & (0xFFFFFFFFu >> (31 - lane))) - 1], e);
-            below += __popc(__ballot_sync(kFull, start && (e >> 2) < vloc));
-            runs += __popc(ball);
+            const uint32_t vr = __shfl_sync(kFull, vloc, row);
+            const unsigned low = __ballot_sync(kFull, start && (e >> 2) < vr);
+            if (ok) {
+                const unsigned mine = ball & (0xFFFFFFFFu >> (31 - lane)) & ~((1u << first) - 1u);
+                atomicOr(&merged[rb + __popc(mine) - 1], e);
+            }
+            if (in) {
+                const int n = (int)Rl;
+                const unsigned seg = n ? (n == kWarp ? kFull : ((1u << n) - 1u) << pre) : 0u;
+                deg[v] = __popc(ball & seg);
+                lo[v] = __popc(low & seg);
+            }
         }
-        if (lane == 0) {
-            deg[v] = runs;
-            lo[v] = below;
-        }
-        __syncwarp();
     }
 }
 
@@ -968,8 +1038,8 @@ long long more_ranges(const BuildBufs &bb, IntRanges &r) {
     long long longest = 0;
     for (int i = 0; i < 6; i++)
         if (bb.zero[i]) {
-            r.p[4 + i] = bb.zero[i];
-            r.n[4 + i] = bb.nzero[i];
+            r.p[r.count] = bb.zero[i];
+            r.n[r.count++] = bb.nzero[i];
             longest = max(longest, bb.nzero[i]);
         }
     return longest;

@@ -612,9 +612,11 @@ struct Walker {
 //
 // k = 5 runs the same passes over the wedges with any middle and the root as
 // the smaller end (K_{2,3}, banners and houses), for one graph.
-template <int K, int PHASE, bool HASH>
+// (BESIDE: k = 4 counted for k = 5, beside the 5-cycles.)
+template <int K, int PHASE, bool HASH, bool BESIDE>
 __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArgs a) {
-    grid_dep_wait();
+    const typename std::conditional<BESIDE, JoinsPrevious, WaitsForPrevious>::type order;
+    if (K == 5) grid_dep_launch();  // k_partial_finish, then k_vertex5 and its followers run beside
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint4 item;
     __shared__ uint32_t bounds[2];
@@ -627,6 +629,8 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArg
     unsigned long long *unit = K == 5 ? ctr + kCtrPairUnit : (ctr ? ctr + kCtrUnit4 : &a.info->unit_ctr),
                        *qtail = K == 5 ? ctr + kCtrPairTail : (ctr ? ctr + kCtrTail4 : &a.info->queue_tail),
                        *qhead = K == 5 ? ctr + kCtrPairHead : (ctr ? ctr + kCtrHead4 : &a.info->queue_head);
+    // (k = 5: the second half of the queue has the 5-cycles' parts)
+    const unsigned long long queue_cap = ctr ? a.queue_cap / 2 : a.queue_cap;
     uint32_t *root_wedges = K == 5 ? a.p5.pair_wedges : a.wedges;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
@@ -691,13 +695,13 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArg
                 unsigned long long base = 0;
                 if (lane == 0) base = atomicAdd(qtail, (unsigned long long)tot);
                 base = __shfl_sync(kFull, base, 0) + (unsigned long long)pre;
-                if (base + parts <= a.queue_cap) {
+                if (base + parts <= queue_cap) {
                     for (uint32_t c = 0; c < parts; c++)
                         a.queue[base + c] = make_uint4((uint32_t)vg, parts == 1u ? W : c, parts, (uint32_t)gi);
                     if (parts) root_wedges[vg] = 0u;
                 } else {
                     for (uint32_t c = 0; c < parts; c++)
-                        if (base + c < a.queue_cap) a.queue[base + c] = make_uint4(0u, 0u, 0u, 0u);
+                        if (base + c < queue_cap) a.queue[base + c] = make_uint4(0u, 0u, 0u, 0u);
                 }
             }
             unsigned todo = __ballot_sync(kFull, W > 0u) & ~heavy;
@@ -830,7 +834,7 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArg
                 end = hi - lo > 2u * width ? lo + 2u * width : hi;
             }
         };
-        const unsigned long long pushed = *qtail, tail = min(pushed, a.queue_cap);
+        const unsigned long long pushed = *qtail, tail = min(pushed, queue_cap);
         for (;;) {
             __syncthreads();
             if (threadIdx.x == 0) {
@@ -842,7 +846,7 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArg
             if (it.x == 0xFFFFFFFFu) break;
             if (it.z) run_part(it.x, it.y, it.y, it.z, (int)it.w);
         }
-        if (pushed > a.queue_cap) {
+        if (pushed > queue_cap) {
             for (long long vg = blockIdx.x; vg < a.gs.NV; vg += gridDim.x)
                 for (uint32_t c = 0; c < 2u && root_wedges[vg] > (uint32_t)kFill; c++)
                     run_part((uint32_t)vg, 0u, c, 2u, a.gs.graph_of((int)vg));
@@ -1002,7 +1006,7 @@ __device__ void induced(const PartialArgs &a, int g, uint32_t *res, unsigned lon
 // dense block it also zeroes the marked chunks (k_clear_chunks).
 template <int K, bool INDUCED>
 __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) {
-    grid_dep_wait();
+    const typename std::conditional<INDUCED, WaitsForPrevious, JoinsPrevious>::type order;  // (beside k_wedges<5, 1>)
     constexpr int N = num_classes(K);
     __shared__ uint32_t hist[2 * N];
     __shared__ unsigned long long sums[N];
@@ -1168,23 +1172,28 @@ int scaled_grid(int per_sm, int num_sms, int grid_num, int grid_den) {
     return (int)(g < num_sms ? num_sms : g);
 }
 
-template <int K, bool HASH>
-int wedges(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+template <int K, int PHASE, bool HASH, bool BESIDE>
+int wedge_phase(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
     static bool smem_opt_in = false;
     if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_wedges<K, 1, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)wedge_smem(K, 1)) != cudaSuccess ||
-            cudaFuncSetAttribute(k_wedges<K, 2, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)wedge_smem(K, 2)) != cudaSuccess)
+        if (cudaFuncSetAttribute(k_wedges<K, PHASE, HASH, BESIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)wedge_smem(K, PHASE)) != cudaSuccess)
             return ACC_ERR_CUDA;
         smem_opt_in = true;
     }
     // (no kernel waits on another block, so the grid need not be resident as a whole)
     const int grid = scaled_grid(K == 5 ? 3 : 4, num_sms, grid_num, grid_den);
-    launch_pdl(k_wedges<K, 1, HASH>, grid, kPThreads, wedge_smem(K, 1), s, a);
-    if (!launched()) return ACC_ERR_CUDA;
-    launch_pdl(k_wedges<K, 2, HASH>, grid, kPThreads, wedge_smem(K, 2), s, a);
-    return launched() ? 2 : ACC_ERR_CUDA;
+    launch_pdl(k_wedges<K, PHASE, HASH, BESIDE>, grid, kPThreads, wedge_smem(K, PHASE), s, a);
+    return launched() ? 1 : ACC_ERR_CUDA;
+}
+
+template <int K, bool BESIDE>
+int wedges(const PartialArgs &a, int phase, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+    if (a.nh)
+        return phase == 1 ? wedge_phase<K, 1, true, BESIDE>(a, num_sms, s, grid_num, grid_den)
+                          : wedge_phase<K, 2, true, BESIDE>(a, num_sms, s, grid_num, grid_den);
+    return phase == 1 ? wedge_phase<K, 1, false, BESIDE>(a, num_sms, s, grid_num, grid_den)
+                      : wedge_phase<K, 2, false, BESIDE>(a, num_sms, s, grid_num, grid_den);
 }
 
 int grid_prep(long long max_entries, int num_sms) {
@@ -1264,10 +1273,11 @@ int launch_partial(int k, PartialArgs &a, long long max_entries, int num_sms, cu
         if (!launched()) return ACC_ERR_CUDA;
         launches++;
     } else {
-        const int rc = a.nh ? wedges<4, true>(a, num_sms, s, grid_num, grid_den)
-                            : wedges<4, false>(a, num_sms, s, grid_num, grid_den);
-        if (rc < 0) return rc;
-        launches += rc;
+        for (int phase = 1; phase <= 2; phase++) {
+            const int rc = wedges<4, false>(a, phase, num_sms, s, grid_num, grid_den);
+            if (rc < 0) return rc;
+            launches += rc;
+        }
     }
     const int fin = finish_grid(a, max_entries, num_sms);
     if (k == 3) launch_pdl(k_partial_finish<3, true>, fin, kFThreads, 0, s, a);
@@ -1275,21 +1285,23 @@ int launch_partial(int k, PartialArgs &a, long long max_entries, int num_sms, cu
     return launched() ? launches + 1 : ACC_ERR_CUDA;
 }
 
-int launch_partial5_wedges(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num,
-                           int grid_den) {
+int launch_partial5_prep(const PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s) {
     launch_pdl(k_partial_prep<5>, grid_prep(max_entries, num_sms), 256, 0, s, a);
-    if (!launched()) return ACC_ERR_CUDA;
-    const int rc = a.nh ? wedges<4, true>(a, num_sms, s, grid_num, grid_den)
-                        : wedges<4, false>(a, num_sms, s, grid_num, grid_den);
-    if (rc < 0) return rc;
-    const int fin = finish_grid(a, max_entries, num_sms);
-    launch_pdl(k_partial_finish<4, false>, fin, kFThreads, 0, s, a);
-    return launched() ? rc + 2 : ACC_ERR_CUDA;
+    return launched() ? 1 : ACC_ERR_CUDA;
 }
 
-int launch_partial5_pairs(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
-    return a.nh ? wedges<5, true>(a, num_sms, s, grid_num, grid_den)
-                : wedges<5, false>(a, num_sms, s, grid_num, grid_den);
+int launch_partial5_wedges(const PartialArgs &a, int phase, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+    return wedges<4, true>(a, phase, num_sms, s, grid_num, grid_den);
+}
+
+int launch_partial5_finish(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s) {
+    const int fin = finish_grid(a, max_entries, num_sms);
+    launch_pdl(k_partial_finish<4, false>, fin, kFThreads, 0, s, a);
+    return launched() ? 1 : ACC_ERR_CUDA;
+}
+
+int launch_partial5_pairs(const PartialArgs &a, int phase, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+    return wedges<5, false>(a, phase, num_sms, s, grid_num, grid_den);
 }
 
 }  // namespace acc

@@ -249,9 +249,11 @@ void partial5_tables(const uint32_t *code5, const uint32_t *code4, const uint32_
 // when ctr[kCtrScan] is set) the counts from them.
 int launch_partial5(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num, int grid_den);
 int launch_partial5_counts(const PartialArgs &a, int num_sms, cudaStream_t s);
-// (partial.cu) typed degrees, 4-cycles, triangles and the partial counts of
-// k = 4, then the pair pass.
-int launch_partial5_wedges(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num, int grid_den);
-int launch_partial5_pairs(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den);
+// (partial.cu) typed degrees; 4-cycles and triangles by phase; the other partial
+// counts of k = 4; the pair pass by phase.
+int launch_partial5_prep(const PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s);
+int launch_partial5_wedges(const PartialArgs &a, int phase, int num_sms, cudaStream_t s, int grid_num, int grid_den);
+int launch_partial5_finish(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s);
+int launch_partial5_pairs(const PartialArgs &a, int phase, int num_sms, cudaStream_t s, int grid_num, int grid_den);
 
 }  // namespace acc

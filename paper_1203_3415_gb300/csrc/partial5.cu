@@ -147,7 +147,7 @@ __device__ void vertex_term(int o, const int16_t *lut3, uint32_t *code, uint32_t
 }
 
 __global__ void __launch_bounds__(kVThreads) k_vertex5(PartialArgs a) {
-    grid_dep_wait();
+    const JoinsPrevious beside;  // k_wedges<5, 2>
     if (scan_instead(a)) return;
     constexpr int kTerms = kTreeTerms + kTriTerms, kPer = (kTerms + kVThreads - 1) / kVThreads;
     __shared__ unsigned long long F[kVTile][kF];
@@ -353,7 +353,7 @@ __device__ void corner_sums(const PartialArgs &a, const PView &g, const Bins5 &b
 }
 
 __global__ void __launch_bounds__(256) k_closed5(PartialArgs a) {
-    grid_dep_wait();
+    const JoinsPrevious beside;  // k_wedges<5, 2>
     if (scan_instead(a)) return;
     const unsigned long long tris = a.p5.ctr[kCtrTris];
     if (!tris) return;
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(256) k_closed5(PartialArgs a) {
 // ---------------------------------------------------------------------------
 template <bool HASH>
 __global__ void __launch_bounds__(256, 2) k_diamonds5(PartialArgs a) {
-    grid_dep_wait();
+    const JoinsPrevious beside;  // k_wedges<5, 2>
     if (scan_instead(a)) return;
     const unsigned long long units = 3ull * a.p5.ctr[kCtrTris];
     if (!units) return;
@@ -665,8 +665,12 @@ struct CycleWarp {
 template <int PHASE>
 __global__ void __launch_bounds__(kCThreads, PHASE == 1 ? 3 : 2) k_cycles5(PartialArgs a) {
     grid_dep_wait();
+    grid_dep_launch();  // k_wedges<4, PHASE> runs beside
     if (scan_instead(a)) return;
     unsigned long long *ctr = a.p5.ctr;
+    // (the second half of the queue: k_wedges<4> has the first)
+    const unsigned long long cap = a.queue_cap / 2;
+    uint4 *queue = a.queue + cap;
     if (PHASE == 2 && ctr[kCtrCycTail] == 0) return;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ uint4 item;
@@ -707,9 +711,9 @@ __global__ void __launch_bounds__(kCThreads, PHASE == 1 ? 3 : 2) k_cycles5(Parti
                 const uint32_t r = W <= (uint32_t)kCFill ? 1u : min(W / (uint32_t)(kCFill / 2) + 1u, 5u);
                 const uint32_t parts = min(r * (r + 1u) / 2u, (uint32_t)kCParts);
                 const unsigned long long i = atomicAdd(&ctr[kCtrCycTail], (unsigned long long)parts);
-                if (i + parts > a.queue_cap) ctr[kCtrScan] = 1ull;
-                for (uint32_t c = 0; c < parts && i + c < a.queue_cap; c++)
-                    a.queue[i + c] = make_uint4((uint32_t)vl, W, c, parts);
+                if (i + parts > cap) ctr[kCtrScan] = 1ull;
+                for (uint32_t c = 0; c < parts && i + c < cap; c++)
+                    queue[i + c] = make_uint4((uint32_t)vl, W, c, parts);
             }
             unsigned todo = __ballot_sync(kFull, W > 0u) & ~heavy;
             while (todo) {
@@ -734,12 +738,12 @@ __global__ void __launch_bounds__(kCThreads, PHASE == 1 ? 3 : 2) k_cycles5(Parti
             }
         }
     } else {
-        const unsigned long long tail = min(ctr[kCtrCycTail], a.queue_cap);
+        const unsigned long long tail = min(ctr[kCtrCycTail], cap);
         for (;;) {
             __syncthreads();
             if (threadIdx.x == 0) {
                 const unsigned long long i = atomicAdd(&ctr[kCtrCycHead], 1ull);
-                item = i < tail ? a.queue[i] : make_uint4(0u, 0u, 0u, 0u);
+                item = i < tail ? queue[i] : make_uint4(0u, 0u, 0u, 0u);
             }
             __syncthreads();
             const uint4 it = item;
@@ -1052,9 +1056,28 @@ int launch_partial5(PartialArgs &a, long long max_entries, int num_sms, cudaStre
             return ACC_ERR_CUDA;
         smem_opt_in = true;
     }
-    int rc = launch_partial5_wedges(a, max_entries, num_sms, s, grid_num, grid_den);
+    // Most of these passes wait on memory or on their last few blocks, so they run
+    // side by side where the data allows (JoinsPrevious): the 5-cycles beside the
+    // wedges of k = 4, then the pairs' first phase beside the finish, then its second
+    // beside the products (5000 vertices, regulatory: MEASURED).
+    int launches = launch_partial5_prep(a, max_entries, num_sms, s);
+    if (launches < 0) return launches;
+    const int grid = share(3, num_sms, grid_num, grid_den);
+    launch_pdl(k_cycles5<1>, grid, kCThreads, cycle_smem(1), s, a);
+    if (!launched()) return ACC_ERR_CUDA;
+    int rc = launch_partial5_wedges(a, 1, num_sms, s, grid_num, grid_den);
     if (rc < 0) return rc;
-    int launches = rc;
+    launch_pdl(k_cycles5<2>, share(2, num_sms, grid_num, grid_den), kCThreads, cycle_smem(2), s, a);
+    if (!launched()) return ACC_ERR_CUDA;
+    rc = launch_partial5_wedges(a, 2, num_sms, s, grid_num, grid_den);
+    if (rc < 0) return rc;
+    rc = launch_partial5_pairs(a, 1, num_sms, s, grid_num, grid_den);
+    if (rc < 0) return rc;
+    rc = launch_partial5_finish(a, max_entries, num_sms, s);
+    if (rc < 0) return rc;
+    rc = launch_partial5_pairs(a, 2, num_sms, s, grid_num, grid_den);
+    if (rc < 0) return rc;
+    launches += 7;
     int tiles = (a.gs.one.n + kVTile - 1) / kVTile;
     if (tiles > 2 * num_sms) tiles = 2 * num_sms;
     launch_pdl(k_vertex5, tiles < 1 ? 1 : tiles, kVThreads, 0, s, a);
@@ -1064,15 +1087,8 @@ int launch_partial5(PartialArgs &a, long long max_entries, int num_sms, cudaStre
     if (a.nh) launch_pdl(k_diamonds5<true>, share(2, num_sms, grid_num, grid_den), 256, kN5 * 4, s, a);
     else launch_pdl(k_diamonds5<false>, share(2, num_sms, grid_num, grid_den), 256, kN5 * 4, s, a);
     if (!launched()) return ACC_ERR_CUDA;
-    rc = launch_partial5_pairs(a, num_sms, s, grid_num, grid_den);
-    if (rc < 0) return rc;
-    launches += rc;
-    launch_pdl(k_cycles5<1>, share(3, num_sms, grid_num, grid_den), kCThreads, cycle_smem(1), s, a);
-    if (!launched()) return ACC_ERR_CUDA;
-    launch_pdl(k_cycles5<2>, share(2, num_sms, grid_num, grid_den), kCThreads, cycle_smem(2), s, a);
-    if (!launched()) return ACC_ERR_CUDA;
     launch_pdl(k_quotients, num_sms * 4, 256, 0, s, a);
-    return launched() ? launches + 6 : ACC_ERR_CUDA;
+    return launched() ? launches + 4 : ACC_ERR_CUDA;
 }
 
 int launch_partial5_counts(const PartialArgs &a, int num_sms, cudaStream_t s) {
