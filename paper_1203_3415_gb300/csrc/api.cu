@@ -141,7 +141,7 @@ int ensure_lut(acc_ctx *c, int k, cudaStream_t s);
 // k = 5 by partial patterns reads the tables of every k, and each class's
 // divisor and the smaller classes' automorphisms (built with the k = 5 table).
 int ensure_tab5(acc_ctx *c, cudaStream_t s) {
-    for (int k = 3; k <= 5; k++) {
+    for (int k = 5; k >= 3; k--) {
         const int rc = ensure_lut(c, k, s);
         if (rc) return rc;
     }

@@ -49,15 +49,17 @@ __device__ __forceinline__ int warp_excl_scan(int x, int lane, int *total) {
     return incl - x;
 }
 
-constexpr int kRanges = 10;
+// Arrays of ints to clear: the build's own, and up to six of the caller's.
+template <int N>
 struct IntRanges {
-    int *p[kRanges];
-    long long n[kRanges];
-    int count = 4;  // ranges in use, at least 4
+    int *p[N];
+    long long n[N];
 };
+constexpr int kRanges = 4, kMoreRanges = kRanges + 6;
 
+template <int N>
 __global__ void k_zero(uint4 *p, size_t n16, unsigned char *tail, size_t ntail, int *status,
-                       unsigned long long *counts, long long ncounts, IntRanges ints) {
+                       unsigned long long *counts, long long ncounts, IntRanges<N> ints) {
     grid_dep_wait();
     size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
     size_t stride = (size_t)gridDim.x * blockDim.x;
@@ -65,9 +67,7 @@ __global__ void k_zero(uint4 *p, size_t n16, unsigned char *tail, size_t ntail, 
     if (i < ntail) tail[i] = 0;
     for (size_t j = i; j < (size_t)ncounts; j += stride) counts[j] = 0;
 #pragma unroll
-    for (int r = 0; r < 4; r++)
-        for (size_t j = i; j < (size_t)ints.n[r]; j += stride) ints.p[r][j] = 0;
-    for (int r = 4; r < ints.count; r++)
+    for (int r = 0; r < N; r++)
         for (size_t j = i; j < (size_t)ints.n[r]; j += stride) ints.p[r][j] = 0;
     if (i == 0 && status) *status = 0;
 }
@@ -179,8 +179,8 @@ __global__ void k_ingest(GSet gs, uint32_t *state, const int *__restrict__ label
 // The marked chunks of the set's pair-state rows back to zero (clear_chunks).
 __global__ void k_clear_chunks(GSet gs, uint32_t *state, const uint32_t *__restrict__ occ, int occ_w) {
     grid_dep_wait();
-    clear_chunks(gs, state, occ, occ_w, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
-                 ((long long)gridDim.x * blockDim.x) >> 5, threadIdx.x & 31);
+    clear_chunks(gs, state, occ, occ_w, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                 (long long)gridDim.x * blockDim.x);
 }
 
 // Renumbering of large graphs (above kRelabelSmemMax vertices) by descending
@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(1024) k_scan_degrees(const int *__restrict__ d
                 for (int j = 0; j < 3; j++) tb[j] += warp_bound[w][j];
             const double bound = count_bound(k, max_n, warp_max[0], tb);
             if (bound > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
-            info->large = bound > kCountLimit / 32;
+            if (k == 5) info->large = bound > kCountLimit / 32;
         }
         info->maxdeg = warp_max[0];
         info->big_rows = 0;
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(1024) k_scan_top(long long *tile_sum, int ntil
         if (k) {
             const double bound = count_bound(k, max_n, info->maxdeg, info->bound);
             if (bound > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
-            info->large = bound > kCountLimit / 32;
+            if (k == 5) info->large = bound > kCountLimit / 32;
         }
         info->big_rows = 0;
         info->big_head = 0;
@@ -739,7 +739,7 @@ __device__ __forceinline__ void flip_sort(uint32_t *x, int n, int t, int nt, Syn
 // first).  Shorter rows: consecutive ones share a warp, an entry a lane, up to
 // 32 entries and 16 rows, sorted across the lanes by (row, entry).  With a warp
 // per row all through, 10^6 vertices of 6 entries took 705 us, most lanes idle;
-// now SORTUS.
+// now 154.
 constexpr int kPackRows = 16;  // rows that share a warp: 4 bits beside an entry's 28
 __global__ void __launch_bounds__(kSortWarps * kWarp) k_sp_sort_small(GSet gs, const long long *__restrict__ roff,
                                                                    const uint32_t *__restrict__ raw,
@@ -1033,13 +1033,18 @@ int grid_for(long long work_items, int per_block, int num_sms) {
     return (int)b;
 }
 
-// Append the caller's arrays to a build's cleared ranges; the longest.
-long long more_ranges(const BuildBufs &bb, IntRanges &r) {
+// The build's cleared ranges followed by the caller's; the longest of those.
+long long more_ranges(const BuildBufs &bb, const IntRanges<kRanges> &own, IntRanges<kMoreRanges> &r) {
     long long longest = 0;
+    r = {};
+    for (int i = 0; i < kRanges; i++) {
+        r.p[i] = own.p[i];
+        r.n[i] = own.n[i];
+    }
     for (int i = 0; i < 6; i++)
         if (bb.zero[i]) {
-            r.p[r.count] = bb.zero[i];
-            r.n[r.count++] = bb.nzero[i];
+            r.p[kRanges + i] = bb.zero[i];
+            r.n[kRanges + i] = bb.nzero[i];
             longest = max(longest, bb.nzero[i]);
         }
     return longest;
@@ -1049,10 +1054,10 @@ long long more_ranges(const BuildBufs &bb, IntRanges &r) {
 
 int launch_zero(void *p, size_t bytes, int num_sms, cudaStream_t s, int *status, unsigned long long *counts,
                 long long ncounts, int *ints, long long nints) {
-    IntRanges r = {{ints}, {ints ? nints : 0}};
+    const IntRanges<1> r = {{ints}, {ints ? nints : 0}};
     const size_t n16 = bytes / 16, ntail = bytes % 16;
     const int grid = grid_for((long long)(n16 > 0 ? n16 : 1), 256 * 4, num_sms);
-    launch_pdl(k_zero, grid, 256, 0, s, reinterpret_cast<uint4 *>(p), n16,
+    launch_pdl(k_zero<1>, grid, 256, 0, s, reinterpret_cast<uint4 *>(p), n16,
                                 reinterpret_cast<unsigned char *>(p) + n16 * 16, ntail, status, counts, ncounts, r);
     return cudaGetLastError() == cudaSuccess ? 1 : ACC_ERR_CUDA;
 }
@@ -1084,14 +1089,17 @@ int launch_build_graph(const GSet &gs, const BuildBufs &bb, int max_n, int *stat
     {
         const size_t bytes = bb.state_clean ? 0 : (size_t)bb.state_words * 4;
         const long long nocc = NV * bb.occ_w;
-        IntRanges r = {{bb.deg, bb.lo, bb.deg_in, reinterpret_cast<int *>(bb.occ)},
+        const IntRanges<kRanges> r = {{bb.deg, bb.lo, bb.deg_in, reinterpret_cast<int *>(bb.occ)},
                        {NV, NV, relabel ? NV : 0, nocc}};
-        const long long extra = more_ranges(bb, r);
+        IntRanges<kMoreRanges> all;
+        const long long extra = more_ranges(bb, r, all);
         const size_t n16 = bytes / 16, ntail = bytes % 16;
         const long long items = (long long)max((size_t)1, max(n16, (size_t)max(max(max(NV, ncounts), nocc), extra)));
-        launch_pdl(k_zero, grid_for(items, 256 * 4, num_sms), 256, 0, s, reinterpret_cast<uint4 *>(bb.state), n16,
-                                                                 reinterpret_cast<unsigned char *>(bb.state) + n16 * 16,
-                                                                 ntail, status, counts, ncounts, r);
+        uint4 *state = reinterpret_cast<uint4 *>(bb.state);
+        unsigned char *tail = reinterpret_cast<unsigned char *>(bb.state) + n16 * 16;
+        const int grid = grid_for(items, 256 * 4, num_sms);
+        if (extra) launch_pdl(k_zero<kMoreRanges>, grid, 256, 0, s, state, n16, tail, ntail, status, counts, ncounts, all);
+        else launch_pdl(k_zero<kRanges>, grid, 256, 0, s, state, n16, tail, ntail, status, counts, ncounts, r);
         if (!launch_ok()) return ACC_ERR_CUDA;
         launches++;
     }
@@ -1167,9 +1175,10 @@ int launch_build_graph_sparse(const GSet &gs, const BuildBufs &bb, const SparseB
     const int arcs_grid = grid_for(max(gs.M, NV), 256, num_sms);
     int *cnt = bb.lo, *cur = bb.deg;  // raw entries per row, then the final neighbours below each vertex
     {
-        IntRanges r = {{bb.deg, bb.lo, bb.deg_in, nullptr}, {NV, NV, relabel ? NV : 0, 0}};
-        const long long items = max(max(max(NV, ncounts), more_ranges(bb, r)), 1ll);
-        launch_pdl(k_zero, grid_for(items, 256 * 4, num_sms), 256, 0, s, nullptr, 0, nullptr, 0, status, counts, ncounts, r);
+        const IntRanges<kRanges> r = {{bb.deg, bb.lo, bb.deg_in, nullptr}, {NV, NV, relabel ? NV : 0, 0}};
+        IntRanges<kMoreRanges> all;
+        const long long items = max(max(max(NV, ncounts), more_ranges(bb, r, all)), 1ll);
+        launch_pdl(k_zero<kMoreRanges>, grid_for(items, 256 * 4, num_sms), 256, 0, s, nullptr, 0, nullptr, 0, status, counts, ncounts, all);
         if (!launch_ok()) return ACC_ERR_CUDA;
         launches++;
     }

@@ -34,8 +34,13 @@ constexpr int kPWarps = 8;           // warps per block
 constexpr int kPThreads = kPWarps * kWarp;
 // Wedge tables, 16 bytes a slot: one a warp for the roots with few wedges, one
 // a block for the others (k = 5: smaller, beside the block's sums).
-constexpr int kSlots = 192;
-constexpr int kFill = 144;           // most keys a warp's table takes
+// A warp's table: of a set of graphs three times as many slots, at half the
+// warps an SM.  A root on a warp takes less work than on a block, whose warps
+// each have their fixed part, so where roots are plenty the warps keep those of
+// up to 384 wedges: 4008 graphs, phases 1 + 2: 1.3 + 9.9 ms with 192 slots, 2.6 +
+// 8.2 with 576.
+constexpr int kSlots = 192, kSetSlots = 576;
+__host__ __device__ constexpr int warp_fill(int slots) { return slots == kSetSlots ? 384 : 144; }  // most keys it takes
 __host__ __device__ constexpr int block_slots(int K) { return K == 5 ? 1024 : 2048; }
 __host__ __device__ constexpr int wide_slots(int K) { return block_slots(K) / 2; }  // 28-byte slots: key, three words of 21-bit counts
 constexpr int kRowParts = 1024;      // k = 4: rows whose part of a range of ends is kept
@@ -613,11 +618,12 @@ struct Walker {
 // k = 5 runs the same passes over the wedges with any middle and the root as
 // the smaller end (K_{2,3}, banners and houses), for one graph.
 // (BESIDE: k = 4 counted for k = 5, beside the 5-cycles.)
-template <int K, int PHASE, bool HASH, bool BESIDE>
-__global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : 4) k_wedges(PartialArgs a) {
+template <int K, int PHASE, bool HASH, bool BESIDE, int SLOTS>
+__global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : (SLOTS == kSetSlots && PHASE == 1 ? 2 : 4)) k_wedges(PartialArgs a) {
     const typename std::conditional<BESIDE, JoinsPrevious, WaitsForPrevious>::type order;
     if (K == 5) grid_dep_launch();  // k_partial_finish, then k_vertex5 and its followers run beside
     extern __shared__ __align__(16) unsigned char smem[];
+    constexpr int kSlots = SLOTS, kFill = warp_fill(SLOTS);
     __shared__ uint4 item;
     __shared__ uint32_t bounds[2];
     constexpr int kBlockSlots = block_slots(K), kBlockFill = kBlockSlots * 2 / 3, kWideFill = wide_slots(K) * 2 / 3,
@@ -933,7 +939,7 @@ __device__ __forceinline__ void warp_add(uint32_t *hist, const int16_t *lut, int
 struct EdgeEnds {
     uint32_t s;
     bool flip;
-    unsigned long long b[3], c[3];
+    uint32_t b[3], c[3];  // (32 bits: their products are one wide multiply each)
 };
 
 __device__ __forceinline__ EdgeEnds edge_ends(uint32_t s, unsigned long long nb, unsigned long long nc) {
@@ -944,8 +950,8 @@ __device__ __forceinline__ EdgeEnds edge_ends(uint32_t s, unsigned long long nb,
     const unsigned long long n0 = x.flip ? nc : nb, n1 = x.flip ? nb : nc;
 #pragma unroll
     for (uint32_t i = 0; i < 3; i++) {
-        x.b[i] = nd_of(n0, i + 1u) - (x.s == i + 1u ? 1u : 0u);
-        x.c[i] = nd_of(n1, i + 1u) - (r == i + 1u ? 1u : 0u);
+        x.b[i] = (uint32_t)nd_of(n0, i + 1u) - (x.s == i + 1u ? 1u : 0u);
+        x.c[i] = (uint32_t)nd_of(n1, i + 1u) - (r == i + 1u ? 1u : 0u);
     }
     return x;
 }
@@ -1110,7 +1116,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
                     for (int i = 0; i < 3; i++)
 #pragma unroll
                         for (int j = 0; j < 3; j++) {
-                            const unsigned long long y = x.b[i] * x.c[j];
+                            const unsigned long long y = (unsigned long long)x.b[i] * x.c[j];
                             p4[3 * i + j] += x.s == 3u ? 0ull : y;
                             p4[9 + 3 * i + j] += x.s == 3u ? y : 0ull;
                         }
@@ -1149,8 +1155,8 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
         __syncthreads();
     }
     if (INDUCED && a.occ)
-        clear_chunks(a.gs, a.state_w, a.occ, a.occ_w, (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5,
-                     ((long long)gridDim.x * blockDim.x) >> 5, lane);
+        clear_chunks(a.gs, a.state_w, a.occ, a.occ_w, blockIdx.x * (long long)blockDim.x + threadIdx.x,
+                     (long long)gridDim.x * blockDim.x);
 }
 
 bool launched() {
@@ -1160,8 +1166,8 @@ bool launched() {
 }
 
 // Dynamic shared memory of k_wedges.
-constexpr size_t wedge_smem(int K, int phase) {
-    return (phase == 1 ? kPWarps * kSlots : block_slots(K)) * 16 + kPWarps * (kRingP * 16 + (K == 4 ? 8 * kHits : 0)) +
+constexpr size_t wedge_smem(int K, int phase, int slots) {
+    return (phase == 1 ? kPWarps * slots : block_slots(K)) * 16 + kPWarps * (kRingP * 16 + (K == 4 ? 8 * kHits : 0)) +
            (K == 5 ? 4 * num_classes(5) : (phase == 1 ? kPWarps : 1) * 8 * num_classes(4)) +
            (phase == 2 && K == 4 ? 8 * kRowParts : 0);
 }
@@ -1172,23 +1178,31 @@ int scaled_grid(int per_sm, int num_sms, int grid_num, int grid_den) {
     return (int)(g < num_sms ? num_sms : g);
 }
 
-template <int K, int PHASE, bool HASH, bool BESIDE>
+template <int K, int PHASE, bool HASH, bool BESIDE, int SLOTS = kSlots>
 int wedge_phase(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
     static bool smem_opt_in = false;
     if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_wedges<K, PHASE, HASH, BESIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)wedge_smem(K, PHASE)) != cudaSuccess)
+        if (cudaFuncSetAttribute(k_wedges<K, PHASE, HASH, BESIDE, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)wedge_smem(K, PHASE, SLOTS)) != cudaSuccess)
             return ACC_ERR_CUDA;
         smem_opt_in = true;
     }
     // (no kernel waits on another block, so the grid need not be resident as a whole)
-    const int grid = scaled_grid(K == 5 ? 3 : 4, num_sms, grid_num, grid_den);
-    launch_pdl(k_wedges<K, PHASE, HASH, BESIDE>, grid, kPThreads, wedge_smem(K, PHASE), s, a);
+    const int grid = scaled_grid(K == 5 ? 3 : (SLOTS == kSetSlots && PHASE == 1 ? 2 : 4), num_sms, grid_num, grid_den);
+    launch_pdl(k_wedges<K, PHASE, HASH, BESIDE, SLOTS>, grid, kPThreads, wedge_smem(K, PHASE, SLOTS), s, a);
     return launched() ? 1 : ACC_ERR_CUDA;
 }
 
 template <int K, bool BESIDE>
 int wedges(const PartialArgs &a, int phase, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
+    if constexpr (K == 4 && !BESIDE) {
+        if (a.gs.B > 1 && a.nh)
+            return phase == 1 ? wedge_phase<K, 1, true, BESIDE, kSetSlots>(a, num_sms, s, grid_num, grid_den)
+                              : wedge_phase<K, 2, true, BESIDE, kSetSlots>(a, num_sms, s, grid_num, grid_den);
+        if (a.gs.B > 1)
+            return phase == 1 ? wedge_phase<K, 1, false, BESIDE, kSetSlots>(a, num_sms, s, grid_num, grid_den)
+                              : wedge_phase<K, 2, false, BESIDE, kSetSlots>(a, num_sms, s, grid_num, grid_den);
+    }
     if (a.nh)
         return phase == 1 ? wedge_phase<K, 1, true, BESIDE>(a, num_sms, s, grid_num, grid_den)
                           : wedge_phase<K, 2, true, BESIDE>(a, num_sms, s, grid_num, grid_den);
@@ -1210,7 +1224,7 @@ int finish_grid(PartialArgs &a, long long max_entries, int num_sms) {
     if (sl > per) sl = per;
     a.slices = (int)(sl < 1 ? 1 : sl);
     long long fin = (long long)a.gs.B * a.slices;
-    const long long rows = (a.gs.NV * kWarp + kFThreads - 1) / kFThreads;  // a warp a row to clear
+    const long long rows = (a.gs.NV * kWarp + kFThreads - 1) / kFThreads;  // (to clear them)
     if (a.occ && fin < rows) fin = rows;
     if (fin > (long long)num_sms * 8) fin = (long long)num_sms * 8;
     return (int)fin;
