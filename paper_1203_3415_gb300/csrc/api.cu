@@ -287,6 +287,29 @@ bool uses_partial5(const acc_ctx *c, int k, int n, long long arcs, bool relabel,
            (arcs >= 2ll * n || arcs >= ACC_PARTIAL_MIN_ARCS1);
 }
 
+// One graph counted by partial patterns that is large enough for its dense block
+// to cost more than sorted rows and hashed tables do takes the sparse build
+// (ACC_ADJ_AUTO).  Measured, dense / sparse, us: k = 3, 250000 arcs on 50000
+// vertices 221 / 235 with hubs, 164 / 152 uniform; 300000 on 100000 296 / 212 and
+// 218 / 155; k = 4, 260000 on 66000 361 / 381 and 229 / 202; 200000 on 100000 298 /
+// 248 and 205 / 162.
+#ifndef ACC_SPARSE_MIN_N
+#define ACC_SPARSE_MIN_N 98304
+#endif
+bool sparse_auto(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
+    return c->adjacency == ACC_ADJ_AUTO && B == 1 && max_n >= ACC_SPARSE_MIN_N &&
+           uses_partial(c, k, max_n, arcs, relabel, B);
+}
+bool sparse_path(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
+    return sparse_build(c, max_n) || sparse_auto(c, k, max_n, arcs, relabel, B);
+}
+// The sparse build waits for the largest degree, which sizes the scan's
+// overflow lists; partial patterns have none, and hold any degree of a graph of
+// kNdMax vertices.
+bool sparse_waits(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
+    return !(uses_partial(c, k, max_n, arcs, relabel, B) && max_n <= kNdMax);
+}
+
 // Size limit of one graph: the dense block's, or the sparse build's for the
 // count mode (local ids fill 26 bits of the extension-list entries).
 int size_check(const acc_ctx *c, long long n) {
@@ -305,7 +328,7 @@ long long sparse_list_entries(int maxdeg) { return (3LL * maxdeg + 64 + 31) & ~3
 int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long arcs, int max_n, int k, int B,
                      bool relabel) {
     int rc;
-    const bool sparse = sparse_build(c, max_n);
+    const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
     const bool partial = uses_partial(c, k, max_n, arcs, relabel, B);
     const bool partial5 = uses_partial5(c, k, max_n, arcs, relabel, B);
     if (partial5) {
@@ -319,7 +342,7 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
         if (k >= 4 && (rc = grow(&c->pp_wedges, &c->pp_wedges_cap, (size_t)NV + 1))) return rc;
         if (k >= 4 && (rc = grow(&c->pp_tri, &c->pp_tri_cap, 3 * (size_t)(2 * arcs) + 1))) return rc;
     }
-    if (uses_hash(c, k, max_n) && (rc = grow(&c->nh, &c->nh_cap, (size_t)kNhWords * (size_t)(2 * arcs) + 4)))
+    if ((sparse || uses_hash(c, k, max_n)) && (rc = grow(&c->nh, &c->nh_cap, (size_t)kNhWords * (size_t)(2 * arcs) + 4)))
         return rc;
     if (sparse) {
         if ((rc = grow(&c->sp_raw, &c->sp_raw_cap, (size_t)(2 * arcs) + 1))) return rc;
@@ -389,7 +412,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     c->timed_call = c->timing;
     if (c->timing && !ok(cudaEventRecord(c->ev[0], s))) return ACC_ERR_CUDA;
     const bool clean = c->state_clean;
-    const bool sparse = sparse_build(c, max_n);
+    const bool sparse = sparse_path(c, k, max_n, gs.M, relabel, gs.B);
     if (!sparse) c->state_clean = false;  // until the closing clear below is enqueued
     // a buffer not known to be clean is swept whole (capacity, not just this
     // set's blocks): a later, larger set may use any part of it
@@ -442,7 +465,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     if (rc < 0) return rc;
     launches += rc;
     long long spw = scratch_per_warp(max_n);
-    if (sparse) {
+    if (sparse && sparse_waits(c, k, max_n, gs.M, relabel, gs.B)) {
         // overflow lists sized by the largest degree: wait for the build
         if (!ok(cudaMemcpyAsync(c->maxdeg_host, &c->info->maxdeg, sizeof(int), cudaMemcpyDeviceToHost, s)) ||
             !ok(cudaStreamSynchronize(s)))
@@ -455,7 +478,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
     }
     // count mode on a large set: probes read hashed tables, built from the
     // sorted neighbour lists
-    const bool hash = gs.NV > 0 && uses_hash(c, k, max_n);
+    const bool hash = gs.NV > 0 && (sparse || uses_hash(c, k, max_n));
     if (hash) {
         rc = launch_nh_build(c->nptr, c->deg, c->nbr, c->src, c->info, 2 * gs.M, c->nh, c->num_sms, s);
         if (rc < 0) return rc;
@@ -611,7 +634,8 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     int rc = uses_partial5(c, k, n, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
-    if ((rc = ensure_workspace(c, n, sparse_build(c, n) ? 0 : (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN)))
+    const bool sparse = sparse_path(c, k, n, m, n >= kRelabelMinN, 1);
+    if ((rc = ensure_workspace(c, n, sparse ? 0 : (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN)))
         return rc;
     GSet gs = {};
     gs.one.rowptr = reinterpret_cast<const long long *>(rowptr);
@@ -627,7 +651,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     gs.M = m;
     int *status = status_user ? status_user : c->status_dev;
     const bool relabel = n >= kRelabelMinN;
-    if (c->graphs && !c->timing && c->state_clean && n > 0 && !sparse_build(c, n)) {
+    if (c->graphs && !c->timing && n > 0 && (sparse ? !sparse_waits(c, k, n, m, relabel, 1) : c->state_clean)) {
         // repeat counts replay one CUDA graph of the whole launch sequence;
         // it is captured (on the context's stream, not run) at the second
         // count with the same key, and only while the pair-state buffer is
@@ -647,10 +671,10 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
         key.grid_num = c->grid_num;
         key.grid_den = c->grid_den;
         key.adjacency = c->adjacency;
-        const void *ws[28] = {c->state, c->deg, c->lo, c->label, c->deg_in, c->nptr, c->tiles, c->nbr, c->occ,
+        const void *ws[32] = {c->state, c->deg, c->lo, c->label, c->deg_in, c->nptr, c->tiles, c->nbr, c->occ,
                               c->info, c->queue, c->scratch, c->lut[k], c->lut_sv[k], c->class_code_dev[k],
                               c->f5_pre, c->status_dev, c->src, c->nh, c->rev, c->pp_nd, c->pp_tri, c->pp_part,
-                              c->pp_wedges, c->pp_done, c->p5_vert, c->p5_sums, c->tab5};
+                              c->pp_wedges, c->pp_done, c->p5_vert, c->p5_sums, c->tab5, c->sp_raw, c->sp_merged, c->sp_roff, c->sp_big};
         memcpy(key.ws, ws, sizeof(ws));
         bool have = c->cg_exec && memcmp(&key, &c->cg_key, sizeof(key)) == 0;
         // capture only when a count repeats: a one-off count runs one by one
@@ -663,7 +687,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
             if (ok(cudaStreamBeginCapture(c->own, cudaStreamCaptureModeRelaxed))) {
                 rc = run_set(c, gs, n, k, relabel, c->own, counts, status);
                 const cudaError_t ce = cudaStreamEndCapture(c->own, &g);
-                c->state_clean = true;  // nothing ran
+                if (!sparse) c->state_clean = true;  // nothing ran
                 if (rc) {
                     if (g) cudaGraphDestroy(g);
                     return rc;
@@ -683,7 +707,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
         }
         if (have) {
             if (!ok(cudaGraphLaunch(c->cg_exec, s))) return ACC_ERR_CUDA;
-            c->state_clean = true;  // the sequence ends with the clear
+            if (!sparse) c->state_clean = true;  // the sequence ends with the clear
             c->last_launches = c->cg_launches;
             c->last_k = k;
             c->last_units = c->cg_units;
@@ -702,7 +726,8 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
 // build): grows nothing when they are the same.
 int batch_workspace(acc_ctx *c) {
     if (size_check(c, c->batch_max_n)) return ACC_ERR_TOO_LARGE;
-    return ensure_workspace(c, c->batch_set.NV, sparse_build(c, c->batch_max_n) ? 0 : c->batch_words, c->batch_arcs,
+    return ensure_workspace(c, c->batch_set.NV,
+                            sparse_path(c, c->batch_k, c->batch_max_n, c->batch_arcs, true, c->batch_set.B) ? 0 : c->batch_words, c->batch_arcs,
                             c->batch_max_n, c->batch_k, c->batch_set.B, true);
 }
 
@@ -713,8 +738,9 @@ namespace acc {
 long long ctx_footprint(const acc_ctx *c, long long n, long long m, int k) {
     const long long pitch = state_pitch((int)n);
     const long long warps = enum_grid_warps(k, c->num_sms);
-    const long long hash_bytes = uses_hash(c, k, (int)n) ? 4LL * kNhWords * (2 * m + 1) : 0;
+    // (a graph that takes the sparse build by sparse_auto needs less than this)
     const bool sparse = sparse_build(c, (int)n);
+    const long long hash_bytes = uses_hash(c, k, (int)n) ? 4LL * kNhWords * (2 * m + 1) : 0;
     // the sparse build keeps raw and merged rows (2 m words each) and row
     // offsets instead of the dense block and its bitmap; its overflow lists
     // are bounded by the largest degree, itself at most 2m and n
@@ -735,7 +761,9 @@ int ctx_reserve(acc_ctx *c, long long n, long long m, int k) {
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     const int rc = ensure_tab5(c, c->own);
     if (rc) return rc;
-    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, n >= kRelabelMinN);
+    const bool relabel = n >= kRelabelMinN;
+    return ensure_workspace(c, n, sparse_path(c, k, (int)n, m, relabel, 1) ? 0 : n * state_pitch((int)n), m, (int)n, k, 1,
+                            relabel);
 }
 
 }  // namespace acc
@@ -910,7 +938,7 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     // (k = 5: also for a run after the mode changed to the count mode)
     int rc = k == 5 && B == 1 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
-    if ((rc = ensure_workspace(c, NV, sparse_build(c, max_n) ? 0 : words, arcs, max_n, k, B, true))) return rc;
+    if ((rc = ensure_workspace(c, NV, sparse_path(c, k, max_n, arcs, true, B) ? 0 : words, arcs, max_n, k, B, true))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;
     if ((rc = grow(&c->gid, &c->gid_cap, (size_t)NV + 1))) return rc;
     if (B > 0 && !ok(cudaMemcpy(c->meta_dev, metas.data(), sizeof(GMeta) * (size_t)B, cudaMemcpyHostToDevice)))

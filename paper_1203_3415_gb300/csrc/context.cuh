@@ -119,7 +119,7 @@ struct acc_ctx {
         const void *rowptr, *col, *counts, *status;
         long long m, light, target;
         int n, k, mode, grid_num, grid_den, adjacency;
-        const void *ws[28];
+        const void *ws[32];
     } cg_key = {}, cg_seen = {};  // the captured graph's key; the last key counted one by one
     int cg_launches = 0;
     long long cg_units = 0;

@@ -667,7 +667,8 @@ __global__ void k_fill(GSet gs, const uint32_t *__restrict__ state, const uint32
 // compacted into the lists.
 // ---------------------------------------------------------------------------
 
-constexpr int kSortSmall = 2048;  // raw entries of a row one warp sorts in shared memory
+constexpr int kSortSmall = 128;   // raw entries of a row one warp sorts in shared memory
+constexpr int kSortShared = 2048; // of a row one block sorts in shared memory
 constexpr int kSortWarps = 4;     // warps per block of the small-row sort
 
 // Raw entries per row (cnt[v], both directions of each arc), after the row
@@ -735,8 +736,7 @@ __device__ __forceinline__ void flip_sort(uint32_t *x, int n, int t, int nt, Syn
 // neighbours of v, those below v.
 //
 // Rows of more than 32 entries: a warp each, sorted in its shared buffer (the
-// rows of one warp lie a grid apart: the hubs, whose rows are long, come
-// first).  Shorter rows: consecutive ones share a warp, an entry a lane, up to
+// rows of one warp lie a grid apart: the longer rows come first).  Shorter rows: consecutive ones share a warp, an entry a lane, up to
 // 32 entries and 16 rows, sorted across the lanes by (row, entry).  With a warp
 // per row all through, 10^6 vertices of 6 entries took 705 us, most lanes idle;
 // now 154.
@@ -839,11 +839,14 @@ __global__ void __launch_bounds__(kSortWarps * kWarp) k_sp_sort_small(GSet gs, c
 }
 
 // Block per listed long row (taken one at a time through info->big_head):
-// the same sort in place in raw (global memory), then the same merge.
+// sorted in shared memory up to kSortShared entries, above that in place in raw
+// (global memory), then merged as above.  (Rows of up to 2048 entries on one
+// warp kept a graph of 50000 vertices with hubs of 500 waiting for 91 us.)
 __global__ void k_sp_sort_big(GSet gs, const long long *__restrict__ roff, uint32_t *raw, uint32_t *merged, int *deg,
                               int *lo, const int *__restrict__ big, GraphInfo *info) {
     grid_dep_wait();
     __shared__ int row, warp_cnt[32], warp_below[32];
+    __shared__ uint32_t buf[kSortShared];
     const int t = threadIdx.x, lane = t & 31, wid = t >> 5, nwarps = blockDim.x >> 5;
     for (;;) {
         if (t == 0) {
@@ -856,6 +859,11 @@ __global__ void k_sp_sort_big(GSet gs, const long long *__restrict__ roff, uint3
         const long long r0 = roff[v];
         const int R = (int)(roff[v + 1] - r0);
         uint32_t *x = raw + r0;
+        if (R <= kSortShared) {
+            for (int i = t; i < R; i += (int)blockDim.x) buf[i] = x[i];
+            x = buf;
+            __syncthreads();
+        }
         flip_sort(x, R, t, (int)blockDim.x, [] {
             __threadfence_block();
             __syncthreads();
@@ -1234,7 +1242,7 @@ int launch_build_graph_sparse(const GSet &gs, const BuildBufs &bb, const SparseB
     launch_pdl(k_sp_sort_small, grid_for((NV + kSortWarps - 1) / kSortWarps, 1, num_sms), kSortWarps * kWarp, 0, s, 
         gs, sb.roff, sb.raw, sb.merged, bb.deg, bb.lo, sb.big, bb.info);
     if (!launch_ok()) return ACC_ERR_CUDA;
-    launch_pdl(k_sp_sort_big, num_sms, 256, 0, s, gs, sb.roff, sb.raw, sb.merged, bb.deg, bb.lo, sb.big, bb.info);
+    launch_pdl(k_sp_sort_big, num_sms * 6, 256, 0, s, gs, sb.roff, sb.raw, sb.merged, bb.deg, bb.lo, sb.big, bb.info);
     if (!launch_ok()) return ACC_ERR_CUDA;
     launches += 2;
     if ((rc = scan(bb.deg, bb.nptr, bb.k)) < 0) return rc;

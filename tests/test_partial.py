@@ -154,5 +154,32 @@ def test_partial_patterns_equal_the_walk(rows, ends, pool):
         c.close()
 
 
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [98303, 98304])
+def test_sparse_build_from_98304_vertices(n):
+    """k = 3, 4 on either side of the size from which partial patterns are
+    counted on sorted rows: the dense block's counts, also when repeated (the
+    count is replayed) and after another graph."""
+    import torch
+    from paper_1203_3415_gb300 import build
+    build.build()
+    import paper_1203_3415_gb300 as acc
+    g = synth.chung_lu(n, 2 * n, 2.2, 300, 10, 31)
+    rowptr, col = g.csr()
+    r, cl = torch.from_numpy(rowptr).cuda(), torch.from_numpy(col).cuda()
+    a, dense = acc.Counter(0), acc.Counter(0)
+    dense.set_adjacency(acc.ACC_ADJ_DENSE)
+    try:
+        for k in (3, 4):
+            want = dense.count(r, cl, g.n, k).cpu().numpy().tolist()
+            out = torch.zeros(acc.NUM_CLASSES[k], dtype=torch.int64, device="cuda")
+            for _ in range(4):
+                out.zero_()
+                assert a.count(r, cl, g.n, k, counts=out).cpu().numpy().tolist() == want
+    finally:
+        a.close()
+        dense.close()
+
+
 if __name__ == "__main__":
     host_main(sys.argv[1], int(sys.argv[2]))
