@@ -373,7 +373,10 @@ ACC_API int acc_motif_copy_table(acc_ctx *ctx, int k, int16_t *h_table);
  *   neighbour-list positions for k = 4, 5), [2] chunks heavy units were split
  *   into, [3] undirected edges |E*|, [4] largest degree in G*, [5] blocks of
  *   each enumeration launch, [6] neighbour entries the last two levels
- *   scanned (ACC_MODE_COUNT; 0 in ACC_MODE_ENUMERATE).
+ *   scanned (ACC_MODE_COUNT; 0 in ACC_MODE_ENUMERATE); where the count mode
+ *   counts by partial patterns (see ACC_MODE_COUNT) [2] is the parts of the
+ *   roots with many wedges and [6] the neighbour entries its wedge and
+ *   triangle passes read.
  */
 #define ACC_STATS_LEN 7
 ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);
@@ -388,6 +391,15 @@ ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);
  *   set of at least 8192 arcs the build also stores, per neighbour entry
  *   v -> x, where x's list passes v (8 bytes per entry), so the scans of
  *   the root's neighbours' lists start without a search.
+ *   Larger sets are counted by partial patterns instead: non-induced
+ *   occurrences of each class, from typed degrees, wedges, triangles and (k =
+ *   5) 5-cycles and diamonds, and the induced counts from them by inclusion
+ *   and exclusion.  Taken from 8192 arcs on for k = 3 and for sets of several
+ *   graphs (k = 4), from 12288 for one graph of k = 4, and for one graph of k = 5
+ *   from 8192 (below 12288: of at least two arcs a vertex); one graph of fewer
+ *   than 1024 vertices is never counted so.  A k = 5 graph with a vertex of over
+ *   1023 neighbours after it in degree order, with more triangles than the
+ *   workspace lists, or with a count bound above 2^57 is left to the lists.
  *  ACC_MODE_ENUMERATE: every k-subset is visited and classified on its own.
  *  ACC_MODE_FORMULA: for k = 3, the paper's per-vertex formulas (Thm teo3,
  *   Algorithm s3, Table starb): open triples from the sizes of each vertex's
@@ -428,12 +440,14 @@ ACC_API int acc_ctx_set_mode(acc_ctx *ctx, int mode);
  *   the lists), one 16-byte load per probe in the common case.
  *  ACC_ADJ_SPARSE: the same hashed tables, and the neighbour lists built
  *   without the dense block: every arc puts a raw entry in both endpoints'
- *   rows, each row is sorted (one warp in shared memory up to 2048 raw
- *   entries, one block in global memory above) and its repeated neighbours
- *   merged.  Memory O(n + m); the call waits once for the build (the
- *   per-warp overflow lists are sized by the largest degree it finds), so it
- *   is never replayed from a launch graph.
- *  ACC_ADJ_AUTO (default): sparse above ACC_MAX_N vertices; hashed when the
+ *   rows, each row is sorted (short rows several to a warp, rows of over 128
+ *   raw entries by a block, in shared memory up to 2048) and its repeated
+ *   neighbours merged.  Memory O(n + m).  Where the lists are scanned (see
+ *   ACC_MODE_COUNT) the call waits once for the build (the per-warp overflow
+ *   lists are sized by the largest degree it finds) and is never replayed from
+ *   a launch graph.
+ *  ACC_ADJ_AUTO (default): sparse above ACC_MAX_N vertices, and from 98304 for
+ *   one graph of k = 3, 4 counted by partial patterns; hashed when the
  *   largest graph of the count or batch has at least 49152 vertices for
  *   k = 5, 131072 for k = 3, 4 (where the dense probes, out of L2, get slower
  *   than the hashed ones); dense otherwise.
@@ -453,7 +467,8 @@ ACC_API int acc_ctx_set_adjacency(acc_ctx *ctx, int adjacency);
  * estimated work is at most `light` runs whole on one warp; a heavier one is
  * cut into row tiles of about `target` work that any warp may take.  Work is
  * counted in scanned neighbour entries (count mode) or leaves (enumerate
- * mode).  0 selects the built-in default: light 2048 and target 4096, except
+ * mode); counting by partial patterns does not read it.  0 selects the built-in
+ * default: light 2048 and target 4096, except
  * in the count mode light 6144 for k = 4 and target 16384 for k = 5 (whose
  * tiles share one scan of the level-2 rows, so longer tiles save work).
  * Values above 2^40 or negative are ACC_ERR_ARG.  The schedule changes speed

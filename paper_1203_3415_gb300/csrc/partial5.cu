@@ -51,6 +51,8 @@ __device__ __forceinline__ PView view5(const PartialArgs &a) { return pview(a, a
 // sums of four of them from their neighbours, then a thread per product adds
 // its term for each.
 // ---------------------------------------------------------------------------
+// 60000 vertices: 81 us (211 with the stars' binomials on 15 threads and tiles of
+// 32 vertices); bound by the gather's loads and, on small graphs, by its few tiles.
 constexpr int kVWarps = 8, kVThreads = kVWarps * kWarp, kVTile = 16;
 constexpr int kF = 49;  // n[3], q[9], t[27], 1, n choose 2, 3, 4 [3 each]
 constexpr int kTreeTerms = 54 + 45 + 15 + 8, kTriTerms = 27 * 6 + 27 * 9 + 378;
@@ -249,7 +251,10 @@ __global__ void __launch_bounds__(kVThreads) k_vertex5(PartialArgs a) {
 // Products at an edge with common neighbours and at a triangle.
 // ---------------------------------------------------------------------------
 
-// Thread per edge (upper entry): triangles on it with a pendant at both ends
+// Thread per edge (upper entry), and per triangle corner below: 27 us on 866
+// triangles, 88 on 16000 (157 with a thread per triangle over all type pairs, not
+// only the nonzero ones); bound by the chains of class lookups and adds.
+// On an edge: triangles on it with a pendant at both ends
 // (twice: the ends may be swapped), two of them with a pendant at one end, and
 // three of them.
 __device__ void edge_sums(const PartialArgs &a, const PView &g, const Bins5 &bins, long long pos) {
@@ -375,7 +380,9 @@ __global__ void __launch_bounds__(256) k_closed5(PartialArgs a) {
 // Diamonds.  A warp takes a triangle's edge as the spine x < y and its third
 // vertex a as a tip, finds the other tips b > a among the neighbours of y
 // (adjacent to x too), and for each reads the neighbours z of b adjacent to a:
-// with them everything that holds the diamond and a vertex on both tips.
+// with them everything that holds the diamond and a vertex on both tips.  208 us
+// for 1.9e5 diamonds (1899 vertices, 20296 arcs), 18 us for 1600: the reads of the
+// tips' lists and two to four states an entry, from L2.
 // ---------------------------------------------------------------------------
 template <bool HASH>
 __global__ void __launch_bounds__(256, 2) k_diamonds5(PartialArgs a) {
@@ -473,7 +480,10 @@ __global__ void __launch_bounds__(256, 2) k_diamonds5(PartialArgs a) {
 // their end x (a table, as in partial.cu, with the state of c and x in the
 // first word's top bits), then for every edge x - y between two ends the pairs
 // of a wedge to x and a wedge to y.  Wedges through the other end are left out
-// there; pairs through one vertex are taken off by triangle_sums.
+// there; pairs through one vertex are taken off by corner_sums.  Bound by the
+// latency of the list entries and table lookups; roots with up to 128 wedges take
+// a warp, the others a block (60000 vertices: 116 + 214 us; with 25 roots a grab
+// phase 1 took 1809, with two searched ranges for every root phase 2 took 372).
 // ---------------------------------------------------------------------------
 constexpr int kCWarps = 8, kCThreads = kCWarps * kWarp;
 #ifndef ACC_CYCLE_SLOTS
@@ -864,7 +874,8 @@ __device__ __forceinline__ uint32_t partition_of(int i) {
 
 // Thread per (pattern, states, partition of its vertices): the sum counts the
 // maps that join the partition's vertices, as many as the injective maps of
-// the quotient pattern: automorphisms times its partial count.
+// the quotient pattern: automorphisms times its partial count.  17 us (64 with the
+// partitions decoded by a loop).
 __global__ void k_quotients(PartialArgs a) {
     grid_dep_wait();
     if (scan_instead(a)) return;
@@ -945,7 +956,7 @@ __global__ void k_quotients(PartialArgs a) {
 
 // Inclusion and exclusion: class c with partial count P adds (-1)^(edges left
 // out) P to the class of every subset of its edges that connects the five
-// vertices.  Thread per (class, subset).
+// vertices.  Warp per class, a lane a subset: 12 to 30 us by the classes present.
 __global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {
     grid_dep_wait();
     if (scan_instead(a)) return;
@@ -1059,7 +1070,8 @@ int launch_partial5(PartialArgs &a, long long max_entries, int num_sms, cudaStre
     // Most of these passes wait on memory or on their last few blocks, so they run
     // side by side where the data allows (JoinsPrevious): the 5-cycles beside the
     // wedges of k = 4, then the pairs' first phase beside the finish, then its second
-    // beside the products (5000 vertices, regulatory: MEASURED).
+    // beside the products (5000 vertices, regulatory: 506 us one
+    // after another, 459 side by side; 1899 vertices, 20296 arcs: 1657 and 1411).
     int launches = launch_partial5_prep(a, max_entries, num_sms, s);
     if (launches < 0) return launches;
     const int grid = share(3, num_sms, grid_num, grid_den);
