@@ -483,7 +483,7 @@ def measure_single(env, workload, steps, warmup, mode="count", schedule="", cpu_
                    "parallelism": f"replicas{env.world}"},
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_gops, "unit": "Gop/s",
                      "frac": achieved / peak_gops, "traffic": traffic,
-                     "kernel": "k_formula3" if eff == "formula" and k == 3 else f"k_enum<{k}> (phase 1 + phase 2)",
+                     "kernel": "k_formula3" if eff == "formula" and k == 3 else f"the passes after the build (k = {k})",
                      "work_unit": unit_name, "units_per_launch": units, "ops_per_unit": per_unit,
                      "peak_source": peak_src,
                      # what a kernel visiting every leaf would have to sustain for this rate
@@ -692,7 +692,7 @@ def measure_batch(env, steps, warmup, cpu_baseline=True, cpu_budget_s=10.0):
                                  "how": "acc_motif_count per graph, same stream, same GPU"},
         "batched_over_single": value / single_rate,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_gops, "unit": "Gop/s",
-                     "frac": achieved / peak_gops, "traffic": None, "kernel": "k_enum<4> (phase 1 + phase 2)",
+                     "frac": achieved / peak_gops, "traffic": None, "kernel": "the passes after the build (k = 4)",
                      "work_unit": "neighbour entries the count's passes read", "units_per_launch": scanned,
                      "ops_per_unit": ops_per_scanned_entry(4), "peak_source": peak_src,
                      "enumerate_ms": statistics.mean(enum_ms)},
