@@ -641,7 +641,7 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : (SLOTS == kSetSlots &&
     uint32_t *root_wedges = K == 5 ? a.p5.pair_wedges : a.wedges;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
-    if (K == 5 && *(volatile unsigned long long *)(ctr + kCtrScan)) return;
+    if (K == 5 && scan_instead(a)) return;
     if (PHASE == 2 && *qtail == 0) return;
     uint4 *tabs = reinterpret_cast<uint4 *>(smem);
     Walker<K, HASH> wk;

@@ -219,6 +219,20 @@ __device__ __forceinline__ EdgeTri edge_tri(const PartialArgs &a, long long p, b
     return EdgeTri{{a.tri[3 * q], a.tri[3 * q + 1], a.tri[3 * q + 2]}, !upper};
 }
 
+// k = 5: whether the list scan counts the set instead (or the build refused it).
+// One answer for the whole block, which every thread must ask for before any
+// other barrier: the flag may be raised while a kernel's blocks start, by the
+// kernel itself or one beside it, and a warp that left while others of its block
+// stayed would leave its share of the tables uncleared.
+__device__ __forceinline__ bool scan_instead(const PartialArgs &a) {
+    __shared__ int instead;
+    if (threadIdx.x == 0)
+        instead = *(volatile unsigned long long *)(a.p5.ctr + kCtrScan) != 0ull ||
+                  (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW);
+    __syncthreads();
+    return instead != 0;
+}
+
 // Nonzero types of an edge's common neighbours: bit 3 i + j for states i + 1 and
 // j + 1 to the ends the edge is seen from.
 __device__ __forceinline__ uint32_t types_of(const EdgeTri &t) {

@@ -33,10 +33,6 @@ namespace {
 
 constexpr int kN5 = num_classes(5);
 
-__device__ __forceinline__ bool scan_instead(const PartialArgs &a) {
-    return *(volatile unsigned long long *)(a.p5.ctr + kCtrScan) != 0ull ||
-           (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW);
-}
 
 __device__ __forceinline__ Bins5 bins5(const PartialArgs &a, uint32_t *lo) {
     return Bins5{lo, a.p5.sums, a.p5.lut5, a.status};

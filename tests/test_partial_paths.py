@@ -1,0 +1,166 @@
+"""The ways a count by partial patterns (csrc/partial.cu, csrc/partial5.cu) can
+take besides the common one, on the host: the library's own source runs there
+(tests/emu) with the size threshold at 0, against the oracle.
+
+The graphs that take these ways in earnest are too large for the host, so the
+sources' limits are read from the environment where EDITS puts emu_env (their
+own value where the variable is not set), and k_cycles5 can be told to find the
+return to the list scan raised while the warps of its first block start."""
+import ctypes
+import json
+import os
+import shutil
+import subprocess
+import sys
+
+import numpy as np
+import pytest
+
+import oracle
+from tests.test_partial import fan
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+HOOKS = r"""
+#include "shim.h"
+inline unsigned long long emu_env(const char *name, unsigned long long own) {
+    const char *e = getenv(name);
+    return e ? strtoull(e, nullptr, 10) : own;
+}
+extern unsigned long long emu_scans;  // k = 5 counts left to the list scan
+// k_cycles5<phase>: what other blocks left in shared memory, as the first thread
+// of a block finds it, and the flag raised when thread EMU_RAISE_AT of the first block
+// arrives
+template <class A> inline void emu_cycles_enter(const A &a, unsigned long long *flag, int phase, size_t smem) {
+    static unsigned entered = 0;
+    if (emu_env("EMU_RAISE_PHASE", 0) != (unsigned long long)phase) return;
+    if (entered % blockDim.x == 0) memset(emu_dyn_smem, 0xA5, smem);
+    if (entered++ < blockDim.x && threadIdx.x == emu_env("EMU_RAISE_AT", 0)) *flag = 1;
+}
+"""
+
+# (source file, text in it, what stands there for these tests)
+EDITS = [
+    ("partial5.cu", "    grid_dep_launch();  // k_wedges<4, PHASE> runs beside\n",
+     "    emu_cycles_enter(a, a.p5.ctr + kCtrScan, PHASE, cycle_smem(PHASE));\n"),
+    ("partial5.cu", "template <int PHASE>\n__global__ void __launch_bounds__(kCThreads",
+     "constexpr size_t cycle_smem(int phase);\ntemplate <int PHASE>\n__global__ void __launch_bounds__(kCThreads"),
+    ("partial5.cu", "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n    grid_dep_wait();\n",
+     "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n"
+     "    if (threadIdx.x == 0 && blockIdx.x == 0 && a.p5.ctr[kCtrScan]) emu_scans++;\n"),
+]
+
+
+@pytest.fixture(scope="module")
+def host_lib(tmp_path_factory):
+    if shutil.which("g++") is None:
+        pytest.skip("g++ not available")
+    from tests.test_cpu_emulation import CSRC, EMU, _launches_to_calls
+    out = tmp_path_factory.mktemp("partial_paths")
+    units = [os.path.join(EMU, "emu_rt.cpp"), str(out / "hooks.cpp")]
+    open(out / "hooks.h", "w").write("#pragma once\n" + HOOKS)
+    open(units[1], "w").write('#include "hooks.h"\nunsigned long long emu_scans = 0;\n'
+                              'extern "C" unsigned long long emu_scan_count() { return emu_scans; }\n')
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith(".cu"):
+            src = open(os.path.join(CSRC, name)).read()
+            for file, text, there in EDITS:
+                if file == name:
+                    assert src.count(text) == 1, (file, text)
+                    src = src.replace(text, there)
+            units.append(str(out / (name[:-3] + ".cpp")))
+            open(units[-1], "w").write('#include "hooks.h"\n' + _launches_to_calls(src))
+    asan = subprocess.run(["g++", "-print-file-name=libasan.so"], capture_output=True, text=True).stdout.strip()
+    san = ["-fsanitize=address", "-DEMU_EXACT_ALLOC", "-DEMU_LANE_STACK=65536"] if os.path.isabs(asan) else []
+    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0",
+                               "-DEMU_NUM_SMS=1", "-I", str(out), "-I", EMU, "-I", os.path.join(EMU, "fake"), "-I", CSRC,
+                               "-c", u, "-o", str(out / f"u{i}.o")], stderr=subprocess.PIPE, text=True)
+             for i, u in enumerate(units)]
+    for p in procs:
+        err = p.communicate()[1]
+        assert p.returncode == 0, err[-3000:]
+    so = str(out / "lib.so")
+    subprocess.run(["g++", "-shared", "-pthread", *san[:1], "-o", so] +
+                   [str(out / f"u{i}.o") for i in range(len(units))], check=True)
+    return so, dict(os.environ, PYTHONPATH=ROOT, **({"LD_PRELOAD": asan, "ASAN_OPTIONS": "detect_leaks=0"} if san else {}))
+
+
+# test -> (function host_<name> of this file, environment): each in a process of
+# its own, all side by side
+RUNS = {}
+
+
+@pytest.fixture(scope="module")
+def on_host(host_lib):
+    so, base = host_lib
+    procs = {k: subprocess.Popen([sys.executable, os.path.abspath(__file__), so, name], cwd=ROOT,
+                                 env=dict(base, **{e: str(v) for e, v in env.items()}), stdout=subprocess.PIPE,
+                                 stderr=subprocess.STDOUT, text=True) for k, (name, env) in RUNS.items()}
+    yield lambda key: finish(procs[key])
+    for p in procs.values():
+        p.kill()
+        p.wait()
+
+
+def finish(p):
+    """What a process's function returned."""
+    out = p.communicate(timeout=300)[0]
+    assert p.returncode == 0, out[-3000:]
+    return json.loads(out.strip().splitlines()[-1])
+
+
+# --------------------------------------------------------------------------
+# in the process with the host library
+# --------------------------------------------------------------------------
+
+def count_set(lib, c, gs, k):
+    """Counts of one set (renumbered by degree, whatever its size), status 0."""
+    from tests.emu.lib_scenarios import NCLS, P, _descs, ok, sync
+    descs, keep = _descs(gs)
+    ok(lib.acc_motif_batch_prepare(c.h, descs, len(gs), k, None), "batch_prepare")
+    out, st = np.zeros((len(gs), NCLS[k]), np.int64), np.full(1, -1, np.int32)
+    ok(lib.acc_motif_batch_run(c.h, None, P(out), P(st)), "batch_run")
+    sync(lib)
+    assert st[0] == 0, st
+    for o, g in zip(out, gs):
+        assert np.array_equal(o, oracle.count(*g, k))
+    return out
+
+
+def host_k5_scans(lib):
+    """Counts of a k = 5 graph; how often the list scan counted it."""
+    from tests.emu.lib_scenarios import Ctx
+    c = Ctx(lib)
+    count_set(lib, c, [fan(13, 12, 20, 1)], 5)
+    c.close()
+    return lib.emu_scan_count()
+
+
+# --------------------------------------------------------------------------
+# tests
+# --------------------------------------------------------------------------
+
+# (EMU_SCHED 0: the threads of a block arrive in ascending order, so warps 0 and 1
+# have passed when thread 64 does; 1: in descending order, all but warp 0)
+RAISED = [(phase, order, at) for phase in (1, 2) for order, at in ((0, 64), (1, 31))]
+for phase, order, at in RAISED:
+    RUNS["raised", phase, order, at] = ("k5_scans", dict(EMU_SCHED=order, EMU_RAISE_PHASE=phase, EMU_RAISE_AT=at))
+RUNS["not raised"] = ("k5_scans", {})
+
+
+@pytest.mark.parametrize("phase,order,at", RAISED)
+def test_return_to_the_scan_raised_as_a_block_starts(on_host, phase, order, at):
+    """The 5-cycle pass while another block or kernel raises the return to the
+    list scan: each block goes on or leaves as a whole."""
+    assert on_host(("raised", phase, order, at)) == 1
+
+
+def test_no_return_to_the_scan(on_host):
+    assert on_host("not raised") == 0
+
+
+if __name__ == "__main__":
+    import paper_1203_3415_gb300 as acc
+    lib = acc.declare(ctypes.CDLL(sys.argv[1]))
+    print(json.dumps(globals()["host_" + sys.argv[2]](lib)))
