@@ -83,6 +83,10 @@ __global__ void k_partial_prep(PartialArgs a) {
             atomicAdd(&a.nd[v], (unsigned long long)__popc(same & m1) |
                                     ((unsigned long long)__popc(same & m2) << kNdBits) |
                                     ((unsigned long long)__popc(same & m3) << (2 * kNdBits)));
+        // k = 5: a root with more rows than the 5-cycle tables count leaves the graph to
+        // the scan.  Decided here, before the passes, so that they are not run for
+        // nothing.
+        if (K == 5 && leader && a.deg[v] - a.lo[v] > kCycleRows) a.p5.ctr[kCtrScan] = 1ull;
         if constexpr (K >= 4) {
             uint2 rv = make_uint2(0u, 0u);
             if (ok && (K == 5 || !(r >> 31))) {
@@ -641,7 +645,7 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : (SLOTS == kSetSlots &&
     uint32_t *root_wedges = K == 5 ? a.p5.pair_wedges : a.wedges;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
-    if (K == 5 && scan_instead(a)) return;
+    if ((K == 5 || BESIDE) && scan_instead(a)) return;
     if (PHASE == 2 && *qtail == 0) return;
     uint4 *tabs = reinterpret_cast<uint4 *>(smem);
     Walker<K, HASH> wk;
@@ -1026,6 +1030,7 @@ __global__ void __launch_bounds__(kFThreads, 3) k_partial_finish(PartialArgs a) 
     __shared__ __align__(16) int16_t lut_s[1 << code_bits(K)];
     __shared__ int last;
     const int lane = threadIdx.x & 31;
+    if (!INDUCED && scan_instead(a)) return;
     if ((long long)blockIdx.x < (long long)a.gs.B * a.slices)
         for (int i = threadIdx.x; i < (1 << code_bits(K)) / 8; i += blockDim.x)
             reinterpret_cast<uint4 *>(lut_s)[i] = __ldg(reinterpret_cast<const uint4 *>(a.lut) + i);

@@ -14,6 +14,10 @@ namespace acc {
 constexpr int kNdBits = 21;
 constexpr int kNdMax = (1 << kNdBits) - 1;
 
+// k = 5: most neighbours above a root (rows of its pass); the 5-cycle tables count
+// a root's wedges to one end in 10 bits, and no more of them than its rows.
+constexpr int kCycleRows = 1023;
+
 // k = 5: what the passes share besides the graph (one graph, not a set).
 struct Partial5 {
     // counters, zeroed by the caller: triangles listed; set when the set must

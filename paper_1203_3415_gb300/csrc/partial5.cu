@@ -705,11 +705,7 @@ __global__ void __launch_bounds__(kCThreads, PHASE == 1 ? 3 : 2) k_cycles5(Parti
             if ((long long)u0 >= g.n) break;
             const int vl = (int)u0 + lane;
             uint32_t W = 0;
-            if (lane < grab && vl < g.n) {
-                W = a.p5.cycle_wedges[vl];
-                // a count of an end is at most the root's rows
-                if (g.deg[vl] - g.lo[vl] > 1023) ctr[kCtrScan] = 1ull;
-            }
+            if (lane < grab && vl < g.n) W = a.p5.cycle_wedges[vl];
             const bool big = W > (uint32_t)kLFill;
             const unsigned heavy = __ballot_sync(kFull, big);
             if (big) {

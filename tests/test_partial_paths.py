@@ -46,6 +46,7 @@ EDITS = [
      "    emu_cycles_enter(a, a.p5.ctr + kCtrScan, PHASE, cycle_smem(PHASE));\n"),
     ("partial5.cu", "template <int PHASE>\n__global__ void __launch_bounds__(kCThreads",
      "constexpr size_t cycle_smem(int phase);\ntemplate <int PHASE>\n__global__ void __launch_bounds__(kCThreads"),
+    ("partial.cu", "- a.lo[v] > kCycleRows", "- a.lo[v] > (int)emu_env(\"EMU_ROWS\", kCycleRows)"),
     ("partial5.cu", "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n    grid_dep_wait();\n",
      "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n"
      "    if (threadIdx.x == 0 && blockIdx.x == 0 && a.p5.ctr[kCtrScan]) emu_scans++;\n"),
@@ -137,6 +138,21 @@ def host_k5_scans(lib):
     return lib.emu_scan_count()
 
 
+def host_k5_scanned(lib):
+    """Neighbour entries read for a k = 5 graph: on its own, and by the list scan
+    of a set with a second, empty graph; how often a scan followed the passes."""
+    from tests.emu.lib_scenarios import Ctx, P, ok
+    c = Ctx(lib)
+    stats = np.zeros(7, np.int64)
+    read = []
+    for gs in ([fan(13, 12, 20, 1)], [fan(13, 12, 20, 1), (1, np.zeros(0, np.int64), np.zeros(0, np.int64))]):
+        count_set(lib, c, gs, 5)
+        ok(lib.acc_motif_last_stats(c.h, P(stats)), "last_stats")
+        read.append(int(stats[6]))
+    c.close()
+    return read + [lib.emu_scan_count()]
+
+
 # --------------------------------------------------------------------------
 # tests
 # --------------------------------------------------------------------------
@@ -158,6 +174,16 @@ def test_return_to_the_scan_raised_as_a_block_starts(on_host, phase, order, at):
 
 def test_no_return_to_the_scan(on_host):
     assert on_host("not raised") == 0
+
+
+RUNS["rows"] = ("k5_scanned", dict(EMU_ROWS=8))
+
+
+def test_graphs_with_large_hubs_pay_for_the_scan_alone(on_host):
+    """k = 5, a root of more rows than the 5-cycle tables count: the passes leave at
+    once, and what is read is what the list scan reads."""
+    alone, scan, returned = on_host("rows")
+    assert returned == 1 and alone == scan > 0
 
 
 if __name__ == "__main__":
