@@ -207,8 +207,11 @@ ACC_API int acc_motif_count_batch(acc_ctx *ctx, const acc_graph_desc *h_graphs, 
  * Tune the schedule for the prepared batch: runs the batch once for each of
  * a fixed set of candidate (light, target) pairs, timed with CUDA events on
  * `stream`, and keeps the fastest in the context (acc_ctx_set_schedule).
+ * A batch that no list scan counts (counted by partial patterns or by the
+ * formulas, see acc_ctx_set_mode) reads no schedule: it is run and timed, and the
+ * context's schedule stays as it was.
  * Waits for the device.  h_light, h_target, h_ms (nullable) receive the
- * chosen pair and its time.  Errors: ACC_ERR_ARG (no prepared batch), any
+ * pair in effect and its time.  Errors: ACC_ERR_ARG (no prepared batch), any
  * error a batch run returns (the previous schedule is then kept).
  */
 ACC_API int acc_motif_batch_autotune(acc_ctx *ctx, void *stream, int64_t *h_light, int64_t *h_target,

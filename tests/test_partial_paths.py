@@ -153,6 +153,30 @@ def host_k5_scanned(lib):
     return read + [lib.emu_scan_count()]
 
 
+def host_autotune(lib):
+    """The schedule before and after the autotuner, and what it returned, by what
+    counts the batch."""
+    import paper_1203_3415_gb300 as acc
+    from tests.emu.lib_scenarios import Ctx, _descs, ok
+    c = Ctx(lib)
+    seen = []
+    g = fan(6, 4, 8, 1)
+    for mode, k, gs in ((acc.ACC_MODE_COUNT, 4, [g, g]), (acc.ACC_MODE_COUNT, 5, [g]), (acc.ACC_MODE_FORMULA, 3, [g, g]),
+                        (acc.ACC_MODE_ENUMERATE, 3, [g, g])):
+        light, target, ms = ctypes.c_int64(), ctypes.c_int64(), ctypes.c_float()
+        ok(lib.acc_ctx_set_mode(c.h, mode), "set_mode")
+        ok(lib.acc_ctx_set_schedule(c.h, 777, 999), "set_schedule")
+        descs, keep = _descs(gs)
+        ok(lib.acc_motif_batch_prepare(c.h, descs, len(gs), k, None), "batch_prepare")
+        ok(lib.acc_motif_batch_autotune(c.h, None, ctypes.byref(light), ctypes.byref(target), ctypes.byref(ms)), "autotune")
+        pair = [light.value, target.value]
+        ok(lib.acc_ctx_get_schedule(c.h, ctypes.byref(light), ctypes.byref(target)), "get_schedule")
+        assert pair == [light.value, target.value] and ms.value > 0.0
+        seen.append(pair)
+    c.close()
+    return seen
+
+
 # --------------------------------------------------------------------------
 # tests
 # --------------------------------------------------------------------------
@@ -184,6 +208,14 @@ def test_graphs_with_large_hubs_pay_for_the_scan_alone(on_host):
     once, and what is read is what the list scan reads."""
     alone, scan, returned = on_host("rows")
     assert returned == 1 and alone == scan > 0
+
+
+RUNS["autotune"] = ("autotune", {})
+
+
+def test_autotuner_keeps_the_schedule_that_no_scan_reads(on_host):
+    *unread, scanned = on_host("autotune")
+    assert unread == [[777, 999]] * 3 and scanned != [777, 999]
 
 
 if __name__ == "__main__":
