@@ -402,7 +402,10 @@ ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);
  *   from 8192 (below 12288: of at least two arcs a vertex); one graph of fewer
  *   than 1024 vertices is never counted so.  A k = 5 graph with a vertex of over
  *   1023 neighbours after it in degree order, with more triangles than the
- *   workspace lists, or with a count bound above 2^57 is left to the lists.
+ *   workspace lists, or with a count bound above 2^57 is left to the lists.  So
+ *   is a set whose pattern counters (24 bytes a neighbour entry) find no device
+ *   memory, with the context's later sets of as many arcs until the next
+ *   acc_motif_prepare or acc_motif_batch_prepare.
  *  ACC_MODE_ENUMERATE: every k-subset is visited and classified on its own.
  *  ACC_MODE_FORMULA: for k = 3, the paper's per-vertex formulas (Thm teo3,
  *   Algorithm s3, Table starb): open triples from the sizes of each vertex's

@@ -36,6 +36,9 @@ constexpr int kAutoFormulaMaxN = 16384;
 
 bool ok(cudaError_t e) { return e == cudaSuccess; }
 
+// Whether the last failed allocation met a stream capture, not a lack of memory.
+thread_local bool t_alloc_in_capture = false;
+
 template <typename T>
 int grow(T **p, size_t *cap, size_t need) {
     if (need <= *cap && *p) return ACC_OK;
@@ -43,9 +46,11 @@ int grow(T **p, size_t *cap, size_t need) {
     *p = nullptr;
     *cap = 0;
     const size_t alloc = need + need / 4 + 64;
-    if (!ok(cudaMalloc((void **)p, alloc * sizeof(T)))) {
+    const cudaError_t e = cudaMalloc((void **)p, alloc * sizeof(T));
+    if (!ok(e)) {
         cudaGetLastError();
         *p = nullptr;
+        t_alloc_in_capture = e == cudaErrorStreamCaptureUnsupported;
         return ACC_ERR_NOMEM;
     }
     *cap = alloc;
@@ -271,7 +276,7 @@ bool uses_formula(const acc_ctx *c, int k, int max_n) {
 #define ACC_PARTIAL_MIN_ARCS1 (ACC_PARTIAL_MIN_ARCS * 3 / 2)
 #endif
 bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
-    return count_family(c) && k <= 4 && relabel && !uses_formula(c, k, max_n) &&
+    return count_family(c) && k <= 4 && relabel && arcs < c->partial_arcs_end && !uses_formula(c, k, max_n) &&
            arcs >= (k == 4 && B == 1 ? ACC_PARTIAL_MIN_ARCS1 : ACC_PARTIAL_MIN_ARCS);
 }
 
@@ -283,7 +288,7 @@ bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relab
 // ACC_PARTIAL_MIN_ARCS1 (scan / partial, us: 8300 uniform arcs on 4000 vertices 182 /
 // 150, 9000 on 6000 105 / 145; with hubs 820 / 312 and 702 / 246).
 bool uses_partial5(const acc_ctx *c, int k, int n, long long arcs, bool relabel, int B) {
-    return count_family(c) && k == 5 && B == 1 && relabel && arcs >= ACC_PARTIAL_MIN_ARCS &&
+    return count_family(c) && k == 5 && B == 1 && relabel && arcs < c->partial_arcs_end && arcs >= ACC_PARTIAL_MIN_ARCS &&
            (arcs >= 2ll * n || arcs >= ACC_PARTIAL_MIN_ARCS1);
 }
 
@@ -325,7 +330,7 @@ long long sparse_list_entries(int maxdeg) { return (3LL * maxdeg + 64 + 31) & ~3
 
 // Workspace for a set of NV vertices in blocks of state_words words, with at
 // most `arcs` arcs and graphs of at most max_n vertices.
-int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long arcs, int max_n, int k, int B,
+int grow_workspace(acc_ctx *c, long long NV, long long state_words, long long arcs, int max_n, int k, int B,
                      bool relabel) {
     int rc;
     const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
@@ -403,6 +408,48 @@ int ensure_workspace(acc_ctx *c, long long NV, long long state_words, long long 
         return rc;
     if (!c->maxdeg_host && !ok(cudaMallocHost(&c->maxdeg_host, sizeof(int)))) return ACC_ERR_NOMEM;
     return ACC_OK;
+}
+
+// Gives back what only partial patterns need (a free waits for the device).
+void free_partial(acc_ctx *c, bool sparse) {
+    auto drop = [](auto **p, size_t *cap) {
+        cudaFree(*p);
+        *p = nullptr;
+        *cap = 0;
+    };
+    drop(&c->pp_nd, &c->pp_nd_cap);
+    drop(&c->pp_part, &c->pp_part_cap);
+    drop(&c->pp_done, &c->pp_done_cap);
+    drop(&c->pp_wedges, &c->pp_wedges_cap);
+    drop(&c->pp_tri, &c->pp_tri_cap);
+    drop(&c->p5_vert, &c->p5_vert_cap);
+    drop(&c->p5_sums, &c->p5_sums_cap);
+    if (c->cg_exec) cudaGraphExecDestroy(c->cg_exec);  // (it may hold their addresses)
+    c->cg_exec = nullptr;
+    memset(&c->cg_seen, 0, sizeof(c->cg_seen));
+    if (!sparse) return;
+    drop(&c->nh, &c->nh_cap);
+    drop(&c->sp_raw, &c->sp_raw_cap);
+    drop(&c->sp_merged, &c->sp_merged_cap);
+    drop(&c->sp_roff, &c->sp_roff_cap);
+    drop(&c->sp_big, &c->sp_big_cap);
+}
+
+// The workspace of a set whose dense block has `words` words (see
+// grow_workspace).  Partial patterns take 24 bytes a neighbour entry more than the
+// list scan, and 40 more where sparse_auto takes the sparse build: where the device has no room for them the set is counted by
+// the scan, as are the context's later sets of as many arcs (until the next
+// acc_motif_prepare or acc_motif_batch_prepare).
+int ensure_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel) {
+    const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
+    const int rc = grow_workspace(c, NV, sparse ? 0 : words, arcs, max_n, k, B, relabel);
+    if (rc != ACC_ERR_NOMEM || t_alloc_in_capture ||
+        !(uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B)))
+        return rc;
+    c->partial_arcs_end = arcs;
+    const bool still = sparse_path(c, k, max_n, arcs, relabel, B);
+    free_partial(c, sparse && !still);
+    return grow_workspace(c, NV, still ? 0 : words, arcs, max_n, k, B, relabel);
 }
 
 // Build + enumerate one graph set into counts[B * num_classes(k)].
@@ -634,9 +681,8 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     int rc = uses_partial5(c, k, n, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
+    if ((rc = ensure_workspace(c, n, (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN))) return rc;
     const bool sparse = sparse_path(c, k, n, m, n >= kRelabelMinN, 1);
-    if ((rc = ensure_workspace(c, n, sparse ? 0 : (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN)))
-        return rc;
     GSet gs = {};
     gs.one.rowptr = reinterpret_cast<const long long *>(rowptr);
     gs.one.col = col;
@@ -665,6 +711,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
         key.m = m;
         key.light = c->sched_light;
         key.target = c->sched_target;
+        key.partial_end = c->partial_arcs_end;
         key.n = n;
         key.k = k;
         key.mode = c->mode;
@@ -726,9 +773,8 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
 // build): grows nothing when they are the same.
 int batch_workspace(acc_ctx *c) {
     if (size_check(c, c->batch_max_n)) return ACC_ERR_TOO_LARGE;
-    return ensure_workspace(c, c->batch_set.NV,
-                            sparse_path(c, c->batch_k, c->batch_max_n, c->batch_arcs, true, c->batch_set.B) ? 0 : c->batch_words, c->batch_arcs,
-                            c->batch_max_n, c->batch_k, c->batch_set.B, true);
+    return ensure_workspace(c, c->batch_set.NV, c->batch_words, c->batch_arcs, c->batch_max_n, c->batch_k,
+                            c->batch_set.B, true);
 }
 
 }  // namespace
@@ -762,8 +808,7 @@ int ctx_reserve(acc_ctx *c, long long n, long long m, int k) {
     const int rc = ensure_tab5(c, c->own);
     if (rc) return rc;
     const bool relabel = n >= kRelabelMinN;
-    return ensure_workspace(c, n, sparse_path(c, k, (int)n, m, relabel, 1) ? 0 : n * state_pitch((int)n), m, (int)n, k, 1,
-                            relabel);
+    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, relabel);
 }
 
 }  // namespace acc
@@ -864,6 +909,7 @@ int acc_motif_prepare(acc_ctx *c, int k, void *stream) {
     if (!valid_k(k)) return ACC_ERR_K;
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
+    c->partial_arcs_end = INT64_MAX;
     int rc = k == 5 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     return ok(cudaStreamSynchronize(s)) ? ACC_OK : ACC_ERR_CUDA;
@@ -938,7 +984,8 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     // (k = 5: also for a run after the mode changed to the count mode)
     int rc = k == 5 && B == 1 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
-    if ((rc = ensure_workspace(c, NV, sparse_path(c, k, max_n, arcs, true, B) ? 0 : words, arcs, max_n, k, B, true))) return rc;
+    c->partial_arcs_end = INT64_MAX;
+    if ((rc = ensure_workspace(c, NV, words, arcs, max_n, k, B, true))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;
     if ((rc = grow(&c->gid, &c->gid_cap, (size_t)NV + 1))) return rc;
     if (B > 0 && !ok(cudaMemcpy(c->meta_dev, metas.data(), sizeof(GMeta) * (size_t)B, cudaMemcpyHostToDevice)))

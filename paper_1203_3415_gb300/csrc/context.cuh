@@ -73,6 +73,9 @@ struct acc_ctx {
     size_t p5_vert_cap = 0;
     unsigned long long *p5_sums = nullptr;  // k = 5: sums, small patterns, counters
     size_t p5_sums_cap = 0;
+    // sets of at least this many arcs are counted by the list scan: the device had
+    // no memory for the counters of one
+    long long partial_arcs_end = INT64_MAX;
     int mode = 0;             // ACC_MODE_COUNT, _ENUMERATE, _FORMULA or _AUTO
     long long sched_light = 0;   // enumeration schedule (0: the kernels' default)
     long long sched_target = 0;
@@ -117,7 +120,7 @@ struct acc_ctx {
     cudaGraphExec_t cg_exec = nullptr;
     struct CountKey {
         const void *rowptr, *col, *counts, *status;
-        long long m, light, target;
+        long long m, light, target, partial_end;
         int n, k, mode, grid_num, grid_den, adjacency;
         const void *ws[32];
     } cg_key = {}, cg_seen = {};  // the captured graph's key; the last key counted one by one

@@ -28,6 +28,28 @@ inline unsigned long long emu_env(const char *name, unsigned long long own) {
     const char *e = getenv(name);
     return e ? strtoull(e, nullptr, 10) : own;
 }
+// device memory: bytes held, and the most that may be
+extern unsigned long long emu_held, emu_most;
+std::map<void *, size_t> &emu_sizes();
+template <class T> inline cudaError_t emu_counted_malloc(T **p, size_t bytes) {
+    if (emu_held + bytes > emu_most) {
+        *p = nullptr;
+        return 2;  // out of memory
+    }
+    const cudaError_t e = cudaMalloc(p, bytes);
+    if (e == cudaSuccess) emu_held += emu_sizes()[*p] = bytes;
+    return e;
+}
+template <class T> inline cudaError_t emu_counted_free(T *p) {
+    auto it = emu_sizes().find((void *)p);
+    if (it != emu_sizes().end()) {
+        emu_held -= it->second;
+        emu_sizes().erase(it);
+    }
+    return cudaFree((void *)p);
+}
+#define cudaMalloc emu_counted_malloc
+#define cudaFree emu_counted_free
 extern unsigned long long emu_scans;  // k = 5 counts left to the list scan
 // k_cycles5<phase>: what other blocks left in shared memory, as the first thread
 // of a block finds it, and the flag raised when thread EMU_RAISE_AT of the first block
@@ -38,6 +60,18 @@ template <class A> inline void emu_cycles_enter(const A &a, unsigned long long *
     if (entered % blockDim.x == 0) memset(emu_dyn_smem, 0xA5, smem);
     if (entered++ < blockDim.x && threadIdx.x == emu_env("EMU_RAISE_AT", 0)) *flag = 1;
 }
+"""
+
+GLOBALS = r"""
+#include "hooks.h"
+unsigned long long emu_scans = 0, emu_held = 0, emu_most = ~0ull;
+std::map<void *, size_t> &emu_sizes() {
+    static std::map<void *, size_t> m;
+    return m;
+}
+extern "C" unsigned long long emu_scan_count() { return emu_scans; }
+extern "C" unsigned long long emu_bytes() { return emu_held; }
+extern "C" void emu_limit(unsigned long long most) { emu_most = most; }
 """
 
 # (source file, text in it, what stands there for these tests)
@@ -61,8 +95,7 @@ def host_lib(tmp_path_factory):
     out = tmp_path_factory.mktemp("partial_paths")
     units = [os.path.join(EMU, "emu_rt.cpp"), str(out / "hooks.cpp")]
     open(out / "hooks.h", "w").write("#pragma once\n" + HOOKS)
-    open(units[1], "w").write('#include "hooks.h"\nunsigned long long emu_scans = 0;\n'
-                              'extern "C" unsigned long long emu_scan_count() { return emu_scans; }\n')
+    open(units[1], "w").write(GLOBALS)
     for name in sorted(os.listdir(CSRC)):
         if name.endswith(".cu"):
             src = open(os.path.join(CSRC, name)).read()
@@ -74,7 +107,7 @@ def host_lib(tmp_path_factory):
             open(units[-1], "w").write('#include "hooks.h"\n' + _launches_to_calls(src))
     asan = subprocess.run(["g++", "-print-file-name=libasan.so"], capture_output=True, text=True).stdout.strip()
     san = ["-fsanitize=address", "-DEMU_EXACT_ALLOC", "-DEMU_LANE_STACK=65536"] if os.path.isabs(asan) else []
-    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0",
+    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0", "-DACC_QUEUE_CAP=1024ull",
                                "-DEMU_NUM_SMS=1", "-I", str(out), "-I", EMU, "-I", os.path.join(EMU, "fake"), "-I", CSRC,
                                "-c", u, "-o", str(out / f"u{i}.o")], stderr=subprocess.PIPE, text=True)
              for i, u in enumerate(units)]
@@ -177,6 +210,44 @@ def host_autotune(lib):
     return seen
 
 
+def host_short_memory(lib):
+    """Counts of sets that fit the device's memory until their pattern counters are
+    added: bytes held where there is no limit, and the least limit under which the
+    counts are right (below it the call says so)."""
+    import paper_1203_3415_gb300 as acc
+    from tests.emu.lib_scenarios import Ctx, NCLS, P, _descs
+    lib.emu_bytes.restype = ctypes.c_ulonglong
+    lib.emu_limit.argtypes = [ctypes.c_ulonglong]
+    out = []
+    for k, gs, steps in ((4, [fan(40, 20, 30, 2)] * 2, 10), (5, [fan(8, 6, 10, 1)], 4)):
+        table = Ctx(lib)  # (the class tables stay)
+        for kk in (3, 4, 5):
+            assert lib.acc_motif_prepare(table.h, kk, None) == 0
+        before = lib.emu_bytes()
+        want = [oracle.count(*g, k) for g in gs]
+        descs, keep = _descs(gs)
+        counts, st = np.zeros((len(gs), NCLS[k]), np.int64), np.full(1, -1, np.int32)
+
+        def count(limit):
+            lib.emu_limit(limit)
+            c = Ctx(lib)
+            rc = lib.acc_motif_count_batch(c.h, descs, len(gs), k, None, P(counts), P(st))
+            if rc == 0:
+                assert st[0] == 0 and all(np.array_equal(o, w) for o, w in zip(counts, want)), limit
+            held = lib.emu_bytes() - before
+            c.close()
+            lib.emu_limit(1 << 63)
+            assert rc in (0, acc.ACC_ERR_NOMEM), rc
+            return rc == 0, held
+        held = count(1 << 63)[1]
+        limit = held
+        while count(before + limit - held // steps)[0]:
+            limit -= held // steps
+        out.append([held, limit])
+        table.close()
+    return out
+
+
 # --------------------------------------------------------------------------
 # tests
 # --------------------------------------------------------------------------
@@ -218,7 +289,15 @@ def test_autotuner_keeps_the_schedule_that_no_scan_reads(on_host):
     assert unread == [[777, 999]] * 3 and scanned != [777, 999]
 
 
+RUNS["memory"] = ("short_memory", {})
+
+
+def test_sets_whose_counters_do_not_fit_are_scanned(on_host):
+    for held, least in on_host("memory"):
+        assert least < 0.8 * held
+
+
 if __name__ == "__main__":
     import paper_1203_3415_gb300 as acc
     lib = acc.declare(ctypes.CDLL(sys.argv[1]))
-    print(json.dumps(globals()["host_" + sys.argv[2]](lib)))
+    print("\n" + json.dumps(globals()["host_" + sys.argv[2]](lib)))
