@@ -400,7 +400,8 @@ ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);
  *   and exclusion.  Taken from 8192 arcs on for k = 3 and for sets of several
  *   graphs (k = 4), from 12288 for one graph of k = 4, and for one graph of k = 5
  *   from 8192 (below 12288: of at least two arcs a vertex); one graph of fewer
- *   than 1024 vertices is never counted so.  A k = 5 graph with a vertex of over
+ *   than 1024 vertices is never counted so (outside a batch), nor are sets of many
+ *   graphs of a few dozen arcs.  A k = 5 graph with a vertex of over
  *   1023 neighbours after it in degree order, with more triangles than the
  *   workspace lists, or with a count bound above 2^57 is left to the lists.  So
  *   is a set whose pattern counters (24 bytes a neighbour entry) find no device

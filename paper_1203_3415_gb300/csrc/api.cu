@@ -275,9 +275,23 @@ bool uses_formula(const acc_ctx *c, int k, int max_n) {
 #ifndef ACC_PARTIAL_MIN_ARCS1
 #define ACC_PARTIAL_MIN_ARCS1 (ACC_PARTIAL_MIN_ARCS * 3 / 2)
 #endif
+// Many tiny graphs: the finish takes a block a graph, and its fixed part (the
+// graph's sums, its class matrix) more than the scan of the graph does.  Sets of
+// more graphs than the finish has blocks at once are scanned below 64 arcs a graph
+// (96 where the graphs have fewer than 32 vertices; scan / partial, us, k = 4: 4000
+// graphs of 10 vertices and 20 arcs 267 / 368, of 40 and 40 326 / 400, of 20 and
+// 80 487 / 524, of 40 and 80 468 / 450, of 80 and 160 747 / 567; 300 graphs of 20
+// and 40 97 / 82).  k = 3, whose finish is short: from 16 graphs an SM on, below 48
+// (16000 graphs of 20 vertices and 40 arcs 792 / 837, of 40 and 80 1001 / 968).
+bool tiny_graphs(const acc_ctx *c, int k, int max_n, long long arcs, int B) {
+    return k == 3 ? B > 16 * c->num_sms && arcs < 48ll * B
+                  : B > 4 * c->num_sms && arcs < (max_n < 32 ? 96ll : 64ll) * B;
+}
+
 bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
     return count_family(c) && k <= 4 && relabel && arcs < c->partial_arcs_end && !uses_formula(c, k, max_n) &&
-           arcs >= (k == 4 && B == 1 ? ACC_PARTIAL_MIN_ARCS1 : ACC_PARTIAL_MIN_ARCS);
+           arcs >= (k == 4 && B == 1 ? ACC_PARTIAL_MIN_ARCS1 : ACC_PARTIAL_MIN_ARCS) &&
+           !tiny_graphs(c, k, max_n, arcs, B);
 }
 
 // The same for k = 5 (partial5.cu), of one graph; its launches are followed by

@@ -51,6 +51,7 @@ template <class T> inline cudaError_t emu_counted_free(T *p) {
 #define cudaMalloc emu_counted_malloc
 #define cudaFree emu_counted_free
 extern unsigned long long emu_scans;  // k = 5 counts left to the list scan
+extern unsigned long long emu_partials;  // k = 3, 4 sets counted by partial patterns
 // k_cycles5<phase>: what other blocks left in shared memory, as the first thread
 // of a block finds it, and the flag raised when thread EMU_RAISE_AT of the first block
 // arrives
@@ -64,12 +65,13 @@ template <class A> inline void emu_cycles_enter(const A &a, unsigned long long *
 
 GLOBALS = r"""
 #include "hooks.h"
-unsigned long long emu_scans = 0, emu_held = 0, emu_most = ~0ull;
+unsigned long long emu_scans = 0, emu_partials = 0, emu_held = 0, emu_most = ~0ull;
 std::map<void *, size_t> &emu_sizes() {
     static std::map<void *, size_t> m;
     return m;
 }
 extern "C" unsigned long long emu_scan_count() { return emu_scans; }
+extern "C" unsigned long long emu_partial_count() { return emu_partials; }
 extern "C" unsigned long long emu_bytes() { return emu_held; }
 extern "C" void emu_limit(unsigned long long most) { emu_most = most; }
 """
@@ -81,6 +83,7 @@ EDITS = [
     ("partial5.cu", "template <int PHASE>\n__global__ void __launch_bounds__(kCThreads",
      "constexpr size_t cycle_smem(int phase);\ntemplate <int PHASE>\n__global__ void __launch_bounds__(kCThreads"),
     ("partial.cu", "- a.lo[v] > kCycleRows", "- a.lo[v] > (int)emu_env(\"EMU_ROWS\", kCycleRows)"),
+    ("partial.cu", "    if (k == 3) launch_pdl(k_partial_prep<3>", "    emu_partials++;\n    if (k == 3) launch_pdl(k_partial_prep<3>"),
     ("partial5.cu", "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n    grid_dep_wait();\n",
      "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n"
      "    if (threadIdx.x == 0 && blockIdx.x == 0 && a.p5.ctr[kCtrScan]) emu_scans++;\n"),
@@ -248,6 +251,25 @@ def host_short_memory(lib):
     return out
 
 
+def host_many_graphs(lib):
+    """Sets of `graphs` graphs of n vertices and m arcs: counted by partial patterns?"""
+    from tests.emu.lib_scenarios import Ctx
+    rng = np.random.default_rng(5)
+    c = Ctx(lib)
+    seen = []
+    for k, graphs, n, m in SETS:
+        gs = []
+        for _ in range(graphs):
+            key = rng.permutation(n * (n - 1))[:m]
+            s, d = key // (n - 1), key % (n - 1)
+            gs.append((n, s, d + (d >= s)))
+        before = lib.emu_partial_count()
+        count_set(lib, c, gs, k)
+        seen.append(lib.emu_partial_count() > before)
+    c.close()
+    return seen
+
+
 # --------------------------------------------------------------------------
 # tests
 # --------------------------------------------------------------------------
@@ -295,6 +317,16 @@ RUNS["memory"] = ("short_memory", {})
 def test_sets_whose_counters_do_not_fit_are_scanned(on_host):
     for held, least in on_host("memory"):
         assert least < 0.8 * held
+
+
+# (one emulated SM: k = 4 from 5 graphs on, k = 3 from 17)
+SETS = [(4, 5, 32, 63), (4, 5, 32, 64), (4, 5, 31, 95), (4, 5, 31, 96), (4, 4, 10, 20), (3, 17, 12, 47), (3, 17, 12, 48),
+        (3, 16, 12, 20)]
+RUNS["many"] = ("many_graphs", {})
+
+
+def test_sets_of_many_tiny_graphs_are_scanned(on_host):
+    assert on_host("many") == [False, True, False, True, True, False, True, True]
 
 
 if __name__ == "__main__":
