@@ -403,7 +403,8 @@ ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);
  *   than 1024 vertices is never counted so (outside a batch), nor are sets of many
  *   graphs of a few dozen arcs.  A k = 5 graph with a vertex of over
  *   1023 neighbours after it in degree order, with more triangles than the
- *   workspace lists, or with a count bound above 2^57 is left to the lists.  So
+ *   workspace lists, or with a count bound above 2^57 is left to the lists, and
+ *   one with few paths of three edges (sparse uniform graphs).  So
  *   is a set whose pattern counters (24 bytes a neighbour entry) find no device
  *   memory, with the context's later sets of as many arcs until the next
  *   acc_motif_prepare or acc_motif_batch_prepare.

@@ -296,11 +296,12 @@ bool uses_partial(const acc_ctx *c, int k, int max_n, long long arcs, bool relab
 
 // The same for k = 5 (partial5.cu), of one graph; its launches are followed by
 // the scan's, which run only when the device finds that it must (more
-// triangles than the list holds, a root with over 1023 neighbours above it, a
-// count bound near the 64-bit limit).
+// triangles than the list holds, a root with over kCycleRows neighbours above it,
+// left_to_scan).
 // From ACC_PARTIAL_MIN_ARCS arcs on, of at least two a vertex below
 // ACC_PARTIAL_MIN_ARCS1 (scan / partial, us: 8300 uniform arcs on 4000 vertices 182 /
-// 150, 9000 on 6000 105 / 145; with hubs 820 / 312 and 702 / 246).
+// 150, 9000 on 6000 105 / 145).  Only n and m are known here: graphs with hubs below
+// the line would gain too (820 / 312 and 702 / 246 at those sizes).
 bool uses_partial5(const acc_ctx *c, int k, int n, long long arcs, bool relabel, int B) {
     return count_family(c) && k == 5 && B == 1 && relabel && arcs < c->partial_arcs_end && arcs >= ACC_PARTIAL_MIN_ARCS &&
            (arcs >= 2ll * n || arcs >= ACC_PARTIAL_MIN_ARCS1);

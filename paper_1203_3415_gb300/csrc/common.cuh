@@ -55,7 +55,7 @@ struct GraphInfo {
     unsigned big_rows;              // sparse build: rows listed for the block sort
     unsigned big_head;              // sparse build: listed rows taken
     float bound[3];                 // degree sums of the count bound (count_bound_terms)
-    int large;                      // the count bound exceeds kCountLimit / 32
+    int to_scan;                    // k = 5: not for partial patterns (left_to_scan)
 };
 
 // Largest count the library reports: a set whose upper bound on N_k (below)
@@ -94,6 +94,22 @@ __host__ __device__ inline double count_bound(int k, int max_n, int maxdeg, cons
     double c = max_n >= k ? 1.0 : 0.0;
     for (int i = 0; i < k; i++) c = c * (double)(max_n - i) / (double)(i + 1);
     return c < b ? c : b;
+}
+
+// k = 5, one graph of n vertices with count bound `bound` (degree sums s): whether
+// the list scan counts it rather than the partial patterns (partial5.cu).  Because
+// sums come near the 64-bit limit (a pattern's sum counts an occurrence up to 24
+// times before it is divided), or because the scan has little to do: its time grows
+// with sum d (d - 1) (d - 2) = 2 s[1], that of the passes is mostly fixed.  The line
+// is drawn through uniform graphs (scan / patterns, us: 12600 arcs on 12000 vertices,
+// s[1] = 6 n, 104 / 209; 14400 on 9000, 15 n, 120 / 199 or, with a larger largest
+// degree, 175 / 188; 21000 on 12000, 20 n, 211 / 218; 28000 on 20000, 2.1e5, 165 / 227;
+// 30000 on 20000, 2.5e5, 245 / 227; 39000 on 30000, 2.5e5, 212 / 253; 48000 on 40000,
+// 2.6e5, 275 / 262).  Graphs with hubs lie above it (12600 arcs on 12000 vertices,
+// degrees up to 8, 24 n, 275 / 211).  A graph left to the scan pays about 16 us beside
+// it, the launches of the passes that leave at once (104 -> 121).
+__host__ __device__ inline bool left_to_scan(double bound, int n, const float *s) {
+    return bound > kCountLimit / 32 || s[1] < fminf(15.0f * (float)n, 2.2e5f);
 }
 
 // One graph of a set.  Its vertices are the global ids [voff, voff + n); its

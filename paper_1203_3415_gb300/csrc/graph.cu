@@ -387,7 +387,7 @@ __global__ void __launch_bounds__(1024) k_scan_degrees(const int *__restrict__ d
                 for (int j = 0; j < 3; j++) tb[j] += warp_bound[w][j];
             const double bound = count_bound(k, max_n, warp_max[0], tb);
             if (bound > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
-            if (k == 5) info->large = bound > kCountLimit / 32;
+            if (k == 5) info->to_scan = left_to_scan(bound, max_n, tb);
         }
         info->maxdeg = warp_max[0];
         info->big_rows = 0;
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(1024) k_scan_top(long long *tile_sum, int ntil
         if (k) {
             const double bound = count_bound(k, max_n, info->maxdeg, info->bound);
             if (bound > kCountLimit) set_status(status, ACC_ERR_OVERFLOW);
-            if (k == 5) info->large = bound > kCountLimit / 32;
+            if (k == 5) info->to_scan = left_to_scan(bound, max_n, info->bound);
         }
         info->big_rows = 0;
         info->big_head = 0;

@@ -63,9 +63,7 @@ __global__ void k_partial_prep(PartialArgs a) {
     grid_dep_wait();
     const long long nnz = a.info->nnz;
     const int lane = threadIdx.x & 31;
-    // k = 5: sums near the 64-bit limit (a pattern's sum counts an occurrence
-    // up to 24 times before it is divided) are left to the scan
-    if (K == 5 && blockIdx.x == 0 && threadIdx.x == 0 && a.info->large) a.p5.ctr[kCtrScan] = 1ull;
+    if (K == 5 && blockIdx.x == 0 && threadIdx.x == 0 && a.info->to_scan) a.p5.ctr[kCtrScan] = 1ull;
     for (long long p0 = blockIdx.x * (long long)blockDim.x + threadIdx.x - lane; p0 < nnz;
          p0 += (long long)gridDim.x * blockDim.x) {
         const long long pos = p0 + lane;

@@ -174,6 +174,22 @@ def host_k5_scans(lib):
     return lib.emu_scan_count()
 
 
+def host_k5_sparse(lib):
+    """How often the list scan counted a uniform graph of 90 arcs on 80 vertices, and
+    one of 400 arcs (k = 5)."""
+    from tests.emu.lib_scenarios import Ctx
+    rng = np.random.default_rng(8)
+    scans = []
+    for m in (90, 400):
+        key = rng.permutation(80 * 79)[:m]
+        s, d = key // 79, key % 79
+        c = Ctx(lib)
+        count_set(lib, c, [(80, s, d + (d >= s))], 5)
+        c.close()
+        scans.append(lib.emu_scan_count())
+    return scans
+
+
 def host_k5_scanned(lib):
     """Neighbour entries read for a k = 5 graph: on its own, and by the list scan
     of a set with a second, empty graph; how often a scan followed the passes."""
@@ -327,6 +343,14 @@ RUNS["many"] = ("many_graphs", {})
 
 def test_sets_of_many_tiny_graphs_are_scanned(on_host):
     assert on_host("many") == [False, True, False, True, True, False, True, True]
+
+
+RUNS["sparse"] = ("k5_sparse", {})
+
+
+def test_sparse_uniform_graphs_are_scanned(on_host):
+    """k = 5, sum of d (d - 1) (d - 2) / 2 below 15 a vertex: left to the scan."""
+    assert on_host("sparse") == [1, 1]
 
 
 if __name__ == "__main__":
