@@ -25,6 +25,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "../../include/acc_motif.h"
 
 namespace acc {
@@ -274,6 +276,23 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
 }
 #endif
+
+// What is set up once on each device, by its bit (0 from 64 devices on: always
+// again).
+inline unsigned long long device_bit() {
+    int device = 0;
+    return cudaGetDevice(&device) == cudaSuccess && device >= 0 && device < 64 ? 1ull << device : 0ull;
+}
+// Raises a kernel's limit of dynamic shared memory to `bytes`, which the current
+// device keeps for itself; `done`: the devices that have it.
+template <typename Kernel>
+inline bool raise_shared_limit(Kernel kernel, size_t bytes, std::atomic<unsigned long long> &done) {
+    const unsigned long long bit = device_bit();
+    if (done.load(std::memory_order_acquire) & bit) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess) return false;
+    done.fetch_or(bit, std::memory_order_release);
+    return true;
+}
 
 // Orders this thread's writes before its later ones for the whole device.
 __device__ __forceinline__ void fence_device() {

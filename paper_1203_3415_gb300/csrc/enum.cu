@@ -1662,11 +1662,10 @@ __global__ void __launch_bounds__(kThreads, K == 5 ? ACC_MINB5 : (COUNT ? (SET ?
 
 template <int K, bool COUNT, int PHASE, bool SET, bool HASH>
 int blocks_per_sm() {
-    static int cached = 0;
-    if (cached) return cached;
-    if (cudaFuncSetAttribute(k_enum<K, COUNT, PHASE, SET, HASH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)Layout<K>::total) != cudaSuccess)
-        return -1;
+    static std::atomic<unsigned long long> limit{0};
+    if (!raise_shared_limit(k_enum<K, COUNT, PHASE, SET, HASH>, Layout<K>::total, limit)) return -1;
+    static std::atomic<int> cached{0};
+    if (const int known = cached) return known;
     int b = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, k_enum<K, COUNT, PHASE, SET, HASH>, kThreads,
                                                       Layout<K>::total) != cudaSuccess ||
@@ -1711,6 +1710,10 @@ int launch_k(const EnumArgs &a, int num_sms, int phase, cudaStream_t s, int grid
 // overflow lists).
 template <int K>
 int bps_max() {
+    static std::atomic<unsigned long long> done{0};
+    static std::atomic<int> most{0};
+    const unsigned long long bit = device_bit();
+    if (done.load(std::memory_order_acquire) & bit) return most;
     const int b[12] = {blocks_per_sm<K, false, 1, false, false>(), blocks_per_sm<K, false, 2, false, false>(),
                        blocks_per_sm<K, true, 1, false, false>(),  blocks_per_sm<K, true, 2, false, false>(),
                        blocks_per_sm<K, false, 1, true, false>(),  blocks_per_sm<K, false, 2, true, false>(),
@@ -1722,6 +1725,8 @@ int bps_max() {
         if (x < 1) return -1;
         if (x > m) m = x;
     }
+    most = m;
+    done.fetch_or(bit, std::memory_order_release);
     return m;
 }
 

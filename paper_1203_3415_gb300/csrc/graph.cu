@@ -1041,6 +1041,12 @@ int grid_for(long long work_items, int per_block, int num_sms) {
     return (int)b;
 }
 
+bool raise_build_limits() {
+    static std::atomic<unsigned long long> limit[2];
+    return raise_shared_limit(k_scan_degrees, (size_t)kScanSingleMax * 4, limit[0]) &&
+           raise_shared_limit(k_relabel_graph, (size_t)kRelabelSmemMax * 4, limit[1]);
+}
+
 // The build's cleared ranges followed by the caller's; the longest of those.
 long long more_ranges(const BuildBufs &bb, const IntRanges<kRanges> &own, IntRanges<kMoreRanges> &r) {
     long long longest = 0;
@@ -1080,15 +1086,7 @@ long long scan_tiles_needed(long long NV) { return NV <= kScanSingleMax ? 0 : (N
 
 int launch_build_graph(const GSet &gs, const BuildBufs &bb, int max_n, int *status, unsigned long long *counts,
                        long long ncounts, bool relabel, int num_sms, cudaStream_t s) {
-    static bool smem_opt_in = false;
-    if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_scan_degrees, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kScanSingleMax * 4)) != cudaSuccess ||
-            cudaFuncSetAttribute(k_relabel_graph, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kRelabelSmemMax * 4) != cudaSuccess)
-            return ACC_ERR_CUDA;
-        smem_opt_in = true;
-    }
+    if (!raise_build_limits()) return ACC_ERR_CUDA;
     int launches = 0;
     const long long NV = gs.NV;
     const int arcs_grid = grid_for(max(gs.M, NV), 256, num_sms);
@@ -1169,15 +1167,7 @@ int sparse_big_rows_cap(long long arcs) { return (int)(2 * arcs / kSortSmall + 2
 int launch_build_graph_sparse(const GSet &gs, const BuildBufs &bb, const SparseBufs &sb, int max_n, int *status,
                               unsigned long long *counts, long long ncounts, bool relabel, int num_sms,
                               cudaStream_t s) {
-    static bool smem_opt_in = false;
-    if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_scan_degrees, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(kScanSingleMax * 4)) != cudaSuccess ||
-            cudaFuncSetAttribute(k_relabel_graph, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 kRelabelSmemMax * 4) != cudaSuccess)
-            return ACC_ERR_CUDA;
-        smem_opt_in = true;
-    }
+    if (!raise_build_limits()) return ACC_ERR_CUDA;
     int launches = 0;
     const long long NV = gs.NV;
     const int arcs_grid = grid_for(max(gs.M, NV), 256, num_sms);

@@ -1189,13 +1189,8 @@ int scaled_grid(int per_sm, int num_sms, int grid_num, int grid_den) {
 
 template <int K, int PHASE, bool HASH, bool BESIDE, int SLOTS = kSlots>
 int wedge_phase(const PartialArgs &a, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
-    static bool smem_opt_in = false;
-    if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_wedges<K, PHASE, HASH, BESIDE, SLOTS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)wedge_smem(K, PHASE, SLOTS)) != cudaSuccess)
-            return ACC_ERR_CUDA;
-        smem_opt_in = true;
-    }
+    static std::atomic<unsigned long long> limit{0};
+    if (!raise_shared_limit(k_wedges<K, PHASE, HASH, BESIDE, SLOTS>, wedge_smem(K, PHASE, SLOTS), limit)) return ACC_ERR_CUDA;
     // (no kernel waits on another block, so the grid need not be resident as a whole)
     const int grid = scaled_grid(K == 5 ? 3 : (SLOTS == kSetSlots && PHASE == 1 ? 2 : 4), num_sms, grid_num, grid_den);
     launch_pdl(k_wedges<K, PHASE, HASH, BESIDE, SLOTS>, grid, kPThreads, wedge_smem(K, PHASE, SLOTS), s, a);

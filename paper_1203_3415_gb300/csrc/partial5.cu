@@ -1052,13 +1052,9 @@ void partial5_tables(const uint32_t *code5, const uint32_t *code4, const uint32_
 }
 
 int launch_partial5(PartialArgs &a, long long max_entries, int num_sms, cudaStream_t s, int grid_num, int grid_den) {
-    static bool smem_opt_in = false;
-    if (!smem_opt_in) {
-        if (cudaFuncSetAttribute(k_cycles5<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cycle_smem(1)) != cudaSuccess ||
-            cudaFuncSetAttribute(k_cycles5<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)cycle_smem(2)) != cudaSuccess)
-            return ACC_ERR_CUDA;
-        smem_opt_in = true;
-    }
+    static std::atomic<unsigned long long> limit[2];
+    if (!raise_shared_limit(k_cycles5<1>, cycle_smem(1), limit[0]) || !raise_shared_limit(k_cycles5<2>, cycle_smem(2), limit[1]))
+        return ACC_ERR_CUDA;
     // Most of these passes wait on memory or on their last few blocks, so they run
     // side by side where the data allows (JoinsPrevious): the 5-cycles beside the
     // wedges of k = 4, then the pairs' first phase beside the finish, then its second

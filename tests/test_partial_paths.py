@@ -48,6 +48,25 @@ template <class T> inline cudaError_t emu_counted_free(T *p) {
     }
     return cudaFree((void *)p);
 }
+// two devices; a kernel's limit of shared memory is set on the current one
+extern int emu_device;
+void emu_limit_set(const void *kernel, int bytes);
+inline cudaError_t emu_set_device(int d) {
+    if (d < 0 || d > 1) return 1;
+    emu_device = d;
+    return cudaSuccess;
+}
+inline cudaError_t emu_get_device(int *d) {
+    *d = emu_device;
+    return cudaSuccess;
+}
+template <class T> inline cudaError_t emu_set_limit(T kernel, cudaFuncAttribute, int bytes) {
+    emu_limit_set((const void *)kernel, bytes);
+    return cudaSuccess;
+}
+#define cudaSetDevice emu_set_device
+#define cudaGetDevice emu_get_device
+#define cudaFuncSetAttribute emu_set_limit
 #define cudaMalloc emu_counted_malloc
 #define cudaFree emu_counted_free
 extern unsigned long long emu_scans;  // k = 5 counts left to the list scan
@@ -69,6 +88,15 @@ unsigned long long emu_scans = 0, emu_partials = 0, emu_held = 0, emu_most = ~0u
 std::map<void *, size_t> &emu_sizes() {
     static std::map<void *, size_t> m;
     return m;
+}
+int emu_device = 0;
+static std::map<const void *, int> emu_limits[2];
+void emu_limit_set(const void *kernel, int bytes) { emu_limits[emu_device][kernel] = bytes; }
+// kernels whose limit was raised on device 0, and on both devices alike
+extern "C" void emu_limit_counts(int *first, int *both) {
+    *first = (int)emu_limits[0].size();
+    *both = 0;
+    for (auto &l : emu_limits[0]) *both += emu_limits[1].count(l.first) && emu_limits[1][l.first] == l.second;
 }
 extern "C" unsigned long long emu_scan_count() { return emu_scans; }
 extern "C" unsigned long long emu_partial_count() { return emu_partials; }
@@ -267,6 +295,28 @@ def host_short_memory(lib):
     return out
 
 
+def host_two_devices(lib):
+    """The same counts on device 0, then on device 1: kernels whose limit of shared
+    memory was raised on the first, and on both."""
+    from tests.emu.lib_scenarios import Ctx, ok
+
+    class On(Ctx):
+        def __init__(self, lib, device):
+            self.lib, self.h = lib, ctypes.c_void_p()
+            ok(lib.acc_ctx_create(ctypes.byref(self.h), device), "acc_ctx_create")
+    g, big = fan(6, 4, 8, 1), fan(13, 12, 1200, 1)
+    for device in (0, 1):
+        c = On(lib, device)
+        count_set(lib, c, [big, big], 3)
+        count_set(lib, c, [g, g], 4)
+        count_set(lib, c, [g], 4)
+        count_set(lib, c, [g], 5)
+        c.close()
+    first, both = ctypes.c_int(), ctypes.c_int()
+    lib.emu_limit_counts(ctypes.byref(first), ctypes.byref(both))
+    return [first.value, both.value]
+
+
 def host_many_graphs(lib):
     """Sets of `graphs` graphs of n vertices and m arcs: counted by partial patterns?"""
     from tests.emu.lib_scenarios import Ctx
@@ -351,6 +401,14 @@ RUNS["sparse"] = ("k5_sparse", {})
 def test_sparse_uniform_graphs_are_scanned(on_host):
     """k = 5, sum of d (d - 1) (d - 2) / 2 below 15 a vertex: left to the scan."""
     assert on_host("sparse") == [1, 1]
+
+
+RUNS["devices"] = ("two_devices", {})
+
+
+def test_every_device_gets_the_kernels_shared_memory(on_host):
+    first, both = on_host("devices")
+    assert first == both > 20
 
 
 if __name__ == "__main__":
