@@ -299,7 +299,8 @@ ACC_API int acc_ctx_set_randomise_memory(acc_ctx *ctx, int64_t bytes);
  * admitted as soon as one of the server's slots is free and the slot's device
  * workspace for it fits the memory budget, in the order of the admission
  * policy (acc_server_set_policy; a request that cannot fit even with every
- * slot idle fails with ACC_ERR_NOMEM).  Each slot has its own
+ * slot idle fails with ACC_ERR_NOMEM; one that fits without the counters of the
+ * partial patterns alone is counted by the lists, see ACC_MODE_COUNT).  Each slot has its own
  * context and CUDA stream, so admitted requests overlap on the device; a
  * request on a graph of at most 4096 vertices takes 1/8 of the GPU's
  * enumeration grid (its few work units cannot fill more) and so runs beside

@@ -343,67 +343,94 @@ int size_check(const acc_ctx *c, long long n) {
 // and the neighbours of w2; k = 4: two neighbour lists; k = 3: one).
 long long sparse_list_entries(int maxdeg) { return (3LL * maxdeg + 64 + 31) & ~31LL; }
 
-// Workspace for a set of NV vertices in blocks of state_words words, with at
-// most `arcs` arcs and graphs of at most max_n vertices.
-int grow_workspace(acc_ctx *c, long long NV, long long state_words, long long arcs, int max_n, int k, int B,
-                     bool relabel) {
-    int rc;
+// What a set of NV vertices in a dense block of `words` words, with at most `arcs`
+// arcs and graphs of at most max_n vertices, needs: need(&buffer, &capacity,
+// elements) for each buffer.  (The sparse build's overflow lists are sized by the
+// largest degree, once it is known: run_set.)
+template <typename Need>
+void workspace_needs(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
+                     int warps, Need need) {
     const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
     const bool partial = uses_partial(c, k, max_n, arcs, relabel, B);
     const bool partial5 = uses_partial5(c, k, max_n, arcs, relabel, B);
+    const size_t n1 = (size_t)NV + 1, entries = (size_t)(2 * arcs);
     if (partial5) {
-        if ((rc = grow(&c->p5_vert, &c->p5_vert_cap, 3 * ((size_t)NV + 1)))) return rc;
-        if ((rc = grow(&c->p5_sums, &c->p5_sums_cap, (size_t)num_classes(5) + 16 + kCtrs))) return rc;
+        need(&c->p5_vert, &c->p5_vert_cap, 3 * n1);
+        need(&c->p5_sums, &c->p5_sums_cap, (size_t)num_classes(5) + 16 + kCtrs);
     }
     if (partial || partial5) {
-        if ((rc = grow(&c->pp_nd, &c->pp_nd_cap, (size_t)NV + 1))) return rc;
-        if ((rc = grow(&c->pp_part, &c->pp_part_cap, (size_t)B * num_classes(k == 5 ? 4 : k)))) return rc;
-        if ((rc = grow(&c->pp_done, &c->pp_done_cap, (size_t)B))) return rc;
-        if (k >= 4 && (rc = grow(&c->pp_wedges, &c->pp_wedges_cap, (size_t)NV + 1))) return rc;
-        if (k >= 4 && (rc = grow(&c->pp_tri, &c->pp_tri_cap, 3 * (size_t)(2 * arcs) + 1))) return rc;
+        need(&c->pp_nd, &c->pp_nd_cap, n1);
+        need(&c->pp_part, &c->pp_part_cap, (size_t)B * num_classes(k == 5 ? 4 : k));
+        need(&c->pp_done, &c->pp_done_cap, (size_t)B);
+        if (k >= 4) need(&c->pp_wedges, &c->pp_wedges_cap, n1);
+        if (k >= 4) need(&c->pp_tri, &c->pp_tri_cap, 3 * entries + 1);
     }
-    if ((sparse || uses_hash(c, k, max_n)) && (rc = grow(&c->nh, &c->nh_cap, (size_t)kNhWords * (size_t)(2 * arcs) + 4)))
-        return rc;
+    if (sparse || uses_hash(c, k, max_n)) need(&c->nh, &c->nh_cap, (size_t)kNhWords * entries + 4);
     if (sparse) {
-        if ((rc = grow(&c->sp_raw, &c->sp_raw_cap, (size_t)(2 * arcs) + 1))) return rc;
-        if ((rc = grow(&c->sp_merged, &c->sp_merged_cap, (size_t)(2 * arcs) + 1))) return rc;
-        if ((rc = grow(&c->sp_roff, &c->sp_roff_cap, (size_t)NV + 1))) return rc;
-        if ((rc = grow(&c->sp_big, &c->sp_big_cap, (size_t)sparse_big_rows_cap(arcs)))) return rc;
+        need(&c->sp_raw, &c->sp_raw_cap, entries + 1);
+        need(&c->sp_merged, &c->sp_merged_cap, entries + 1);
+        need(&c->sp_roff, &c->sp_roff_cap, n1);
+        need(&c->sp_big, &c->sp_big_cap, (size_t)sparse_big_rows_cap(arcs));
+    } else {
+        need(&c->state, &c->state_cap, (size_t)words + 4);
+        need(&c->occ, &c->occ_cap, (size_t)NV * (size_t)occ_words(max_n) + 1);
     }
-    if (!sparse) {
-        // a reallocation (the capacity changes; the address may not) brings
-        // memory that is not zero: the next build sweeps it
-        const size_t cap_before = c->state_cap;
-        if ((rc = grow(&c->state, &c->state_cap, (size_t)state_words + 4))) {
-            c->state_clean = false;
-            return rc;
-        }
-        if (c->state_cap != cap_before) c->state_clean = false;
-    }
-    if ((size_t)NV + 1 > c->n_cap || !c->deg) {
-        size_t a = 0, b = 0, d = 0, e = 0;
-        cudaFree(c->deg);
-        cudaFree(c->lo);
-        cudaFree(c->nptr);
-        cudaFree(c->label);
-        cudaFree(c->deg_in);
-        c->deg = c->lo = c->label = c->deg_in = nullptr;
-        c->nptr = nullptr;
-        c->n_cap = 0;
-        if ((rc = grow(&c->deg, &a, (size_t)NV + 1))) return rc;
-        if ((rc = grow(&c->lo, &b, (size_t)NV + 1))) return rc;
-        if ((rc = grow(&c->nptr, &d, (size_t)NV + 1))) return rc;
-        if ((rc = grow(&c->label, &e, (size_t)NV + 1))) return rc;
-        e = 0;
-        if ((rc = grow(&c->deg_in, &e, (size_t)NV + 1))) return rc;
-        c->n_cap = a;
-    }
-    if ((rc = grow(&c->tiles, &c->tiles_cap, (size_t)scan_tiles_needed(NV) + 1))) return rc;
-    if ((rc = grow(&c->f5_pre, &c->f5_pre_cap, (size_t)NV + 1))) return rc;
-    if ((rc = grow(&c->nbr, &c->nbr_cap, (size_t)(2 * arcs) + 1))) return rc;
-    if ((rc = grow(&c->src, &c->src_cap, (size_t)(2 * arcs) + 1))) return rc;
-    if ((uses_rev(c, arcs) || (partial && k == 4) || partial5) && (rc = grow(&c->rev, &c->rev_cap, (size_t)(2 * arcs) + 1))) return rc;
-    if (!sparse && (rc = grow(&c->occ, &c->occ_cap, (size_t)NV * (size_t)occ_words(max_n) + 1))) return rc;
+    need(&c->deg, &c->deg_cap, n1);
+    need(&c->lo, &c->lo_cap, n1);
+    need(&c->nptr, &c->nptr_cap, n1);
+    need(&c->label, &c->label_cap, n1);
+    need(&c->deg_in, &c->deg_in_cap, n1);
+    need(&c->tiles, &c->tiles_cap, (size_t)scan_tiles_needed(NV) + 1);
+    need(&c->f5_pre, &c->f5_pre_cap, n1);
+    need(&c->nbr, &c->nbr_cap, entries + 1);
+    need(&c->src, &c->src_cap, entries + 1);
+    if (uses_rev(c, arcs) || (partial && k == 4) || partial5) need(&c->rev, &c->rev_cap, entries + 1);
+    // (partial patterns have no extension lists)
+    if (!sparse && !partial) need(&c->scratch, &c->scratch_cap, (size_t)scratch_per_warp(max_n) * (size_t)warps);
+}
+
+// Every buffer that workspace_needs may ask for: each(&buffer, &capacity).
+template <typename Each>
+void workspace_buffers(acc_ctx *c, Each each) {
+    each(&c->p5_vert, &c->p5_vert_cap);
+    each(&c->p5_sums, &c->p5_sums_cap);
+    each(&c->pp_nd, &c->pp_nd_cap);
+    each(&c->pp_part, &c->pp_part_cap);
+    each(&c->pp_done, &c->pp_done_cap);
+    each(&c->pp_wedges, &c->pp_wedges_cap);
+    each(&c->pp_tri, &c->pp_tri_cap);
+    each(&c->nh, &c->nh_cap);
+    each(&c->sp_raw, &c->sp_raw_cap);
+    each(&c->sp_merged, &c->sp_merged_cap);
+    each(&c->sp_roff, &c->sp_roff_cap);
+    each(&c->sp_big, &c->sp_big_cap);
+    each(&c->state, &c->state_cap);
+    each(&c->occ, &c->occ_cap);
+    each(&c->deg, &c->deg_cap);
+    each(&c->lo, &c->lo_cap);
+    each(&c->nptr, &c->nptr_cap);
+    each(&c->label, &c->label_cap);
+    each(&c->deg_in, &c->deg_in_cap);
+    each(&c->tiles, &c->tiles_cap);
+    each(&c->f5_pre, &c->f5_pre_cap);
+    each(&c->nbr, &c->nbr_cap);
+    each(&c->src, &c->src_cap);
+    each(&c->rev, &c->rev_cap);
+    each(&c->scratch, &c->scratch_cap);
+}
+
+int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel) {
+    const int warps = enum_grid_warps(k, c->num_sms);
+    if (warps < 0) return warps;
+    int rc = ACC_OK;
+    // a reallocation (the capacity changes; the address may not) brings
+    // memory that is not zero: the next build sweeps it
+    const size_t state_before = c->state_cap;
+    workspace_needs(c, NV, words, arcs, max_n, k, B, relabel, warps, [&](auto **p, size_t *cap, size_t need) {
+        if (!rc) rc = grow(p, cap, need);
+    });
+    if (c->state_cap != state_before) c->state_clean = false;
+    if (rc) return rc;
     if (!c->info) {
         if (!ok(cudaMalloc(&c->info, sizeof(GraphInfo)))) return ACC_ERR_NOMEM;
         if (!ok(cudaMemset(c->info, 0, sizeof(GraphInfo)))) return ACC_ERR_CUDA;
@@ -415,12 +442,6 @@ int grow_workspace(acc_ctx *c, long long NV, long long state_words, long long ar
     if (!c->status_dev) {
         if (!ok(cudaMalloc(&c->status_dev, sizeof(int)))) return ACC_ERR_NOMEM;
     }
-    const int warps = enum_grid_warps(k, c->num_sms);
-    if (warps < 0) return warps;
-    // the sparse build sizes the overflow lists by the largest degree, once
-    // it is known (run_set); partial patterns have no extension lists
-    if (!sparse && !partial && (rc = grow(&c->scratch, &c->scratch_cap, (size_t)scratch_per_warp(max_n) * (size_t)warps)))
-        return rc;
     if (!c->maxdeg_host && !ok(cudaMallocHost(&c->maxdeg_host, sizeof(int)))) return ACC_ERR_NOMEM;
     return ACC_OK;
 }
@@ -457,14 +478,14 @@ void free_partial(acc_ctx *c, bool sparse) {
 // acc_motif_prepare or acc_motif_batch_prepare).
 int ensure_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel) {
     const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
-    const int rc = grow_workspace(c, NV, sparse ? 0 : words, arcs, max_n, k, B, relabel);
+    const int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel);
     if (rc != ACC_ERR_NOMEM || t_alloc_in_capture ||
         !(uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B)))
         return rc;
     c->partial_arcs_end = arcs;
     const bool still = sparse_path(c, k, max_n, arcs, relabel, B);
     free_partial(c, sparse && !still);
-    return grow_workspace(c, NV, still ? 0 : words, arcs, max_n, k, B, relabel);
+    return grow_workspace(c, NV, words, arcs, max_n, k, B, relabel);
 }
 
 // Build + enumerate one graph set into counts[B * num_classes(k)].
@@ -796,33 +817,44 @@ int batch_workspace(acc_ctx *c) {
 
 namespace acc {
 
-long long ctx_footprint(const acc_ctx *c, long long n, long long m, int k) {
+long long ctx_footprint(acc_ctx *c, long long n, long long m, int k, bool partial) {
     const long long pitch = state_pitch((int)n);
-    const long long warps = enum_grid_warps(k, c->num_sms);
-    // (a graph that takes the sparse build by sparse_auto needs less than this)
+    const long long warps = enum_grid_warps(k, c->num_sms) > 0 ? enum_grid_warps(k, c->num_sms) : 0;
+    const long long arcs_end = c->partial_arcs_end;
+    ctx_allow_partial(c, partial);
+    // the list scan's share, whichever way the graph is counted, so that admission
+    // does not depend on it.  The sparse build keeps raw and merged rows (2 m words
+    // each) and row offsets instead of the dense block and its bitmap; its overflow
+    // lists are bounded by the largest degree, itself at most 2m and n
     const bool sparse = sparse_build(c, (int)n);
     const long long hash_bytes = uses_hash(c, k, (int)n) ? 4LL * kNhWords * (2 * m + 1) : 0;
-    // the sparse build keeps raw and merged rows (2 m words each) and row
-    // offsets instead of the dense block and its bitmap; its overflow lists
-    // are bounded by the largest degree, itself at most 2m and n
     const long long list_n = sparse ? (2 * m < n ? 2 * m : n) : n;
-    const long long lists = (sparse ? 2 * sparse_list_entries((int)list_n) + 2 * kPartBRows : scratch_per_warp((int)n)) *
-                            (warps > 0 ? warps : 0) * 4;
-    // k = 3, 4 by partial patterns hold counters per entry instead of the
-    // scan's lists; a slot is sized for either, so that admission does not
-    // depend on the path
-    const long long counters = 12 * (n + 1) + (k == 4 ? (24 + 8) * (2 * m + 1) : 0);
-    const long long bytes = (sparse ? 16 * (m + 1) + 8 * (n + 1) : n * pitch * 4 + 4 * n * occ_words((int)n)) +
-                            5 * 4 * (n + 1) + 8 * (n + 1) + (uses_rev(c, m) ? 16 : 8) * (2 * m + 1) + hash_bytes +
-                            (long long)kQueueCap * 16 + (lists > counters ? lists : counters);
-    return bytes + bytes / 4;
+    const long long list_words =
+        (sparse ? 2 * sparse_list_entries((int)list_n) + 2 * kPartBRows : scratch_per_warp((int)n)) * warps;
+    const long long scan = (sparse ? 16 * (m + 1) + 8 * (n + 1) : n * pitch * 4 + 4 * n * occ_words((int)n)) +
+                           5 * 4 * (n + 1) + 8 * (n + 1) + (uses_rev(c, m) ? 16 : 8) * (2 * m + 1) + hash_bytes +
+                           (long long)kQueueCap * 16 + list_words * 4;
+    // what the context holds already, and what would grow
+    long long held = (long long)kQueueCap * 16;
+    workspace_buffers(c, [&](auto **p, size_t *cap) { held += (long long)(*cap * sizeof(**p)); });
+    const bool relabel = n >= kRelabelMinN;
+    const auto grown = [](size_t need) { return need + need / 4 + 64; };
+    workspace_needs(c, n, n * pitch, m, (int)n, k, 1, relabel, (int)warps, [&](auto **p, size_t *cap, size_t need) {
+        if (need > *cap) held += (long long)((grown(need) - *cap) * sizeof(**p));
+    });
+    if (sparse_path(c, k, (int)n, m, relabel, 1) && sparse_waits(c, k, (int)n, m, relabel, 1) &&
+        (size_t)list_words > c->scratch_cap)
+        held += (long long)(grown((size_t)list_words) - c->scratch_cap) * 4;
+    c->partial_arcs_end = arcs_end;
+    return held > scan + scan / 4 ? held : scan + scan / 4;
 }
 
-int ctx_reserve(acc_ctx *c, long long n, long long m, int k) {
+int ctx_reserve(acc_ctx *c, long long n, long long m, int k, bool partial) {
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     const int rc = ensure_tab5(c, c->own);
     if (rc) return rc;
     const bool relabel = n >= kRelabelMinN;
+    ctx_allow_partial(c, partial);
     return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, relabel);
 }
 

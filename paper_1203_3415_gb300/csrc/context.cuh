@@ -33,7 +33,7 @@ struct acc_ctx {
     bool state_clean = false;  // every pair-state word is zero (each call clears what it set)
     int *deg = nullptr, *lo = nullptr, *label = nullptr, *deg_in = nullptr;
     long long *nptr = nullptr;
-    size_t n_cap = 0;
+    size_t deg_cap = 0, lo_cap = 0, label_cap = 0, deg_in_cap = 0, nptr_cap = 0;
     long long *tiles = nullptr;
     size_t tiles_cap = 0;
     long long *f5_pre = nullptr;  // k = 5 formula path: prefix of C(deg, 2)
@@ -146,9 +146,14 @@ struct acc_ctx {
 
 
 namespace acc {
-// Device bytes a context's workspace needs for one graph of n vertices and m
-// arcs at k (with the growth margin), and pre-sizing it (plus the tables of
-// every k) so later counts of graphs up to that size allocate nothing.
-long long ctx_footprint(const acc_ctx *c, long long n, long long m, int k);
-int ctx_reserve(acc_ctx *c, long long n, long long m, int k);
+// Device bytes a context may hold for a count of one graph of n vertices and m arcs
+// at k: what it holds already and what would grow (with the growth margin), and no
+// less than the list scan's share.  partial: with the counters of the partial
+// patterns, where the count takes them.
+long long ctx_footprint(acc_ctx *c, long long n, long long m, int k, bool partial);
+// Pre-sizes a context (and the tables of every k) so that later counts of graphs up
+// to that size allocate nothing.
+int ctx_reserve(acc_ctx *c, long long n, long long m, int k, bool partial);
+// From which arcs on the context's sets are counted by the list scan alone.
+inline void ctx_allow_partial(acc_ctx *c, bool partial) { c->partial_arcs_end = partial ? INT64_MAX : 0; }
 }  // namespace acc

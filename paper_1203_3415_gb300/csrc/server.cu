@@ -159,18 +159,23 @@ int progress(acc_server *sv) {
         const long long id = sv->queue[pick];
         Req &r = sv->reqs[(size_t)id];
         const Graph &g = sv->graphs[(size_t)r.graph];
-        // the free slot that needs the least growth and stays within budget
+        // the free slot that needs the least growth and stays within budget; where
+        // none does with the counters of the partial patterns, without them
         int best = -1;
         long long best_fp = 0;
-        for (size_t i = 0; i < sv->slots.size(); i++) {
-            Slot &sl = sv->slots[i];
-            if (sl.req >= 0) continue;
-            const long long need = acc::ctx_footprint(sl.ctx, g.n, g.m, r.k);
-            const long long fp = need > sl.footprint ? need : sl.footprint;
-            if (used_except(sv, i) + fp > sv->budget) continue;
-            if (best < 0 || fp < best_fp) {
-                best = (int)i;
-                best_fp = fp;
+        bool partial = true;
+        for (int pass = 0; pass < 2 && best < 0; pass++) {
+            partial = pass == 0;
+            for (size_t i = 0; i < sv->slots.size(); i++) {
+                Slot &sl = sv->slots[i];
+                if (sl.req >= 0) continue;
+                const long long need = acc::ctx_footprint(sl.ctx, g.n, g.m, r.k, partial);
+                const long long fp = need > sl.footprint ? need : sl.footprint;
+                if (used_except(sv, i) + fp > sv->budget) continue;
+                if (best < 0 || fp < best_fp) {
+                    best = (int)i;
+                    best_fp = fp;
+                }
             }
         }
         if (best < 0) {
@@ -187,6 +192,7 @@ int progress(acc_server *sv) {
         sl.footprint = best_fp;
         sl.ctx->grid_num = g.n <= kSmallGraph ? kSmallShare : kBigShare;
         sl.ctx->grid_den = 8;
+        acc::ctx_allow_partial(sl.ctx, partial);
         r.t_start = now_s();
         const int rc = acc_motif_count(sl.ctx, g.rowptr, g.col, g.n, g.m, r.k, sl.s, sl.d_counts, sl.d_status);
         sv->queue.erase(sv->queue.begin() + (long)pick);
@@ -293,13 +299,19 @@ int acc_server_reserve(acc_server *sv) {
     for (size_t i = 0; i < sv->slots.size(); i++) {
         Slot &sl = sv->slots[i];
         long long fp = 0;
-        for (int k = 3; k <= 5; k++) {
-            const long long f = acc::ctx_footprint(sl.ctx, n, m, k);
-            if (f > fp) fp = f;
+        bool partial = true;
+        for (int pass = 0; pass < 2; pass++) {
+            partial = pass == 0;
+            fp = 0;
+            for (int k = 3; k <= 5; k++) {
+                const long long f = acc::ctx_footprint(sl.ctx, n, m, k, partial);
+                if (f > fp) fp = f;
+            }
+            if (used_except(sv, i) + fp <= sv->budget) break;
         }
         if (used_except(sv, i) + fp > sv->budget) continue;  // this slot grows on demand
         for (int k = 3; k <= 5; k++) {
-            const int rc = acc::ctx_reserve(sl.ctx, n, m, k);
+            const int rc = acc::ctx_reserve(sl.ctx, n, m, k, partial);
             if (rc) return rc;
         }
         if (fp > sl.footprint) sl.footprint = fp;

@@ -84,6 +84,13 @@ template <class A> inline void emu_cycles_enter(const A &a, unsigned long long *
 
 GLOBALS = r"""
 #include "hooks.h"
+#include "context.cuh"
+extern "C" long long emu_footprint(acc_ctx *c, long long n, long long m, int k, int partial) {
+    return acc::ctx_footprint(c, n, m, k, partial != 0);
+}
+extern "C" int emu_reserve(acc_ctx *c, long long n, long long m, int k, int partial) {
+    return acc::ctx_reserve(c, n, m, k, partial != 0);
+}
 unsigned long long emu_scans = 0, emu_partials = 0, emu_held = 0, emu_most = ~0ull;
 std::map<void *, size_t> &emu_sizes() {
     static std::map<void *, size_t> m;
@@ -138,7 +145,7 @@ def host_lib(tmp_path_factory):
             open(units[-1], "w").write('#include "hooks.h"\n' + _launches_to_calls(src))
     asan = subprocess.run(["g++", "-print-file-name=libasan.so"], capture_output=True, text=True).stdout.strip()
     san = ["-fsanitize=address", "-DEMU_EXACT_ALLOC", "-DEMU_LANE_STACK=65536"] if os.path.isabs(asan) else []
-    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0", "-DACC_QUEUE_CAP=1024ull",
+    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0", "-DACC_QUEUE_CAP=1024ull", "-DACC_SPARSE_MIN_N=20000",
                                "-DEMU_NUM_SMS=1", "-I", str(out), "-I", EMU, "-I", os.path.join(EMU, "fake"), "-I", CSRC,
                                "-c", u, "-o", str(out / f"u{i}.o")], stderr=subprocess.PIPE, text=True)
              for i, u in enumerate(units)]
@@ -295,6 +302,61 @@ def host_short_memory(lib):
     return out
 
 
+def host_footprint(lib):
+    """Bytes held by a slot's context after it was made ready for a sequence of
+    (n, m, k), over its footprint before the last; the most of all sequences."""
+    from tests.emu.lib_scenarios import Ctx, ok
+    lib.emu_bytes.restype = lib.emu_footprint.restype = ctypes.c_longlong
+    lib.emu_footprint.argtypes = lib.emu_reserve.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong,
+                                                             ctypes.c_int, ctypes.c_int]
+    tables = Ctx(lib)
+    ok(lib.acc_motif_prepare(tables.h, 5, None), "prepare")
+    most = 0.0
+    for graphs in ([(3000, 400000)], [(3000, 9000)], [(20000, 300000)], [(19000, 90000), (2000, 500000)]):
+        for ks in ((3, 4, 5), (5, 4, 3), (4, 5), (5,), (4,)):
+            for partial in (1, 0):
+                c = Ctx(lib)
+                before = lib.emu_bytes()
+                for n, m in graphs:
+                    for k in ks:
+                        fp = lib.emu_footprint(c.h, n, m, k, partial)
+                        ok(lib.emu_reserve(c.h, n, m, k, partial), "reserve")
+                        most = max(most, (lib.emu_bytes() - before) / (fp + 4096.0))
+                c.close()
+    tables.close()
+    return most
+
+
+def host_server_budget(lib):
+    """A server whose budget holds the list scan's workspace, not the pattern
+    counters: the request's state, and whether patterns counted it."""
+    from tests.emu.lib_scenarios import Ctx, P, csr, ok
+    n = 1024
+    key = np.random.default_rng(3).permutation(n * (n - 1))[:8000]
+    src, dst = key // (n - 1), key % (n - 1)
+    dst = dst + (dst >= src)
+    rp, cl = csr(n, src, dst)
+    lib.emu_footprint.restype = ctypes.c_longlong
+    lib.emu_footprint.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    c = Ctx(lib)
+    scan, patterns = (lib.emu_footprint(c.h, n, len(cl), 4, partial) for partial in (0, 1))
+    c.close()
+    seen = []
+    for budget in (scan, patterns):
+        srv, gid, rid, state = ctypes.c_void_p(), ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int32()
+        out = np.zeros(199, np.int64)
+        before = lib.emu_partial_count()
+        ok(lib.acc_server_create(ctypes.byref(srv), 0, 1, budget), "server_create")
+        ok(lib.acc_server_add_graph(srv, P(rp), P(cl), n, len(cl), ctypes.byref(gid)), "add_graph")
+        ok(lib.acc_server_submit(srv, gid.value, 4, ctypes.byref(rid)), "submit")
+        ok(lib.acc_server_drain(srv), "drain")
+        ok(lib.acc_server_poll(srv, rid, ctypes.byref(state), P(out), None), "poll")
+        lib.acc_server_destroy(srv)
+        assert state.value < 0 or np.array_equal(out, oracle.count(n, src, dst, 4))
+        seen.append([state.value, lib.emu_partial_count() > before])
+    return [scan < patterns] + seen
+
+
 def host_two_devices(lib):
     """The same counts on device 0, then on device 1: kernels whose limit of shared
     memory was raised on the first, and on both."""
@@ -409,6 +471,20 @@ RUNS["devices"] = ("two_devices", {})
 def test_every_device_gets_the_kernels_shared_memory(on_host):
     first, both = on_host("devices")
     assert first == both > 20
+
+
+RUNS["footprint"] = ("footprint", {})
+RUNS["budget"] = ("server_budget", {})
+
+
+def test_footprint_covers_what_a_slot_holds(on_host):
+    assert on_host("footprint") <= 1.0
+
+
+def test_requests_that_fit_by_the_scan_alone_are_served(on_host):
+    import paper_1203_3415_gb300 as acc
+    done = acc.ACC_REQ_DONE
+    assert on_host("budget") == [True, [done, False], [done, True]]
 
 
 if __name__ == "__main__":
