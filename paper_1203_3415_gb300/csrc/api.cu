@@ -346,13 +346,15 @@ long long sparse_list_entries(int maxdeg) { return (3LL * maxdeg + 64 + 31) & ~3
 // What a set of NV vertices in a dense block of `words` words, with at most `arcs`
 // arcs and graphs of at most max_n vertices, needs: need(&buffer, &capacity,
 // elements) for each buffer.  (The sparse build's overflow lists are sized by the
-// largest degree, once it is known: run_set.)
+// largest degree, once it is known: run_set.)  either: for the list scan and, where a
+// set of no more arcs may take them, the partial patterns.
 template <typename Need>
 void workspace_needs(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
-                     int warps, Need need) {
+                     int warps, bool either, Need need) {
     const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
-    const bool partial = uses_partial(c, k, max_n, arcs, relabel, B);
-    const bool partial5 = uses_partial5(c, k, max_n, arcs, relabel, B);
+    const bool may = either && count_family(c) && relabel && arcs >= ACC_PARTIAL_MIN_ARCS && arcs < c->partial_arcs_end;
+    const bool partial = uses_partial(c, k, max_n, arcs, relabel, B) || (may && k <= 4);
+    const bool partial5 = uses_partial5(c, k, max_n, arcs, relabel, B) || (may && k == 5 && B == 1);
     const size_t n1 = (size_t)NV + 1, entries = (size_t)(2 * arcs);
     if (partial5) {
         need(&c->p5_vert, &c->p5_vert_cap, 3 * n1);
@@ -386,7 +388,7 @@ void workspace_needs(acc_ctx *c, long long NV, long long words, long long arcs, 
     need(&c->src, &c->src_cap, entries + 1);
     if (uses_rev(c, arcs) || (partial && k == 4) || partial5) need(&c->rev, &c->rev_cap, entries + 1);
     // (partial patterns have no extension lists)
-    if (!sparse && !partial) need(&c->scratch, &c->scratch_cap, (size_t)scratch_per_warp(max_n) * (size_t)warps);
+    if (!sparse && (!partial || either)) need(&c->scratch, &c->scratch_cap, (size_t)scratch_per_warp(max_n) * (size_t)warps);
 }
 
 // Every buffer that workspace_needs may ask for: each(&buffer, &capacity).
@@ -419,14 +421,15 @@ void workspace_buffers(acc_ctx *c, Each each) {
     each(&c->scratch, &c->scratch_cap);
 }
 
-int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel) {
+int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
+                   bool either) {
     const int warps = enum_grid_warps(k, c->num_sms);
     if (warps < 0) return warps;
     int rc = ACC_OK;
     // a reallocation (the capacity changes; the address may not) brings
     // memory that is not zero: the next build sweeps it
     const size_t state_before = c->state_cap;
-    workspace_needs(c, NV, words, arcs, max_n, k, B, relabel, warps, [&](auto **p, size_t *cap, size_t need) {
+    workspace_needs(c, NV, words, arcs, max_n, k, B, relabel, warps, either, [&](auto **p, size_t *cap, size_t need) {
         if (!rc) rc = grow(p, cap, need);
     });
     if (c->state_cap != state_before) c->state_clean = false;
@@ -476,16 +479,17 @@ void free_partial(acc_ctx *c, bool sparse) {
 // list scan, and 40 more where sparse_auto takes the sparse build: where the device has no room for them the set is counted by
 // the scan, as are the context's later sets of as many arcs (until the next
 // acc_motif_prepare or acc_motif_batch_prepare).
-int ensure_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel) {
+int ensure_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
+                     bool either = false) {
     const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
-    const int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel);
+    const int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, either);
     if (rc != ACC_ERR_NOMEM || t_alloc_in_capture ||
-        !(uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B)))
+        !(either || uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B)))
         return rc;
     c->partial_arcs_end = arcs;
     const bool still = sparse_path(c, k, max_n, arcs, relabel, B);
     free_partial(c, sparse && !still);
-    return grow_workspace(c, NV, words, arcs, max_n, k, B, relabel);
+    return grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, either);
 }
 
 // Build + enumerate one graph set into counts[B * num_classes(k)].
@@ -817,45 +821,57 @@ int batch_workspace(acc_ctx *c) {
 
 namespace acc {
 
-long long ctx_footprint(acc_ctx *c, long long n, long long m, int k, bool partial) {
-    const long long pitch = state_pitch((int)n);
-    const long long warps = enum_grid_warps(k, c->num_sms) > 0 ? enum_grid_warps(k, c->num_sms) : 0;
-    const long long arcs_end = c->partial_arcs_end;
-    ctx_allow_partial(c, partial);
-    // the list scan's share, whichever way the graph is counted, so that admission
-    // does not depend on it.  The sparse build keeps raw and merged rows (2 m words
-    // each) and row offsets instead of the dense block and its bitmap; its overflow
-    // lists are bounded by the largest degree, itself at most 2m and n
-    const bool sparse = sparse_build(c, (int)n);
-    const long long hash_bytes = uses_hash(c, k, (int)n) ? 4LL * kNhWords * (2 * m + 1) : 0;
-    const long long list_n = sparse ? (2 * m < n ? 2 * m : n) : n;
-    const long long list_words =
-        (sparse ? 2 * sparse_list_entries((int)list_n) + 2 * kPartBRows : scratch_per_warp((int)n)) * warps;
-    const long long scan = (sparse ? 16 * (m + 1) + 8 * (n + 1) : n * pitch * 4 + 4 * n * occ_words((int)n)) +
-                           5 * 4 * (n + 1) + 8 * (n + 1) + (uses_rev(c, m) ? 16 : 8) * (2 * m + 1) + hash_bytes +
-                           (long long)kQueueCap * 16 + list_words * 4;
-    // what the context holds already, and what would grow
-    long long held = (long long)kQueueCap * 16;
-    workspace_buffers(c, [&](auto **p, size_t *cap) { held += (long long)(*cap * sizeof(**p)); });
+long long ctx_footprint(acc_ctx *c, long long n, long long m, int k0, int k1, Ways ways) {
+    const long long pitch = state_pitch((int)n), arcs_end = c->partial_arcs_end;
     const bool relabel = n >= kRelabelMinN;
-    const auto grown = [](size_t need) { return need + need / 4 + 64; };
-    workspace_needs(c, n, n * pitch, m, (int)n, k, 1, relabel, (int)warps, [&](auto **p, size_t *cap, size_t need) {
-        if (need > *cap) held += (long long)((grown(need) - *cap) * sizeof(**p));
-    });
-    if (sparse_path(c, k, (int)n, m, relabel, 1) && sparse_waits(c, k, (int)n, m, relabel, 1) &&
-        (size_t)list_words > c->scratch_cap)
-        held += (long long)(grown((size_t)list_words) - c->scratch_cap) * 4;
+    ctx_allow_partial(c, ways != Ways::kScan);
+    // what the context holds already
+    long long held = (long long)kQueueCap * 16, least = 0;
+    workspace_buffers(c, [&](auto **p, size_t *cap) { held += (long long)(*cap * sizeof(**p)); });
+    // what would grow, by the buffer's capacity
+    std::vector<std::pair<const size_t *, long long>> growth;
+    auto grows = [&](const size_t *cap, size_t need, size_t bytes) {
+        if (need <= *cap) return;
+        const long long more = (long long)((need + need / 4 + 64 - *cap) * bytes);
+        for (auto &g : growth)
+            if (g.first == cap) {
+                g.second = g.second > more ? g.second : more;
+                return;
+            }
+        growth.push_back({cap, more});
+    };
+    for (int k = k0; k <= k1; k++) {
+        const long long warps = enum_grid_warps(k, c->num_sms) > 0 ? enum_grid_warps(k, c->num_sms) : 0;
+        // the list scan's share, whichever way the graph is counted, so that admission
+        // does not depend on it.  The sparse build keeps raw and merged rows (2 m words
+        // each) and row offsets instead of the dense block and its bitmap; its overflow
+        // lists are bounded by the largest degree, itself at most 2m and n
+        const bool sparse = sparse_build(c, (int)n);
+        const long long hash_bytes = uses_hash(c, k, (int)n) ? 4LL * kNhWords * (2 * m + 1) : 0;
+        const long long list_n = sparse ? (2 * m < n ? 2 * m : n) : n;
+        const long long lists =
+            (sparse ? 2 * sparse_list_entries((int)list_n) + 2 * kPartBRows : scratch_per_warp((int)n)) * warps;
+        const long long scan = (sparse ? 16 * (m + 1) + 8 * (n + 1) : n * pitch * 4 + 4 * n * occ_words((int)n)) +
+                               5 * 4 * (n + 1) + 8 * (n + 1) + (uses_rev(c, m) ? 16 : 8) * (2 * m + 1) + hash_bytes +
+                               (long long)kQueueCap * 16 + lists * 4;
+        least = least > scan + scan / 4 ? least : scan + scan / 4;
+        workspace_needs(c, n, n * pitch, m, (int)n, k, 1, relabel, (int)warps, ways == Ways::kEither,
+                        [&](auto **p, size_t *cap, size_t need) { grows(cap, need, sizeof(**p)); });
+        if (sparse_path(c, k, (int)n, m, relabel, 1) && sparse_waits(c, k, (int)n, m, relabel, 1))
+            grows(&c->scratch_cap, (size_t)lists, sizeof(*c->scratch));
+    }
     c->partial_arcs_end = arcs_end;
-    return held > scan + scan / 4 ? held : scan + scan / 4;
+    for (const auto &g : growth) held += g.second;
+    return held > least ? held : least;
 }
 
-int ctx_reserve(acc_ctx *c, long long n, long long m, int k, bool partial) {
+int ctx_reserve(acc_ctx *c, long long n, long long m, int k, Ways ways) {
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     const int rc = ensure_tab5(c, c->own);
     if (rc) return rc;
     const bool relabel = n >= kRelabelMinN;
-    ctx_allow_partial(c, partial);
-    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, relabel);
+    ctx_allow_partial(c, ways != Ways::kScan);
+    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, relabel, ways == Ways::kEither);
 }
 
 }  // namespace acc

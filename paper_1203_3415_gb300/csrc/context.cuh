@@ -146,14 +146,17 @@ struct acc_ctx {
 
 
 namespace acc {
-// Device bytes a context may hold for a count of one graph of n vertices and m arcs
-// at k: what it holds already and what would grow (with the growth margin), and no
-// less than the list scan's share.  partial: with the counters of the partial
-// patterns, where the count takes them.
-long long ctx_footprint(acc_ctx *c, long long n, long long m, int k, bool partial);
+// The ways a graph may be counted: by the list scan, as the rules have it for the
+// graph, or as they may have it for any graph of no more vertices and arcs (the
+// rules look at arcs a vertex too, so a smaller graph may take the other way).
+enum class Ways { kScan, kRuled, kEither };
+// Device bytes a context may hold for counts of one graph of n vertices and m arcs
+// at k0 to k1: what it holds already and what would grow (with the growth margin),
+// and no less than the list scan's share.
+long long ctx_footprint(acc_ctx *c, long long n, long long m, int k0, int k1, Ways ways);
 // Pre-sizes a context (and the tables of every k) so that later counts of graphs up
 // to that size allocate nothing.
-int ctx_reserve(acc_ctx *c, long long n, long long m, int k, bool partial);
+int ctx_reserve(acc_ctx *c, long long n, long long m, int k, Ways ways);
 // From which arcs on the context's sets are counted by the list scan alone.
 inline void ctx_allow_partial(acc_ctx *c, bool partial) { c->partial_arcs_end = partial ? INT64_MAX : 0; }
 }  // namespace acc

@@ -169,7 +169,8 @@ int progress(acc_server *sv) {
             for (size_t i = 0; i < sv->slots.size(); i++) {
                 Slot &sl = sv->slots[i];
                 if (sl.req >= 0) continue;
-                const long long need = acc::ctx_footprint(sl.ctx, g.n, g.m, r.k, partial);
+                const acc::Ways ways = partial ? acc::Ways::kRuled : acc::Ways::kScan;
+                const long long need = acc::ctx_footprint(sl.ctx, g.n, g.m, r.k, r.k, ways);
                 const long long fp = need > sl.footprint ? need : sl.footprint;
                 if (used_except(sv, i) + fp > sv->budget) continue;
                 if (best < 0 || fp < best_fp) {
@@ -299,19 +300,15 @@ int acc_server_reserve(acc_server *sv) {
     for (size_t i = 0; i < sv->slots.size(); i++) {
         Slot &sl = sv->slots[i];
         long long fp = 0;
-        bool partial = true;
-        for (int pass = 0; pass < 2; pass++) {
-            partial = pass == 0;
-            fp = 0;
-            for (int k = 3; k <= 5; k++) {
-                const long long f = acc::ctx_footprint(sl.ctx, n, m, k, partial);
-                if (f > fp) fp = f;
-            }
+        acc::Ways ways = acc::Ways::kScan;
+        for (const acc::Ways w : {acc::Ways::kEither, acc::Ways::kScan}) {
+            ways = w;
+            fp = acc::ctx_footprint(sl.ctx, n, m, 3, 5, ways);
             if (used_except(sv, i) + fp <= sv->budget) break;
         }
         if (used_except(sv, i) + fp > sv->budget) continue;  // this slot grows on demand
         for (int k = 3; k <= 5; k++) {
-            const int rc = acc::ctx_reserve(sl.ctx, n, m, k, partial);
+            const int rc = acc::ctx_reserve(sl.ctx, n, m, k, ways);
             if (rc) return rc;
         }
         if (fp > sl.footprint) sl.footprint = fp;

@@ -85,11 +85,11 @@ template <class A> inline void emu_cycles_enter(const A &a, unsigned long long *
 GLOBALS = r"""
 #include "hooks.h"
 #include "context.cuh"
-extern "C" long long emu_footprint(acc_ctx *c, long long n, long long m, int k, int partial) {
-    return acc::ctx_footprint(c, n, m, k, partial != 0);
+extern "C" long long emu_footprint(acc_ctx *c, long long n, long long m, int k0, int k1, int ways) {
+    return acc::ctx_footprint(c, n, m, k0, k1, (acc::Ways)ways);
 }
-extern "C" int emu_reserve(acc_ctx *c, long long n, long long m, int k, int partial) {
-    return acc::ctx_reserve(c, n, m, k, partial != 0);
+extern "C" int emu_reserve(acc_ctx *c, long long n, long long m, int k, int ways) {
+    return acc::ctx_reserve(c, n, m, k, (acc::Ways)ways);
 }
 unsigned long long emu_scans = 0, emu_partials = 0, emu_held = 0, emu_most = ~0ull;
 std::map<void *, size_t> &emu_sizes() {
@@ -117,6 +117,8 @@ EDITS = [
      "    emu_cycles_enter(a, a.p5.ctr + kCtrScan, PHASE, cycle_smem(PHASE));\n"),
     ("partial5.cu", "template <int PHASE>\n__global__ void __launch_bounds__(kCThreads",
      "constexpr size_t cycle_smem(int phase);\ntemplate <int PHASE>\n__global__ void __launch_bounds__(kCThreads"),
+    ("api.cu", "(arcs >= 2ll * n || arcs >= ACC_PARTIAL_MIN_ARCS1);",
+     "(arcs >= 2ll * n || arcs >= (long long)emu_env(\"EMU_ARCS1\", ACC_PARTIAL_MIN_ARCS1));"),
     ("partial.cu", "- a.lo[v] > kCycleRows", "- a.lo[v] > (int)emu_env(\"EMU_ROWS\", kCycleRows)"),
     ("partial.cu", "    if (k == 3) launch_pdl(k_partial_prep<3>", "    emu_partials++;\n    if (k == 3) launch_pdl(k_partial_prep<3>"),
     ("partial5.cu", "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n    grid_dep_wait();\n",
@@ -307,22 +309,25 @@ def host_footprint(lib):
     (n, m, k), over its footprint before the last; the most of all sequences."""
     from tests.emu.lib_scenarios import Ctx, ok
     lib.emu_bytes.restype = lib.emu_footprint.restype = ctypes.c_longlong
-    lib.emu_footprint.argtypes = lib.emu_reserve.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong,
-                                                             ctypes.c_int, ctypes.c_int]
+    lib.emu_reserve.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    lib.emu_footprint.argtypes = lib.emu_reserve.argtypes + [ctypes.c_int]
     tables = Ctx(lib)
     ok(lib.acc_motif_prepare(tables.h, 5, None), "prepare")
     most = 0.0
     for graphs in ([(3000, 400000)], [(3000, 9000)], [(20000, 300000)], [(19000, 90000), (2000, 500000)]):
         for ks in ((3, 4, 5), (5, 4, 3), (4, 5), (5,), (4,)):
-            for partial in (1, 0):
-                c = Ctx(lib)
-                before = lib.emu_bytes()
-                for n, m in graphs:
-                    for k in ks:
-                        fp = lib.emu_footprint(c.h, n, m, k, partial)
-                        ok(lib.emu_reserve(c.h, n, m, k, partial), "reserve")
-                        most = max(most, (lib.emu_bytes() - before) / (fp + 4096.0))
-                c.close()
+            for ways in range(3):  # (scan, as ruled, either)
+                for at_once in (False, True):
+                    c = Ctx(lib)
+                    before = lib.emu_bytes()
+                    for n, m in graphs:
+                        fp = lib.emu_footprint(c.h, n, m, min(ks), max(ks), ways)
+                        for k in ks:
+                            if not at_once:
+                                fp = lib.emu_footprint(c.h, n, m, k, k, ways)
+                            ok(lib.emu_reserve(c.h, n, m, k, ways), "reserve")
+                            most = max(most, (lib.emu_bytes() - before) / (fp + 4096.0))
+                    c.close()
     tables.close()
     return most
 
@@ -337,9 +342,10 @@ def host_server_budget(lib):
     dst = dst + (dst >= src)
     rp, cl = csr(n, src, dst)
     lib.emu_footprint.restype = ctypes.c_longlong
-    lib.emu_footprint.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    lib.emu_footprint.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int,
+                                  ctypes.c_int]
     c = Ctx(lib)
-    scan, patterns = (lib.emu_footprint(c.h, n, len(cl), 4, partial) for partial in (0, 1))
+    scan, patterns = (lib.emu_footprint(c.h, n, len(cl), 4, 4, ways) for ways in (0, 1))
     c.close()
     seen = []
     for budget in (scan, patterns):
@@ -355,6 +361,34 @@ def host_server_budget(lib):
         assert state.value < 0 or np.array_equal(out, oracle.count(n, src, dst, 4))
         seen.append([state.value, lib.emu_partial_count() > before])
     return [scan < patterns] + seen
+
+
+def host_reserved(lib):
+    """Bytes a server grows by when it serves, after the reserve, a k = 5 request on
+    the smaller of two graphs, which has more arcs a vertex; whether it was scanned."""
+    from tests.emu.lib_scenarios import P, csr, ok
+    lib.emu_bytes.restype = ctypes.c_longlong
+    rng = np.random.default_rng(3)
+    srv, gid, rid, state = ctypes.c_void_p(), ctypes.c_int32(), ctypes.c_int64(), ctypes.c_int32()
+    ok(lib.acc_server_create(ctypes.byref(srv), 0, 1, 1 << 30), "server_create")
+    graphs = []
+    for n, m in ((3000, 2600), (1024, 2500)):
+        key = rng.permutation(n * (n - 1))[:m]
+        src, dst = key // (n - 1), key % (n - 1)
+        graphs.append((n, src, dst + (dst >= src)))
+        arrays = csr(*graphs[-1])
+        graphs.append(arrays)
+        ok(lib.acc_server_add_graph(srv, P(arrays[0]), P(arrays[1]), n, m, ctypes.byref(gid)), "add_graph")
+    ok(lib.acc_server_reserve(srv), "reserve")
+    before = lib.emu_bytes()
+    ok(lib.acc_server_submit(srv, gid.value, 5, ctypes.byref(rid)), "submit")
+    ok(lib.acc_server_drain(srv), "drain")
+    more = lib.emu_bytes() - before
+    out = np.zeros(9364, np.int64)
+    ok(lib.acc_server_poll(srv, rid, ctypes.byref(state), P(out), None), "poll")
+    lib.acc_server_destroy(srv)
+    assert np.array_equal(out, oracle.count(*graphs[2], 5))
+    return [more, lib.emu_scan_count()]
 
 
 def host_two_devices(lib):
@@ -485,6 +519,15 @@ def test_requests_that_fit_by_the_scan_alone_are_served(on_host):
     import paper_1203_3415_gb300 as acc
     done = acc.ACC_REQ_DONE
     assert on_host("budget") == [True, [done, False], [done, True]]
+
+
+RUNS["reserved"] = ("reserved", dict(EMU_ARCS1=10000))
+
+
+def test_serving_allocates_nothing_after_the_reserve(on_host):
+    """k = 5, a registered graph that is counted by partial patterns where the
+    largest of both sizes would not be."""
+    assert on_host("reserved") == [0, 0]
 
 
 if __name__ == "__main__":
