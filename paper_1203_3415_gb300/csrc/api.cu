@@ -114,7 +114,8 @@ int build_table(int k, cudaStream_t s, SharedTable &t) {
         std::vector<uint32_t> m;
         partial_matrix(k, lut_host, cc_host, m);
         if (!ok(cudaMalloc(&inv, m.size() * 4)) ||
-            !ok(cudaMemcpy(inv, m.data(), m.size() * 4, cudaMemcpyHostToDevice))) {
+            !ok(cudaMemcpyAsync(inv, m.data(), m.size() * 4, cudaMemcpyHostToDevice, s)) ||
+            !ok(cudaStreamSynchronize(s))) {
             rc = inv ? ACC_ERR_CUDA : ACC_ERR_NOMEM;
             goto fail;
         }
@@ -163,7 +164,7 @@ int ensure_tab5(acc_ctx *c, cudaStream_t s) {
             cudaGetLastError();
             return ACC_ERR_NOMEM;
         }
-        if (!ok(cudaMemcpy(d, div5.data(), div5.size(), cudaMemcpyHostToDevice))) {
+        if (!ok(cudaMemcpyAsync(d, div5.data(), div5.size(), cudaMemcpyHostToDevice, s)) || !ok(cudaStreamSynchronize(s))) {
             cudaGetLastError();
             cudaFree(d);
             return ACC_ERR_CUDA;
@@ -436,7 +437,8 @@ int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, in
     if (rc) return rc;
     if (!c->info) {
         if (!ok(cudaMalloc(&c->info, sizeof(GraphInfo)))) return ACC_ERR_NOMEM;
-        if (!ok(cudaMemset(c->info, 0, sizeof(GraphInfo)))) return ACC_ERR_CUDA;
+        // (a set returns before it is done; the caller's stream does not wait for it)
+        if (!ok(cudaMemset(c->info, 0, sizeof(GraphInfo))) || !ok(cudaStreamSynchronize(nullptr))) return ACC_ERR_CUDA;
     }
     if (!c->queue) {
         if (!ok(cudaMalloc(&c->queue, kQueueCap * sizeof(uint4)))) return ACC_ERR_NOMEM;
@@ -1051,7 +1053,10 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     if ((rc = ensure_workspace(c, NV, words, arcs, max_n, k, B, true))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;
     if ((rc = grow(&c->gid, &c->gid_cap, (size_t)NV + 1))) return rc;
-    if (B > 0 && !ok(cudaMemcpy(c->meta_dev, metas.data(), sizeof(GMeta) * (size_t)B, cudaMemcpyHostToDevice)))
+    // (copies from pageable memory return when staged: on the stream that reads them,
+    // which need not wait for the legacy stream)
+    if (B > 0 &&
+        !ok(cudaMemcpyAsync(c->meta_dev, metas.data(), sizeof(GMeta) * (size_t)B, cudaMemcpyHostToDevice, s)))
         return ACC_ERR_CUDA;
     GSet gs = {};
     if (B == 1) gs.one = metas[0];
@@ -1146,7 +1151,7 @@ int acc_swap_randomise(acc_ctx *c, const acc_graph_desc *graphs, int32_t G, int3
         if ((rc = grow(&c->rand_meta, &c->rand_meta_cap, (size_t)G + 1))) return rc;
         if ((rc = grow(&c->rand_rows, &c->rand_rows_cap, (size_t)M + 1))) return rc;
         if (G > 0 &&
-            !ok(cudaMemcpy(c->rand_meta, metas.data(), sizeof(RGraph) * (size_t)G, cudaMemcpyHostToDevice)))
+            !ok(cudaMemcpyAsync(c->rand_meta, metas.data(), sizeof(RGraph) * (size_t)G, cudaMemcpyHostToDevice, s)))
             return ACC_ERR_CUDA;
         c->rand_host = metas;
     }

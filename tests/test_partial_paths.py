@@ -64,6 +64,21 @@ template <class T> inline cudaError_t emu_set_limit(T kernel, cudaFuncAttribute,
     emu_limit_set((const void *)kernel, bytes);
     return cudaSuccess;
 }
+// deferred mode (EMU_DEFER=1): a copy from pageable memory and a set return before
+// they are done, and a stream of its own does not wait for the legacy stream
+inline cudaError_t emu_late_memcpy(void *d, const void *s, size_t n, cudaMemcpyKind kind) {
+    if (kind != cudaMemcpyHostToDevice || !emu_defer() || emu_is_pinned(s)) return cudaMemcpy(d, s, n, kind);
+    emu_flush(nullptr);
+    std::vector<char> staged((const char *)s, (const char *)s + n);
+    emu_submit(nullptr, [=] { memcpy(d, staged.data(), n); });
+    return cudaSuccess;
+}
+inline cudaError_t emu_late_memset(void *d, int v, size_t n) {
+    emu_submit(nullptr, [=] { memset(d, v, n); });
+    return cudaSuccess;
+}
+#define cudaMemcpy emu_late_memcpy
+#define cudaMemset emu_late_memset
 #define cudaSetDevice emu_set_device
 #define cudaGetDevice emu_get_device
 #define cudaFuncSetAttribute emu_set_limit
@@ -391,6 +406,36 @@ def host_reserved(lib):
     return [more, lib.emu_scan_count()]
 
 
+def host_own_stream(lib):
+    """Batches and randomised copies on a stream that does not wait for the legacy
+    one; edges of the last batch's graphs, as the statistics have them."""
+    import paper_1203_3415_gb300 as acc
+    from tests.emu.lib_scenarios import Ctx, NCLS, P, _descs, csr, ok
+    lib.emu_stream_create.restype = ctypes.c_void_p
+    s = ctypes.c_void_p(lib.emu_stream_create())
+    c = Ctx(lib)
+    for gs in ([fan(6, 4, 8, 1), fan(5, 3, 9, 2)], [fan(4, 4, 7, 3), fan(7, 2, 8, 4), fan(3, 3, 3, 5)]):
+        descs, keep = _descs(gs)
+        counts = np.full((len(gs), NCLS[4]), -1, np.int64)
+        ok(lib.acc_motif_batch_prepare(c.h, descs, len(gs), 4, s), "batch_prepare")
+        ok(lib.acc_motif_batch_run(c.h, s, P(counts), None), "batch_run")
+        for o, g in zip(counts, gs):
+            assert np.array_equal(o, oracle.count(*g, 4))
+        arrays = [csr(*g) for g in gs]
+        R, seeds, m = 2, np.arange(len(gs), dtype=np.uint64), sum(len(a[1]) for a in arrays)
+        out, accepted = np.zeros(R * m, np.int32), np.zeros(len(gs) * R, np.int64)
+        ok(lib.acc_swap_randomise(c.h, descs, len(gs), R, 2, P(seeds), acc.ACC_RAND_SWAP, s, P(out), P(accepted), None),
+           "swap_randomise")
+        want = [oracle.swap_randomise(g[0], *a, 2 * len(a[1]), i + r)[0] for i, (g, a) in enumerate(zip(gs, arrays))
+                for r in range(R)]
+        assert np.array_equal(out, np.concatenate(want))
+    stats = np.zeros(7, np.int64)
+    ok(lib.acc_motif_last_stats(c.h, P(stats)), "last_stats")
+    c.close()
+    pairs = [np.unique(np.minimum(g[1], g[2]) * g[0] + np.maximum(g[1], g[2])) for g in gs]
+    return [int(stats[3]), sum(len(p) for p in pairs)]
+
+
 def host_two_devices(lib):
     """The same counts on device 0, then on device 1: kernels whose limit of shared
     memory was raised on the first, and on both."""
@@ -528,6 +573,14 @@ def test_serving_allocates_nothing_after_the_reserve(on_host):
     """k = 5, a registered graph that is counted by partial patterns where the
     largest of both sizes would not be."""
     assert on_host("reserved") == [0, 0]
+
+
+RUNS["stream"] = ("own_stream", dict(EMU_DEFER=1))
+
+
+def test_host_tables_are_copied_on_the_stream_that_reads_them(on_host):
+    seen, edges = on_host("stream")
+    assert seen == edges
 
 
 if __name__ == "__main__":
