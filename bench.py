@@ -67,8 +67,9 @@ def ops_per_subgraph(k: int) -> int:
 # List scan: the entry's load and its test against the root (2 ops), its k-2
 # pair states to the prefix (4 ops each: address, load, shift, mask), then one
 # table load and one histogram increment: 4(k-2) + 4.  By partial patterns
-# (k = 4, 5 from 12288 arcs) the entry ends a wedge or a triangle: its load and
-# row lookup, one pair state, a hashed table slot and its counter, about as many.
+# (k = 4 from 12288 arcs, k = 5 from 8192) the entry ends a wedge or a triangle:
+# its load and row lookup, one pair state, a hashed table slot and its counter,
+# about as many.
 def ops_per_scanned_entry(k: int) -> int:
     return 4 * (k - 2) + 4
 
@@ -456,7 +457,7 @@ def measure_single(env, workload, steps, warmup, mode="count", schedule="", cpu_
     leaf_achieved = ops_per_subgraph(k) * n_k / enum_s / 1e9
     if eff == "count":
         units, per_unit = int(stats["scanned_entries"]), ops_per_scanned_entry(k)
-        unit_name = "neighbour entries the count's passes read"
+        unit_name = "neighbour entries the count's wedge and triangle passes or its list scan read"
     elif eff == "formula" and k == 3:
         units, per_unit = n_k, ops_per_subgraph(k)
         unit_name = "classified subgraphs (leaf-equivalent: the formula path visits none)"
@@ -695,7 +696,7 @@ def measure_batch(env, steps, warmup, cpu_baseline=True, cpu_budget_s=10.0):
         "batched_over_single": value / single_rate,
         "roofline": {"bound": "alu", "achieved": achieved, "peak": peak_gops, "unit": "Gop/s",
                      "frac": achieved / peak_gops, "traffic": None, "kernel": "the passes after the build (k = 4)",
-                     "work_unit": "neighbour entries the count's passes read", "units_per_launch": scanned,
+                     "work_unit": "neighbour entries the count's wedge and triangle passes or its list scan read", "units_per_launch": scanned,
                      "ops_per_unit": ops_per_scanned_entry(4), "peak_source": peak_src,
                      "enumerate_ms": statistics.mean(enum_ms)},
         "cpu_baseline": cpu,

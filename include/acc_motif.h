@@ -379,8 +379,9 @@ ACC_API int acc_motif_copy_table(acc_ctx *ctx, int k, int16_t *h_table);
  *   each enumeration launch, [6] neighbour entries the last two levels
  *   scanned (ACC_MODE_COUNT; 0 in ACC_MODE_ENUMERATE); where the count mode
  *   counts by partial patterns (see ACC_MODE_COUNT) [2] is the parts of the
- *   roots with many wedges and [6] the neighbour entries its wedge and
- *   triangle passes read.
+ *   roots with many wedges (of every pass) and [6] the neighbour entries its
+ *   wedge and triangle passes read (k = 5: not those of the 5-cycle and diamond
+ *   passes), with what a list scan that follows them reads.
  */
 #define ACC_STATS_LEN 7
 ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);

@@ -698,6 +698,7 @@ int run_set(acc_ctx *c, const GSet &gs, int max_n, int k, bool relabel, cudaStre
         c->state_clean = true;
     }
     c->last_launches = launches;
+    c->last_partial5 = partial5;
     c->last_k = k;
     c->last_units = gs.NV;
     c->last_blocks = enum_grid_warps(k, c->num_sms) / kWarpsPerBlock * c->grid_num / c->grid_den;
@@ -784,6 +785,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
                 if (ce == cudaSuccess && g && ok(cudaGraphInstantiate(&c->cg_exec, g, 0))) {
                     c->cg_key = key;
                     c->cg_launches = c->last_launches;
+                    c->cg_partial5 = c->last_partial5;
                     c->cg_units = c->last_units;
                     c->cg_blocks = c->last_blocks;
                     have = true;
@@ -798,6 +800,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
             if (!ok(cudaGraphLaunch(c->cg_exec, s))) return ACC_ERR_CUDA;
             if (!sparse) c->state_clean = true;  // the sequence ends with the clear
             c->last_launches = c->cg_launches;
+            c->last_partial5 = c->cg_partial5;
             c->last_k = k;
             c->last_units = c->cg_units;
             c->last_blocks = c->cg_blocks;
@@ -1246,6 +1249,11 @@ int acc_motif_last_stats(acc_ctx *c, int64_t *h_stats) {
     h_stats[0] = c->last_launches;
     h_stats[1] = c->last_k == 3 ? (int64_t)c->last_units : (int64_t)gi.nnz;
     h_stats[2] = (int64_t)gi.queue_tail;
+    if (c->last_partial5 && c->p5_sums) {
+        unsigned long long ctr[kCtrs];
+        if (!ok(cudaMemcpy(ctr, c->p5_sums + num_classes(5) + 16, sizeof(ctr), cudaMemcpyDeviceToHost))) return ACC_ERR_CUDA;
+        h_stats[2] += (int64_t)(ctr[kCtrPairTail] + ctr[kCtrTail4] + ctr[kCtrCycTail]);
+    }
     h_stats[3] = (int64_t)(gi.nnz / 2);
     h_stats[4] = gi.maxdeg;
     h_stats[5] = c->last_blocks;

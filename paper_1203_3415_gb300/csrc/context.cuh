@@ -125,6 +125,7 @@ struct acc_ctx {
         const void *ws[32];
     } cg_key = {}, cg_seen = {};  // the captured graph's key; the last key counted one by one
     int cg_launches = 0;
+    bool cg_partial5 = false;
     long long cg_units = 0;
     int cg_blocks = 0;
 
@@ -135,6 +136,7 @@ struct acc_ctx {
 
     // statistics of the last count
     int last_launches = 0;
+    bool last_partial5 = false;  // k = 5 by partial patterns: its queues have their own counters
     int last_k = 0;
     long long last_units = 0;
     int last_blocks = 0;

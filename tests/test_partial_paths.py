@@ -226,6 +226,18 @@ def host_k5_scans(lib):
     return lib.emu_scan_count()
 
 
+def host_k5_parts(lib):
+    """Parts of the roots with many wedges of a k = 5 graph, as the statistics have
+    them."""
+    from tests.emu.lib_scenarios import Ctx, P, ok
+    c = Ctx(lib)
+    stats = np.zeros(7, np.int64)
+    count_set(lib, c, [fan(13, 12, 20, 1)], 5)
+    ok(lib.acc_motif_last_stats(c.h, P(stats)), "last_stats")
+    c.close()
+    return int(stats[2])
+
+
 def host_k5_sparse(lib):
     """How often the list scan counted a uniform graph of 90 arcs on 80 vertices, and
     one of 400 arcs (k = 5)."""
@@ -581,6 +593,13 @@ RUNS["stream"] = ("own_stream", dict(EMU_DEFER=1))
 def test_host_tables_are_copied_on_the_stream_that_reads_them(on_host):
     seen, edges = on_host("stream")
     assert seen == edges
+
+
+RUNS["parts"] = ("k5_parts", {})
+
+
+def test_statistics_have_the_parts_of_every_pass(on_host):
+    assert on_host("parts") >= 1
 
 
 if __name__ == "__main__":
