@@ -833,17 +833,20 @@ long long ctx_footprint(acc_ctx *c, long long n, long long m, int k0, int k1, Wa
     // what the context holds already
     long long held = (long long)kQueueCap * 16, least = 0;
     workspace_buffers(c, [&](auto **p, size_t *cap) { held += (long long)(*cap * sizeof(**p)); });
-    // what would grow, by the buffer's capacity
-    std::vector<std::pair<const size_t *, long long>> growth;
+    // what would grow, by the buffer's capacity (workspace_needs names 25)
+    struct {
+        const size_t *cap;
+        long long more;
+    } growth[32] = {};
     auto grows = [&](const size_t *cap, size_t need, size_t bytes) {
         if (need <= *cap) return;
         const long long more = (long long)((need + need / 4 + 64 - *cap) * bytes);
         for (auto &g : growth)
-            if (g.first == cap) {
-                g.second = g.second > more ? g.second : more;
+            if (!g.cap || g.cap == cap) {
+                g.cap = cap;
+                g.more = g.more > more ? g.more : more;
                 return;
             }
-        growth.push_back({cap, more});
     };
     for (int k = k0; k <= k1; k++) {
         const long long warps = enum_grid_warps(k, c->num_sms) > 0 ? enum_grid_warps(k, c->num_sms) : 0;
@@ -866,7 +869,7 @@ long long ctx_footprint(acc_ctx *c, long long n, long long m, int k0, int k1, Wa
             grows(&c->scratch_cap, (size_t)lists, sizeof(*c->scratch));
     }
     c->partial_arcs_end = arcs_end;
-    for (const auto &g : growth) held += g.second;
+    for (const auto &g : growth) held += g.more;
     return held > least ? held : least;
 }
 
