@@ -17,6 +17,7 @@ import numpy as np
 import pytest
 
 import oracle
+from tests.graph_helpers import random_digraph
 from tests.test_partial import fan
 
 HERE = os.path.dirname(os.path.abspath(__file__))
@@ -134,6 +135,10 @@ EDITS = [
      "constexpr size_t cycle_smem(int phase);\ntemplate <int PHASE>\n__global__ void __launch_bounds__(kCThreads"),
     ("api.cu", "(arcs >= 2ll * n || arcs >= ACC_PARTIAL_MIN_ARCS1);",
      "(arcs >= 2ll * n || arcs >= (long long)emu_env(\"EMU_ARCS1\", ACC_PARTIAL_MIN_ARCS1));"),
+    ("api.cu", "q.tri_cap = c->scratch_cap / 4;", "q.tri_cap = emu_env(\"EMU_TRIANGLES\", c->scratch_cap / 4);"),
+    ("partial.cu", "return d > kFieldMax ?", "return d > (int)emu_env(\"EMU_FIELD\", kFieldMax) ?"),
+    ("partial.cu", "const bool wide = rows > kFieldMax;", "const bool wide = rows > (int)emu_env(\"EMU_FIELD\", kFieldMax);"),
+    ("partial5.cu", "lo < n && nr < kCRanges", "lo < n && nr < (int)emu_env(\"EMU_RANGES\", kCRanges)"),
     ("partial.cu", "- a.lo[v] > kCycleRows", "- a.lo[v] > (int)emu_env(\"EMU_ROWS\", kCycleRows)"),
     ("partial.cu", "    if (k == 3) launch_pdl(k_partial_prep<3>", "    emu_partials++;\n    if (k == 3) launch_pdl(k_partial_prep<3>"),
     ("partial5.cu", "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n    grid_dep_wait();\n",
@@ -162,7 +167,7 @@ def host_lib(tmp_path_factory):
             open(units[-1], "w").write('#include "hooks.h"\n' + _launches_to_calls(src))
     asan = subprocess.run(["g++", "-print-file-name=libasan.so"], capture_output=True, text=True).stdout.strip()
     san = ["-fsanitize=address", "-DEMU_EXACT_ALLOC", "-DEMU_LANE_STACK=65536"] if os.path.isabs(asan) else []
-    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0", "-DACC_QUEUE_CAP=1024ull", "-DACC_SPARSE_MIN_N=20000",
+    procs = [subprocess.Popen(["g++", "-std=c++20", "-O1", "-fPIC", "-pthread", "-w", *san, "-DACC_PARTIAL_MIN_ARCS=0", "-DACC_QUEUE_CAP=1024ull", "-DACC_SPARSE_MIN_N=20000", "-DACC_CYCLE_SLOTS=256",
                                "-DEMU_NUM_SMS=1", "-I", str(out), "-I", EMU, "-I", os.path.join(EMU, "fake"), "-I", CSRC,
                                "-c", u, "-o", str(out / f"u{i}.o")], stderr=subprocess.PIPE, text=True)
              for i, u in enumerate(units)]
@@ -222,6 +227,32 @@ def host_k5_scans(lib):
     from tests.emu.lib_scenarios import Ctx
     c = Ctx(lib)
     count_set(lib, c, [fan(13, 12, 20, 1)], 5)
+    c.close()
+    return lib.emu_scan_count()
+
+
+def host_returns(lib):
+    """How often the list scan counted: a k = 5 graph of many triangles, one with a
+    root of more wedges than a 5-cycle table takes."""
+    from tests.emu.lib_scenarios import Ctx
+    s, d = random_digraph(np.random.default_rng(9), 14, p=0.4, recip=0.5)
+    seen = []
+    for g in ((14, np.asarray(s, np.int64), np.asarray(d, np.int64)), fan(40, 6, 150, 1)):
+        c = Ctx(lib)
+        before = lib.emu_scan_count()
+        count_set(lib, c, [g], 5)
+        c.close()
+        seen.append(lib.emu_scan_count() - before)
+    return seen
+
+
+def host_wide(lib):
+    """Sets with roots of more rows than a table's 10-bit fields count (20 of them)."""
+    from tests.emu.lib_scenarios import Ctx
+    c = Ctx(lib)
+    count_set(lib, c, [fan(40, 20, 30, 2), fan(12, 12, 40, 3), fan(60, 30, 900, 3)], 4)
+    count_set(lib, c, [fan(40, 20, 30, 2)], 4)
+    count_set(lib, c, [fan(22, 9, 20, 1)], 5)
     c.close()
     return lib.emu_scan_count()
 
@@ -600,6 +631,48 @@ RUNS["parts"] = ("k5_parts", {})
 
 def test_statistics_have_the_parts_of_every_pass(on_host):
     assert on_host("parts") >= 1
+
+
+RUNS["returns", 0] = ("returns", {})
+RUNS["returns", 1] = ("returns", dict(EMU_TRIANGLES=5))
+RUNS["returns", 2] = ("returns", dict(EMU_RANGES=1))
+RUNS["wide"] = ("wide", dict(EMU_FIELD=20))
+
+
+@pytest.mark.parametrize("limit,scans", [(0, [0, 0]), (1, [1, 0]), (2, [0, 1])], ids=["none", "triangles", "ranges"])
+def test_full_lists_return_to_the_scan(on_host, limit, scans):
+    assert on_host(("returns", limit)) == scans
+
+
+def test_sets_with_wide_roots(on_host):
+    assert on_host("wide") == 0
+
+
+@pytest.mark.gpu
+def test_set_with_a_root_of_1100_rows():
+    """k = 3, 4, a set of graphs, one with a root of more rows than a table's 10-bit
+    fields count, against the enumerate mode."""
+    import torch
+    from paper_1203_3415_gb300 import build
+    build.build()
+    import paper_1203_3415_gb300 as acc
+    import synth
+    gs = [fan(1100, 3, 900, 1), fan(300, 6, 500, 2)]
+    small = synth.chung_lu(500, 2000, 2.2, 60, 10, 5)
+    gs.append((small.n, small.src, small.dst))
+    from tests.emu.lib_scenarios import csr
+    dev = [(torch.from_numpy(r).cuda(), torch.from_numpy(c).cuda(), g[0]) for g in gs for r, c in [csr(*g)]]
+    c = acc.Counter(0)
+    try:
+        for k in (3, 4):
+            got = {}
+            for mode in (acc.ACC_MODE_COUNT, acc.ACC_MODE_ENUMERATE):
+                c.set_mode(mode)
+                c.prepare_batch(dev, k)
+                got[mode] = c.run_batch().cpu().numpy().tolist()
+            assert got[acc.ACC_MODE_COUNT] == got[acc.ACC_MODE_ENUMERATE], k
+    finally:
+        c.close()
 
 
 if __name__ == "__main__":
