@@ -457,7 +457,8 @@ ACC_API int acc_ctx_set_mode(acc_ctx *ctx, int mode);
  *   lists are sized by the largest degree it finds) and is never replayed from
  *   a launch graph.
  *  ACC_ADJ_AUTO (default): sparse above ACC_MAX_N vertices, and from 98304 for
- *   one graph of k = 3, 4 counted by partial patterns; hashed when the
+ *   one graph of k = 3, 4 counted by partial patterns, of up to 20 (k = 3) or 10 (k
+ *   = 4) arcs a vertex; hashed when the
  *   largest graph of the count or batch has at least 49152 vertices for
  *   k = 5, 131072 for k = 3, 4 (where the dense probes, out of L2, get slower
  *   than the hashed ones); dense otherwise.

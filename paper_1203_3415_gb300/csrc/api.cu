@@ -313,12 +313,18 @@ bool uses_partial5(const acc_ctx *c, int k, int n, long long arcs, bool relabel,
 // (ACC_ADJ_AUTO).  Measured, dense / sparse, us: k = 3, 250000 arcs on 50000
 // vertices 221 / 235 with hubs, 164 / 152 uniform; 300000 on 100000 296 / 212 and
 // 218 / 155; k = 4, 260000 on 66000 361 / 381 and 229 / 202; 200000 on 100000 298 /
-// 248 and 205 / 162.
+// 248 and 205 / 162.  Up to kSparseArcs arcs a vertex, above which the rows' sort and
+// the hashed probes take longer than the block (98304 vertices, with hubs of up to
+// 500, 1000 and 2000, and uniform: 10 a vertex k = 3 604 / 489 and 499 / 306, k = 4
+// 1610 / 1670 and 860 / 702; 20 a vertex k = 3 1070 / 1097 and 848 / 667, k = 4 6647 /
+// 8955 and 2179 / 2036; 40 a vertex k = 3 2231 / 3007 and 1681 / 1468; 100 a vertex,
+// uniform, k = 3 4637 / 6290).
+constexpr long long kSparseArcs[5] = {0, 0, 0, 20, 10};
 #ifndef ACC_SPARSE_MIN_N
 #define ACC_SPARSE_MIN_N 98304
 #endif
 bool sparse_auto(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
-    return c->adjacency == ACC_ADJ_AUTO && B == 1 && max_n >= ACC_SPARSE_MIN_N &&
+    return c->adjacency == ACC_ADJ_AUTO && B == 1 && max_n >= ACC_SPARSE_MIN_N && k <= 4 && arcs <= kSparseArcs[k] * max_n &&
            uses_partial(c, k, max_n, arcs, relabel, B);
 }
 bool sparse_path(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {

@@ -390,6 +390,25 @@ def host_footprint(lib):
     return most
 
 
+def host_dense_block(lib):
+    """Whether the workspace of a graph of 20000 vertices and m arcs has the dense
+    block."""
+    from tests.emu.lib_scenarios import Ctx, ok
+    lib.emu_bytes.restype = ctypes.c_longlong
+    lib.emu_reserve.argtypes = [ctypes.c_void_p, ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int, ctypes.c_int]
+    tables = Ctx(lib)
+    ok(lib.acc_motif_prepare(tables.h, 5, None), "prepare")
+    seen = []
+    for k, m in ((3, 400000), (3, 400001), (4, 200000), (4, 200001)):
+        c = Ctx(lib)
+        before = lib.emu_bytes()
+        ok(lib.emu_reserve(c.h, 20000, m, k, 1), "reserve")
+        seen.append(lib.emu_bytes() - before > 20000 ** 2 // 4)
+        c.close()
+    tables.close()
+    return seen
+
+
 def host_server_budget(lib):
     """A server whose budget holds the list scan's workspace, not the pattern
     counters: the request's state, and whether patterns counted it."""
@@ -673,6 +692,14 @@ def test_set_with_a_root_of_1100_rows():
             assert got[acc.ACC_MODE_COUNT] == got[acc.ACC_MODE_ENUMERATE], k
     finally:
         c.close()
+
+
+RUNS["dense"] = ("dense_block", {})
+
+
+def test_sparse_build_up_to_its_arcs_a_vertex(on_host):
+    """(from 20000 vertices here)"""
+    assert on_host("dense") == [False, True, False, True]
 
 
 if __name__ == "__main__":
