@@ -269,7 +269,11 @@ bool uses_formula(const acc_ctx *c, int k, int max_n) {
 // of k = 4: the passes of a small graph take longer than its list scan
 // (scan / partial, us: k = 4, 8300 arcs on 4000 vertices 60 / 69 uniform, 73 / 82
 // with hubs; 12000 on 3000 65 / 67 and 117 / 104; 20000 on 5000 78 / 80 and 199 /
-// 119).
+// 119).  Only n and m are known here.  From 12288 to about 32000 arcs, graphs of 1 to
+// 3 arcs a vertex with light tails still lose (12600 on 12000 vertices, uniform 74 /
+// 83, degrees up to 25 76 / 92; 24000 on 12000, up to 25, 91 / 99), and those with hubs
+// gain more (up to 60 115 / 102; up to 100, 12400 on 6000, 126 / 98; up to 1000, 30000
+// on 20000, 260 / 148).
 #ifndef ACC_PARTIAL_MIN_ARCS
 #define ACC_PARTIAL_MIN_ARCS 8192
 #endif

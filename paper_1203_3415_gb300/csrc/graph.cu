@@ -736,10 +736,11 @@ __device__ __forceinline__ void flip_sort(uint32_t *x, int n, int t, int nt, Syn
 // neighbours of v, those below v.
 //
 // Rows of more than 32 entries: a warp each, sorted in its shared buffer (the
-// rows of one warp lie a grid apart: the longer rows come first).  Shorter rows: consecutive ones share a warp, an entry a lane, up to
-// 32 entries and 16 rows, sorted across the lanes by (row, entry).  With a warp
+// rows of one warp lie a grid apart: the longer rows come first).  Shorter rows:
+// consecutive ones share a warp, an entry a lane, up to 32 entries and 16 rows,
+// sorted across the lanes by (row, entry).  With a warp
 // per row all through, 10^6 vertices of 6 entries took 705 us, most lanes idle;
-// now 154.
+// now 100 (and 65 for the rows of over 128).
 constexpr int kPackRows = 16;  // rows that share a warp: 4 bits beside an entry's 28
 __global__ void __launch_bounds__(kSortWarps * kWarp) k_sp_sort_small(GSet gs, const long long *__restrict__ roff,
                                                                    const uint32_t *__restrict__ raw,

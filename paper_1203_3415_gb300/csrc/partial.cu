@@ -1,5 +1,5 @@
-// Counting by partial patterns (k = 3, 4): the count mode of sets of at least
-// kPartialMinArcs arcs whose vertices are renumbered by descending degree.
+// Counting by partial patterns (k = 3, 4): the count mode of the larger sets
+// (uses_partial) whose vertices are renumbered by descending degree.
 //
 // A partial pattern fixes the pair states of some pairs of a k-set (its
 // edges, which connect the set) and leaves the other pairs open.  With P(c)
@@ -64,6 +64,7 @@ __global__ void k_partial_prep(PartialArgs a) {
     const long long nnz = a.info->nnz;
     const int lane = threadIdx.x & 31;
     if (K == 5 && blockIdx.x == 0 && threadIdx.x == 0 && a.info->to_scan) a.p5.ctr[kCtrScan] = 1ull;
+    const bool hubs = K == 5 && a.info->maxdeg > kCycleRows;
     for (long long p0 = blockIdx.x * (long long)blockDim.x + threadIdx.x - lane; p0 < nnz;
          p0 += (long long)gridDim.x * blockDim.x) {
         const long long pos = p0 + lane;
@@ -84,7 +85,7 @@ __global__ void k_partial_prep(PartialArgs a) {
         // k = 5: a root with more rows than the 5-cycle tables count leaves the graph to
         // the scan.  Decided here, before the passes, so that they are not run for
         // nothing.
-        if (K == 5 && leader && a.deg[v] - a.lo[v] > kCycleRows) a.p5.ctr[kCtrScan] = 1ull;
+        if (K == 5 && hubs && leader && a.deg[v] - a.lo[v] > kCycleRows) a.p5.ctr[kCtrScan] = 1ull;
         if constexpr (K >= 4) {
             uint2 rv = make_uint2(0u, 0u);
             if (ok && (K == 5 || !(r >> 31))) {
@@ -185,7 +186,7 @@ struct Walker {
     // b < c, common neighbour x: word state(b, x), field state(c, x)), and the
     // 4-cliques v < u < w < x are found among the neighbours of w above w: the
     // triangles' lists as one flat sequence, kAhead entries a lane in flight
-    // (phase 2 of 20000 vertices, 1.5e4 triangles: 109 us; 190 us with a lane
+    // (phase 2 of 20000 vertices, 1.5e4 triangles: 85 us; 190 us with a lane
     // walking its own triangle's list, which waits for one entry at a time).
     __device__ __forceinline__ void triangles(int n) {
         constexpr int kAhead = 4;

@@ -139,6 +139,7 @@ EDITS = [
     ("partial.cu", "return d > kFieldMax ?", "return d > (int)emu_env(\"EMU_FIELD\", kFieldMax) ?"),
     ("partial.cu", "const bool wide = rows > kFieldMax;", "const bool wide = rows > (int)emu_env(\"EMU_FIELD\", kFieldMax);"),
     ("partial5.cu", "lo < n && nr < kCRanges", "lo < n && nr < (int)emu_env(\"EMU_RANGES\", kCRanges)"),
+    ("partial.cu", "a.info->maxdeg > kCycleRows", "a.info->maxdeg > (int)emu_env(\"EMU_ROWS\", kCycleRows)"),
     ("partial.cu", "- a.lo[v] > kCycleRows", "- a.lo[v] > (int)emu_env(\"EMU_ROWS\", kCycleRows)"),
     ("partial.cu", "    if (k == 3) launch_pdl(k_partial_prep<3>", "    emu_partials++;\n    if (k == 3) launch_pdl(k_partial_prep<3>"),
     ("partial5.cu", "__global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {\n    grid_dep_wait();\n",
