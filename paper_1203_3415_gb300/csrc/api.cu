@@ -433,7 +433,7 @@ void workspace_buffers(acc_ctx *c, Each each) {
 }
 
 int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
-                   bool either) {
+                   cudaStream_t s, bool either) {
     const int warps = enum_grid_warps(k, c->num_sms);
     if (warps < 0) return warps;
     int rc = ACC_OK;
@@ -447,8 +447,7 @@ int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, in
     if (rc) return rc;
     if (!c->info) {
         if (!ok(cudaMalloc(&c->info, sizeof(GraphInfo)))) return ACC_ERR_NOMEM;
-        // (a set returns before it is done; the caller's stream does not wait for it)
-        if (!ok(cudaMemset(c->info, 0, sizeof(GraphInfo))) || !ok(cudaStreamSynchronize(nullptr))) return ACC_ERR_CUDA;
+        if (!ok(cudaMemsetAsync(c->info, 0, sizeof(GraphInfo), s))) return ACC_ERR_CUDA;
     }
     if (!c->queue) {
         if (!ok(cudaMalloc(&c->queue, kQueueCap * sizeof(uint4)))) return ACC_ERR_NOMEM;
@@ -492,16 +491,16 @@ void free_partial(acc_ctx *c, bool sparse) {
 // the scan, as are the context's later sets of as many arcs (until the next
 // acc_motif_prepare or acc_motif_batch_prepare).
 int ensure_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
-                     bool either = false) {
+                     cudaStream_t s, bool either = false) {
     const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
-    const int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, either);
+    const int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, s, either);
     if (rc != ACC_ERR_NOMEM || t_alloc_in_capture ||
         !(either || uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B)))
         return rc;
     c->partial_arcs_end = arcs;
     const bool still = sparse_path(c, k, max_n, arcs, relabel, B);
     free_partial(c, sparse && !still);
-    return grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, either);
+    return grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, s, either);
 }
 
 // Build + enumerate one graph set into counts[B * num_classes(k)].
@@ -734,7 +733,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     int rc = uses_partial5(c, k, n, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
-    if ((rc = ensure_workspace(c, n, (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN))) return rc;
+    if ((rc = ensure_workspace(c, n, (long long)n * pitch, m, n, k, 1, n >= kRelabelMinN, s))) return rc;
     const bool sparse = sparse_path(c, k, n, m, n >= kRelabelMinN, 1);
     GSet gs = {};
     gs.one.rowptr = reinterpret_cast<const long long *>(rowptr);
@@ -826,10 +825,10 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
 // current mode and adjacency choice, which may differ from those at the
 // prepare (the count mode's reverse positions, hashed tables or sparse
 // build): grows nothing when they are the same.
-int batch_workspace(acc_ctx *c) {
+int batch_workspace(acc_ctx *c, cudaStream_t s) {
     if (size_check(c, c->batch_max_n)) return ACC_ERR_TOO_LARGE;
     return ensure_workspace(c, c->batch_set.NV, c->batch_words, c->batch_arcs, c->batch_max_n, c->batch_k,
-                            c->batch_set.B, true);
+                            c->batch_set.B, true, s);
 }
 
 }  // namespace
@@ -889,7 +888,7 @@ int ctx_reserve(acc_ctx *c, long long n, long long m, int k, Ways ways) {
     if (rc) return rc;
     const bool relabel = n >= kRelabelMinN;
     ctx_allow_partial(c, ways != Ways::kScan);
-    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, relabel, ways == Ways::kEither);
+    return ensure_workspace(c, n, n * state_pitch((int)n), m, (int)n, k, 1, relabel, c->own, ways == Ways::kEither);
 }
 
 }  // namespace acc
@@ -1066,7 +1065,7 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     int rc = k == 5 && B == 1 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     c->partial_arcs_end = INT64_MAX;
-    if ((rc = ensure_workspace(c, NV, words, arcs, max_n, k, B, true))) return rc;
+    if ((rc = ensure_workspace(c, NV, words, arcs, max_n, k, B, true, s))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;
     if ((rc = grow(&c->gid, &c->gid_cap, (size_t)NV + 1))) return rc;
     // (copies from pageable memory return when staged: on the stream that reads them,
@@ -1097,7 +1096,7 @@ int acc_motif_batch_run(acc_ctx *c, void *stream, int64_t *d_counts, int32_t *d_
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     if (c->batch_set.B == 0) return ACC_OK;
-    int rc = batch_workspace(c);
+    int rc = batch_workspace(c, s);
     if (rc) return rc;
     int *status = d_status ? d_status : c->status_dev;
     rc = run_set(c, c->batch_set, c->batch_max_n, c->batch_k, true, s, d_counts, status);
@@ -1337,7 +1336,7 @@ int acc_motif_batch_autotune(acc_ctx *c, void *stream, int64_t *h_light, int64_t
         best = 0.0f;
         goto done;
     }
-    if ((rc = batch_workspace(c))) return rc;
+    if ((rc = batch_workspace(c, s))) return rc;
     if (!ok(cudaMalloc(&counts, (size_t)B * num_classes(c->batch_k) * sizeof(int64_t)))) return ACC_ERR_NOMEM;
     if (!ok(cudaEventCreate(&e0)) || !ok(cudaEventCreate(&e1))) {
         rc = ACC_ERR_CUDA;
