@@ -404,8 +404,8 @@ ACC_API int acc_motif_last_stats(acc_ctx *ctx, int64_t *h_stats);
  *   from 8192 (below 12288: of at least two arcs a vertex); one graph of fewer
  *   than 1024 vertices is never counted so (outside a batch), nor are sets of many
  *   graphs of a few dozen arcs.  A k = 5 graph with a vertex of over
- *   1023 neighbours after it in degree order, with more triangles than the
- *   workspace lists, or with a count bound above 2^57 is left to the lists, and
+ *   1023 neighbours after it in degree order, with more triangles (or parts of its
+ *   5-cycle pass) than the workspace lists, or with a count bound above 2^57 is left to the lists, and
  *   one with few paths of three edges (sparse uniform graphs).  So
  *   is a set whose pattern counters (24 bytes a neighbour entry) find no device
  *   memory, with the context's later sets of as many arcs until the next
@@ -458,7 +458,7 @@ ACC_API int acc_ctx_set_mode(acc_ctx *ctx, int mode);
  *   a launch graph.
  *  ACC_ADJ_AUTO (default): sparse above ACC_MAX_N vertices, and from 98304 for
  *   one graph of k = 3, 4 counted by partial patterns, of up to 20 (k = 3) or 10 (k
- *   = 4) arcs a vertex; hashed when the
+ *   = 4) arcs a vertex or without device memory for the dense block; hashed when the
  *   largest graph of the count or batch has at least 49152 vertices for
  *   k = 5, 131072 for k = 3, 4 (where the dense probes, out of L2, get slower
  *   than the hashed ones); dense otherwise.

@@ -328,7 +328,8 @@ constexpr long long kSparseArcs[5] = {0, 0, 0, 20, 10};
 #define ACC_SPARSE_MIN_N 98304
 #endif
 bool sparse_auto(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
-    return c->adjacency == ACC_ADJ_AUTO && B == 1 && max_n >= ACC_SPARSE_MIN_N && k <= 4 && arcs <= kSparseArcs[k] * max_n &&
+    return c->adjacency == ACC_ADJ_AUTO && B == 1 && max_n >= ACC_SPARSE_MIN_N && k <= 4 &&
+           (c->sparse_any || arcs <= kSparseArcs[k] * max_n) &&
            uses_partial(c, k, max_n, arcs, relabel, B);
 }
 bool sparse_path(const acc_ctx *c, int k, int max_n, long long arcs, bool relabel, int B) {
@@ -460,13 +461,23 @@ int grow_workspace(acc_ctx *c, long long NV, long long words, long long arcs, in
     return ACC_OK;
 }
 
-// Gives back what only partial patterns need (a free waits for the device).
+template <typename T>
+void drop(T **p, size_t *cap) {  // (a free waits for the device)
+    cudaFree(*p);
+    *p = nullptr;
+    *cap = 0;
+}
+
+// The launch graph may hold the addresses of buffers that are given back.
+void drop_launch_graph(acc_ctx *c) {
+    if (c->cg_exec) cudaGraphExecDestroy(c->cg_exec);
+    c->cg_exec = nullptr;
+    memset(&c->cg_seen, 0, sizeof(c->cg_seen));
+}
+
+// Gives back what only partial patterns need, with the sparse build's buffers.
 void free_partial(acc_ctx *c, bool sparse) {
-    auto drop = [](auto **p, size_t *cap) {
-        cudaFree(*p);
-        *p = nullptr;
-        *cap = 0;
-    };
+    drop_launch_graph(c);
     drop(&c->pp_nd, &c->pp_nd_cap);
     drop(&c->pp_part, &c->pp_part_cap);
     drop(&c->pp_done, &c->pp_done_cap);
@@ -474,9 +485,6 @@ void free_partial(acc_ctx *c, bool sparse) {
     drop(&c->pp_tri, &c->pp_tri_cap);
     drop(&c->p5_vert, &c->p5_vert_cap);
     drop(&c->p5_sums, &c->p5_sums_cap);
-    if (c->cg_exec) cudaGraphExecDestroy(c->cg_exec);  // (it may hold their addresses)
-    c->cg_exec = nullptr;
-    memset(&c->cg_seen, 0, sizeof(c->cg_seen));
     if (!sparse) return;
     drop(&c->nh, &c->nh_cap);
     drop(&c->sp_raw, &c->sp_raw_cap);
@@ -486,20 +494,34 @@ void free_partial(acc_ctx *c, bool sparse) {
 }
 
 // The workspace of a set whose dense block has `words` words (see
-// grow_workspace).  Partial patterns take 24 bytes a neighbour entry more than the
-// list scan, and 40 more where sparse_auto takes the sparse build: where the device has no room for them the set is counted by
-// the scan, as are the context's later sets of as many arcs (until the next
-// acc_motif_prepare or acc_motif_batch_prepare).
+// grow_workspace).  Where the device has no room for the way that the rules choose,
+// another one is taken, for the context's later sets too (until the next
+// acc_motif_prepare or acc_motif_batch_prepare): the sparse build for a graph
+// that sparse_auto leaves to the dense block for its density, then the list scan for
+// sets of as many arcs (partial patterns take 24 bytes a neighbour entry more, and
+// the sparse build 40 more).
 int ensure_workspace(acc_ctx *c, long long NV, long long words, long long arcs, int max_n, int k, int B, bool relabel,
                      cudaStream_t s, bool either = false) {
-    const bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
-    const int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, s, either);
-    if (rc != ACC_ERR_NOMEM || t_alloc_in_capture ||
-        !(either || uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B)))
-        return rc;
+    int rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, s, either);
+    if (rc != ACC_ERR_NOMEM || t_alloc_in_capture) return rc;
+    bool sparse = sparse_path(c, k, max_n, arcs, relabel, B);
+    if (!sparse && !c->sparse_any) {
+        c->sparse_any = true;
+        if (sparse_path(c, k, max_n, arcs, relabel, B)) {
+            drop_launch_graph(c);
+            drop(&c->state, &c->state_cap);
+            drop(&c->occ, &c->occ_cap);
+            c->state_clean = false;
+            rc = grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, s, either);
+            if (rc != ACC_ERR_NOMEM) return rc;
+            sparse = true;
+        } else {
+            c->sparse_any = false;
+        }
+    }
+    if (!(either || uses_partial(c, k, max_n, arcs, relabel, B) || uses_partial5(c, k, max_n, arcs, relabel, B))) return rc;
     c->partial_arcs_end = arcs;
-    const bool still = sparse_path(c, k, max_n, arcs, relabel, B);
-    free_partial(c, sparse && !still);
+    free_partial(c, sparse && !sparse_path(c, k, max_n, arcs, relabel, B));
     return grow_workspace(c, NV, words, arcs, max_n, k, B, relabel, s, either);
 }
 
@@ -764,6 +786,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
         key.light = c->sched_light;
         key.target = c->sched_target;
         key.partial_end = c->partial_arcs_end;
+        key.sparse_any = c->sparse_any;
         key.n = n;
         key.k = k;
         key.mode = c->mode;
@@ -990,6 +1013,7 @@ int acc_motif_prepare(acc_ctx *c, int k, void *stream) {
     if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     c->partial_arcs_end = INT64_MAX;
+    c->sparse_any = false;
     int rc = k == 5 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     return ok(cudaStreamSynchronize(s)) ? ACC_OK : ACC_ERR_CUDA;
@@ -1065,6 +1089,7 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
     int rc = k == 5 && B == 1 ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     c->partial_arcs_end = INT64_MAX;
+    c->sparse_any = false;
     if ((rc = ensure_workspace(c, NV, words, arcs, max_n, k, B, true, s))) return rc;
     if ((rc = grow(&c->meta_dev, &c->meta_cap, (size_t)B + 1))) return rc;
     if ((rc = grow(&c->gid, &c->gid_cap, (size_t)NV + 1))) return rc;

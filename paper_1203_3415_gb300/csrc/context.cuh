@@ -76,6 +76,9 @@ struct acc_ctx {
     // sets of at least this many arcs are counted by the list scan: the device had
     // no memory for the counters of one
     long long partial_arcs_end = INT64_MAX;
+    // the sparse build at any density (sparse_auto): there was no memory for the
+    // dense block of such a graph
+    bool sparse_any = false;
     int mode = 0;             // ACC_MODE_COUNT, _ENUMERATE, _FORMULA or _AUTO
     long long sched_light = 0;   // enumeration schedule (0: the kernels' default)
     long long sched_target = 0;
@@ -121,7 +124,7 @@ struct acc_ctx {
     struct CountKey {
         const void *rowptr, *col, *counts, *status;
         long long m, light, target, partial_end;
-        int n, k, mode, grid_num, grid_den, adjacency;
+        int n, k, mode, grid_num, grid_den, adjacency, sparse_any;
         const void *ws[32];
     } cg_key = {}, cg_seen = {};  // the captured graph's key; the last key counted one by one
     int cg_launches = 0;

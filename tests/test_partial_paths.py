@@ -406,6 +406,15 @@ def host_dense_block(lib):
         ok(lib.emu_reserve(c.h, 20000, m, k, 1), "reserve")
         seen.append(lib.emu_bytes() - before > 20000 ** 2 // 4)
         c.close()
+    # no memory for the block: the sparse build after all
+    lib.emu_limit.argtypes = [ctypes.c_ulonglong]
+    c = Ctx(lib)
+    before = lib.emu_bytes()
+    lib.emu_limit(before + 20000 ** 2 // 4)
+    ok(lib.emu_reserve(c.h, 20000, 200001, 4, 1), "reserve")
+    lib.emu_limit(1 << 63)
+    seen.append(lib.emu_bytes() - before > 20000 ** 2 // 4)
+    c.close()
     tables.close()
     return seen
 
@@ -700,7 +709,7 @@ RUNS["dense"] = ("dense_block", {})
 
 def test_sparse_build_up_to_its_arcs_a_vertex(on_host):
     """(from 20000 vertices here)"""
-    assert on_host("dense") == [False, True, False, True]
+    assert on_host("dense") == [False, True, False, True, False]
 
 
 if __name__ == "__main__":
