@@ -751,7 +751,7 @@ int count_impl(acc_ctx *c, const int64_t *rowptr, const int32_t *col, int32_t n,
     if (!valid_k(k)) return ACC_ERR_K;
     if (n < 0 || m < 0 || m >= (1ll << 31)) return ACC_ERR_INPUT;
     if (size_check(c, n)) return ACC_ERR_TOO_LARGE;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     int rc = uses_partial5(c, k, n, m, n >= kRelabelMinN, 1) ? ensure_tab5(c, s) : ensure_lut(c, k, s);
     if (rc) return rc;
     const long long pitch = state_pitch(n);
@@ -906,7 +906,7 @@ long long ctx_footprint(acc_ctx *c, long long n, long long m, int k0, int k1, Wa
 }
 
 int ctx_reserve(acc_ctx *c, long long n, long long m, int k, Ways ways) {
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     const int rc = ensure_tab5(c, c->own);
     if (rc) return rc;
     const bool relabel = n >= kRelabelMinN;
@@ -942,7 +942,7 @@ int acc_ctx_create(acc_ctx **out, int device) {
     acc_ctx *c = new (std::nothrow) acc_ctx();
     if (!c) return ACC_ERR_NOMEM;
     c->device = device;
-    if (!ok(cudaSetDevice(device)) ||
+    if (!set_device(device) ||
         !ok(cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device)) ||
         !ok(cudaStreamCreateWithFlags(&c->own, cudaStreamNonBlocking)) ||
         !ok(cudaMallocHost(&c->status_host, sizeof(int)))) {
@@ -1010,7 +1010,7 @@ void acc_ctx_destroy(acc_ctx *c) {
 int acc_motif_prepare(acc_ctx *c, int k, void *stream) {
     if (!c) return ACC_ERR_ARG;
     if (!valid_k(k)) return ACC_ERR_K;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     c->partial_arcs_end = INT64_MAX;
     c->sparse_any = false;
@@ -1030,7 +1030,7 @@ int acc_motif_count_host(acc_ctx *c, const int64_t *h_rowptr, const int32_t *h_c
     if (!valid_k(k)) return ACC_ERR_K;
     if (n < 0 || m < 0 || m >= (1ll << 31)) return ACC_ERR_INPUT;
     if (size_check(c, n)) return ACC_ERR_TOO_LARGE;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     int rc;
     size_t cnt_cap = c->h2d_counts ? 9364 : 0;
     if ((rc = grow(&c->h2d_rowptr, &c->h2d_rowptr_cap, (size_t)n + 1))) return rc;
@@ -1055,7 +1055,7 @@ int acc_motif_count_host(acc_ctx *c, const int64_t *h_rowptr, const int32_t *h_c
 int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B, int k, void *stream) {
     if (!c || (B > 0 && !graphs) || B < 0) return ACC_ERR_ARG;
     if (!valid_k(k)) return ACC_ERR_K;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     c->batch_ready = false;
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<GMeta> metas((size_t)B);
@@ -1118,7 +1118,7 @@ int acc_motif_batch_prepare(acc_ctx *c, const acc_graph_desc *graphs, int32_t B,
 
 int acc_motif_batch_run(acc_ctx *c, void *stream, int64_t *d_counts, int32_t *d_status) {
     if (!c || !d_counts || !c->batch_ready) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     if (c->batch_set.B == 0) return ACC_OK;
     int rc = batch_workspace(c, s);
@@ -1152,7 +1152,7 @@ int acc_swap_randomise(acc_ctx *c, const acc_graph_desc *graphs, int32_t G, int3
     if (!c || G < 0 || R < 0 || attempts_per_arc < 0) return ACC_ERR_ARG;
     if (mode != ACC_RAND_SWAP && mode != ACC_RAND_MUTUAL) return ACC_ERR_ARG;
     if (G > 0 && (!graphs || !seeds)) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     std::vector<RGraph> metas((size_t)G);
     long long M = 0, NV = 0, bwords = 0;
@@ -1249,7 +1249,7 @@ int acc_motif_class_code(acc_ctx *c, int k, int32_t cls, uint32_t *code) {
     if (!c || !code) return ACC_ERR_ARG;
     if (!valid_k(k)) return ACC_ERR_K;
     if (cls < 0 || cls >= num_classes(k)) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     int rc = ensure_lut(c, k, c->own);
     if (rc) return rc;
     *code = c->class_code_host[k][cls];
@@ -1260,7 +1260,7 @@ int acc_motif_classify_code(acc_ctx *c, int k, uint32_t code, int32_t *cls) {
     if (!c || !cls) return ACC_ERR_ARG;
     if (!valid_k(k)) return ACC_ERR_K;
     if (code >= (1u << code_bits(k))) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     int rc = ensure_lut(c, k, c->own);
     if (rc) return rc;
     *cls = c->lut_host[k][code];
@@ -1270,7 +1270,7 @@ int acc_motif_classify_code(acc_ctx *c, int k, uint32_t code, int32_t *cls) {
 int acc_motif_copy_table(acc_ctx *c, int k, int16_t *h_table) {
     if (!c || !h_table) return ACC_ERR_ARG;
     if (!valid_k(k)) return ACC_ERR_K;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     int rc = ensure_lut(c, k, c->own);
     if (rc) return rc;
     memcpy(h_table, c->lut_host[k], (size_t(1) << code_bits(k)) * 2);
@@ -1280,7 +1280,7 @@ int acc_motif_copy_table(acc_ctx *c, int k, int16_t *h_table) {
 int acc_motif_last_stats(acc_ctx *c, int64_t *h_stats) {
     if (!c || !h_stats) return ACC_ERR_ARG;
     if (!c->info) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device)) || !ok(cudaDeviceSynchronize())) return ACC_ERR_CUDA;
+    if (!set_device(c->device) || !ok(cudaDeviceSynchronize())) return ACC_ERR_CUDA;
     GraphInfo gi;
     if (!ok(cudaMemcpy(&gi, c->info, sizeof(gi), cudaMemcpyDeviceToHost))) return ACC_ERR_CUDA;
     h_stats[0] = c->last_launches;
@@ -1331,7 +1331,7 @@ int acc_ctx_get_schedule(acc_ctx *c, int64_t *light, int64_t *target) {
 
 int acc_motif_batch_autotune(acc_ctx *c, void *stream, int64_t *h_light, int64_t *h_target, float *h_ms) {
     if (!c || !c->batch_ready) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     const long long B = c->batch_set.B;
     const long long light0 = c->sched_light, target0 = c->sched_target;
@@ -1422,7 +1422,7 @@ done:
 
 int acc_ctx_set_timing(acc_ctx *c, int on) {
     if (!c) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device))) return ACC_ERR_CUDA;
+    if (!set_device(c->device)) return ACC_ERR_CUDA;
     if (on && !c->ev[0]) {
         for (int i = 0; i < 4; i++)
             if (!ok(cudaEventCreate(&c->ev[i]))) {
@@ -1436,7 +1436,7 @@ int acc_ctx_set_timing(acc_ctx *c, int on) {
 
 int acc_motif_last_timing(acc_ctx *c, float *h_ms) {
     if (!c || !h_ms || !c->timed_call) return ACC_ERR_ARG;
-    if (!ok(cudaSetDevice(c->device)) || !ok(cudaEventSynchronize(c->ev[2]))) return ACC_ERR_CUDA;
+    if (!set_device(c->device) || !ok(cudaEventSynchronize(c->ev[2]))) return ACC_ERR_CUDA;
     if (!ok(cudaEventElapsedTime(&h_ms[0], c->ev[0], c->ev[1])) ||
         !ok(cudaEventElapsedTime(&h_ms[1], c->ev[1], c->ev[2])) ||
         !ok(cudaEventElapsedTime(&h_ms[2], c->ev[1], c->ev[3])) ||

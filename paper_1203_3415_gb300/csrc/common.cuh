@@ -277,11 +277,20 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+// The device that the library made current on this thread for the call under way
+// (-1: not known), so that the launchers need not ask the runtime.
+inline thread_local int t_device = -1;
+inline bool set_device(int device) {
+    if (cudaSetDevice(device) != cudaSuccess) return false;
+    t_device = device;
+    return true;
+}
 // What is set up once on each device, by its bit (0 from 64 devices on: always
 // again).
 inline unsigned long long device_bit() {
-    int device = 0;
-    return cudaGetDevice(&device) == cudaSuccess && device >= 0 && device < 64 ? 1ull << device : 0ull;
+    int device = t_device;
+    if (device < 0 && cudaGetDevice(&device) != cudaSuccess) return 0ull;
+    return device >= 0 && device < 64 ? 1ull << device : 0ull;
 }
 // Raises a kernel's limit of dynamic shared memory to `bytes`, which the current
 // device keeps for itself; `done`: the devices that have it.
