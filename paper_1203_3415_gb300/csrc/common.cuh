@@ -108,8 +108,8 @@ __host__ __device__ inline double count_bound(int k, int max_n, int maxdeg, cons
 // degree, 175 / 188; 21000 on 12000, 20 n, 211 / 218; 28000 on 20000, 2.1e5, 165 / 227;
 // 30000 on 20000, 2.5e5, 245 / 227; 39000 on 30000, 2.5e5, 212 / 253; 48000 on 40000,
 // 2.6e5, 275 / 262).  Graphs with hubs lie above it (12600 arcs on 12000 vertices,
-// degrees up to 8, 24 n, 275 / 211).  A graph left to the scan pays about 16 us beside
-// it, the launches of the passes that leave at once (104 -> 121).
+// degrees up to 8, 24 n, 275 / 211).  A graph left to the scan pays 15 to 20 us beside
+// it, the launches of the passes that leave at once (105 -> 122).
 __host__ __device__ inline bool left_to_scan(double bound, int n, const float *s) {
     return bound > kCountLimit / 32 || s[1] < fminf(15.0f * (float)n, 2.2e5f);
 }

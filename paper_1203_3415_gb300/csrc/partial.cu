@@ -644,7 +644,8 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : (SLOTS == kSetSlots &&
     uint32_t *root_wedges = K == 5 ? a.p5.pair_wedges : a.wedges;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     if (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW) return;
-    if ((K == 5 || BESIDE) && scan_instead(a)) return;
+    __shared__ int instead;
+    if (K == 5 || BESIDE) ask_scan(a, &instead);
     if (PHASE == 2 && *qtail == 0) return;
     uint4 *tabs = reinterpret_cast<uint4 *>(smem);
     Walker<K, HASH> wk;
@@ -670,6 +671,7 @@ __global__ void __launch_bounds__(kPThreads, K == 5 ? 3 : (SLOTS == kSetSlots &&
     else
         for (int i = lane; i < 2 * N; i += kWarp) wk.hist[i] = 0u;
     __syncthreads();
+    if ((K == 5 || BESIDE) && instead) return;
     // first row of root v (k = 4: of the vertices above it)
     auto first_row = [&](uint32_t v) -> long long { return wk.g.nptr[v] + (K == 5 ? 0 : wk.g.lo[v]); };
     // parts of a root with W wedges and d rows

@@ -224,15 +224,21 @@ __device__ __forceinline__ EdgeTri edge_tri(const PartialArgs &a, long long p, b
 }
 
 // k = 5: whether the list scan counts the set instead (or the build refused it).
-// One answer for the whole block, which every thread must ask for before any
-// other barrier: the flag may be raised while a kernel's blocks start, by the
-// kernel itself or one beside it, and a warp that left while others of its block
-// stayed would leave its share of the tables uncleared.
+__device__ __forceinline__ bool scan_flag(const PartialArgs &a) {
+    return *(volatile unsigned long long *)(a.p5.ctr + kCtrScan) != 0ull ||
+           (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW);
+}
+// One answer for the whole block: thread 0 asks, and every thread reads it after the
+// kernel's first barrier, before any other thread of the block may have left.  The
+// flag may be raised while a kernel's blocks start, by the kernel itself or one beside
+// it, and a warp that left while others of its block stayed would leave its share of
+// the tables uncleared.  (The answer is on its way while the tables are cleared.)
+__device__ __forceinline__ void ask_scan(const PartialArgs &a, int *instead) {
+    if (threadIdx.x == 0) *instead = scan_flag(a);
+}
 __device__ __forceinline__ bool scan_instead(const PartialArgs &a) {
     __shared__ int instead;
-    if (threadIdx.x == 0)
-        instead = *(volatile unsigned long long *)(a.p5.ctr + kCtrScan) != 0ull ||
-                  (a.status && *(volatile int *)a.status == ACC_ERR_OVERFLOW);
+    ask_scan(a, &instead);
     __syncthreads();
     return instead != 0;
 }

@@ -355,12 +355,14 @@ __device__ void corner_sums(const PartialArgs &a, const PView &g, const Bins5 &b
 
 __global__ void __launch_bounds__(256) k_closed5(PartialArgs a) {
     const JoinsPrevious beside;  // k_wedges<5, 2>
-    if (scan_instead(a)) return;
     const unsigned long long tris = a.p5.ctr[kCtrTris];
     if (!tris) return;
+    __shared__ int instead;
+    ask_scan(a, &instead);
     extern __shared__ __align__(16) unsigned char smem[];
     const Bins5 bins = bins5(a, reinterpret_cast<uint32_t *>(smem));
     bins.clear();
+    if (instead) return;
     const PView g = view5(a);
     // (thread t of block b takes item t gridDim + b: few items still reach every SM)
     const long long t0 = threadIdx.x * (long long)gridDim.x + blockIdx.x, step = (long long)gridDim.x * blockDim.x;
@@ -383,12 +385,14 @@ __global__ void __launch_bounds__(256) k_closed5(PartialArgs a) {
 template <bool HASH>
 __global__ void __launch_bounds__(256, 2) k_diamonds5(PartialArgs a) {
     const JoinsPrevious beside;  // k_wedges<5, 2>
-    if (scan_instead(a)) return;
     const unsigned long long units = 3ull * a.p5.ctr[kCtrTris];
     if (!units) return;
+    __shared__ int instead;
+    ask_scan(a, &instead);
     extern __shared__ __align__(16) unsigned char smem[];
     const Bins5 bins = bins5(a, reinterpret_cast<uint32_t *>(smem));
     bins.clear();
+    if (instead) return;
     const PView g = view5(a);
     const int lane = threadIdx.x & 31;
     for (;;) {
@@ -672,7 +676,8 @@ template <int PHASE>
 __global__ void __launch_bounds__(kCThreads, PHASE == 1 ? 3 : 2) k_cycles5(PartialArgs a) {
     grid_dep_wait();
     grid_dep_launch();  // k_wedges<4, PHASE> runs beside
-    if (scan_instead(a)) return;
+    __shared__ int instead;
+    ask_scan(a, &instead);
     unsigned long long *ctr = a.p5.ctr;
     // (the second half of the queue: k_wedges<4> has the first)
     const unsigned long long cap = a.queue_cap / 2;
@@ -694,6 +699,7 @@ __global__ void __launch_bounds__(kCThreads, PHASE == 1 ? 3 : 2) k_cycles5(Parti
     cw.tab = CycleTable{PHASE == 1 ? table + 4 * kLSlots * wib : table, (uint32_t)kLSlots};
     for (int i = threadIdx.x; i < 4 * kTable; i += kCThreads) table[i] = 0u;
     cw.bins.clear();
+    if (instead) return;  // (after the clear's barrier)
     const PView &g = cw.g;
     if constexpr (PHASE == 1) {
         const long long warps = 4ll * gridDim.x * kCWarps;  // (grabs as in k_wedges)
@@ -870,7 +876,7 @@ __device__ __forceinline__ uint32_t partition_of(int i) {
 // partitions decoded by a loop).
 __global__ void k_quotients(PartialArgs a) {
     grid_dep_wait();
-    if (scan_instead(a)) return;
+    if (scan_flag(a)) return;  // (no pass that may raise it is left, and no barrier follows)
     // the scan's kernels, launched next, find no unit left
     if (blockIdx.x == 0 && threadIdx.x == 0) a.info->unit_ctr = 1ull << 62;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kSigma * kParts; i += gridDim.x * blockDim.x) {
@@ -951,11 +957,13 @@ __global__ void k_quotients(PartialArgs a) {
 // vertices.  Warp per class, a lane a subset: 12 to 30 us by the classes present.
 __global__ void __launch_bounds__(256) k_counts5(PartialArgs a) {
     grid_dep_wait();
-    if (scan_instead(a)) return;
+    __shared__ int instead;
+    ask_scan(a, &instead);
     extern __shared__ __align__(16) unsigned char smem[];
     Bins5 bins = bins5(a, reinterpret_cast<uint32_t *>(smem));
     bins.sums = a.counts;
     bins.clear();
+    if (instead) return;
     const int warp = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), warps = (int)((gridDim.x * blockDim.x) >> 5),
               lane = threadIdx.x & 31;
     for (int c = warp; c < kN5; c += warps) {
